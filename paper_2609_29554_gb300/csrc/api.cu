@@ -115,8 +115,7 @@ void Workspace::release() {
     cap = 0;
 }
 
-int plan_for(ozlu_handle* h, int p, int K, const ozlu_opts* o, const Plan** out,
-             const DevTable** tab) {
+int plan_for(ozlu_handle* h, int p, int K, const ozlu_opts* o, const PlanEntry** out) {
     ozlu_opts d;
     memset(&d, 0, sizeof d);
     if (!o) o = &d;
@@ -127,10 +126,10 @@ int plan_for(ozlu_handle* h, int p, int K, const ozlu_opts* o, const Plan** out,
         int rc = make_plan(p, K, o, e.plan);
         if (rc) return rc;
         fill_table(e.plan, e.table);
+        if (e.plan.backend != OZLU_BE_FP64) fill_conv(e.table, e.conv);
         it = h->plans.emplace(key, e).first;
     }
-    *out = &it->second.plan;
-    *tab = &it->second.table;
+    *out = &it->second;
     return OZLU_OK;
 }
 
@@ -287,16 +286,19 @@ int gemm_device(ozlu_handle* h, int nc, int p, int m, int n, int k, int alpha, c
         if (rc0) return rc0;
         if (o.nslice == 0) o.nslice = S;
     }
-    const Plan* pl;
-    const DevTable* tab;
-    int rc = plan_for(h, p, k, &o, &pl, &tab);
+    const PlanEntry* pe;
+    int rc = plan_for(h, p, k, &o, &pe);
     if (rc) return rc;
+    const Plan* pl = &pe->plan;
+    const DevTable* tab = &pe->table;
     const int be = pl->backend;
     const int mode = be == OZLU_BE_INT8 ? 0 : be == OZLU_BE_FP8 ? 1 : be == OZLU_BE_FP16 ? 2 : 3;
     const int P = mode == 1 ? 3 : 1, esz = mode == 2 ? 2 : (mode == 3 ? 8 : 1);
     const int tsz = mode == 3 ? 4 : 1;  // bytes per t value
     const int Mpad = (m + 127) / 128 * 128, Npad = (n + 127) / 128 * 128;
-    const int Kpad = pl->Kpad;
+    // K padded to the GEMM's step: 64 elements (INT8, FP16; the binary64 kernel
+    // takes any), 128 for FP8 (the accumulator conditions hold for the plan's 128)
+    const int Kpad = mode == 1 ? pl->Kpad : (k + 63) / 64 * 64;
     GemmLayout& L = h->last;
     L.m = m; L.n = n; L.k = k; L.Mpad = Mpad; L.Npad = Npad; L.Kpad = Kpad;
     L.N = pl->N; L.S = pl->S; L.G = pl->G; L.backend = be;
@@ -318,14 +320,13 @@ int gemm_device(ozlu_handle* h, int nc, int p, int m, int n, int k, int alpha, c
     uint8_t* T = (uint8_t*)(base + L.t);
     const int prev = h->open_phase;
     h->phase(PH_CONVERT);
-    // B's exponents and residues on the side stream, beside A's (disjoint
-    // workspace regions)
-    cudaStream_t sb = side_fork(h, s);
-    launch_col_shifts(B, ldb, nc, k, n, pl->Q, nu, sb);
-    launch_convert(B, ldb, nc, k, n, true, nu, *tab, Kpad, Npad, RB, mode, sb);
-    launch_row_shifts(A, lda, nc, m, k, pl->Q, mu, s);
-    launch_convert(A, lda, nc, m, k, false, mu, *tab, Kpad, Mpad, RA, mode, s);
-    if (!side_join(h, s, sb)) return OZLU_ERR_CUDA;
+    launch_shifts(A, lda, m, B, ldb, n, nc, k, pl->Q, mu, nu, nullptr, s);
+    if (mode == 3) {
+        launch_convert64(A, lda, nc, m, k, false, mu, *tab, Kpad, Mpad, (double*)RA, s);
+        launch_convert64(B, ldb, nc, k, n, true, nu, *tab, Kpad, Npad, (double*)RB, s);
+    } else {
+        launch_convert(A, lda, m, B, ldb, n, nc, k, mu, nu, pe->conv, Kpad, Mpad, Npad, RA, RB, mode, s);
+    }
     h->phase(PH_GEMM);
     if (mode == 0) {
         launch_gemm_imma((const int8_t*)RA, (const int8_t*)RB, m, n, Mpad, Npad, Kpad, *tab, T, s);
@@ -346,7 +347,7 @@ int gemm_device(ozlu_handle* h, int nc, int p, int m, int n, int k, int alpha, c
     h->stats.crt_bytes += (double)pl->G * pl->N * m * n + 8.0 * nc * m * n * (beta ? 2 : 1);
     h->stats.convert_bytes += 8.0 * nc * ((double)m * k + (double)k * n) +
                               (double)pl->N * pl->S * ((double)Mpad + Npad) * Kpad;
-    h->count(6);
+    h->count(mode == 3 ? 5 : 4);
     if (cudaGetLastError() != cudaSuccess) return OZLU_ERR_CUDA;
     return OZLU_OK;
 }

@@ -33,6 +33,7 @@
 #include <mutex>
 
 #include "ozlu_internal.h"
+#include "tables.h"
 
 namespace ozlu {
 namespace {
@@ -106,6 +107,8 @@ extern "C" int ozlu_gemm_noalloc(int nc, int p, int m, int n, int k, int alpha, 
     int Kpad = 0;
     int rc = plan_noalloc(p, k, tab, Kpad);
     if (rc) return rc;
+    ConvTab conv;
+    fill_conv(tab, conv);
     const int Mpad = (m + 127) / 128 * 128, Npad = (n + 127) / 128 * 128;
     size_t off = 0;
     const size_t o_mu = off; off = up256(off + sizeof(int) * (size_t)m);
@@ -114,6 +117,7 @@ extern "C" int ozlu_gemm_noalloc(int nc, int p, int m, int n, int k, int alpha, 
     const size_t o_rb = off; off = up256(off + (size_t)tab.N * tab.S * Npad * Kpad);
     const size_t o_t = off;  off = up256(off + (size_t)tab.G * tab.N * m * n);
     if (off > NOALLOC_SCRATCH_BYTES) return OZLU_ERR_CAPACITY;  // problem too large for the array
+    Kpad = (k + 63) / 64 * 64;  // the GEMM's K step (the regions are sized for the plan's 128)
     void* base = nullptr;
     if ((rc = scratch_ptr(&base))) return rc;
     char* sb = (char*)base;
@@ -123,10 +127,8 @@ extern "C" int ozlu_gemm_noalloc(int nc, int p, int m, int n, int k, int alpha, 
     int8_t* RB = (int8_t*)(sb + o_rb);
     uint8_t* T = (uint8_t*)(sb + o_t);
     cudaStream_t s = (cudaStream_t)stream;
-    launch_row_shifts(A, lda, nc, m, k, tab.Q, mu, s);
-    launch_col_shifts(B, ldb, nc, k, n, tab.Q, nu, s);
-    launch_convert(A, lda, nc, m, k, false, mu, tab, Kpad, Mpad, RA, 0, s);
-    launch_convert(B, ldb, nc, k, n, true, nu, tab, Kpad, Npad, RB, 0, s);
+    launch_shifts(A, lda, m, B, ldb, n, nc, k, tab.Q, mu, nu, nullptr, s);
+    launch_convert(A, lda, m, B, ldb, n, nc, k, mu, nu, conv, Kpad, Mpad, Npad, RA, RB, 0, s);
     launch_gemm_imma(RA, RB, m, n, Mpad, Npad, Kpad, tab, T, s);
     launch_crt(T, false, m, n, mu, nu, tab, nc, alpha, beta, C, ldc, s);
     return cudaGetLastError() == cudaSuccess ? OZLU_OK : OZLU_ERR_CUDA;

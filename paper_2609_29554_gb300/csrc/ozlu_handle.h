@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "ozlu_internal.h"
+#include "tables.h"
 
 namespace ozlu {
 
@@ -20,6 +21,7 @@ struct Workspace {
 struct PlanEntry {
     Plan plan;
     DevTable table;
+    ConvTab conv;
 };
 
 // byte offsets of the last ozlu_gemm's intermediates inside the workspace

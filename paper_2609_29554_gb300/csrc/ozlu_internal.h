@@ -94,19 +94,23 @@ void fill_table(const Plan& pl, DevTable& t);
 int plan_noalloc(int p, int K, DevTable& t, int& Kpad);
 
 // ---------------------------------------------------------------- kernels --
-// (S1) shared exponents: mu[i] over rows of A (m x k), nu[j] over columns of B.
-void launch_row_shifts(const double* A, long long lda, int nc, int m, int k, int Q,
-                       int* mu, cudaStream_t s);
-void launch_col_shifts(const double* B, long long ldb, int nc, int k, int n, int Q,
-                       int* nu, cudaStream_t s);
-// (S2)+(S3) fused: expansions -> Q-bit integers -> S digits -> residue planes.
-// A side: planes [l][t][Mpad][Kpad] (row i, K contiguous); B side: [l][t][Npad][Kpad].
-// mode 0: int8 residues (1 plane); 1: E4M3 base-17 digits d0, d1, d0+d1 (3 planes);
-// 2: binary16 residues (1 plane, 2-byte elements); 3: binary64 residues (8-byte).
+struct ConvTab;  // tables.h
+
+// (S1) shared exponents: mu[i] over rows of A (m x k), nu[j] over columns of B
+// (k x n); `clear`: a device error word to zero, or null.
+void launch_shifts(const double* A, long long lda, int m, const double* B, long long ldb, int n, int nc, int k, int Q,
+                   int* mu, int* nu, int* clear, cudaStream_t s);
+// (S2)+(S3) fused, both operands: expansions -> Q-bit integers -> S digits ->
+// residue planes, A planes [l][t][Mpad][Kpad] (row i, K contiguous), B planes
+// [l][t][Npad][Kpad].  mode 0: int8 residues (1 plane); 1: E4M3 base-17 digits
+// d0, d1, d0+d1 (3 planes); 2: binary16 residues (1 plane, 2-byte elements).
 // Plane index (l * S + t) * P + p.
-void launch_convert(const double* X, long long ld, int nc, int rows, int cols,
-                    bool is_b, const int* shifts, const DevTable& tab, int Kpad,
-                    int Rpad, void* planes, int mode, cudaStream_t s);
+void launch_convert(const double* A, long long lda, int m, const double* B, long long ldb, int n, int nc, int k,
+                    const int* mu, const int* nu, const ConvTab& t, int Kpad, int Mpad, int Npad, void* RA, void* RB,
+                    int mode, cudaStream_t s);
+// the binary64 back-end's residues (8-byte) of one operand
+void launch_convert64(const double* X, long long ld, int nc, int rows, int cols, bool is_b, const int* shifts,
+                      const DevTable& tab, int Kpad, int Rpad, double* planes, cudaStream_t s);
 // (S4) on tcgen05: FP8 base-17 Karatsuba (fp8 = true) or FP16 residues
 int launch_gemm_tc05(bool fp8, const void* RA, const void* RB, int m, int n, int Mpad, int Npad,
                      int Kpad, const DevTable& tab, uint8_t* T, int* err, cudaStream_t s);
