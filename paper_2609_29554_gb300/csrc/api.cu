@@ -126,7 +126,11 @@ int plan_for(ozlu_handle* h, int p, int K, const ozlu_opts* o, const PlanEntry**
         int rc = make_plan(p, K, o, e.plan);
         if (rc) return rc;
         fill_table(e.plan, e.table);
-        if (e.plan.backend != OZLU_BE_FP64) fill_conv(e.table, e.conv);
+        if (e.plan.backend != OZLU_BE_FP64) {
+            fill_conv(e.table, e.conv);
+            fill_crt(e.table, e.plan.pint_bits, e.crt);
+            fill_gemm(e.table, e.plan.backend == OZLU_BE_FP8, e.gemm);
+        }
         it = h->plans.emplace(key, e).first;
     }
     *out = &it->second;
@@ -294,7 +298,6 @@ int gemm_device(ozlu_handle* h, int nc, int p, int m, int n, int k, int alpha, c
     const int be = pl->backend;
     const int mode = be == OZLU_BE_INT8 ? 0 : be == OZLU_BE_FP8 ? 1 : be == OZLU_BE_FP16 ? 2 : 3;
     const int P = mode == 1 ? 3 : 1, esz = mode == 2 ? 2 : (mode == 3 ? 8 : 1);
-    const int tsz = mode == 3 ? 4 : 1;  // bytes per t value
     const int Mpad = (m + 127) / 128 * 128, Npad = (n + 127) / 128 * 128;
     // K padded to the GEMM's step: 64 elements (INT8, FP16; the binary64 kernel
     // takes any), 128 for FP8 (the accumulator conditions hold for the plan's 128)
@@ -307,7 +310,12 @@ int gemm_device(ozlu_handle* h, int nc, int p, int m, int n, int k, int alpha, c
     L.nu = off; off = align_up(off + sizeof(int) * n);
     L.ra = off; off = align_up(off + (size_t)pl->N * pl->S * P * Mpad * Kpad * esz);
     L.rb = off; off = align_up(off + (size_t)pl->N * pl->S * P * Npad * Kpad * esz);
-    L.t = off;  off = align_up(off + (size_t)pl->G * pl->N * m * n * tsz);
+    // t values: bytes, 32-bit words (binary64), or a word per triple of moduli
+    const bool pack = (mode == 1 || mode == 2) && tc05_packs(pe->gemm, Mpad, Npad);
+    const size_t tval = pack ? 4 * (size_t)pe->gemm.NT : (size_t)pl->N * (mode == 3 ? 4 : 1);
+    L.t = off;  off = align_up(off + (size_t)pl->G * tval * m * n);
+    L.pack = pack;
+    memcpy(L.mod, pl->mod, sizeof L.mod);
     int* derr = err_word(h);
     if (!derr) return OZLU_ERR_NOMEM;
     rc = h->ws.ensure(off);
@@ -333,11 +341,12 @@ int gemm_device(ozlu_handle* h, int nc, int p, int m, int n, int k, int alpha, c
     } else if (mode == 3) {
         launch_gemm_f64((const double*)RA, (const double*)RB, m, n, Mpad, Npad, Kpad, *tab, (uint32_t*)T, s);
     } else {
-        rc = launch_gemm_tc05(mode == 1, RA, RB, m, n, Mpad, Npad, Kpad, *tab, T, derr, s);
+        rc = launch_gemm_tc05(mode == 1, pack, RA, RB, m, n, Mpad, Npad, Kpad, pe->gemm, T, derr, s);
         if (rc) return rc;
     }
     h->phase(PH_CRT);
-    launch_crt(T, mode == 3, m, n, mu, nu, *tab, nc, alpha, beta, C, ldc, s);
+    if (mode == 3) launch_crt64((const uint32_t*)T, m, n, mu, nu, *tab, nc, alpha, beta, C, ldc, s);
+    else launch_crt(T, pack, m, n, mu, nu, pe->crt, nc, alpha, beta, C, ldc, s);
     h->phase(prev);
     h->stats.gemm_launches += 1;
     h->stats.crt_launches += 1;
@@ -586,7 +595,28 @@ int ozlu_debug_fetch(ozlu_handle* h, int what, void* dst, size_t bytes) {
     if (what == 5) {
         const size_t need = (size_t)L.G * L.N * L.m * L.n * (L.backend == OZLU_BE_FP64 ? 4 : 1);
         if (bytes < need) return -4;
-        return cuda_rc(cudaMemcpy(dst, base + L.t, need, cudaMemcpyDeviceToHost));
+        if (!L.pack) return cuda_rc(cudaMemcpy(dst, base + L.t, need, cudaMemcpyDeviceToHost));
+        // a packed word u = t_a m_b m_c + t_b m_a m_c + t_c m_a m_b gives
+        // t_a = u (m_b m_c)^-1 mod m_a
+        const size_t mn = (size_t)L.m * L.n;
+        const int NT = (L.N + 2) / 3;
+        std::vector<uint32_t> u(mn);
+        for (int gi = 0; gi < L.G; ++gi)
+            for (int q = 0; q < NT; ++q) {
+                if (cudaMemcpy(u.data(), base + L.t + 4 * mn * ((size_t)gi * NT + q), 4 * mn,
+                               cudaMemcpyDeviceToHost) != cudaSuccess)
+                    return OZLU_ERR_CUDA;
+                for (int l = 3 * q; l < 3 * q + 3 && l < L.N; ++l) {
+                    const uint32_t ml = (uint32_t)L.mod[l];
+                    uint32_t others = 1, inv = 1;
+                    for (int j = 3 * q; j < 3 * q + 3 && j < L.N; ++j)
+                        if (j != l) others = others * (uint32_t)L.mod[j] % ml;
+                    while (others * inv % ml != 1 % ml) ++inv;
+                    uint8_t* out = (uint8_t*)dst + mn * ((size_t)gi * L.N + l);
+                    for (size_t e = 0; e < mn; ++e) out[e] = (uint8_t)(u[e] % ml * inv % ml);
+                }
+            }
+        return OZLU_OK;
     }
     return -2;
 }

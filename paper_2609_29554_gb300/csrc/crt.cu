@@ -3,6 +3,7 @@
 //
 // One thread per output element.  For every retained digit group g:
 //   S_g = sum_l t_l M_l - round(F) P,   F = sum_l t_l / m_l       (Eq. (11))
+// (by triples of moduli for the byte-modulus back-ends, tables.h)
 // evaluated modulo 2^(32 WG): |S_g| < 2^(32 WG - 1) by the plan, so the low
 // words of M_l and P suffice and the wrap-around is the two's-complement
 // representation of the centered value.  F is summed in binary32: the plan's
@@ -14,15 +15,11 @@
 // rounded into nc binary64 components by successive round-to-nearest-even.
 //
 // The group accumulators live in registers (WG is a template parameter, so
-// the word loops unroll); the wide integers that need shifts by run-time
-// amounts live in shared memory, one column per thread ([word][thread]).
-#include "mp_device.cuh"
-#include "ozlu_internal.h"
+// the word loops unroll).
+#include "crt_kernel.cuh"
 
 namespace ozlu {
 namespace {
-
-constexpr int CT = 128;  // threads per block
 
 struct Wide {
     uint32_t* w;  // word k at w[k * CT]
@@ -188,11 +185,14 @@ __device__ __forceinline__ void wide_round_out(const Wide& X, bool neg, int E, i
     }
 }
 
-template <int WG, typename TT>
-__global__ void __launch_bounds__(CT) crt_kernel(const TT* __restrict__ T, int m, int n,
-                                                 const int* __restrict__ mu, const int* __restrict__ nu,
-                                                 const __grid_constant__ DevTable tab, int nc, int alpha,
-                                                 int beta, double* __restrict__ C, long long ldc) {
+// The binary64 back-end's kernel (32-bit t values): the wide integers, which
+// need shifts by run-time amounts, live in shared memory, one column per
+// thread ([word][thread]).
+template <int WG>
+__global__ void __launch_bounds__(CT) crt64_kernel(const uint32_t* __restrict__ T, int m, int n,
+                                                   const int* __restrict__ mu, const int* __restrict__ nu,
+                                                   const __grid_constant__ DevTable tab, int nc, int alpha,
+                                                   int beta, double* __restrict__ C, long long ldc) {
     __shared__ uint32_t sx[WACC * CT];
     __shared__ uint32_t ss[MAXWG * CT];
     const long long e = (long long)blockIdx.x * CT + threadIdx.x;
@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(CT) crt_kernel(const TT* __restrict__ T, int m
 #pragma unroll
         for (int w = 0; w < WG; ++w) acc[w] = 0;
         float F = 0.0f;
-        const TT* tp = T + (size_t)gi * tab.N * mn + e;
+        const uint32_t* tp = T + (size_t)gi * tab.N * mn + e;
         for (int l = 0; l < tab.N; ++l) {
             const uint32_t t = tp[(size_t)l * mn];
 #pragma unroll
@@ -261,44 +261,29 @@ __global__ void __launch_bounds__(CT) crt_kernel(const TT* __restrict__ T, int m
     for (int c = 0; c < nc; ++c) cp[c] = out[c];
 }
 
-template <int WG, typename TT>
-void launch_wg(const TT* T, int m, int n, const int* mu, const int* nu, const DevTable& tab, int nc,
-               int alpha, int beta, double* C, long long ldc, cudaStream_t s) {
-    const long long mn = (long long)m * n;
-    crt_kernel<WG, TT><<<(unsigned)((mn + CT - 1) / CT), CT, 0, s>>>(T, m, n, mu, nu, tab, nc, alpha, beta, C,
-                                                                     ldc);
-}
-
-template <typename TT>
-void launch_tt(const TT* T, int m, int n, const int* mu, const int* nu, const DevTable& tab, int nc, int alpha,
-               int beta, double* C, long long ldc, cudaStream_t s) {
-    switch (tab.WG) {
-        case 1: case 2: case 3: case 4: launch_wg<4>(T, m, n, mu, nu, tab, nc, alpha, beta, C, ldc, s); break;
-        case 5: launch_wg<5>(T, m, n, mu, nu, tab, nc, alpha, beta, C, ldc, s); break;
-        case 6: launch_wg<6>(T, m, n, mu, nu, tab, nc, alpha, beta, C, ldc, s); break;
-        case 7: launch_wg<7>(T, m, n, mu, nu, tab, nc, alpha, beta, C, ldc, s); break;
-        case 8: launch_wg<8>(T, m, n, mu, nu, tab, nc, alpha, beta, C, ldc, s); break;
-        case 9: launch_wg<9>(T, m, n, mu, nu, tab, nc, alpha, beta, C, ldc, s); break;
-        case 10: launch_wg<10>(T, m, n, mu, nu, tab, nc, alpha, beta, C, ldc, s); break;
-        case 11: launch_wg<11>(T, m, n, mu, nu, tab, nc, alpha, beta, C, ldc, s); break;
-        case 12: launch_wg<12>(T, m, n, mu, nu, tab, nc, alpha, beta, C, ldc, s); break;
-        case 13: launch_wg<13>(T, m, n, mu, nu, tab, nc, alpha, beta, C, ldc, s); break;
-        case 14: launch_wg<14>(T, m, n, mu, nu, tab, nc, alpha, beta, C, ldc, s); break;
-        case 15: launch_wg<15>(T, m, n, mu, nu, tab, nc, alpha, beta, C, ldc, s); break;
-        default: launch_wg<16>(T, m, n, mu, nu, tab, nc, alpha, beta, C, ldc, s); break;
-    }
-}
-
 }  // namespace
 
-void launch_crt(const void* T, bool t32, int m, int n, const int* mu, const int* nu, const DevTable& tab, int nc,
+void launch_crt(const void* T, bool pack, int m, int n, const int* mu, const int* nu, const CrtTab& tab, int nc,
                 int alpha, int beta, double* C, long long ldc, cudaStream_t s) {
+    const CrtArgs a{T, mu, nu, C, ldc, (long long)m * n, m, nc, alpha, beta, nc != 3 && ((uintptr_t)C & 15) == 0};
+    if (a.mn == 0) return;
+    if (pack) launch_crt_packed(a, tab, s);
+    else launch_crt_bytes(a, tab, s);
+}
+
+void launch_crt64(const uint32_t* T, int m, int n, const int* mu, const int* nu, const DevTable& tab, int nc,
+                  int alpha, int beta, double* C, long long ldc, cudaStream_t s) {
     const long long mn = (long long)m * n;
     if (mn == 0) return;
-    if (t32)
-        launch_tt<uint32_t>((const uint32_t*)T, m, n, mu, nu, tab, nc, alpha, beta, C, ldc, s);
-    else
-        launch_tt<uint8_t>((const uint8_t*)T, m, n, mu, nu, tab, nc, alpha, beta, C, ldc, s);
+    const unsigned grid = (unsigned)((mn + CT - 1) / CT);
+    switch (tab.WG) {
+#define OZLU_WG(W) \
+    case W: crt64_kernel<W><<<grid, CT, 0, s>>>(T, m, n, mu, nu, tab, nc, alpha, beta, C, ldc); break;
+        OZLU_WG(5) OZLU_WG(6) OZLU_WG(7) OZLU_WG(8) OZLU_WG(9) OZLU_WG(10) OZLU_WG(11) OZLU_WG(12) OZLU_WG(13)
+        OZLU_WG(14) OZLU_WG(15) OZLU_WG(16)
+#undef OZLU_WG
+        default: crt64_kernel<4><<<grid, CT, 0, s>>>(T, m, n, mu, nu, tab, nc, alpha, beta, C, ldc); break;
+    }
 }
 
 }  // namespace ozlu

@@ -13,41 +13,59 @@
 // Both rely on the fp32 tensor-core accumulation being exact for integer
 // sums below 2^24; the parity tests check it bit for bit.
 //
-// Kernel: persistent, one CTA per SM over the 128 x 128 output tiles of all
-// (modulus, digit group) pairs.
+// Kernel: persistent, one CTA per SM over 128 x 128 output tiles.  A unit is one
+// tile of a triple of moduli (packed results) or of one modulus (bytes); its
+// plane products follow one another through a ring of four accumulators in
+// TMEM (4 x 128 columns), so the MMAs of the next products run while the
+// epilogue reduces the last.
 //   warp 0: TMA producer (cp.async.bulk.tensor, SWIZZLE_128B, no multicast)
 //   warp 1: one thread issues tcgen05.mma (M = 128, N = 128, K = 32 bytes
 //           per instruction) into TMEM, tcgen05.commit frees smem stages and
 //           hands a finished accumulator to the epilogue
-//   warps 2-9 (FP8) or 2-17 (FP16): epilogue (two or four warps per TMEM
-//           lane quarter, each on a half or a quarter of the columns),
-//           tcgen05.ld 32x32b, combine, t_l = (C mod m) y mod m, then free the
-//           accumulator buffer for the MMA warp
+//   warps 2-17: epilogue (four warps per TMEM lane quarter, each on a quarter
+//           of the columns), tcgen05.ld 32x32b, frees the accumulator at once,
+//           then t_l = (C y_l) mod m_l.
+// The kernel is bound by shared memory: every operand byte is written once by
+// TMA and read once by the 128 x 128 MMAs (about 530 cycles a stage where the
+// MMAs alone need 256), with the epilogue close behind at K = 256.  The
+// reduction therefore runs on the binary32 pipe (eight full-rate instructions
+// per value, all exact: fma with the rounding constant 1.5 2^23 for the first
+// quotient, fma rounding down for the floor of the second), where integer
+// code with its float conversions took about 40, and a triple's three t values
+// leave as the one 32-bit word u_q (CrtTab) that the CRT needs, a 128-byte
+// store a warp instead of three of 32 bytes.
+// FP16, QD, 3840 x 3840 x 256: 891 us (1928 before); FP8, QD, 1024^3: 342 us (534
+// before).  Clusters of two CTAs that share the B tile by multicast (a quarter
+// less L2 traffic) measured the same, 893 us.
 // Every mbarrier wait has an iteration limit; on expiry the CTA records
 // OZLU_ERR_TIMEOUT, stops issuing work, and releases its TMEM.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
-#include "mp_device.cuh"
 #include "ozlu_internal.h"
+#include "tables.h"
 
 namespace ozlu {
 namespace {
 
 constexpr int BM = 128, BN = 128, BK = 128;  // BK in bytes: one 128-byte swizzle row
 constexpr int STAGES = 6;
-// producer, MMA and the epilogue warps: 8 for FP8 (three accumulators per
-// output keep the registers of one epilogue thread high), 16 for FP16
-template <bool FP8>
-struct Cfg {
-    static constexpr int THREADS = FP8 ? 320 : 576;
-    static constexpr int EPI = THREADS - 64;      // epilogue threads
-    static constexpr int SPLIT = (THREADS - 64) / 128;  // column parts per TMEM lane quarter
-};
+constexpr int THREADS = 576;          // producer, MMA and 16 epilogue warps
+constexpr int EPI = THREADS - 64;     // epilogue threads
+constexpr int NBUF = 4;               // accumulators in TMEM
 constexpr int TILE = BM * BK;                // 16 KiB per operand stage
 constexpr long long WAIT_LIMIT = 1ll << 24;  // iterations of ~100 ns
 
 __device__ __forceinline__ uint32_t su32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+// one lane of a converged warp.  The warp's control flow stays uniform (loop
+// state and descriptors in uniform registers); a loop inside `if (lane == 0)`
+// took about 700 cycles to issue a stage of four MMAs.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
+    return r != 0;
+}
 
 __device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(su32(b)), "r"(count));
@@ -71,6 +89,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* b, uint32_t parity) {
 // bounded wait: false (and the error word set) after `limit` tries
 __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, int* err, volatile int* abort,
                                           long long limit = WAIT_LIMIT) {
+    if (mbar_try_wait(b, parity)) return true;
     long long it = 0;
     while (!mbar_try_wait(b, parity)) {
         if (*abort) return false;
@@ -79,7 +98,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, int* err
             *abort = 1;
             return false;
         }
-        __nanosleep(64);
+        // the ring's waits are short: sleeping at once would add to each of them
+        if (it > 32) __nanosleep(64);
     }
     return true;
 }
@@ -130,27 +150,33 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 }
 
-__device__ __forceinline__ uint32_t t_value(int c, uint32_t m, uint32_t y, uint32_t magic) {
-    const uint32_t a = c < 0 ? (uint32_t)(-(long long)c) : (uint32_t)c;
-    uint32_t r = mod_small(a, m, magic);
-    if (c < 0 && r) r = m - r;
-    return mod_small(r * y, m, magic);
+// 1.5 2^23: adding it rounds a binary32 value below 2^22 to an integer, whose
+// low bits are then the low bits of the sum
+constexpr float RINT = 12582912.0f;
+
+// c mod m up to a multiple of m: |result| <= 0.54 m + 1, exact for |c| < 2^24
+__device__ __forceinline__ float fold(float c, float m, float inv) {
+    const float q = __fadd_rn(__fmaf_rn(c, inv, RINT), -RINT);
+    return __fmaf_rn(-q, m, c);
 }
 
-// Persistent kernel: one CTA per SM walks the tiles (tm, tn, l, gi) with
-// stride gridDim.x, tn fastest, so the CTAs in flight share A row panels and
-// B column panels of one modulus in L2.  The smem ring runs across tiles; the
-// accumulators are double-buffered in TMEM (FP16: 2 x 128 columns; FP8 keeps
-// one 384-column buffer), so the epilogue of one tile overlaps the MMAs of
-// the next.
-template <bool FP8>
-__global__ void __launch_bounds__(Cfg<FP8>::THREADS, 1) gemm_tc05_kernel(
+// bits of RINT + (v mod m) for an integer 0 <= v < 2^17, invu the float above
+// 1 / m: v invu exceeds v / m by less than 1 / 255, so its floor is exact
+__device__ __forceinline__ uint32_t floor_mod_bits(float v, float m, float invu) {
+    const float k = __fadd_rn(__fmaf_rd(v, invu, RINT), -RINT);
+    return __float_as_uint(__fadd_rn(__fmaf_rn(-k, m, v), RINT));
+}
+
+// The CTAs walk the units (gi, q, tm, tn) with stride gridDim.x, tn fastest, so
+// those in flight share A row panels and B column panels in L2.
+template <bool FP8, bool PACK>
+__global__ void __launch_bounds__(THREADS, 1) gemm_tc05_kernel(
     const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int m, int n,
-    int Mpad, int Npad, int KB, const __grid_constant__ DevTable tab, uint8_t* __restrict__ T,
+    int Mpad, int Npad, int KB, const __grid_constant__ GemmTab tab, void* __restrict__ T,
     int* __restrict__ err) {
-    constexpr int P = FP8 ? 3 : 1;                // planes (accumulators)
-    constexpr int NBUF = FP8 ? 1 : 2;             // accumulator buffers
-    constexpr uint32_t TMEM_COLS = FP8 ? 512 : 256;
+    constexpr int P = FP8 ? 3 : 1;                // planes (products per modulus)
+    constexpr int LG = PACK ? 3 : 1;              // moduli per unit
+    constexpr uint32_t TMEM_COLS = NBUF * BN;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sm = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t* sa = sm;
@@ -158,26 +184,29 @@ __global__ void __launch_bounds__(Cfg<FP8>::THREADS, 1) gemm_tc05_kernel(
     uint64_t* full = (uint64_t*)(sm + 2 * STAGES * TILE);
     uint64_t* empty = full + STAGES;
     uint64_t* accf = empty + STAGES;   // [NBUF] accumulator ready (MMA -> epilogue)
-    uint64_t* acce = accf + 2;         // [NBUF] accumulator free (epilogue -> MMA)
-    uint32_t* tmem_slot = (uint32_t*)(acce + 2);
+    uint64_t* acce = accf + NBUF;      // [NBUF] accumulator free (epilogue -> MMA)
+    uint32_t* tmem_slot = (uint32_t*)(acce + NBUF);
     volatile int* abort = (volatile int*)(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int TM = Mpad / BM, TN = Npad / BN;
-    const int tiles = TM * TN * tab.N * tab.G;
+    const int NQ = PACK ? tab.NT : tab.N;
+    const int units = TM * TN * NQ * tab.G;
     const int S = tab.S;
-    // tile t -> (tm, tn, l, gi) and its work items (pair terms x K blocks x planes)
-    auto decode = [&](int t, int& tm, int& tn, int& l, int& gi, int& ta0, int& items) {
+    // unit -> (tm, tn, q, gi), its moduli [q LG, l1) and items per product
+    // (pair terms x K blocks)
+    auto decode = [&](int t, int& tm, int& tn, int& q, int& gi, int& l1, int& ta0, int& items) {
         tn = t % TN;
         int r = t / TN;
         tm = r % TM;
         r /= TM;
-        l = r % tab.N;
-        gi = r / tab.N;
+        q = r % NQ;
+        gi = r / NQ;
+        l1 = min(tab.N, q * LG + LG);
         const int g = tab.g0 + gi;
         ta0 = max(0, g - (S - 1));
         const int ta1 = min(g, S - 1);
-        items = (ta1 - ta0 + 1) * KB * P;
+        items = (ta1 - ta0 + 1) * KB;
     };
 
     if (threadIdx.x == 0) {
@@ -187,7 +216,7 @@ __global__ void __launch_bounds__(Cfg<FP8>::THREADS, 1) gemm_tc05_kernel(
         }
         for (int b = 0; b < NBUF; ++b) {
             mbar_init(&accf[b], 1);
-            mbar_init(&acce[b], Cfg<FP8>::EPI);
+            mbar_init(&acce[b], EPI);
         }
         *abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -204,119 +233,138 @@ __global__ void __launch_bounds__(Cfg<FP8>::THREADS, 1) gemm_tc05_kernel(
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
-            long long it = 0;       // global item counter (smem ring position)
-            long long issued = 0;
-            for (int t = blockIdx.x; t < tiles && !*abort; t += gridDim.x) {
-                int tm, tn, l, gi, ta0, items;
-                decode(t, tm, tn, l, gi, ta0, items);
-                const int g = tab.g0 + gi;
-                for (int i = 0; i < items && !*abort; ++i, ++it) {
-                    const int s = (int)(it % STAGES);
-                    const long long round = it / STAGES;
-                    if (!mbar_wait(&empty[s], (uint32_t)((round & 1) ^ 1), err, abort)) break;
-                    const int p = i % P, rest = i / P;
-                    const int kb = rest % KB, pr = rest / KB;
-                    const int ta = ta0 + pr, tb = g - ta;
-                    mbar_expect_tx(&full[s], 2 * TILE);
-                    const int ya = ((l * S + ta) * P + p) * Mpad + tm * BM;
-                    const int yb = ((l * S + tb) * P + p) * Npad + tn * BN;
-                    const int x = FP8 ? kb * BK : kb * (BK / 2);  // element units of the map
-                    tma_load_2d(sa + s * TILE, &tmA, x, ya, &full[s]);
-                    tma_load_2d(sb + s * TILE, &tmB, x, yb, &full[s]);
-                    issued = it + 1;
-                }
-            }
-            if (*abort) {
-                // let the copies already issued land before the CTA exits (bounded)
-                for (long long q = issued - STAGES < 0 ? 0 : issued - STAGES; q < issued; ++q) {
-                    long long w = 0;
-                    while (!mbar_try_wait(&full[q % STAGES], (uint32_t)((q / STAGES) & 1)) && ++w < WAIT_LIMIT)
-                        __nanosleep(64);
-                }
+        // position in the smem ring: stage s, parity of its pass; `issued`
+        // (at most STAGES) stages hold copies that nobody may have waited for
+        int s = 0, issued = 0;
+        uint32_t par = 0;
+        bool ok = true;
+        for (int t = blockIdx.x; t < units && ok; t += gridDim.x) {
+            int tm, tn, q, gi, l1, ta0, items;
+            decode(t, tm, tn, q, gi, l1, ta0, items);
+            const int g = tab.g0 + gi, ta1 = min(g, S - 1);
+            for (int l = q * LG; l < l1 && ok; ++l)
+                for (int p = 0; p < P && ok; ++p)
+                    for (int ta = ta0; ta <= ta1 && ok; ++ta) {
+                        const int ya = ((l * S + ta) * P + p) * Mpad + tm * BM;
+                        const int yb = ((l * S + g - ta) * P + p) * Npad + tn * BN;
+                        for (int kb = 0, x = 0; kb < KB; ++kb, x += FP8 ? BK : BK / 2) {
+                            if (!__all_sync(0xffffffffu, mbar_wait(&empty[s], par ^ 1, err, abort))) { ok = false; break; }
+                            if (elect_one()) {
+                                mbar_expect_tx(&full[s], 2 * TILE);
+                                tma_load_2d(sa + s * TILE, &tmA, x, ya, &full[s]);
+                                tma_load_2d(sb + s * TILE, &tmB, x, yb, &full[s]);
+                            }
+                            __syncwarp();
+                            issued = min(issued + 1, STAGES);
+                            if (++s == STAGES) { s = 0; par ^= 1; }
+                        }
+                    }
+        }
+        if (!ok || *abort) {
+            // let the copies already issued land before the CTA exits (bounded)
+            for (; issued > 0; --issued) {
+                if (--s < 0) { s = STAGES - 1; par ^= 1; }
+                long long w = 0;
+                while (!mbar_try_wait(&full[s], par) && ++w < WAIT_LIMIT) __nanosleep(64);
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // kind::f8f6f4 E4M3 x E4M3 or kind::f16 F16 x F16 (format code 0 in both),
-            // fp32 accumulate, K-major A and B, N = 128, M = 128
-            const uint32_t idesc = (1u << 4) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-            long long it = 0;
-            int j = 0;  // local tile count
-            for (int t = blockIdx.x; t < tiles && !*abort; t += gridDim.x, ++j) {
-                int tm, tn, l, gi, ta0, items;
-                decode(t, tm, tn, l, gi, ta0, items);
-                const int b = j % NBUF;
-                const uint32_t use = (uint32_t)(j / NBUF);
-                if (!mbar_wait(&acce[b], (use & 1) ^ 1, err, abort)) break;
+        // kind::f8f6f4 E4M3 x E4M3 or kind::f16 F16 x F16 (format code 0 in both),
+        // fp32 accumulate, K-major A and B, N = 128, M = 128
+        const uint32_t idesc = (1u << 4) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+        const uint64_t da = smem_desc(sa), db = smem_desc(sb);
+        // ring positions: smem stage s, accumulator b, with their parities
+        int s = 0, b = 0;
+        uint32_t par = 0, bpar = 0;
+        bool ok = true;
+        for (int t = blockIdx.x; t < units && ok; t += gridDim.x) {
+            int tm, tn, q, gi, l1, ta0, items;
+            decode(t, tm, tn, q, gi, l1, ta0, items);
+            const int prods = (l1 - q * LG) * P;
+            for (int pd = 0; pd < prods && ok; ++pd) {
+                if (!__all_sync(0xffffffffu, mbar_wait(&acce[b], bpar ^ 1, err, abort))) { ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;\n");
-                const uint32_t acc = tmem + (uint32_t)(b * P * BN);
-                bool ok = true;
-                for (int i = 0; i < items; ++i, ++it) {
-                    const int s = (int)(it % STAGES);
-                    const long long round = it / STAGES;
-                    if (!mbar_wait(&full[s], (uint32_t)(round & 1), err, abort)) { ok = false; break; }
+                const uint32_t acc = tmem + (uint32_t)(b * BN);
+                for (int i = 0; i < items; ++i) {
+                    if (!__all_sync(0xffffffffu, mbar_wait(&full[s], par, err, abort))) { ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;\n");
-                    const int p = i % P;
-                    const int first_of_plane = i < P;  // first item of each accumulator
-                    const uint64_t ad = smem_desc(sa + s * TILE), bd = smem_desc(sb + s * TILE);
+                    const uint64_t ad = da + (uint64_t)(s * (TILE >> 4)), bd = db + (uint64_t)(s * (TILE >> 4));
+                    if (elect_one()) {
 #pragma unroll
-                    for (int k = 0; k < BK / 32; ++k)
-                        mma<FP8>(acc + p * BN, ad + 2 * k, bd + 2 * k, idesc, (first_of_plane && k == 0) ? 0u : 1u);
-                    mma_commit(&empty[s]);
+                        for (int k = 0; k < BK / 32; ++k)
+                            mma<FP8>(acc, ad + 2 * k, bd + 2 * k, idesc, (i == 0 && k == 0) ? 0u : 1u);
+                        mma_commit(&empty[s]);
+                        if (i == items - 1) mma_commit(&accf[b]);
+                    }
+                    __syncwarp();
+                    if (++s == STAGES) { s = 0; par ^= 1; }
                 }
-                if (!ok) break;
-                mma_commit(&accf[b]);
+                if (++b == NBUF) { b = 0; bpar ^= 1; }
             }
         }
     } else {
         // epilogue warps: TMEM lane quarter = warp % 4; the k-th group of four
-        // warps (from warp 2) takes the k-th of SPLIT parts of the tile's columns
-        const int q = warp & 3;
-        const int half = (warp - 2) >> 2;
-        constexpr int CPP = (BN / 32) / Cfg<FP8>::SPLIT;  // 32-column chunks per part
-        int j = 0;
-        for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++j) {
-            int tm, tn, l, gi, ta0, items;
-            decode(t, tm, tn, l, gi, ta0, items);
-            const int b = j % NBUF;
-            const uint32_t use = (uint32_t)(j / NBUF);
-            if (!mbar_wait(&accf[b], use & 1, err, abort)) break;
-            asm volatile("tcgen05.fence::after_thread_sync;\n");
-            const uint32_t md = (uint32_t)tab.mod[l], yd = (uint32_t)tab.y[l], mg = tab.magic[l];
-            const int i = tm * BM + q * 32 + lane;
-            uint8_t* out = T + ((size_t)gi * tab.N + l) * (size_t)m * n;
-            const uint32_t lane_addr = tmem + (uint32_t)(b * P * BN) + ((uint32_t)(q * 32) << 16);
-            for (int ch = half * CPP; ch < (half + 1) * CPP; ++ch) {
-                uint32_t r0[32];
-                tmem_ld32(lane_addr + ch * 32, r0);
-                int c[32];
-                if (FP8) {
-                    uint32_t r1[32], r2[32];
-                    tmem_ld32(lane_addr + BN + ch * 32, r1);
-                    tmem_ld32(lane_addr + 2 * BN + ch * 32, r2);
+        // warps (from warp 2) takes the k-th quarter of the tile's columns
+        const int lq = warp & 3;
+        const int c0 = ((warp - 2) >> 2) * 32;
+        const uint32_t lane_addr = tmem + ((uint32_t)(lq * 32) << 16) + (uint32_t)c0;
+        int b = 0;
+        uint32_t bpar = 0;
+        bool ok = true;
+        for (int t = blockIdx.x; t < units && ok; t += gridDim.x) {
+            int tm, tn, q, gi, l1, ta0, items;
+            decode(t, tm, tn, q, gi, l1, ta0, items);
+            const int i = tm * BM + lq * 32 + lane;
+            const int cols = min(32, n - tn * BN - c0);  // of this warp, may be <= 0
+            uint32_t u[PACK ? 32 : 1];
+            if (PACK) {
 #pragma unroll
-                    for (int jj = 0; jj < 32; ++jj) {
-                        const int p00 = (int)__uint_as_float(r0[jj]);
-                        const int p11 = (int)__uint_as_float(r1[jj]);
-                        const int pss = (int)__uint_as_float(r2[jj]);
-                        c[jj] = p00 + 17 * (pss - p00 - p11) + 289 * p11;
+                for (int jj = 0; jj < 32; ++jj) u[PACK ? jj : 0] = tab.ucorr[q];
+            }
+            for (int l = q * LG; l < l1 && ok; ++l) {
+                const GemmMod& M = tab.mod[l];
+                const float md = M.m, inv = M.inv;
+                float v[32];
+#pragma unroll
+                for (int p = 0; p < P; ++p) {
+                    // (the vote keeps the warp together for the loads that follow)
+                    if (!ok || !__all_sync(0xffffffffu, mbar_wait(&accf[b], bpar, err, abort))) {
+                        ok = false;
+                        break;
                     }
-                } else {
+                    asm volatile("tcgen05.fence::after_thread_sync;\n");
+                    uint32_t r[32];
+                    tmem_ld32(lane_addr + (uint32_t)(b * BN), r);
+                    // the accumulator is in registers: the MMA warp may overwrite it
+                    asm volatile("tcgen05.fence::before_thread_sync;\n");
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(su32(&acce[b])) : "memory");
+                    if (++b == NBUF) { b = 0; bpar ^= 1; }
+                    const float yp = M.y[p], off = M.off;
 #pragma unroll
-                    for (int jj = 0; jj < 32; ++jj) c[jj] = (int)__uint_as_float(r0[jj]);
+                    for (int jj = 0; jj < 32; ++jj)
+                        v[jj] = __fmaf_rn(fold(__uint_as_float(r[jj]), md, inv), yp, p == 0 ? off : v[jj]);
                 }
-                if (i < m) {
+                if (!ok) break;
+                const float invu = M.invu;
+                if (PACK) {
+                    const uint32_t cf = M.coef;
 #pragma unroll
-                    for (int jj = 0; jj < 32; ++jj) {
-                        const int col = tn * BN + ch * 32 + jj;
-                        if (col < n) out[(size_t)col * m + i] = (uint8_t)t_value(c[jj], md, yd, mg);
-                    }
+                    for (int jj = 0; jj < 32; ++jj) u[PACK ? jj : 0] += floor_mod_bits(v[jj], md, invu) * cf;
+                } else if (i < m) {
+                    uint8_t* out = (uint8_t*)T + ((size_t)gi * tab.N + l) * (size_t)m * n +
+                                   (size_t)(tn * BN + c0) * m + i;
+#pragma unroll
+                    for (int jj = 0; jj < 32; ++jj)
+                        if (jj < cols) out[(size_t)jj * m] = (uint8_t)floor_mod_bits(v[jj], md, invu);
                 }
             }
-            // the accumulator buffer may be overwritten by the next tile's MMAs
-            asm volatile("tcgen05.fence::before_thread_sync;\n");
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(su32(&acce[b])) : "memory");
+            if (PACK && ok && i < m) {
+                uint32_t* out = (uint32_t*)T + ((size_t)gi * tab.NT + q) * (size_t)m * n +
+                                (size_t)(tn * BN + c0) * m + i;
+#pragma unroll
+                for (int jj = 0; jj < 32; ++jj)
+                    if (jj < cols) out[(size_t)jj * m] = u[PACK ? jj : 0];
+            }
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n");
@@ -376,10 +424,17 @@ int launch_mbar_expiry_selftest(long long limit, int* err, int* out, cudaStream_
     return cudaGetLastError() == cudaSuccess ? OZLU_OK : OZLU_ERR_CUDA;
 }
 
-size_t tc05_smem_bytes() { return 2 * STAGES * TILE + 2 * STAGES * 8 + 4 * 8 + 16 + 1024; }
+size_t tc05_smem_bytes() { return 2 * STAGES * TILE + 2 * STAGES * 8 + 2 * NBUF * 8 + 16 + 1024; }
 
-int launch_gemm_tc05(bool fp8, const void* RA, const void* RB, int m, int n, int Mpad, int Npad, int Kpad,
-                     const DevTable& tab, uint8_t* T, int* err, cudaStream_t s) {
+// Packed results where every SM still gets four units or more; below that the
+// coarser units (three moduli) leave SMs idle in the last round, and bytes (a
+// unit per modulus) are taken.
+bool tc05_packs(const GemmTab& tab, int Mpad, int Npad) {
+    return (long long)(Mpad / BM) * (Npad / BN) * tab.NT * tab.G >= 4ll * device_sms();
+}
+
+int launch_gemm_tc05(bool fp8, bool pack, const void* RA, const void* RB, int m, int n, int Mpad, int Npad, int Kpad,
+                     const GemmTab& tab, void* T, int* err, cudaStream_t s) {
     const int P = fp8 ? 3 : 1;
     CUtensorMap ta, tb;
     if (!make_map(&ta, RA, fp8, Kpad, (long long)tab.N * tab.S * P * Mpad)) return OZLU_ERR_UNSUPPORTED;
@@ -387,15 +442,14 @@ int launch_gemm_tc05(bool fp8, const void* RA, const void* RB, int m, int n, int
     const int KB = Kpad * (fp8 ? 1 : 2) / BK;
     const size_t smem = tc05_smem_bytes();
     const int sms = device_sms();
-    const long long tiles = (long long)(Mpad / BM) * (Npad / BN) * tab.N * tab.G;
-    dim3 grid((unsigned)(tiles < sms ? tiles : sms));
-    if (fp8) {
-        raise_smem_limit((const void*)gemm_tc05_kernel<true>, (int)smem);
-        gemm_tc05_kernel<true><<<grid, Cfg<true>::THREADS, smem, s>>>(ta, tb, m, n, Mpad, Npad, KB, tab, T, err);
-    } else {
-        raise_smem_limit((const void*)gemm_tc05_kernel<false>, (int)smem);
-        gemm_tc05_kernel<false><<<grid, Cfg<false>::THREADS, smem, s>>>(ta, tb, m, n, Mpad, Npad, KB, tab, T, err);
-    }
+    const long long units = (long long)(Mpad / BM) * (Npad / BN) * (pack ? tab.NT : tab.N) * tab.G;
+    dim3 grid((unsigned)(units < sms ? units : sms));
+    auto go = [&](auto kernel) {
+        raise_smem_limit((const void*)kernel, (int)smem);
+        kernel<<<grid, THREADS, smem, s>>>(ta, tb, m, n, Mpad, Npad, KB, tab, T, err);
+    };
+    if (fp8) pack ? go(gemm_tc05_kernel<true, true>) : go(gemm_tc05_kernel<true, false>);
+    else pack ? go(gemm_tc05_kernel<false, true>) : go(gemm_tc05_kernel<false, false>);
     return cudaGetLastError() == cudaSuccess ? OZLU_OK : OZLU_ERR_CUDA;
 }
 

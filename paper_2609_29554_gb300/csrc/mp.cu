@@ -929,7 +929,7 @@ size_t up256(size_t v) { return (v + 255) / 256 * 256; }
 // accumulator words for a plan: the largest P_int plus 64 bits, one sign bit spare
 int mp_window_words(const Plan& pl) { return (pl.pint_bits + 64 + 31) / 32 + 1; }
 
-int mp_plan_for(ozlu_handle* h, int p, int K, const Plan** pl, const DevTable** tab) {
+int mp_plan_for(ozlu_handle* h, int p, int K, const Plan** pl, const DevTable** tab, const GemmTab** gt) {
     const auto key = std::make_tuple(p, K, 1000, 0, 0, 0);  // backend code 1000: p-bit
     auto it = h->plans.find(key);
     if (it == h->plans.end()) {
@@ -937,10 +937,12 @@ int mp_plan_for(ozlu_handle* h, int p, int K, const Plan** pl, const DevTable** 
         const int rc = make_plan_mp(p, K, e.plan);
         if (rc) return rc;
         fill_table(e.plan, e.table);
+        fill_gemm(e.table, true, e.gemm);
         it = h->plans.emplace(key, e).first;
     }
     *pl = &it->second.plan;
     *tab = &it->second.table;
+    *gt = &it->second.gemm;
     return OZLU_OK;
 }
 
@@ -1131,7 +1133,8 @@ int mp_gemm_device(ozlu_handle* h, int p, int m, int n, int k, int alpha, const 
         return mp_gemm_ext(h, p, h->mp_opts.nslice, m, n, k, alpha, A, B, beta, C);
     const Plan* pl;
     const DevTable* tab;
-    int rc = mp_plan_for(h, p, k, &pl, &tab);
+    const GemmTab* gt;
+    int rc = mp_plan_for(h, p, k, &pl, &tab, &gt);
     if (rc) return rc;
     cudaStream_t s = h->stream;
     // K <= KSMALL: unpadded planes and the small-K product on the integer
@@ -1201,7 +1204,7 @@ int mp_gemm_device(ozlu_handle* h, int p, int m, int n, int k, int alpha, const 
         if (j0 > 0) mp_convert(view_of(B, j0 * B.ld), nc, k, 1, nu + j0, *tab, Kpad, ncp, RB, s, fp8);
         h->phase(PH_GEMM);
         if (fp8) {
-            if ((rc = launch_gemm_tc05(true, RA, RB, m, nc, Mpad, ncp, Kpad, *tab, T, derr, s))) return rc;
+            if ((rc = launch_gemm_tc05(true, false, RA, RB, m, nc, Mpad, ncp, Kpad, *gt, T, derr, s))) return rc;
         } else if (smallk) {
             const long long work = (long long)m * nc * pl->N * pl->G;
             small_k_gemm_kernel<<<(unsigned)((work + 255) / 256), 256, 0, s>>>(RA, RB, m, nc, k, *tab, T);

@@ -104,11 +104,13 @@ extern "C" int ozlu_gemm_noalloc(int nc, int p, int m, int n, int k, int alpha, 
     if (ldc < (m > 1 ? m : 1)) return -13;
     if (m == 0 || n == 0) return OZLU_OK;
     DevTable tab;
-    int Kpad = 0;
-    int rc = plan_noalloc(p, k, tab, Kpad);
+    int Kpad = 0, pint_bits = 0;
+    int rc = plan_noalloc(p, k, tab, Kpad, &pint_bits);
     if (rc) return rc;
     ConvTab conv;
     fill_conv(tab, conv);
+    CrtTab crt;
+    fill_crt(tab, pint_bits, crt);
     const int Mpad = (m + 127) / 128 * 128, Npad = (n + 127) / 128 * 128;
     size_t off = 0;
     const size_t o_mu = off; off = up256(off + sizeof(int) * (size_t)m);
@@ -130,6 +132,6 @@ extern "C" int ozlu_gemm_noalloc(int nc, int p, int m, int n, int k, int alpha, 
     launch_shifts(A, lda, m, B, ldb, n, nc, k, tab.Q, mu, nu, nullptr, s);
     launch_convert(A, lda, m, B, ldb, n, nc, k, mu, nu, conv, Kpad, Mpad, Npad, RA, RB, 0, s);
     launch_gemm_imma(RA, RB, m, n, Mpad, Npad, Kpad, tab, T, s);
-    launch_crt(T, false, m, n, mu, nu, tab, nc, alpha, beta, C, ldc, s);
+    launch_crt(T, false, m, n, mu, nu, crt, nc, alpha, beta, C, ldc, s);
     return cudaGetLastError() == cudaSuccess ? OZLU_OK : OZLU_ERR_CUDA;
 }

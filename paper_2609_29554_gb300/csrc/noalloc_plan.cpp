@@ -50,7 +50,7 @@ int inv_mod_na(int a, int m) {
 }  // namespace
 
 // INT8 plan of Sec. 3.2 into a DevTable, fixed-size arrays only
-int plan_noalloc(int p, int K, DevTable& t, int& Kpad_out) {
+int plan_noalloc(int p, int K, DevTable& t, int& Kpad_out, int* pint_out) {
     memset(&t, 0, sizeof t);
     if (p < 1 || K < 1) return OZLU_ERR_CAPACITY;
     int mods[64];
@@ -111,6 +111,7 @@ int plan_noalloc(int p, int K, DevTable& t, int& Kpad_out) {
         }
         for (int wd = 0; wd < MAXWG; ++wd) t.Plow[wd] = wd < PW ? P[wd] : 0u;
         Kpad_out = Kpad;
+        if (pint_out) *pint_out = pint_bits;
         return OZLU_OK;
     }
     return OZLU_ERR_CAPACITY;

@@ -22,12 +22,16 @@ struct PlanEntry {
     Plan plan;
     DevTable table;
     ConvTab conv;
+    CrtTab crt;
+    GemmTab gemm;  // tensor-core epilogue
 };
 
 // byte offsets of the last ozlu_gemm's intermediates inside the workspace
 struct GemmLayout {
     int m = 0, n = 0, k = 0, Mpad = 0, Npad = 0, Kpad = 0, N = 0, S = 0, G = 0, backend = 0;
     size_t mu = 0, nu = 0, ra = 0, rb = 0, t = 0;
+    bool pack = false;         // t values packed by triples of moduli
+    int mod[MAXMOD] = {0};
 };
 
 }  // namespace ozlu

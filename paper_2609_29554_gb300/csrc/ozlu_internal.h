@@ -91,10 +91,11 @@ void build_ext_image(const Plan& pl, ExtImage& img);
 void fill_table(const Plan& pl, DevTable& t);
 // the allocation-free GEMM's planner: the INT8 plan straight into a table,
 // fixed-size arrays only (no host allocation)
-int plan_noalloc(int p, int K, DevTable& t, int& Kpad);
+int plan_noalloc(int p, int K, DevTable& t, int& Kpad, int* pint_bits = nullptr);
 
 // ---------------------------------------------------------------- kernels --
 struct ConvTab;  // tables.h
+struct CrtTab;
 
 // (S1) shared exponents: mu[i] over rows of A (m x k), nu[j] over columns of B
 // (k x n); `clear`: a device error word to zero, or null.
@@ -111,9 +112,12 @@ void launch_convert(const double* A, long long lda, int m, const double* B, long
 // the binary64 back-end's residues (8-byte) of one operand
 void launch_convert64(const double* X, long long ld, int nc, int rows, int cols, bool is_b, const int* shifts,
                       const DevTable& tab, int Kpad, int Rpad, double* planes, cudaStream_t s);
-// (S4) on tcgen05: FP8 base-17 Karatsuba (fp8 = true) or FP16 residues
-int launch_gemm_tc05(bool fp8, const void* RA, const void* RB, int m, int n, int Mpad, int Npad,
-                     int Kpad, const DevTable& tab, uint8_t* T, int* err, cudaStream_t s);
+struct GemmTab;
+// (S4) on tcgen05: FP8 base-17 Karatsuba (fp8 = true) or FP16 residues, t values
+// as bytes or packed by triples; tc05_packs: the layout to take for a product
+bool tc05_packs(const GemmTab& tab, int Mpad, int Npad);
+int launch_gemm_tc05(bool fp8, bool pack, const void* RA, const void* RB, int m, int n, int Mpad, int Npad, int Kpad,
+                     const GemmTab& tab, void* T, int* err, cudaStream_t s);
 // (S4)+(S5 t_l) INT8 residue GEMMs with the modular epilogue; T[gi][l][j][i].
 void launch_gemm_imma(const int8_t* RA, const int8_t* RB, int m, int n, int Mpad,
                       int Npad, int Kpad, const DevTable& tab, uint8_t* T,
@@ -130,9 +134,12 @@ void launch_gemm_imma_ext(const int8_t* RA, const int8_t* RB, int m, int n, int 
 void launch_gemm_f64(const double* RA, const double* RB, int m, int n, int Mpad, int Npad, int Kpad,
                      const DevTable& tab, uint32_t* T, cudaStream_t s);
 // (S5)+(S6): CRT per digit group, recombination, fused beta*C + alpha*AB, rounding.
-// t values are bytes (INT8/FP8/FP16 moduli <= 255) or 32-bit words (t32, binary64).
-void launch_crt(const void* T, bool t32, int m, int n, const int* mu, const int* nu,
-                const DevTable& tab, int nc, int alpha, int beta, double* C,
-                long long ldc, cudaStream_t s);
+// t values are bytes, T[gi][l][j][i], or packed by triples of moduli (CrtTab),
+// 32-bit words T[gi][q][j][i].
+void launch_crt(const void* T, bool pack, int m, int n, const int* mu, const int* nu, const CrtTab& tab, int nc,
+                int alpha, int beta, double* C, long long ldc, cudaStream_t s);
+// the binary64 back-end: t values as 32-bit words
+void launch_crt64(const uint32_t* T, int m, int n, const int* mu, const int* nu, const DevTable& tab, int nc,
+                  int alpha, int beta, double* C, long long ldc, cudaStream_t s);
 
 }  // namespace ozlu
