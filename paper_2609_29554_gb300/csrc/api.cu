@@ -242,32 +242,6 @@ int autotune(ozlu_handle* h, int nc, int p, int m, int n, int k, const double* A
 
 // The device part of one GEMM, all pointers on the device.
 
-cudaStream_t side_fork(ozlu_handle* h, cudaStream_t s) {
-    // the first call outside a capture creates the stream and its events
-    if (!h->side && !h->capturing) {
-        if (cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking) != cudaSuccess ||
-            cudaEventCreateWithFlags(&h->side_fork, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&h->side_join, cudaEventDisableTiming) != cudaSuccess) {
-            cudaGetLastError();
-            if (h->side) cudaStreamDestroy(h->side);
-            if (h->side_fork) cudaEventDestroy(h->side_fork);
-            h->side = nullptr;
-            h->side_fork = nullptr;
-            h->side_join = nullptr;
-        }
-    }
-    if (h->side && cudaEventRecord(h->side_fork, s) == cudaSuccess &&
-        cudaStreamWaitEvent(h->side, h->side_fork, 0) == cudaSuccess)
-        return h->side;
-    cudaGetLastError();
-    return s;
-}
-
-bool side_join(ozlu_handle* h, cudaStream_t s, cudaStream_t side) {
-    if (side == s) return true;
-    return cudaEventRecord(h->side_join, side) == cudaSuccess && cudaStreamWaitEvent(s, h->side_join, 0) == cudaSuccess;
-}
-
 int gemm_device(ozlu_handle* h, int nc, int p, int m, int n, int k, int alpha, const double* A,
                 long long lda, const double* B, long long ldb, int beta, double* C,
                 long long ldc, const ozlu_opts* opts) {
@@ -444,9 +418,6 @@ int ozlu_destroy(ozlu_handle* h) {
     }
     if (h->fork) cudaEventDestroy(h->fork);
     if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
-    if (h->side) cudaStreamDestroy(h->side);
-    if (h->side_fork) cudaEventDestroy(h->side_fork);
-    if (h->side_join) cudaEventDestroy(h->side_join);
     if (h->dev_err) cudaFree(h->dev_err);
     for (auto& e : h->ext_plans)
         if (e.second.dev) cudaFree(e.second.dev);

@@ -23,16 +23,15 @@
 #include <limits.h>
 #include <string.h>
 
-#include <cuda_fp8.h>
 #include <math.h>
 
+#include "conv_device.cuh"
 #include "mp_device.cuh"
 #include "ozlu_handle.h"
 
 namespace ozlu {
 namespace {
 
-constexpr int MPD = 9;      // words of one digit with its carry (w <= 254)
 constexpr int MPCT = 64;    // threads per block of the CRT kernel
 
 struct MPView {
@@ -61,316 +60,152 @@ __device__ __forceinline__ uint32_t mant32(const MPView& X, long long x, long lo
     return r ? (lo >> r) | (hi << (32 - r)) : lo;
 }
 
-// (S1) shared exponents over rows (is_col = 0: row a, h < len) or columns
-__global__ void mp_shift_kernel(MPView X, int count, int len, int is_col, int Q, int* out) {
-    const int a = blockIdx.x * blockDim.x + threadIdx.x;
-    if (a >= count) return;
-    int emax = INT_MIN;
-    for (int h = 0; h < len; ++h) {
-        const long long x = is_col ? (long long)h + (long long)a * X.ld : (long long)a + (long long)h * X.ld;
-        if (!mp_zero(X, x)) emax = max(emax, X.exps[x]);
-    }
-    out[a] = emax == INT_MIN ? 0 : (Q - 1) - emax;
-}
-
-// centered residue of sign * mag modulo m_l, mag < 2^(16 H)
-template <int H>
-__device__ __forceinline__ int mp_residue(const uint32_t (&mag)[MPD], bool neg, const DevTable& tab, int l) {
-    const uint32_t m = (uint32_t)tab.mod[l];
-    uint32_t acc = 0;
-#pragma unroll
-    for (int j = 0; j < H; ++j) acc += ((mag[j >> 1] >> (16 * (j & 1))) & 0xffffu) * tab.pow16[l][j];
-    uint32_t r = mod_small(acc, m, tab.magic[l]);
-    if (neg && r) r = m - r;
-    int c = (int)r;
-    if (c > (int)(m - 1) / 2) c -= (int)m;
-    return c;
-}
-
-// (S2)+(S3): one element per thread; A side: element (r, h), B side: (h, r);
-// planes [l][t][r][h] (Rpad x Kpad), h < Kc only: the K padding is zeroed by
-// the host beforehand and the padded rows are left untouched (they only
-// reach discarded outputs).  A threads run along r (consecutive elements of
-// a column), B threads along h.
-template <int H>
-__global__ void __launch_bounds__(256) mp_convert_kernel(MPView X, int R, int Kc, int is_b,
-                                                         const int* __restrict__ shifts,
-                                                         const __grid_constant__ DevTable tab, int Kpad,
-                                                         int Rpad, int8_t* __restrict__ planes) {
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)R * Kc) return;
-    const int r = is_b ? (int)(idx / Kc) : (int)(idx % R);
-    const int h = is_b ? (int)(idx % Kc) : (int)(idx / R);
-    const size_t plane = (size_t)Rpad * Kpad, off = (size_t)r * Kpad + h;
-    const int S = tab.S, w = tab.w;
-    const long long x = is_b ? (long long)h + (long long)r * X.ld : (long long)r + (long long)h * X.ld;
-    if (mp_zero(X, x)) {
-        for (int l = 0; l < tab.N; ++l)
-            for (int t = 0; t < S; ++t) planes[(size_t)(l * S + t) * plane + off] = 0;
-        return;
-    }
-    const bool neg = X.signs[x] != 0;
-    // bit b of |X| = trunc(|a| 2^mu) is bit b + sh of the magnitude
-    const long long sh = 32LL * X.L - X.exps[x] - shifts[r];
-    const int nw = (w + 2 + 31) >> 5;
-    uint32_t carry = 0;
-    for (int t = 0; t < S; ++t) {
-        uint32_t D[MPD];
-#pragma unroll
-        for (int k = 0; k < MPD; ++k) D[k] = k < nw ? mant32(X, x, (long long)t * w + 32 * k + sh) : 0u;
-        mask_below<MPD>(D, w);
-        uint64_t c = carry;
-#pragma unroll
-        for (int k = 0; k < MPD; ++k) {
-            const uint64_t s = (uint64_t)D[k] + c;
-            D[k] = (uint32_t)s;
-            c = s >> 32;
-        }
-        // u = D <= 2^w; X >= 0: u >= 2^(w-1) gives the digit u - 2^w;
-        // X < 0: u > 2^(w-1) gives 2^w - u, else -u (Eq. (2) on the signed X)
-        bool dneg = neg;
-        if (t < S - 1) {
-            const bool ge = bit_at<MPD>(D, w - 1) || bit_at<MPD>(D, w);
-            const bool half = bit_at<MPD>(D, w - 1) && !bit_at<MPD>(D, w) && !any_below<MPD>(D, w - 1);
-            const bool wrap = neg ? (ge && !half) : ge;
-            if (wrap) {
-                complement_below<MPD>(D, w);
-                dneg = !neg;
-                carry = 1;
-            } else {
-                carry = 0;
+// (S1) of both operands in one launch: blocks [0, blocks_a) take 32 rows of A
+// each (32 warps share the columns), the others 32 columns of B, one a warp.
+// Four elements in flight per thread; one thread walking a whole row took
+// about a load latency per element.
+__global__ void __launch_bounds__(1024) mp_shift_kernel(MPView A, int m, MPView B, int n, int k, int Q, int* mu,
+                                                         int* nu, int blocks_a) {
+    __shared__ int red[32][33];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int E = INT_MIN;
+    if ((int)blockIdx.x < blocks_a) {
+        const int i = blockIdx.x * 32 + lane;
+        if (i < m) {
+#pragma unroll 4
+            for (int h = warp; h < k; h += 32) {
+                const long long x = (long long)i + (long long)h * A.ld;
+                const int ex = A.exps[x];
+                if (!mp_zero(A, x)) E = max(E, ex);
             }
         }
-        for (int l = 0; l < tab.N; ++l)
-            planes[(size_t)(l * S + t) * plane + off] = (int8_t)mp_residue<H>(D, dneg, tab, l);
-    }
-}
-
-// (S2)+(S3), one warp per element: the element's limbs are staged in shared
-// memory once, lane t forms the raw bits of digit t (bits [t w, (t + 1) w) of
-// |X|, X = trunc(a 2^mu)) with the flags the balanced digits need, lane 0
-// resolves the carries from digit to digit in order (Eq. (2): a digit that
-// reaches 2^(w-1) wraps to D - 2^w, for negative X to 2^w - D, and carries
-// one into the next), and the lanes then take the (digit, modulus) pairs:
-// residue of the raw digit by 16-bit chunks, plus the carry, the wrap
-// applied to the residue, the sign, centered.  The same planes as
-// mp_convert_kernel, whose single thread per element runs the limb loads and
-// the S N residues in sequence; this form keeps narrow products (a few
-// elements) from being latency-bound.
-constexpr int CW = 8;  // warps per block of mp_convert_warp_kernel
-
-__device__ __forceinline__ uint32_t sm_bits32(const uint32_t* lm, int L, long long pos) {
-    if (pos >= 32LL * L || pos <= -32) return 0;
-    const long long q = pos >= 0 ? (pos >> 5) : -((-pos + 31) >> 5);
-    const int r = (int)(pos - 32 * q);
-    const uint32_t lo = (q >= 0 && q < L) ? lm[q] : 0u;
-    const uint32_t hi = (q + 1 >= 0 && q + 1 < L) ? lm[q + 1] : 0u;
-    return r ? (lo >> r) | (hi << (32 - r)) : lo;
-}
-
-template <int H>
-__global__ void __launch_bounds__(32 * CW) mp_convert_warp_kernel(MPView X, int R, int Kc, int is_b,
-                                                                  const int* __restrict__ shifts,
-                                                                  const __grid_constant__ DevTable tab, int Kpad,
-                                                                  int Rpad, int8_t* __restrict__ planes,
-                                                                  int per_warp) {
-    extern __shared__ uint32_t wsm[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long task = (long long)blockIdx.x * CW + warp;
-    if (task >= (long long)R * Kc) return;
-    const int r = is_b ? (int)(task / Kc) : (int)(task % R);
-    const int h = is_b ? (int)(task % Kc) : (int)(task / R);
-    const size_t plane = (size_t)Rpad * Kpad, off = (size_t)r * Kpad + h;
-    const int S = tab.S, w = tab.w, N = tab.N, L = X.L;
-    const long long x = is_b ? (long long)h + (long long)r * X.ld : (long long)r + (long long)h * X.ld;
-    if (mp_zero(X, x)) {
-        for (int q = lane; q < N * S; q += 32) planes[(size_t)q * plane + off] = 0;
-        return;
-    }
-    uint32_t* lm = wsm + (size_t)warp * per_warp;  // L limbs
-    uint32_t* dw = lm + L;                         // S digits x MPD words
-    uint32_t* fl = dw + S * MPD;                   // S flag words
-    for (int k = lane; k < L; k += 32) lm[k] = X.limbs[(long long)k * X.plane + x];
-    __syncwarp();
-    const bool neg = X.signs[x] != 0;
-    const long long sh = 32LL * L - X.exps[x] - shifts[r];
-    const int nw = (w + 31) >> 5;
-    for (int t = lane; t < S; t += 32) {
-        bool lowzero = true, lowones = true;
-        uint32_t top = 0;
+        red[warp][lane] = E;
+        __syncthreads();
+        if (warp == 0 && i < m) {
 #pragma unroll
-        for (int k = 0; k < MPD; ++k) {
-            uint32_t v = k < nw ? sm_bits32(lm, L, (long long)t * w + 32 * k + sh) : 0u;
-            const int hib = w - 32 * k;
-            if (hib < 32) v = hib > 0 ? (v & ((1u << hib) - 1u)) : 0u;
-            dw[t * MPD + k] = v;
-            const int lim = w - 1 - 32 * k;
-            if (lim >= 32) {
-                lowzero &= v == 0;
-                lowones &= v == 0xffffffffu;
-            } else if (lim >= 0) {
-                const uint32_t msk = lim ? (1u << lim) - 1u : 0u;
-                lowzero &= (v & msk) == 0;
-                lowones &= (v & msk) == msk;
-                top = (v >> lim) & 1u;
-            }
+            for (int r = 1; r < 32; ++r) E = max(E, red[r][lane]);
+            mu[i] = E == INT_MIN ? 0 : (Q - 1) - E;
         }
-        fl[t] = top | (lowzero ? 2u : 0u) | (lowones ? 4u : 0u);
-    }
-    __syncwarp();
-    if (lane == 0) {
-        uint32_t carry = 0;
-        for (int t = 0; t < S; ++t) {
-            const uint32_t f = fl[t];
-            const bool top = f & 1u, lz = (f >> 1) & 1u, lo = (f >> 2) & 1u;
-            bool wrap = false;
-            if (t < S - 1) {
-                const bool ge = top || (carry && lo);
-                const bool half = carry ? (!top && lo) : (top && lz);
-                wrap = neg ? (ge && !half) : ge;
-            }
-            const bool dneg = wrap ? !neg : neg;
-            fl[t] = (carry << 3) | (wrap ? 16u : 0u) | (dneg ? 32u : 0u);
-            carry = wrap ? 1u : 0u;
+    } else {
+        const int j = ((int)blockIdx.x - blocks_a) * 32 + warp;
+        if (j >= n) return;
+#pragma unroll 4
+        for (int h = lane; h < k; h += 32) {
+            const long long x = (long long)h + (long long)j * B.ld;
+            const int ex = B.exps[x];
+            if (!mp_zero(B, x)) E = max(E, ex);
         }
-    }
-    __syncwarp();
-    for (int q = lane; q < N * S; q += 32) {
-        const int t = q / N, l = q - t * N;
-        const uint32_t m = (uint32_t)tab.mod[l], mg = tab.magic[l];
-        uint32_t acc = 0;
-#pragma unroll
-        for (int j = 0; j < H; ++j) acc += ((dw[t * MPD + (j >> 1)] >> (16 * (j & 1))) & 0xffffu) * tab.pow16[l][j];
-        uint32_t v = mod_small(acc, m, mg);
-        const uint32_t f = fl[t];
-        v = mod_small(v + ((f >> 3) & 1u), m, mg);
-        if ((f >> 4) & 1u) {
-            const uint32_t pw = mod_small(tab.pow16[l][w >> 4] << (w & 15), m, mg);  // 2^w mod m
-            v = mod_small(pw + m - v, m, mg);
-        }
-        if (((f >> 5) & 1u) && v) v = m - v;
-        int c = (int)v;
-        if (c > (int)(m - 1) / 2) c -= (int)m;
-        planes[(size_t)(l * S + t) * plane + off] = (int8_t)c;
+        E = __reduce_max_sync(0xffffffffu, E);
+        if (lane == 0) nu[j] = E == INT_MIN ? 0 : (Q - 1) - E;
     }
 }
 
-// (S2)+(S3) in plane order: a block takes 32 consecutive positions f of the
-// planes (f = r Kp + h, the K padding included), its 8 warps each form the
-// residues of 4 of them as mp_convert_warp_kernel does (a padding position or
-// a zero element gives zeros) into a shared tile [plane][32], and the block
-// then writes every plane's 32 bytes at once, contiguous.  With Kp = K
-// (unpadded planes of a small-K product) consecutive rows are adjacent, so
-// narrow operands are written as densely as wide ones.
-constexpr int TW = 8;  // warps per block of mp_convert_tile_kernel
+// (S2)+(S3) of both operands: a thread takes E consecutive positions h of one
+// plane row (A side: elements (r, h), B side: (h, r)), reads the words of one
+// digit of |X| = trunc(|a| 2^mu) at a time from the limbs (bits [t w, t w + w),
+// plus the carry; Eq. (2): X >= 0 wraps from 2^(w-1) on, X < 0 above it) and
+// forms its residues for all moduli by four-byte dot products, as the
+// conversion of expansions does.  A negative element's digit enters as its
+// complement with a constant per modulus (ConvMod::k4, picked by a one-hot
+// dot product).  Bound by integer issue.  A block covers eight consecutive rows,
+// so that the limb sectors of A's columns are shared in L1.
+// 512 x 512 each, p = 1024, FP8 digits: @@@ us with the exponents; the former
+// kernel (a warp per element, a lane per residue, the table in constant memory
+// read at 32 addresses at once) 3836 us.
+// E = 4 where that leaves two blocks of 256 threads per SM, else E = 1 and the
+// moduli split over gridDim.y (digits formed again in each slice).
+struct MpConvArgs {
+    MPView A, B;
+    const int* mu;
+    const int* nu;
+    int8_t* RA;
+    int8_t* RB;
+    int m, n, K, Kp, Mpad, Npad;
+    int blocks_a;  // blocks of the A side; the B side follows
+    int hb;        // blocks along h (a warp's lanes cover `lanes_h` position groups)
+    int lanes_h;   // power of two <= 32; a warp covers 32 / lanes_h rows
+    int lper;      // moduli per gridDim.y slice
+};
 
-template <int H, bool FP8>
-__global__ void __launch_bounds__(32 * TW) mp_convert_tile_kernel(MPView X, int R, int Kc, int is_b,
-                                                                  const int* __restrict__ shifts,
-                                                                  const __grid_constant__ DevTable tab, int Kp,
-                                                                  int Rpad, int8_t* __restrict__ planes,
-                                                                  int per_warp) {
-    extern __shared__ uint32_t tsm[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int S = tab.S, w = tab.w, N = tab.N, L = X.L, NS = N * S;
-    int8_t* tile = reinterpret_cast<int8_t*>(tsm);                           // [NS][32]
-    uint32_t* lm = tsm + (NS * 32 + 3) / 4 + (size_t)warp * per_warp;       // L limbs
-    uint32_t* dw = lm + L;                                                   // S x MPD digit words
-    uint32_t* fl = dw + S * MPD;                                             // S flag words
-    const long long f0 = (long long)blockIdx.x * 32;
-    const long long total = (long long)R * Kp;
-    for (int e = warp; e < 32; e += TW) {
-        const long long f = f0 + e;
-        const int r = (int)(f / Kp), h = (int)(f - (long long)r * Kp);
+template <int NW, bool FP8, int E>
+__global__ void __launch_bounds__(256) mp_convert_kernel(const __grid_constant__ MpConvArgs a,
+                                                         const __grid_constant__ ConvTab tab) {
+    const bool is_b = (int)blockIdx.x >= a.blocks_a;
+    const int bid = (int)blockIdx.x - (is_b ? a.blocks_a : 0);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int per = 32 / a.lanes_h;  // rows per warp
+    const int r = (bid / a.hb) * (8 * per) + warp * per + lane / a.lanes_h;
+    const int h0 = ((bid % a.hb) * a.lanes_h + (lane & (a.lanes_h - 1))) * E;
+    if (r >= (is_b ? a.n : a.m) || h0 >= a.Kp) return;
+    const MPView& X = is_b ? a.B : a.A;
+    const int shift = is_b ? a.nu[r] : a.mu[r];
+    const size_t plane = (size_t)(is_b ? a.Npad : a.Mpad) * a.Kp;
+    const size_t off = (size_t)r * a.Kp + h0;
+    const int L = X.L, S = tab.S, w = tab.w;
+    const uint32_t* lp[E];
+    int sh[E];          // bit b of |X| is bit b + sh of the magnitude
+    bool neg[E], live[E];
+    uint32_t carry[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int h = h0 + e;
         const long long x = is_b ? (long long)h + (long long)r * X.ld : (long long)r + (long long)h * X.ld;
-        if (f >= total || h >= Kc || mp_zero(X, x)) {
-            for (int q = lane; q < NS; q += 32) tile[q * 32 + e] = 0;
-            continue;
-        }
-        for (int k = lane; k < L; k += 32) lm[k] = X.limbs[(long long)k * X.plane + x];
-        __syncwarp();
-        const bool neg = X.signs[x] != 0;
-        const long long sh = 32LL * L - X.exps[x] - shifts[r];
-        const int nw = (w + 31) >> 5;
-        for (int t = lane; t < S; t += 32) {
-            bool lowzero = true, lowones = true;
-            uint32_t top = 0;
-#pragma unroll
-            for (int k = 0; k < MPD; ++k) {
-                uint32_t v = k < nw ? sm_bits32(lm, L, (long long)t * w + 32 * k + sh) : 0u;
-                const int hib = w - 32 * k;
-                if (hib < 32) v = hib > 0 ? (v & ((1u << hib) - 1u)) : 0u;
-                dw[t * MPD + k] = v;
-                const int lim = w - 1 - 32 * k;
-                if (lim >= 32) {
-                    lowzero &= v == 0;
-                    lowones &= v == 0xffffffffu;
-                } else if (lim >= 0) {
-                    const uint32_t msk = lim ? (1u << lim) - 1u : 0u;
-                    lowzero &= (v & msk) == 0;
-                    lowones &= (v & msk) == msk;
-                    top = (v >> lim) & 1u;
-                }
-            }
-            fl[t] = top | (lowzero ? 2u : 0u) | (lowones ? 4u : 0u);
-        }
-        __syncwarp();
-        if (lane == 0) {
-            uint32_t carry = 0;
-            for (int t = 0; t < S; ++t) {
-                const uint32_t fg = fl[t];
-                const bool top = fg & 1u, lz = (fg >> 1) & 1u, lo = (fg >> 2) & 1u;
-                bool wrap = false;
-                if (t < S - 1) {
-                    const bool ge = top || (carry && lo);
-                    const bool half = carry ? (!top && lo) : (top && lz);
-                    wrap = neg ? (ge && !half) : ge;
-                }
-                const bool dneg = wrap ? !neg : neg;
-                fl[t] = (carry << 3) | (wrap ? 16u : 0u) | (dneg ? 32u : 0u);
-                carry = wrap ? 1u : 0u;
-            }
-        }
-        __syncwarp();
-        for (int q = lane; q < NS; q += 32) {
-            const int l = q / S, t = q - l * S;  // plane q = l S + t
-            const uint32_t m = (uint32_t)tab.mod[l], mg = tab.magic[l];
-            uint32_t acc = 0;
-#pragma unroll
-            for (int j = 0; j < H; ++j) acc += ((dw[t * MPD + (j >> 1)] >> (16 * (j & 1))) & 0xffffu) * tab.pow16[l][j];
-            uint32_t v = mod_small(acc, m, mg);
-            const uint32_t fg = fl[t];
-            v = mod_small(v + ((fg >> 3) & 1u), m, mg);
-            if ((fg >> 4) & 1u) {
-                const uint32_t pw = mod_small(tab.pow16[l][w >> 4] << (w & 15), m, mg);  // 2^w mod m
-                v = mod_small(pw + m - v, m, mg);
-            }
-            if (((fg >> 5) & 1u) && v) v = m - v;
-            int c = (int)v;
-            if (c > (int)(m - 1) / 2) c -= (int)m;
-            tile[q * 32 + e] = (int8_t)c;
-        }
-        __syncwarp();
+        live[e] = h < a.K && !mp_zero(X, x);
+        lp[e] = X.limbs + x;
+        neg[e] = live[e] && X.signs[x] != 0;
+        // far outside the magnitude every bit is zero: the clamp keeps 32-bit positions
+        const long long s = live[e] ? 32LL * L - X.exps[x] - shift : 0LL;
+        sh[e] = (int)(s > 32LL * L ? 32LL * L : (s < -(1 << 29) ? -(1 << 29) : s));
+        carry[e] = 0;
     }
-    __syncthreads();
-    // plane q: positions f0 .. f0 + 31, rows of Rpad x Kp (rows beyond R are not written);
-    // FP8: the residue r as its balanced base-17 digits in E4M3 (Eq. (15)),
-    // planes 3 q + 0, 1, 2 holding d0, d1, d0 + d1
-    const size_t plane = (size_t)Rpad * Kp;
-    for (int idx = threadIdx.x; idx < NS * 32; idx += 32 * TW) {
-        const int q = idx >> 5, e = idx & 31;
-        const long long f = f0 + e;
-        if (f >= total) continue;
-        const int r = tile[q * 32 + e];
-        if (!FP8) {
-            planes[(size_t)q * plane + f] = (int8_t)r;
-        } else {
-            const int d1 = (2 * r + 17 + 238) / 34 - 7;  // round(r / 17), never a tie (17 is odd)
-            const int d0 = r - 17 * d1;
-            uint8_t* p8 = reinterpret_cast<uint8_t*>(planes) + (size_t)(3 * q) * plane + f;
-            p8[0] = (uint8_t)__nv_cvt_float_to_fp8((float)d0, __NV_SATFINITE, __NV_E4M3);
-            p8[plane] = (uint8_t)__nv_cvt_float_to_fp8((float)d1, __NV_SATFINITE, __NV_E4M3);
-            p8[2 * plane] = (uint8_t)__nv_cvt_float_to_fp8((float)(d0 + d1), __NV_SATFINITE, __NV_E4M3);
+    const int l0 = blockIdx.y * a.lper, l1 = min(tab.N, l0 + a.lper);
+    const uint32_t mk = (1u << (w - 32 * (NW - 1))) - 1u;  // bits of the digit's last word below w
+    for (int t = 0; t < S; ++t) {
+        uint32_t D[E][NW], f[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int pos = t * w + sh[e];
+            const int q = pos >> 5, rr = pos & 31;
+            uint32_t v = live[e] && q >= 0 && q < L ? __ldg(lp[e] + (long long)q * X.plane) : 0u;
+            uint64_t c = carry[e];
+            bool lowzero = true;
+#pragma unroll
+            for (int i = 0; i < NW; ++i) {
+                const int qn = q + i + 1;
+                const uint32_t nx = live[e] && qn >= 0 && qn < L ? __ldg(lp[e] + (long long)qn * X.plane) : 0u;
+                uint32_t d = __funnelshift_r(v, nx, rr);
+                v = nx;
+                if (i == NW - 1) d &= mk;
+                c += d;
+                D[e][i] = (uint32_t)c;
+                c >>= 32;
+            }
+            uint32_t hi = 0, half = 0;  // bits w - 1 and w; bit w - 1 alone
+#pragma unroll
+            for (int i = 0; i < NW; ++i) {
+                const int lim = w - 1 - 32 * i;  // bits of this word below w - 1
+                if (lim >= 32) {
+                    lowzero &= D[e][i] == 0;
+                } else if (lim >= 0) {
+                    lowzero &= (D[e][i] & ((1u << lim) - 1u)) == 0;
+                    half = (D[e][i] >> lim) & 1u;
+                    hi |= half;
+                }
+                if (i == (w >> 5)) hi |= (D[e][i] >> (w & 31)) & 1u;
+            }
+            const bool wrap = t < S - 1 && hi && !(neg[e] && half && lowzero);
+            carry[e] = wrap ? 1u : 0u;
+            f[e] = 1u << (8 * ((neg[e] ? 2 : 0) + (wrap ? 1 : 0)));
+            const uint32_t msk = neg[e] ? 0xffffffffu : 0u;
+#pragma unroll
+            for (int i = 0; i < NW; ++i) D[e][i] ^= msk;
+        }
+        for (int l = l0; l < l1; ++l) {
+            const ConvMod& M = tab.mod[l];
+            uint32_t res[E];
+#pragma unroll
+            for (int e = 0; e < E; ++e) res[e] = conv_residue<NW>(D[e], M, __dp4a(f[e], M.k4, M.half));
+            store_residues<FP8 ? 1 : 0, E>(is_b ? a.RB : a.RA, (size_t)(l * S + t), plane, off, M, res);
         }
     }
 }
@@ -770,155 +605,300 @@ void zero_k_padding(int8_t* planes, long long count, int R, int Rpad, int Kc, in
     cudaMemset2DAsync(planes + Kc, Kpad, 0, Kpad - Kc, (size_t)count * Rpad, s);
 }
 
-// (S5)+(S6) for few outputs: one warp per output, the lanes forming the S_g of
-// different digit groups in parallel (the N WG word products of each),
-// then lane 0 adds them into the NW-word accumulator through the same short
-// window as mp_crt_kernel and finishes with mp_finish.
-constexpr int CWC = 4;  // warps per block of mp_crt_warp_kernel
+// (S5)+(S6), one warp per output.  The lanes share the triples of each digit
+// group (partial word sums combined by shuffles), then every step on the
+// NW-word window is a pass over 32 words at a time with the carries of a pass
+// resolved by one addition on the lanes' generate and propagate ballots: the
+// S_g placed at bit w (g - g0) as unsigned word sums less their sign words, the
+// old C, the negation, the rounding.  The former kernels ran those passes on
+// one thread (about 20 us for 80 words).
+constexpr int CWC = 4;  // warps per block
+// outputs below which a warp takes each (above, a thread each: mp_crt_kernel)
+#ifndef MP_WARP_CRT_N
+#define MP_WARP_CRT_N 16384
+#endif
+constexpr long long MP_WARP_CRT = MP_WARP_CRT_N;
+
+struct MpCrtArgs {
+    const uint8_t* T;
+    const int* mu;
+    const int* nu;
+    long long mn;
+    int m, j0, NW, alpha, beta, p;
+    MPView C;
+};
+
+// A[k] = A[k] + b(k) + carry over words [0, NW) of the warp's window
+template <class F>
+__device__ __forceinline__ void warp_add(uint32_t* A, int NW, int lane, uint32_t cin, F b) {
+    for (int k0 = 0; k0 < NW; k0 += 32) {
+        const int k = k0 + lane;
+        const uint32_t x = k < NW ? A[k] : 0u, s = k < NW ? x + b(k, x) : 0u;
+        const uint32_t G = __ballot_sync(0xffffffffu, s < x), P = __ballot_sync(0xffffffffu, s == 0xffffffffu);
+        const uint64_t t = (uint64_t)P + (((uint64_t)G << 1) | cin);
+        const uint32_t in = (uint32_t)t ^ P;  // carry into each lane's word
+        if (k < NW) A[k] = s + ((in >> lane) & 1u);
+        cin = (uint32_t)(t >> 32) & 1u;
+    }
+    __syncwarp();
+}
+
+// A = -A
+__device__ __forceinline__ void warp_negate(uint32_t* A, int NW, int lane) {
+    // -A = ~A + 1, as a sum of ~A and 0 (the sum of a word and b is ~word)
+    for (int k = lane; k < NW; k += 32) A[k] = ~A[k];
+    __syncwarp();
+    warp_add(A, NW, lane, 1u, [](int, uint32_t) { return 0u; });
+}
+
+__device__ __forceinline__ int warp_bitlen(const uint32_t* A, int NW, int lane) {
+    for (int k0 = (NW - 1) & ~31; k0 >= 0; k0 -= 32) {
+        const uint32_t x = k0 + lane < NW ? A[k0 + lane] : 0u;
+        const uint32_t nz = __ballot_sync(0xffffffffu, x != 0);
+        if (nz) {
+            const int k = 31 - __clz((int)nz);
+            return 32 * (k0 + k) + 32 - __clz((int)__shfl_sync(0xffffffffu, x, k));
+        }
+    }
+    return 0;
+}
+
+// bits [pos, pos + 32), pos >= -31 (zeros outside)
+__device__ __forceinline__ uint32_t win_bits(const uint32_t* A, int NW, long long pos) {
+    const long long q = pos >> 5;
+    const int r = (int)(pos & 31);
+    const uint32_t lo = q >= 0 && q < NW ? A[q] : 0u, hi = q + 1 >= 0 && q + 1 < NW ? A[q + 1] : 0u;
+    return __funnelshift_r(lo, hi, r);
+}
 
 template <int WG>
-__global__ void __launch_bounds__(32 * CWC) mp_crt_warp_kernel(const uint8_t* __restrict__ T, int m, int nchunk,
-                                                               int j0, const int* __restrict__ mu,
-                                                               const int* __restrict__ nu,
-                                                               const __grid_constant__ DevTable tab, int NW,
-                                                               int alpha, int beta, MPView C, int p) {
+__global__ void __launch_bounds__(32 * CWC) mp_crt_warp_kernel(const __grid_constant__ MpCrtArgs a,
+                                                               const __grid_constant__ CrtTab tab) {
     extern __shared__ uint32_t cwsm[];
+    __shared__ uint32_t sM[MAXTRI][WG];  // P / m_q (lanes read different triples)
+    __shared__ uint32_t sc[3 * MAXTRI];
+    __shared__ float si[MAXTRI];
+    for (int i = threadIdx.x; i < tab.NT * WG; i += 32 * CWC) sM[i / WG][i % WG] = tab.Mt[i / WG][i % WG];
+    for (int i = threadIdx.x; i < 3 * tab.NT; i += 32 * CWC) sc[i] = tab.coef[i];
+    for (int i = threadIdx.x; i < tab.NT; i += 32 * CWC) si[i] = tab.inv[i];
+    __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long e = (long long)blockIdx.x * CWC + warp;
-    const long long mn = (long long)m * nchunk;
-    if (e >= mn) return;
-    const int i = (int)(e % m), jj = (int)(e / m), j = j0 + jj;
-    const int G = tab.G;
+    if (e >= a.mn) return;
+    const int i = (int)(e % a.m), j = a.j0 + (int)(e / a.m);
+    const int G = tab.G, NW = a.NW, p = a.p;
     uint32_t* sg = cwsm + (size_t)warp * ((size_t)G * WG + NW);  // S_g words [gi][WG]
-    uint32_t* aw = sg + (size_t)G * WG;                          // the accumulator
-    for (int gi = lane; gi < G; gi += 32) {
-        uint64_t a[WG];
+    uint32_t* A = sg + (size_t)G * WG;                           // the window
+    // `parts` lanes per digit group, 32 / parts groups at a time
+    int parts = 1;
+    while (2 * parts * G <= 32 && parts < 16) parts *= 2;
+    const int part = lane & (parts - 1);
+    for (int g0 = 0; g0 < G; g0 += 32 / parts) {
+        const int gi = g0 + lane / parts;
+        uint64_t acc[WG];
 #pragma unroll
-        for (int wd = 0; wd < WG; ++wd) a[wd] = 0;
+        for (int k = 0; k < WG; ++k) acc[k] = 0;
         float F = 0.0f;
-        const uint8_t* tp = T + (size_t)gi * tab.N * mn + e;
-        for (int l = 0; l < tab.N; ++l) {
-            const uint32_t t = tp[(size_t)l * mn];
+        if (gi < G) {
+            const uint8_t* tp = a.T + (size_t)gi * tab.N * a.mn + e;
+            for (int q = part; q < tab.NT; q += parts) {
+                uint32_t u = (uint32_t)__ldg(tp + (size_t)(3 * q) * a.mn) * sc[3 * q];
+                if (3 * q + 1 < tab.N) u += (uint32_t)__ldg(tp + (size_t)(3 * q + 1) * a.mn) * sc[3 * q + 1];
+                if (3 * q + 2 < tab.N) u += (uint32_t)__ldg(tp + (size_t)(3 * q + 2) * a.mn) * sc[3 * q + 2];
 #pragma unroll
-            for (int wd = 0; wd < WG; ++wd) a[wd] += (uint64_t)t * tab.Mlow[l][wd];
-            F = fmaf((float)t, tab.invm[l], F);
+                for (int k = 0; k < WG; ++k) acc[k] += (uint64_t)u * sM[q][k];
+                F = fmaf((float)u, si[q], F);
+            }
         }
-        const uint32_t R = (uint32_t)rintf(F);
-        long long cy = 0;
+        for (int o = 1; o < parts; o *= 2) {
 #pragma unroll
-        for (int wd = 0; wd < WG; ++wd) {
-            const long long cur = (long long)a[wd] + cy - (long long)((uint64_t)R * tab.Plow[wd]);
-            sg[gi * WG + wd] = (uint32_t)cur;
-            cy = cur >> 32;
+            for (int k = 0; k < WG; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+            F += __shfl_xor_sync(0xffffffffu, F, o);
+        }
+        if (part == 0 && gi < G) {
+            // S_g = sum - R P, carries propagated
+            const uint32_t R = (uint32_t)rintf(F);
+            uint64_t cy = 0;
+#pragma unroll
+            for (int k = 0; k < WG; ++k) {
+                acc[k] += (uint64_t)R * tab.Pneg[k];
+                cy += (uint32_t)acc[k];
+                sg[gi * WG + k] = (uint32_t)cy;
+                cy = (cy >> 32) + (acc[k] >> 32);
+            }
         }
     }
     __syncwarp();
-    if (lane != 0) return;
-    const Acc A{aw, NW, 1};
-    constexpr int WIN = WG + 2;
-    long long win[WIN];
-#pragma unroll
-    for (int k = 0; k < WIN; ++k) win[k] = 0;
-    int base = 0;
-    long long carry = 0;
-    auto retire = [&]() {
-        const long long v = win[0] + carry;
-        if (base < NW) A[base] = (uint32_t)v;
-        carry = v >> 32;  // arithmetic
-#pragma unroll
-        for (int k = 0; k < WIN - 1; ++k) win[k] = win[k + 1];
-        win[WIN - 1] = 0;
-        ++base;
+    // word k of the window: sum over the groups that reach it of word k - q of
+    // S_g 2^r (WG + 1 words, the top one sign-filled), q = (w gi) >> 5.  First
+    // the low halves of the sums, then the high halves one word up, then one
+    // off word q + WG + 1 for every negative group.
+    const int w = tab.w;
+    auto groups = [&](int k, int span, int& ga, int& gb) {  // gi with 0 <= k - q(gi) <= span
+        ga = max(0, (32 * (k - span) + w - 1) / w);
+        if (k <= span) ga = 0;
+        gb = min(G - 1, (32 * k + 31) / w);
     };
-    for (int gi = 0; gi < G; ++gi) {
-        const uint32_t* Sg = sg + gi * WG;
-        const long long pos = (long long)tab.w * gi;
-        const int q = (int)(pos >> 5), r = (int)(pos & 31);
-        while (base < q) retire();
-#pragma unroll
-        for (int k = 0; k < WG; ++k) {
-            const uint32_t lo = k ? Sg[k - 1] : 0u;
-            win[k] += (long long)(r ? (Sg[k] << r) | (lo >> (32 - r)) : Sg[k]);
+    auto word_sum = [&](int k) -> uint64_t {
+        int ga, gb;
+        groups(k, WG, ga, gb);
+        uint64_t v = 0;
+        for (int gi = ga; gi <= gb; ++gi) {
+            const int pos = w * gi, d = k - (pos >> 5), r = pos & 31;
+            if (d < 0 || d > WG) continue;
+            const uint32_t* Sg = sg + gi * WG;
+            const uint32_t hi = d < WG ? Sg[d] : (uint32_t)((int)Sg[WG - 1] >> 31), lo = d ? Sg[d - 1] : 0u;
+            v += __funnelshift_l(lo, hi, r);
         }
-        win[WG] += r ? (long long)((int)Sg[WG - 1] >> (32 - r)) : ((Sg[WG - 1] >> 31) ? -1LL : 0LL);
+        return v;
+    };
+    for (int k = lane; k < NW; k += 32) A[k] = (uint32_t)word_sum(k);
+    __syncwarp();
+    warp_add(A, NW, lane, 0u, [&](int k, uint32_t) { return k ? (uint32_t)(word_sum(k - 1) >> 32) : 0u; });
+    warp_add(A, NW, lane, 1u, [&](int k, uint32_t) {  // A - D = A + ~D + 1
+        int ga, gb, d = 0;
+        groups(k, WG + 1, ga, gb);
+        for (int gi = ga; gi <= gb; ++gi)
+            if (k == ((w * gi) >> 5) + WG + 1) d += (int)(sg[gi * WG + WG - 1] >> 31);
+        return (uint32_t)~d;
+    });
+    // the fused update with the old C and the single rounding to p bits (S6),
+    // P_int on the grid 2^(w g0 - mu_i - nu_j)
+    const MPView& C = a.C;
+    const long long xc = (long long)i + (long long)j * C.ld;
+    long long E = (long long)w * tab.g0 - a.mu[i] - a.nu[j];
+    bool neg = (A[NW - 1] >> 31) != 0;
+    if (neg) warp_negate(A, NW, lane);
+    if (a.alpha < 0) neg = !neg;
+    if (a.beta && !mp_zero(C, xc)) {
+        const int Lp = warp_bitlen(A, NW, lane);
+        const long long etop = max(E + Lp, (long long)C.exps[xc]) + 1;
+        const long long Wb = 32LL * NW - 2;
+        if (etop - E > Wb) {
+            // raise the grid: truncation toward zero of the product
+            const long long E2 = etop - Wb, d = E2 - E;
+            for (int k0 = 0; k0 < NW; k0 += 32) {
+                const uint32_t v = win_bits(A, NW, 32LL * (k0 + lane) + d);
+                __syncwarp();
+                if (k0 + lane < NW) A[k0 + lane] = v;
+                __syncwarp();
+            }
+            E = E2;
+        }
+        if (neg) warp_negate(A, NW, lane);
+        // trunc(C 2^-E): magnitude bit b at bit b + (exps - 32 L) - E of the grid
+        const long long s = (long long)C.exps[xc] - 32LL * C.L - E;
+        const uint32_t f = C.signs[xc] != 0 ? 0xffffffffu : 0u;
+        warp_add(A, NW, lane, f & 1u, [&](int k, uint32_t) { return mant32(C, xc, 32LL * k - s) ^ f; });
+        neg = (A[NW - 1] >> 31) != 0;
+        if (neg) warp_negate(A, NW, lane);
     }
-    while (base < NW) retire();
-    mp_finish(A, NW, (long long)tab.w * tab.g0 - mu[i] - nu[j], alpha, beta, C, (long long)i + (long long)j * C.ld, p);
+    const int Lt = warp_bitlen(A, NW, lane);
+    if (Lt == 0) {
+        for (int k = lane; k < C.L; k += 32) C.limbs[(long long)k * C.plane + xc] = 0;
+        if (lane == 0) {
+            C.exps[xc] = 0;
+            C.signs[xc] = 0;
+        }
+        return;
+    }
+    int Lo = Lt;
+    if (Lt > p) {
+        const int sh = Lt - p;
+        bool st = false;  // any bit below sh - 1
+        for (int k = lane; k < NW && 32 * k < sh - 1; k += 32)
+            st |= (sh - 1 - 32 * k >= 32 ? A[k] : A[k] & ((1u << (sh - 1 - 32 * k)) - 1u)) != 0;
+        const bool sticky = __any_sync(0xffffffffu, st);
+        const bool rb = (win_bits(A, NW, sh - 1) & 1u) != 0;
+        const bool up = rb && (sticky || (win_bits(A, NW, sh) & 1u));
+        __syncwarp();
+        // clear the bits below sh, then add 2^sh if rounding up
+        for (int k = lane; k < NW && 32 * k < sh; k += 32) A[k] = sh - 32 * k >= 32 ? 0u : A[k] & ~((1u << (sh - 32 * k)) - 1u);
+        __syncwarp();
+        if (up) {
+            warp_add(A, NW, lane, 0u, [&](int k, uint32_t) { return k == (sh >> 5) ? 1u << (sh & 31) : 0u; });
+            Lo = warp_bitlen(A, NW, lane);
+        }
+    }
+    const long long first = (long long)Lo - 32LL * C.L;  // bit of A at limb 0, bit 0
+    for (int k = lane; k < C.L; k += 32) {
+        const long long pos = first + 32LL * k;
+        C.limbs[(long long)k * C.plane + xc] = pos <= -32 ? 0u : win_bits(A, NW, pos);
+    }
+    if (lane == 0) {
+        C.exps[xc] = (int)(Lo + E);
+        C.signs[xc] = neg ? 1 : 0;
+    }
 }
 
-template <int H, bool FP8>
-void convert_h(const MPView& X, int R, int Kc, int is_b, const int* shifts, const DevTable& tab, int Kpad, int Rpad,
-               int8_t* planes, cudaStream_t s) {
-    // rows [0, R) only (padded rows reach discarded outputs); zeros in the K padding
-    const long long total = (long long)R * Kc;
-    if (total == 0) return;
-    {
-        // plane-ordered tiles: the K padding is written (zeros) by the kernel
-        const int per_warp = X.L + tab.S * (MPD + 1) + 1;
-        const size_t smem = sizeof(uint32_t) * ((size_t)(tab.N * tab.S * 32 + 3) / 4 + (size_t)per_warp * TW);
-        if (smem <= 220 * 1024 || FP8) {
-            raise_smem_limit((const void*)mp_convert_tile_kernel<H, FP8>, (int)smem);
-            const long long positions = (long long)R * Kpad;
-            mp_convert_tile_kernel<H, FP8><<<(unsigned)((positions + 31) / 32), 32 * TW, smem, s>>>(
-                X, R, Kc, is_b, shifts, tab, Kpad, Rpad, planes, per_warp);
-            return;
-        }
+template <int NW, bool FP8>
+void convert_nw(MpConvArgs a, const ConvTab& t, cudaStream_t s) {
+    const int sms = device_sms();
+    auto blocks = [&](int R, int E) {
+        const int HG = a.Kp / E;
+        a.lanes_h = 1;
+        while (a.lanes_h < HG && a.lanes_h < 32) a.lanes_h *= 2;
+        a.hb = (HG + a.lanes_h - 1) / a.lanes_h;
+        const int rows = 8 * (32 / a.lanes_h);
+        return (R + rows - 1) / rows * a.hb;
+    };
+    if (a.Kp % 4 == 0 && ((long long)a.m + a.n) * a.Kp >= 4ll * 512 * sms) {
+        a.blocks_a = blocks(a.m, 4);
+        a.lper = t.N;
+        mp_convert_kernel<NW, FP8, 4><<<a.blocks_a + blocks(a.n, 4), 256, 0, s>>>(a, t);
+        return;
     }
-    zero_k_padding(planes, (long long)tab.N * tab.S, R, Rpad, Kc, Kpad, s);
-    mp_convert_kernel<H><<<(unsigned)((total + 255) / 256), 256, 0, s>>>(X, R, Kc, is_b, shifts, tab, Kpad, Rpad,
-                                                                         planes);
+    a.blocks_a = blocks(a.m, 1);
+    const int nb = a.blocks_a + blocks(a.n, 1);
+    // few elements: the moduli over up to 16 slices
+    int split = (2 * sms + nb - 1) / nb;
+    if (split > 16) split = 16;
+    if (split > t.N) split = t.N;
+    a.lper = (t.N + split - 1) / split;
+    mp_convert_kernel<NW, FP8, 1><<<dim3(nb, (t.N + a.lper - 1) / a.lper), 256, 0, s>>>(a, t);
 }
 
-void mp_convert(const MPView& X, int R, int Kc, int is_b, const int* shifts, const DevTable& tab, int Kpad, int Rpad,
-                int8_t* planes, cudaStream_t s, bool fp8 = false) {
-    switch (tab.H) {
-#define OZ_H(HH)                                                                                   \
-    case HH:                                                                                       \
-        if (fp8) convert_h<HH, true>(X, R, Kc, is_b, shifts, tab, Kpad, Rpad, planes, s);          \
-        else convert_h<HH, false>(X, R, Kc, is_b, shifts, tab, Kpad, Rpad, planes, s);             \
+// rows [0, m) of A's planes and [0, n) of B's (padded rows reach discarded
+// outputs), zeros in the K padding; m = 0: B alone
+void mp_convert(const MPView& A, int m, const MPView& B, int n, int K, const int* mu, const int* nu, const ConvTab& t,
+                int Kp, int Mpad, int Npad, int8_t* RA, int8_t* RB, bool fp8, cudaStream_t s) {
+    const MpConvArgs a{A, B, mu, nu, RA, RB, m, n, K, Kp, Mpad, Npad, 0, 0, 0, 0};
+    switch (t.NW) {
+#define OZ_N(NN)                                                                       \
+    case NN:                                                                           \
+        if (fp8) convert_nw<NN, true>(a, t, s);                                        \
+        else convert_nw<NN, false>(a, t, s);                                           \
         break;
-        OZ_H(1) OZ_H(2) OZ_H(3) OZ_H(4) OZ_H(5) OZ_H(6) OZ_H(7) OZ_H(8) OZ_H(9) OZ_H(10) OZ_H(11) OZ_H(12)
-        OZ_H(13) OZ_H(14) OZ_H(15)
-#undef OZ_H
-        default:
-            if (fp8) convert_h<16, true>(X, R, Kc, is_b, shifts, tab, Kpad, Rpad, planes, s);
-            else convert_h<16, false>(X, R, Kc, is_b, shifts, tab, Kpad, Rpad, planes, s);
-            break;
+        OZ_N(1) OZ_N(2) OZ_N(3) OZ_N(4) OZ_N(5) OZ_N(6) OZ_N(7) OZ_N(8)
+#undef OZ_N
     }
-}
-
-// shared memory of the tiled conversion (it must fit for the FP8 planes)
-size_t tile_smem(const MPView& X, const DevTable& tab) {
-    const int per_warp = X.L + tab.S * (MPD + 1) + 1;
-    return sizeof(uint32_t) * ((size_t)(tab.N * tab.S * 32 + 3) / 4 + (size_t)per_warp * TW);
 }
 
 template <int WG>
-void crt_wg(const uint8_t* T, int m, int nchunk, int j0, const int* mu, const int* nu, const DevTable& tab, int NW,
-            int alpha, int beta, const MPView& C, int p, cudaStream_t s) {
+void crt_wg(const uint8_t* T, int m, int nchunk, int j0, const int* mu, const int* nu, const DevTable& tab,
+            const CrtTab& ct, int NW, int alpha, int beta, const MPView& C, int p, cudaStream_t s) {
     const long long mn = (long long)m * nchunk;
-    // few outputs: a warp per output (the digit groups in parallel)
     const size_t wsm = sizeof(uint32_t) * ((size_t)tab.G * WG + NW) * CWC;
-    if (mn < 16384 && wsm <= 200 * 1024) {
+    if (mn < MP_WARP_CRT && wsm <= 200 * 1024) {
+        const MpCrtArgs a{T, mu, nu, mn, m, j0, NW, alpha, beta, p, C};
         raise_smem_limit((const void*)mp_crt_warp_kernel<WG>, (int)wsm);
-        mp_crt_warp_kernel<WG><<<(unsigned)((mn + CWC - 1) / CWC), 32 * CWC, wsm, s>>>(T, m, nchunk, j0, mu, nu,
-                                                                                      tab, NW, alpha, beta, C, p);
+        mp_crt_warp_kernel<WG><<<(unsigned)((mn + CWC - 1) / CWC), 32 * CWC, wsm, s>>>(a, ct);
         return;
     }
     const size_t smem = sizeof(uint32_t) * (size_t)NW * MPCT;
-    cudaFuncSetAttribute(mp_crt_kernel<WG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    raise_smem_limit((const void*)mp_crt_kernel<WG>, (int)smem);
     mp_crt_kernel<WG><<<(unsigned)((mn + MPCT - 1) / MPCT), MPCT, smem, s>>>(T, m, nchunk, j0, mu, nu, tab, NW,
                                                                             alpha, beta, C, p);
 }
 
-void mp_crt(const uint8_t* T, int m, int nchunk, int j0, const int* mu, const int* nu, const DevTable& tab, int NW,
-            int alpha, int beta, const MPView& C, int p, cudaStream_t s) {
+void mp_crt(const uint8_t* T, int m, int nchunk, int j0, const int* mu, const int* nu, const DevTable& tab,
+            const CrtTab& ct, int NW, int alpha, int beta, const MPView& C, int p, cudaStream_t s) {
     switch (tab.WG) {
-#define OZ_W(WW) case WW: crt_wg<WW>(T, m, nchunk, j0, mu, nu, tab, NW, alpha, beta, C, p, s); break;
+#define OZ_W(WW) case WW: crt_wg<WW>(T, m, nchunk, j0, mu, nu, tab, ct, NW, alpha, beta, C, p, s); break;
         OZ_W(1) OZ_W(2) OZ_W(3) OZ_W(4) OZ_W(5) OZ_W(6) OZ_W(7) OZ_W(8) OZ_W(9) OZ_W(10) OZ_W(11) OZ_W(12)
         OZ_W(13) OZ_W(14) OZ_W(15)
 #undef OZ_W
-        default: crt_wg<16>(T, m, nchunk, j0, mu, nu, tab, NW, alpha, beta, C, p, s); break;
+        default: crt_wg<16>(T, m, nchunk, j0, mu, nu, tab, ct, NW, alpha, beta, C, p, s); break;
     }
 }
 
@@ -929,7 +909,7 @@ size_t up256(size_t v) { return (v + 255) / 256 * 256; }
 // accumulator words for a plan: the largest P_int plus 64 bits, one sign bit spare
 int mp_window_words(const Plan& pl) { return (pl.pint_bits + 64 + 31) / 32 + 1; }
 
-int mp_plan_for(ozlu_handle* h, int p, int K, const Plan** pl, const DevTable** tab, const GemmTab** gt) {
+int mp_plan_for(ozlu_handle* h, int p, int K, const PlanEntry** out) {
     const auto key = std::make_tuple(p, K, 1000, 0, 0, 0);  // backend code 1000: p-bit
     auto it = h->plans.find(key);
     if (it == h->plans.end()) {
@@ -937,12 +917,12 @@ int mp_plan_for(ozlu_handle* h, int p, int K, const Plan** pl, const DevTable** 
         const int rc = make_plan_mp(p, K, e.plan);
         if (rc) return rc;
         fill_table(e.plan, e.table);
+        fill_conv(e.table, e.conv);
+        fill_crt(e.table, e.plan.pint_bits, e.crt);
         fill_gemm(e.table, true, e.gemm);
         it = h->plans.emplace(key, e).first;
     }
-    *pl = &it->second.plan;
-    *tab = &it->second.table;
-    *gt = &it->second.gemm;
+    *out = &it->second;
     return OZLU_OK;
 }
 
@@ -1036,10 +1016,10 @@ int mp_gemm_ext(ozlu_handle* h, int p, int S, int m, int n, int k, int alpha, co
     memset(&tab, 0, sizeof tab);
     const int prev = h->open_phase;
     h->phase(PH_CONVERT);
-    mp_shift_kernel<<<(m + 127) / 128, 128, 0, s>>>(vA, m, k, 0, pl->Q, mu);
-    mp_shift_kernel<<<(n + 127) / 128, 128, 0, s>>>(vB, n, k, 1, pl->Q, nu);
+    const int ba = (m + 31) / 32, bb = (n + 31) / 32;
+    mp_shift_kernel<<<ba + bb, 1024, 0, s>>>(vA, m, vB, n, k, pl->Q, mu, nu, ba);
     mp_convert_ext(vA, m, k, 0, mu, E, Kpad, Mpad, RA, s);
-    h->count(3);
+    h->count(2);
     for (long long j0 = 0; j0 < n; j0 += nch) {
         const int nc = (int)(n - j0 < nch ? n - j0 : nch);
         const int ncp = (nc + 127) / 128 * 128;
@@ -1131,11 +1111,11 @@ int mp_gemm_device(ozlu_handle* h, int p, int m, int n, int k, int alpha, const 
     if (m == 0 || n == 0) return OZLU_OK;
     if (h->mp_opts.modset == OZLU_MODSET_EXT)
         return mp_gemm_ext(h, p, h->mp_opts.nslice, m, n, k, alpha, A, B, beta, C);
-    const Plan* pl;
-    const DevTable* tab;
-    const GemmTab* gt;
-    int rc = mp_plan_for(h, p, k, &pl, &tab, &gt);
+    const PlanEntry* pe;
+    int rc = mp_plan_for(h, p, k, &pe);
     if (rc) return rc;
+    const Plan* pl = &pe->plan;
+    const DevTable* tab = &pe->table;
     cudaStream_t s = h->stream;
     // K <= KSMALL: unpadded planes and the small-K product on the integer
     // pipe; otherwise residue planes padded in K to a multiple of the GEMM's
@@ -1146,11 +1126,10 @@ int mp_gemm_device(ozlu_handle* h, int p, int m, int n, int k, int alpha, const 
     const MPView vA = view_of(A, 0), vB = view_of(B, 0), vC = view_of(C, 0);
     // FP8 (balanced base-17 digits on tcgen05, three planes per residue, the
     // same plan and so the same results) for wide products when chosen and
-    // admissible: fp32 accumulations below 2^24 and the tiles in shared memory
+    // admissible: fp32 accumulations below 2^24
     int be = h->mp_opts.backend;
     const int kp128 = (k + 127) / 128 * 128;
-    const bool fp8_ok = !smallk && !narrow && (double)kp128 * pl->S * 225.0 < ldexp(1.0, 24) &&
-                        tile_smem(vA, *tab) <= 220 * 1024 && tile_smem(vB, *tab) <= 220 * 1024;
+    const bool fp8_ok = !smallk && !narrow && (double)kp128 * pl->S * 225.0 < ldexp(1.0, 24);
     if (be == OZLU_BE_AUTO && fp8_ok) {
         if ((rc = mp_tune_backend(h, p, m, n, k, A, B, &be))) return rc;
     }
@@ -1186,25 +1165,23 @@ int mp_gemm_device(ozlu_handle* h, int p, int m, int n, int k, int alpha, const 
     if (fp8 && !(derr = err_word(h))) return OZLU_ERR_NOMEM;
     const int prev = h->open_phase;
     h->phase(PH_CONVERT);
-    // B's exponents and first column chunk on the side stream, beside A's
     {
-        cudaStream_t sb = side_fork(h, s);
-        const int nc0 = (int)(n < nch ? n : nch);
-        mp_shift_kernel<<<(n + 127) / 128, 128, 0, sb>>>(vB, n, k, 1, pl->Q, nu);
-        mp_convert(vB, nc0, k, 1, nu, *tab, Kpad, (nc0 + rowq - 1) / rowq * rowq, RB, sb, fp8);
-        mp_shift_kernel<<<(m + 127) / 128, 128, 0, s>>>(vA, m, k, 0, pl->Q, mu);
-        mp_convert(vA, m, k, 0, mu, *tab, Kpad, Mpad, RA, s, fp8);
-        if (!side_join(h, s, sb)) return OZLU_ERR_CUDA;
+        const int nc0 = (int)(n < nch ? n : nch), ba = (m + 31) / 32, bb = (n + 31) / 32;
+        mp_shift_kernel<<<ba + bb, 1024, 0, s>>>(vA, m, vB, n, k, pl->Q, mu, nu, ba);
+        mp_convert(vA, m, vB, nc0, k, mu, nu, pe->conv, Kpad, Mpad, (nc0 + rowq - 1) / rowq * rowq, RA, RB, fp8, s);
     }
-    h->count(3);
+    h->count(2);
     for (long long j0 = 0; j0 < n; j0 += nch) {
         const int nc = (int)(n - j0 < nch ? n - j0 : nch);
         const int ncp = (nc + rowq - 1) / rowq * rowq;
         h->phase(PH_CONVERT);
-        if (j0 > 0) mp_convert(view_of(B, j0 * B.ld), nc, k, 1, nu + j0, *tab, Kpad, ncp, RB, s, fp8);
+        if (j0 > 0) {
+            mp_convert(vA, 0, view_of(B, j0 * B.ld), nc, k, mu, nu + j0, pe->conv, Kpad, Mpad, ncp, RA, RB, fp8, s);
+            h->count(1);
+        }
         h->phase(PH_GEMM);
         if (fp8) {
-            if ((rc = launch_gemm_tc05(true, false, RA, RB, m, nc, Mpad, ncp, Kpad, *gt, T, derr, s))) return rc;
+            if ((rc = launch_gemm_tc05(true, false, RA, RB, m, nc, Mpad, ncp, Kpad, pe->gemm, T, derr, s))) return rc;
         } else if (smallk) {
             const long long work = (long long)m * nc * pl->N * pl->G;
             small_k_gemm_kernel<<<(unsigned)((work + 255) / 256), 256, 0, s>>>(RA, RB, m, nc, k, *tab, T);
@@ -1214,8 +1191,8 @@ int mp_gemm_device(ozlu_handle* h, int p, int m, int n, int k, int alpha, const 
             launch_gemm_imma(RA, RB, m, nc, Mpad, ncp, Kpad, *tab, T, s);
         }
         h->phase(PH_CRT);
-        mp_crt(T, m, nc, (int)j0, mu, nu, *tab, NW, alpha, beta, vC, p, s);
-        h->count(3);
+        mp_crt(T, m, nc, (int)j0, mu, nu, *tab, pe->crt, NW, alpha, beta, vC, p, s);
+        h->count(2);
         h->stats.gemm_launches += 1;
         h->stats.crt_launches += 1;
         h->stats.gemm_ops += 2.0 * m * nc * (double)k * pl->N * pl->pair_terms * P;

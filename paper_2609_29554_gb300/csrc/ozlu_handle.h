@@ -51,10 +51,6 @@ struct ozlu_handle {
     std::map<std::tuple<int, int, int, int, int, int>, ozlu::PlanEntry> plans;
     ozlu::GemmLayout last;
     int* dev_err = nullptr;  // device error word of the tensor-core GEMMs
-    // second stream of the GEMM's conversion: B's exponents and residues run
-    // beside A's (fork / join events on the handle's stream)
-    cudaStream_t side = nullptr;
-    cudaEvent_t side_fork = nullptr, side_join = nullptr;
     bool timing = false;
     ozlu_stats stats = {};
     void* lu_scratch = nullptr;  // pivot-search scratch of ozlu_getrf
@@ -111,11 +107,5 @@ int* err_word(ozlu_handle* h);
 int mp_gemm_device(ozlu_handle* h, int p, int m, int n, int k, int alpha, const ozlu_mp_matrix& A,
                    const ozlu_mp_matrix& B, int beta, const ozlu_mp_matrix& C);
 int clear_err_word(ozlu_handle* h);
-// the handle's second stream, forked from s (made by the first call outside a
-// graph capture); s itself when there is none
-cudaStream_t side_fork(ozlu_handle* h, cudaStream_t s);
-// s waits for the work issued on `side` (nothing when side is s); false on a
-// CUDA error
-bool side_join(ozlu_handle* h, cudaStream_t s, cudaStream_t side);
 int cuda_rc(cudaError_t e);
 }  // namespace ozlu

@@ -21,6 +21,8 @@ void fill_conv(const DevTable& t, ConvTab& c) {
             pw += pw;
             if (pw >= m) pw -= m;
         }
+        const uint32_t kneg = (1 + k.topc) % m;
+        k.k4 = (k.wrapc << 8) | (kneg << 16) | ((kneg + m - k.wrapc) % m << 24);
         k.m = m;
         k.magic = t.magic[l];
         k.half = m / 2;

@@ -23,7 +23,11 @@ struct ConvMod {
     uint32_t wrapc;           // -2^w mod m
     uint32_t topc;            // -2^(32 NW) mod m
     uint32_t h2;              // binary16 pair (1024 + half, 1024 + half)
-    uint32_t pad_[2];
+    // p-bit digits sgn (D - wrap 2^w), D replaced by its complement where
+    // negative: byte neg 2 + wrap is the correction {0, -2^w, 1 - 2^(32 NW),
+    // 1 - 2^(32 NW) + 2^w} mod m
+    uint32_t k4;
+    uint32_t pad_;
 };
 
 struct ConvTab {
