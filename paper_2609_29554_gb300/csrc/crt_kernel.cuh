@@ -3,6 +3,7 @@
 // (two translation units compile side by side).
 #pragma once
 
+#include "carry.cuh"
 #include "mp_device.cuh"
 #include "ozlu_internal.h"
 #include "tables.h"
@@ -46,19 +47,6 @@ constexpr int CT = 128;  // threads per block
 // step), TD 1777 x 611, 78 / 72 / 76 / 80 us.
 template <int NW, bool PACK>
 constexpr int min_blocks() { return PACK && NW <= 13 ? 8 : 6; }
-
-// Carry chains: add_first sets the carry flag, add_next takes and sets it (one
-// instruction a word; the 64-bit sums of a plain loop take three).
-__device__ __forceinline__ uint32_t add_first(uint32_t a, uint32_t b) {
-    uint32_t r;
-    asm volatile("add.cc.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-    return r;
-}
-__device__ __forceinline__ uint32_t add_next(uint32_t a, uint32_t b) {
-    uint32_t r;
-    asm volatile("addc.cc.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-    return r;
-}
 
 // X <<= 32 Q + r
 template <int NW, int Q>

@@ -34,7 +34,6 @@ constexpr int PIV_BLOCKS = 152;
 constexpr int MAXPART = 1024;   // block partials of a column step
 constexpr int STEP_ROWS = 16;   // rows per block of a column step
 constexpr int LCT = 4;          // laswp: columns per block
-constexpr int LHASH = 2048;     // laswp: hash slots (>= 2 x affected rows)
 constexpr int LMAXB = 512;      // laswp: interchanges per call
 constexpr int TRI_SLOTS = 8;    // triangles of base solves converted ahead (256 / BASE)
 
@@ -324,64 +323,81 @@ __global__ void __launch_bounds__(128) column_step_kernel(double* A, long long l
 // ---------------------------------------------------------------------------
 // Cooperative factorisation of one base block: columns [c0, c0 + b) over rows
 // [c0, n).  One block per SM owns a contiguous slice of rows and keeps its
-// b-column slice in shared memory as L-limb floats for the whole block.  A
-// column step needs one exchange: each block publishes its best candidate row
-// for the column (its index and the whole row) in its slot, then one 64-bit
-// word holding the column number and an ordering key of the candidate; every
-// block waits for all G stamp words (one load each when they are there),
-// reduces the same keys to the same pivot, takes the pivot row from the
-// winner's slot, swaps it into place among its rows, scales and updates.
-// The exchange overlaps the trailing update: a block first updates only the
-// rows the next step needs from it (its next candidate and the row that the
-// pivot will replace), publishes them, and only then updates the rest of its
-// rows; meanwhile one thread forms the reciprocal of its candidate and
-// publishes it under a second stamp, which the other blocks wait for (from
-// the winner only) when they need the multipliers.  Waiting on the stamps
-// replaces a grid barrier, and the slots are double-buffered by column
-// parity: a block can only stamp column kc + 2 after every block has stamped
-// kc + 1, i.e. after every block has finished reading the slots of column kc.
+// b-column slice in shared memory as L-limb floats for the whole block.
+//
+// A column is a serial chain (the pivot, its reciprocal, the next column, the
+// next candidate) through every block, so the kernel is bound by latency, and
+// what is off the chain runs beside it on warps of its own:
+//   warp 0      the chain: reduce the blocks' keys to the pivot, fetch the
+//               pivot's reciprocal and its next element, update the next column,
+//               choose and announce the block's candidate, invert it;
+//   warp 1      the multipliers; then column kc + 2, which the chain needs next;
+//   warps 2, 3  the pivot row into shared memory, the interchange;
+//   warps 4 ..  the trailing update of the last column, then the two rows other
+//               blocks may need from this one (its candidate and the row the
+//               pivot will replace), published as they are formed.
+// The next column is updated as y - (x u) / p with x u formed while the
+// reciprocal is on its way (one rounding more of 2^-(32 L), 32 L >= 53 nc + 12);
+// the multipliers x / p are off the chain.
+//
+// Blocks exchange 64-bit words whose upper half is a tag (the column) and whose
+// lower half is data, so that a word announces itself: readers poll the words
+// they need, and neither side pays for a fence (about 1000 cycles each at GPU
+// scope).  Only relaxed accesses to single words are used.  The first word a
+// block announces is its candidate's key, before its row is final.  There are
+// three slots per block, used in turn: a block writes the words of column kc + 3
+// only after every block has announced its key of kc + 2, which a block does after
+// the block-wide barrier of column kc, i.e. when all its warps have read what they
+// need of column kc.  The words are zeroed before every factorisation and tags are
+// column numbers, so a stale word never matches.
+//
+// Measured, QD panels of the n = 1000 / 4096 LU (nb = 256): 5.2 / 23.8 ms, from 13.0 /
+// 58.7 ms with a stamp over a fenced row and the exchange, the reciprocal and the
+// multipliers on the same warp in turn (5.0 against 13 us a column at n = 1000).
+//
 // The interchanges of the columns outside the base block are applied once,
-// after the last column.
-// Every wait is bounded (2 s of the global timer); on expiry the kernel
-// records OZLU_ERR_TIMEOUT in the scratch and every block returns.
+// after the last column, as one permutation (laswp2; by one thread per column
+// swap by swap they took 150 us per 128 columns).  Every wait is bounded (2 s of
+// the global timer); on expiry the kernel records OZLU_ERR_TIMEOUT in the
+// scratch and every block returns.
 constexpr int COOP_MAXG = 304;           // blocks (up to 2 per SM)
 constexpr int COOP_THREADS = 512;
-static_assert(2 * PBASE + 2 <= COOP_THREADS, "one pivot-row element per thread");
+constexpr int COOP_DEPTH = 3;            // slots per block
 constexpr unsigned long long COOP_WAIT_NS = 2000000000ull;
 
 // stamp word of a slot: bits 63..44 the column (c0 + kc + 1, modulo 2^20),
-// bits 43..0 the candidate's key (mpf_key; 0: no candidate).  One 64-bit
-// store publishes both, after the rest of the slot.
+// bits 43..0 the candidate's key (mpf_key; 0: no candidate)
 constexpr int STAMP_SHIFT = 44;
 constexpr unsigned long long KEY_MASK = (1ull << STAMP_SHIFT) - 1;
 
+// tagged words: (tag << 32) | data, tag = c0 + kc + 1
 template <int L>
 struct CoopSlot {
-    unsigned long long stamp;      // column tag and key: idx and row are published
-    unsigned long long stamp_rec;  // column tag: rec is published
-    int idx;                 // the candidate's global row index, -1 if none
-    int pad;
-    MPF<L> rec;              // 1 / the candidate (0 for a zero candidate)
-    MPF<L> row[PBASE];       // the candidate row (all b columns)
+    static constexpr int WORDS = L + 2;       // MPF: limbs, exponent, sign
+    unsigned long long stamp;
+    unsigned long long idx;                   // the candidate's global row
+    unsigned long long rec[WORDS];            // 1 / the candidate (0 for a zero candidate)
+    unsigned long long row[WORDS][PBASE];     // the candidate row (all b columns), word-major
 };
 
 template <int L>
 struct CoopScratch {
     int error;
     int pad[3];
-    CoopSlot<L> part[2][COOP_MAXG];  // double-buffered by column parity
-    MPF<L> orow[2][PBASE];           // old row c, for the owner of the pivot row
+    CoopSlot<L> part[COOP_DEPTH][COOP_MAXG];             // by column modulo COOP_DEPTH
+    unsigned long long orow[COOP_DEPTH][L + 2][PBASE];   // old row c, for the owner of the pivot row
 };
 
-// the error word and every slot stamp start at zero for each factorisation
-// (one thread per slot; the scratch was laid out for L limbs)
+// the error word and every tagged word of G slots start at zero for each
+// factorisation (grid G x COOP_DEPTH; the scratch was laid out for L limbs)
 template <int L>
 __global__ void coop_reset_kernel(CoopScratch<L>* sc) {
-    const int t = threadIdx.x;
-    if (t == 0) sc->error = 0;
-    if (t < 2 * COOP_MAXG) {
-        sc->part[t / COOP_MAXG][t % COOP_MAXG].stamp = 0ull;
-        sc->part[t / COOP_MAXG][t % COOP_MAXG].stamp_rec = 0ull;
+    unsigned long long* w = reinterpret_cast<unsigned long long*>(&sc->part[blockIdx.y][blockIdx.x]);
+    for (int t = threadIdx.x; t < (int)(sizeof(CoopSlot<L>) / 8); t += blockDim.x) w[t] = 0ull;
+    if (blockIdx.x == 0) {
+        unsigned long long* o = &sc->orow[blockIdx.y][0][0];
+        for (int t = threadIdx.x; t < (L + 2) * PBASE; t += blockDim.x) o[t] = 0ull;
+        if (blockIdx.y == 0 && threadIdx.x == 0) sc->error = 0;
     }
 }
 
@@ -391,48 +407,96 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 
-// load with acquire semantics at GPU scope: this thread's later loads see
-// everything the writer of the value made visible before it
-__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long* p) {
+__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long* p) {
     unsigned long long v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
 
-// store with release semantics at GPU scope
-__device__ __forceinline__ void st_release(unsigned long long* p, unsigned long long v) {
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+__device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long long v) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-// wait until the stamp word carries column `want`; returns it, or 0 on
-// expiry after limit_ns of the global timer (the error word is then set) or
-// when another block has given up
+// The bound of a wait, for a polling loop that calls expired() once per failed
+// poll: true after limit_ns of the global timer (the error word is then set) or
+// when another block has given up.  The timer, slow to read, is first read
+// after 256 polls.
+struct WaitBound {
+    unsigned long long t0 = 0;
+    int it = 0;
+    __device__ __forceinline__ bool expired(int* err, unsigned long long limit_ns = COOP_WAIT_NS) {
+        if ((++it & 255) != 0) return false;
+        if (*(volatile int*)err) return true;
+        const unsigned long long t = global_ns();
+        if (it == 256) t0 = t;
+        if (t - t0 <= limit_ns) return false;
+        atomicExch(err, OZLU_ERR_TIMEOUT);
+        return true;
+    }
+};
+
+// wait until the stamp word carries column `want`; returns it, or 0 on expiry
 __device__ __forceinline__ unsigned long long wait_stamp(const unsigned long long* p, unsigned want,
                                                          int* err,
                                                          unsigned long long limit_ns = COOP_WAIT_NS) {
-    const unsigned long long t0 = global_ns();
-    for (int it = 1;; ++it) {
-        const unsigned long long v = ld_acquire(p);
+    WaitBound wb;
+    for (;;) {
+        const unsigned long long v = ld_relaxed(p);
         if ((unsigned)(v >> STAMP_SHIFT) == want) return v;
-        if ((it & 63) == 0) {
-            if (*(volatile int*)err) return 0;
-            if (global_ns() - t0 > limit_ns) {
-                atomicExch(err, OZLU_ERR_TIMEOUT);
-                return 0;
-            }
-        }
+        if (wb.expired(err, limit_ns)) return 0;
     }
 }
 
-// load an L-limb float written by another block (bypassing L1)
-template <int L>
-__device__ __forceinline__ MPF<L> ld_cg(const MPF<L>* p) {
-    MPF<L> v;
-    const unsigned int* w = reinterpret_cast<const unsigned int*>(p);
+// Poll n tagged words a lane (p[i], skipped where null) until all carry `tag`;
+// false on expiry.  All loads of a round are in flight together.  The lanes
+// decide together, so a warp leaves the loop converged.
+template <int n>
+__device__ __forceinline__ bool wait_words(const unsigned long long* const (&p)[n], unsigned tag, uint32_t (&v)[n],
+                                           int* err) {
+    WaitBound wb;
+    unsigned long long w[n];
 #pragma unroll
-    for (int i = 0; i < L; ++i) v.m[i] = __ldcg(w + i);
-    v.e = __ldcg(reinterpret_cast<const int*>(w + L));
-    v.neg = __ldcg(reinterpret_cast<const int*>(w + L + 1));
+    for (int i = 0; i < n; ++i) w[i] = 0;
+    for (;;) {
+        bool miss = false;
+#pragma unroll
+        for (int i = 0; i < n; ++i)
+            if (p[i] && (unsigned)(w[i] >> 32) != tag) w[i] = ld_relaxed(p[i]);
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            v[i] = (uint32_t)w[i];
+            miss |= p[i] && (unsigned)(w[i] >> 32) != tag;
+        }
+        if (!__any_sync(0xffffffffu, miss)) return true;
+        if (__any_sync(0xffffffffu, wb.expired(err))) return false;
+    }
+}
+
+// word i of an L-limb float (limbs, exponent, sign) and its inverse
+template <int L>
+__device__ __forceinline__ uint32_t mpf_word(const MPF<L>& v, int i) {
+    return i < L ? v.m[i < L ? i : 0] : (uint32_t)(i == L ? v.e : v.neg);
+}
+
+// the float whose word i lane i holds, on every lane
+template <int L>
+__device__ __forceinline__ MPF<L> mpf_gather(uint32_t w) {
+    MPF<L> v;
+#pragma unroll
+    for (int i = 0; i < L; ++i) v.m[i] = __shfl_sync(0xffffffffu, w, i);
+    v.e = (int)__shfl_sync(0xffffffffu, w, L);
+    v.neg = (int)__shfl_sync(0xffffffffu, w, L + 1);
+    return v;
+}
+
+// lane src's float on every lane
+template <int L>
+__device__ __forceinline__ MPF<L> mpf_bcast(const MPF<L>& x, int src) {
+    MPF<L> v;
+#pragma unroll
+    for (int i = 0; i < L; ++i) v.m[i] = __shfl_sync(0xffffffffu, x.m[i], src);
+    v.e = __shfl_sync(0xffffffffu, x.e, src);
+    v.neg = __shfl_sync(0xffffffffu, x.neg, src);
     return v;
 }
 
@@ -443,10 +507,11 @@ __device__ __forceinline__ MPF<L> ld_cg(const MPF<L>* p) {
 // highest nonzero key, so that they always go through the full comparison.
 template <int L>
 __device__ __forceinline__ unsigned long long mpf_key(const MPF<L>& v) {
-    if (mpf_zero<L>(v)) return 1ull;
-    if (v.e < -2047) return 1ull << 32;
-    if (v.e > 2047) return KEY_MASK;
-    return ((unsigned long long)(unsigned)(v.e + 2048) << 32) | v.m[L - 1];
+    // (selects, so that the lanes of a warp stay together)
+    const unsigned hi = v.e < -2047 ? 1u : (v.e > 2047 ? 0xfffu : (unsigned)(v.e + 2048));
+    const unsigned lo = v.e < -2047 ? 0u : (v.e > 2047 ? 0xffffffffu : v.m[L - 1]);
+    const unsigned long long k = ((unsigned long long)hi << 32) | lo;
+    return mpf_zero<L>(v) ? 1ull : k;
 }
 
 // |a| > |b|, or equal and ia < ib (first index on ties); ib < 0: b is empty
@@ -474,294 +539,412 @@ __device__ __forceinline__ void warp_best(MPF<L>& v, int& idx, int& aux) {
     }
 }
 
-// warp-wide max of (key, then lowest index); idx < 0: none
-__device__ __forceinline__ void warp_best_key(unsigned long long& k, int& idx, int& aux) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long k2 = __shfl_xor_sync(0xffffffffu, k, o);
-        const int i2 = __shfl_xor_sync(0xffffffffu, idx, o);
-        const int a2 = __shfl_xor_sync(0xffffffffu, aux, o);
-        if (i2 >= 0 && (idx < 0 || k2 > k || (k2 == k && i2 < idx))) { k = k2; idx = i2; aux = a2; }
-    }
+// warp-wide max of (key, then lowest index >= 0) by three integer reductions;
+// idx < 0: none (its key is 0)
+__device__ __forceinline__ void warp_best_key(unsigned long long& k, int& idx) {
+    const unsigned hi = idx >= 0 ? (unsigned)(k >> 32) : 0u;
+    const unsigned H = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned lo = idx >= 0 && hi == H ? (unsigned)k : 0u;
+    const unsigned Lo = __reduce_max_sync(0xffffffffu, lo);
+    const bool mine = idx >= 0 && hi == H && (unsigned)k == Lo;
+    idx = (int)__reduce_min_sync(0xffffffffu, mine ? (unsigned)idx : 0xffffffffu);
+    k = ((unsigned long long)H << 32) | Lo;
 }
 
-// named barrier of warps 1 .. COOP_THREADS / 32 - 1 (warp 0 takes no part)
-__device__ __forceinline__ void bar_rest() {
-    asm volatile("bar.sync 1, %0;" ::"r"(COOP_THREADS - 32) : "memory");
+// named barriers of the kernel below: the count of threads that arrive or wait
+// (whole warps, converged)
+__device__ __forceinline__ void bar_sync(int id, int threads) {
+    __syncwarp();
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int threads) {
+    __syncwarp();
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
-template <int N>
+// Q: rows of warp 0's lanes, nr <= 32 Q
+template <int N, int Q>
 __global__ void __launch_bounds__(COOP_THREADS, 1) base_block_coop_kernel(
-    double* A, long long lda, int n, int c0, int b, int p0, int p1, int rows_per_block,
-    int* ipiv, int* info, CoopScratch<Limbs<N>::L>* sc) {
-    constexpr int L = Limbs<N>::L;
+    double* A, long long lda, int n, int c0, int b, int rows_per_block, int* ipiv, int* info,
+    CoopScratch<Limbs<N>::L>* sc) {
+    constexpr int L = Limbs<N>::L, WORDS = L + 2;
     constexpr int T = COOP_THREADS;
+    constexpr int BAR_PIVOT = 1;  // warps 0 .. 3: the pivot's slot is known
+    constexpr int BAR_COL = 2;    // column kc + 2 is updated (warp 0 waits, the others arrive)
     extern __shared__ __align__(16) unsigned char smraw[];
     MPF<L>* a = reinterpret_cast<MPF<L>*>(smraw);  // [r][k], r < rows_per_block, k < b
     // rows padded to b + 1 entries: threads on consecutive rows of one column
     // then fall on different shared-memory banks
     const int bs = b + 1;
     __shared__ MPF<L> prow[2][PBASE];  // the pivot row, double-buffered by column parity
-    __shared__ MPF<L> otmp[PBASE];     // old row c (for the owner of the pivot row)
-    __shared__ MPF<L> rec;         // 1 / pivot
-    __shared__ MPF<L> cv;          // this block's next candidate
-    __shared__ int ci, s_piv, s_fail;
-    __shared__ int s_pivs[PBASE];
-    const int g = blockIdx.x, G = gridDim.x, tid = threadIdx.x;
+    __shared__ int s_cand, s_slot, s_zero;
+    __shared__ int s_fail[2];  // by column parity: a slow warp still reads the last one
+    const int g = blockIdx.x, G = gridDim.x, tid = threadIdx.x, lane = tid & 31;
+    // (broadcast, so that the compiler sees the warps' branches as uniform: it
+    // then keeps shuffles and reductions in them inline; else each takes an
+    // out-of-line reconvergence, about 250 cycles)
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const int r0 = c0 + g * rows_per_block;
     const int r1 = min(n, r0 + rows_per_block);
     const int nr = max(0, r1 - r0);
-    auto owner = [&](int row) { return (row - c0) / rows_per_block; };
+    auto owns = [&](int row) { return row >= r0 && row < r1; };
+    int* err = &sc->error;
 
+    if (tid < 2) s_fail[tid] = 0;
     for (int p = tid; p < nr * b; p += T) {
         const int r = p / b, k = p - r * b;
         a[r * bs + k] = mpf_from_exp<L, N>(elem(A, lda, N, r0 + r, c0 + k));
     }
     __syncthreads();
 
-    // warp 0: this block's best candidate in local column kc among rows >=
-    // row_lo (cv, ci)
-    auto candidate = [&](int kc, int row_lo) {
+    // warp 0: the block's candidate among the rows >= row_lo for column kc, whose
+    // values the lanes hold (v[q]: row lane + 32 q); announces it and leaves its
+    // row in s_cand; returns its value
+    auto choose = [&](const MPF<L> (&v)[Q], int row_lo, int kc) -> MPF<L> {
         unsigned long long bk = 0;
-        int bi = -1, aux = 0;
-        for (int r = tid; r < nr; r += 32) {
-            const int i = r0 + r;
-            if (i < row_lo) continue;
-            const unsigned long long k = mpf_key<L>(a[r * bs + kc]);
-            if (bi < 0 || k > bk ||
-                (k == bk && mpf_abs_cmp<L>(a[r * bs + kc], a[(bi - r0) * bs + kc]) > 0)) {
-                bk = k;
-                bi = i;
+        int bi = -1;
+        MPF<L> mine = v[0];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            if (32 * q >= nr) break;
+            const int r = lane + 32 * q;
+            const bool in = r < nr && r0 + r >= row_lo;
+            const unsigned long long k = mpf_key<L>(v[q]);
+            bool better = in && (bi < 0 || k > bk);
+            if (q > 0 && __any_sync(0xffffffffu, in && bi >= 0 && k == bk))
+                better = better || (in && bi >= 0 && k == bk && mpf_abs_cmp<L>(v[q], mine) > 0);
+            bk = better ? k : bk;
+            bi = better ? r0 + r : bi;
+            if (q > 0) {
+#pragma unroll
+                for (int i = 0; i < L; ++i) mine.m[i] = better ? v[q].m[i] : mine.m[i];
+                mine.e = better ? v[q].e : mine.e;
+                mine.neg = better ? v[q].neg : mine.neg;
             }
         }
+        __syncwarp();
         unsigned long long K = bk;
         int I = bi;
-        warp_best_key(K, I, aux);
+        warp_best_key(K, I);
         if (__any_sync(0xffffffffu, bi >= 0 && bk == K && bi != I)) {  // equal keys: compare exactly
-            MPF<L> v = (bi >= 0 && bk == K) ? a[(bi - r0) * bs + kc] : mpf_make_zero<L>();
-            int vi = (bi >= 0 && bk == K) ? bi : -1;
-            warp_best<L>(v, vi, aux);
-            I = vi;
+            MPF<L> x = (bi >= 0 && bk == K) ? mine : mpf_make_zero<L>();
+            int xi = (bi >= 0 && bk == K) ? bi : -1, aux = 0;
+            warp_best<L>(x, xi, aux);
+            I = xi;
         }
-        if (tid == 0) {
-            ci = I;
-            cv = I >= 0 ? a[(I - r0) * bs + kc] : mpf_make_zero<L>();
+        const unsigned tag = (unsigned)(c0 + kc + 1);
+        CoopSlot<L>& slot = sc->part[kc % COOP_DEPTH][g];
+        if (lane == 0) {
+            st_relaxed(&slot.stamp, ((unsigned long long)(tag & 0xfffff) << STAMP_SHIFT) | (I >= 0 ? K : 0ull));
+            st_relaxed(&slot.idx, ((unsigned long long)tag << 32) | (unsigned)I);
+            s_cand = I;
         }
+        const MPF<L> best = mpf_bcast<L>(mine, I >= 0 ? (I - r0) & 31 : 0);
+        return I >= 0 ? best : mpf_make_zero<L>();
     };
-    // all threads: publish the candidate of column kc (every column of its row
-    // final) and, from the owner of row c0 + kc, that row's old contents;
-    // stamp A carries the key
-    auto publish = [&](int kc) {
-        CoopSlot<L>& slot = sc->part[kc & 1][g];
-        const int wi = ci;
-        const int c = c0 + kc;
-        if (wi >= 0)
-            for (int k = tid; k < b; k += T) slot.row[k] = a[(wi - r0) * bs + k];
-        if (owner(c) == g)
-            for (int k = tid; k < b; k += T) sc->orow[kc & 1][k] = a[(c - r0) * bs + k];
-        if (tid == 0) slot.idx = wi;
-        __syncthreads();
-        if (tid == 0) {
-            __threadfence();
-            const unsigned long long key = wi >= 0 ? mpf_key<L>(cv) : 0ull;
-            *reinterpret_cast<volatile unsigned long long*>(&slot.stamp) =
-                ((unsigned long long)((c + 1) & 0xfffff) << STAMP_SHIFT) | key;
-        }
+    // warp 0: the reciprocal of the candidate of column kc
+    auto publish_rec = [&](const MPF<L>& cand, int kc) {
+        const MPF<L> r = mpf_zero<L>(cand) ? mpf_make_zero<L>() : mpf_recip<L>(cand);
+        uint32_t w = 0;
+#pragma unroll
+        for (int i = 0; i < WORDS; ++i) w = lane == i ? mpf_word<L>(r, i) : w;
+        if (lane < WORDS)
+            st_relaxed(&sc->part[kc % COOP_DEPTH][g].rec[lane], ((unsigned long long)(unsigned)(c0 + kc + 1) << 32) | w);
     };
-    // thread 0: the reciprocal of the candidate of column kc, then stamp B
-    auto publish_rec = [&](int kc) {
-        CoopSlot<L>& slot = sc->part[kc & 1][g];
-        const MPF<L> r = (ci >= 0 && !mpf_zero<L>(cv)) ? mpf_recip<L, true>(cv) : mpf_make_zero<L>();
-        slot.rec = r;
-        st_release(&slot.stamp_rec, (unsigned long long)((c0 + kc + 1) & 0xfffff) << STAMP_SHIFT);
+    // four warps each for the candidate row (pub 0 .. 3) and, in its owner, row
+    // c0 + kc + 1 (pub 4 .. 7): update it by column kc (kc < 0 or zero: no update)
+    // and publish it for column kc + 1.  None of them shares warp 0's scheduler,
+    // where the reciprocal runs at the same time.
+    const int pub = (warp & 3) == 0 || warp < 5 || warp > 14 ? -1 : (warp - 5) - ((warp - 5) >> 2);
+    auto publish_rows = [&](int kc, bool zero, int pa, int pb) {
+        const unsigned long long tag = (unsigned long long)(unsigned)(c0 + kc + 2) << 32;
+        const int r = pub < 4 ? pa : pb, k = (pub & 3) * 32 + lane;
+        if (r < 0 || (pub >= 4 && pb == pa)) return;
+        unsigned long long* orow = &sc->orow[(kc + 1) % COOP_DEPTH][0][0];
+        unsigned long long* dst = pub < 4 ? &sc->part[(kc + 1) % COOP_DEPTH][g].row[0][0] : orow;
+        if (k < b) {
+            MPF<L> v = a[r * bs + k];
+            if (!zero && k >= kc + 2) {
+                v = mpf_fms_oolv<L>(v, a[r * bs + kc], prow[kc & 1][k]);
+                a[r * bs + k] = v;
+            }
+#pragma unroll
+            for (int i = 0; i < WORDS; ++i) st_relaxed(dst + i * PBASE + k, tag | mpf_word<L>(v, i));
+            if (pb == pa) {  // the candidate is row c0 + kc + 1 itself
+#pragma unroll
+                for (int i = 0; i < WORDS; ++i) st_relaxed(orow + i * PBASE + k, tag | mpf_word<L>(v, i));
+            }
+        }
     };
 
-    if (tid < 32) candidate(0, c0);
+    MPF<L> cand = mpf_make_zero<L>();  // warp 0: this block's candidate
+    if (warp == 0) {
+        MPF<L> v[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) v[q] = lane + 32 * q < nr ? a[(lane + 32 * q) * bs] : mpf_make_zero<L>();
+        cand = choose(v, c0, 0);
+    }
     __syncthreads();
-    publish(0);
-    if (tid == 0) publish_rec(0);
-    // warps that share a scheduler with warp 0 (warp ids 4, 8, ...) leave the
-    // priority rows to the others, so that the reciprocal on thread 0 issues
-    // alone there
-    constexpr int NPRIO_T = 32 * (T / 32 - (T / 32 + 3) / 4);
-    const int warp = tid >> 5;
-    // the update of the rows outside the priority pair by column bulk_kc is
-    // deferred to the next column's exchange (bulk_kc < 0: none pending)
+    if (warp == 0) {
+        publish_rec(cand, 0);
+    } else {
+        if (pub >= 0) publish_rows(-1, true, s_cand >= 0 ? s_cand - r0 : -1, owns(c0) ? c0 - r0 : -1);
+        bar_arrive(BAR_COL, T);
+    }
+
+    // the trailing update by column bulk_kc of the rows outside the pair that
+    // publish_rows took is deferred to the next column (bulk_kc < 0: none)
     int bulk_kc = -1, bulk_lo = 0, bulk_pa = -1, bulk_pb = -1;
     for (int kc = 0; kc < b; ++kc) {
         const int c = c0 + kc;
+        const unsigned tag = (unsigned)(c + 1);
         MPF<L>* pr = prow[kc & 1];
-        if (tid < 32) {
-            // warp 0: wait for every stamp A of column kc, reduce the keys to
-            // the pivot, wait for the winner's stamp B (its reciprocal), then
-            // load the pivot row, its reciprocal and index and old row c
+        const int lo = max(r0, c + 1) - r0;  // first row below the pivot
+        const bool last = kc == b - 1;
+        const unsigned long long* orow = &sc->orow[kc % COOP_DEPTH][0][0];
+        if (warp == 0) {
+            // the rows' elements of column kc, before warp 1 makes them multipliers
+            MPF<L> x[Q];
+#pragma unroll
+            for (int q = 0; q < Q; ++q)
+                if (lane + 32 * q < nr) x[q] = a[(lane + 32 * q) * bs + kc];
+                else x[q] = mpf_make_zero<L>();
+            // every block's key of column kc
             constexpr int PER = (COOP_MAXG + 31) / 32;
-            const unsigned want = (unsigned)((c + 1) & 0xfffff);
+            const unsigned want = tag & 0xfffff;
             unsigned long long key[PER];
+            WaitBound wb;
             bool ok = true;
 #pragma unroll
-            for (int u = 0; u < PER; ++u) {
-                const int q = tid + 32 * u;
-                key[u] = 0;
-                if (q < G) key[u] = ld_acquire(&sc->part[kc & 1][q].stamp);
-            }
-#pragma unroll
-            for (int u = 0; u < PER; ++u) {
-                const int q = tid + 32 * u;
-                if (q < G && ok && (unsigned)(key[u] >> STAMP_SHIFT) != want) {
-                    key[u] = wait_stamp(&sc->part[kc & 1][q].stamp, want, &sc->error);
-                    ok = key[u] != 0;
-                }
-                key[u] &= KEY_MASK;
-            }
-            bool fail = __any_sync(0xffffffffu, !ok);
-            __syncwarp();
-            if (!fail) {
-                // the slots' contents are visible after their stamps (acquire loads)
-                unsigned long long K = 0;
-                int W = -1, dummy = 0;
+            for (int u = 0; u < PER; ++u) key[u] = 0;
+            for (;;) {
+                bool miss = false;
 #pragma unroll
                 for (int u = 0; u < PER; ++u) {
-                    const int q = tid + 32 * u;
+                    const int q = lane + 32 * u;
+                    if (q < G && (unsigned)(key[u] >> STAMP_SHIFT) != want) key[u] = ld_relaxed(&sc->part[kc % COOP_DEPTH][q].stamp);
+                }
+#pragma unroll
+                for (int u = 0; u < PER; ++u)
+                    miss |= lane + 32 * u < G && (unsigned)(key[u] >> STAMP_SHIFT) != want;
+                if (!__any_sync(0xffffffffu, miss)) break;
+                if (__any_sync(0xffffffffu, wb.expired(err))) {
+                    ok = false;
+                    break;
+                }
+            }
+            // (from here on a failed wait only sets ok: the column runs to its end on
+            // whatever was read, with no interchange, and the block leaves after it)
+            int W = -1;
+            {
+                unsigned long long K = 0;
+#pragma unroll
+                for (int u = 0; u < PER; ++u) {
+                    key[u] &= KEY_MASK;
+                    const int q = lane + 32 * u;
                     if (q < G && key[u] > 0 && (W < 0 || key[u] > K)) { K = key[u]; W = q; }
                 }
-                warp_best_key(K, W, dummy);  // lowest slot among equal keys
+                warp_best_key(K, W);  // lowest slot among equal keys
                 int same = 0;
 #pragma unroll
-                for (int u = 0; u < PER; ++u) same += (tid + 32 * u < G && key[u] == K) ? 1 : 0;
+                for (int u = 0; u < PER; ++u) same += (lane + 32 * u < G && key[u] == K) ? 1 : 0;
                 same = __reduce_add_sync(0xffffffffu, same);
                 if (same > 1) {
                     // equal keys: compare the candidates exactly (lowest row on ties)
                     MPF<L> v = mpf_make_zero<L>();
                     int vi = -1, vw = -1;
-#pragma unroll
+#pragma unroll 1
                     for (int u = 0; u < PER; ++u) {
-                        const int q = tid + 32 * u;
-                        if (q >= G || key[u] != K) continue;
-                        const CoopSlot<L>& slot = sc->part[kc & 1][q];
-                        const int iv = __ldcg(&slot.idx);
-                        const MPF<L> x = ld_cg<L>(&slot.row[kc]);
-                        if (mpf_better<L>(x, iv, v, vi)) { v = x; vi = iv; vw = q; }
+                        const int q = lane + 32 * u;
+                        bool mine = false;
+#pragma unroll
+                        for (int t = 0; t < PER; ++t) mine |= t == u && q < G && key[t] == K;
+                        const CoopSlot<L>& slot = sc->part[kc % COOP_DEPTH][mine ? q : 0];
+                        const unsigned long long* p[WORDS + 1];
+                        uint32_t w[WORDS + 1];
+#pragma unroll
+                        for (int i = 0; i < WORDS; ++i) p[i] = mine ? &slot.row[i][kc] : nullptr;
+                        p[WORDS] = mine ? &slot.idx : nullptr;
+                        ok = ok && wait_words<WORDS + 1>(p, tag, w, err);
+                        MPF<L> y;
+#pragma unroll
+                        for (int i = 0; i < L; ++i) y.m[i] = w[i];
+                        y.e = (int)w[L];
+                        y.neg = (int)w[L + 1];
+                        if (mine && mpf_better<L>(y, (int)w[WORDS], v, vi)) { v = y; vi = (int)w[WORDS]; vw = q; }
                     }
                     warp_best<L>(v, vi, vw);
                     W = vw;
                 }
-                if (W < 0) W = 0;  // W >= 0: the owner of row c has a candidate
-                // the pivot row (under stamp A) with all loads in flight before
-                // the first shared-memory store, then the reciprocal (stamp B)
-                const CoopSlot<L>& ws = sc->part[kc & 1][W];
-                const int piv = __ldcg(&ws.idx);
-                constexpr int PL = PBASE / 32;
-                MPF<L> v[PL];
-#pragma unroll
-                for (int q = 0; q < PL; ++q) {
-                    const int k = tid + 32 * q;
-                    if (k < b) v[q] = ld_cg<L>(&ws.row[k]);
-                }
-#pragma unroll
-                for (int q = 0; q < PL; ++q) {
-                    const int k = tid + 32 * q;
-                    if (k < b) pr[k] = v[q];
-                }
-                if (piv != c && owner(piv) == g) {
-#pragma unroll
-                    for (int q = 0; q < PL; ++q) {
-                        const int k = tid + 32 * q;
-                        if (k < b) v[q] = ld_cg<L>(&sc->orow[kc & 1][k]);
-                    }
-#pragma unroll
-                    for (int q = 0; q < PL; ++q) {
-                        const int k = tid + 32 * q;
-                        if (k < b) otmp[k] = v[q];
-                    }
-                }
-                int sb_ok = 1;
-                if (tid == 0) sb_ok = wait_stamp(&ws.stamp_rec, want, &sc->error) != 0;
-                fail = __shfl_sync(0xffffffffu, sb_ok, 0) == 0;
-                if (!fail && tid == 0) {
-                    rec = ld_cg<L>(&ws.rec);
-                    s_piv = piv;
-                }
+                if (W < 0) W = 0;  // (some block has a candidate: row c itself is one)
             }
-            if (tid == 0) s_fail = fail ? 1 : 0;
+            if (lane == 0) {
+                s_slot = W;
+                if (!ok) s_fail[kc & 1] = 1;
+            }
+            bar_sync(BAR_PIVOT, 128);
+            // the pivot's row, its element of column kc + 1, old row c's two
+            // elements (for the owner of the pivot row); then the reciprocal
+            const CoopSlot<L>& ws = sc->part[kc % COOP_DEPTH][W];
+            const bool word = lane < WORDS;
+            uint32_t w[4], wr[1];
+            {
+                const unsigned long long* p[4];
+                p[0] = &ws.idx;
+                p[1] = word && !last ? &ws.row[word ? lane : 0][last ? kc : kc + 1] : nullptr;
+                p[2] = word ? orow + lane * PBASE + kc : nullptr;
+                p[3] = word && !last ? orow + lane * PBASE + kc + 1 : nullptr;
+                ok &= wait_words<4>(p, tag, w, err);
+            }
+            const int piv = ok ? (int)w[0] : c;
+            const MPF<L> u = mpf_gather<L>(w[1]), ox = mpf_gather<L>(w[2]), oy = mpf_gather<L>(w[3]);
+            const bool swapped = piv != c && owns(piv);
+            MPF<L> s[Q];
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                if (swapped && lane + 32 * q == piv - r0) x[q] = ox;
+                s[q] = mpf_make_zero<L>();
+                if (32 * q < nr) s[q] = mpf_mul<L>(x[q], u);
+            }
+            __syncwarp();
+            {
+                const unsigned long long* p[1] = {word ? &ws.rec[word ? lane : 0] : nullptr};
+                ok &= wait_words<1>(p, tag, wr, err);
+            }
+            const MPF<L> rec = mpf_gather<L>(wr[0]);
+            const bool zero = mpf_zero<L>(rec);
+            bar_sync(BAR_COL, T);  // column kc + 1 carries the updates up to kc - 1
+            if (lane == 0) {
+                s_zero = zero ? 1 : 0;
+                if (!ok) s_fail[kc & 1] = 1;
+            }
+            if (!last) {
+                MPF<L> y[Q];
+#pragma unroll
+                for (int q = 0; q < Q; ++q) {
+                    y[q] = mpf_make_zero<L>();
+                    if (32 * q >= nr) break;
+                    const int r = lane + 32 * q;
+                    // (lanes past the last row work on it too, so that the warp stays together)
+                    const MPF<L> old = a[min(r, nr - 1) * bs + kc + 1];
+                    const bool from = !zero && swapped && r0 + r == piv;
+#pragma unroll
+                    for (int i = 0; i < L; ++i) y[q].m[i] = from ? oy.m[i] : old.m[i];
+                    y[q].e = from ? oy.e : old.e;
+                    y[q].neg = from ? oy.neg : old.neg;
+                    if (!zero) {
+                        y[q] = mpf_fms<L>(y[q], s[q], rec);
+                        if (r >= lo && r < nr) a[r * bs + kc + 1] = y[q];
+                    }
+                }
+                __syncwarp();
+                cand = choose(y, c + 1, kc + 1);
+            }
+        } else if (warp < 4) {
+            bar_sync(BAR_PIVOT, 128);
+            const CoopSlot<L>& ws = sc->part[kc % COOP_DEPTH][s_slot];
+            if (warp == 1) {
+                // the multipliers; the rows' elements of column kc as warp 0 has them
+                const bool word = lane < WORDS;
+                const unsigned long long* p[3] = {&ws.idx, word ? &ws.rec[word ? lane : 0] : nullptr,
+                                                  word ? orow + lane * PBASE + kc : nullptr};
+                uint32_t v[3];
+                const bool ok = wait_words<3>(p, tag, v, err);
+                const int piv = ok ? (int)v[0] : c;
+                const MPF<L> rec = mpf_gather<L>(v[1]), ox = mpf_gather<L>(v[2]);
+                const bool zero = mpf_zero<L>(rec);
+                if (lane == 0) {
+                    if (!ok) s_fail[kc & 1] = 1;
+                    if (g == 0) {
+                        ipiv[c] = piv + 1;
+                        if (zero && *info == 0) *info = c + 1;
+                    }
+                }
+                if (!zero)
+                    for (int r = lane; r < nr; r += 32)
+                        if (r >= lo) a[r * bs + kc] = mpf_mul<L>(piv != c && r0 + r == piv ? ox : a[r * bs + kc], rec);
+            } else {
+                // the pivot row, and the interchange (the owner of the pivot row
+                // leaves columns kc and kc + 1 to warps 1 and 0); two elements a lane
+                constexpr int H = PBASE / 64;
+                const int k0 = tid - 64;
+                const unsigned long long* p[H * WORDS + 2];
+                uint32_t v[H * WORDS + 2];
+#pragma unroll
+                for (int h = 0; h < H; ++h)
+#pragma unroll
+                    for (int i = 0; i < WORDS; ++i) p[h * WORDS + i] = k0 + 64 * h < b ? &ws.row[i][(k0 + 64 * h) & (PBASE - 1)] : nullptr;
+                p[H * WORDS] = &ws.idx;
+                p[H * WORDS + 1] = &ws.row[L - 1][kc];  // the pivot's top limb
+                bool ok = wait_words<H * WORDS + 2>(p, tag, v, err);
+                const int piv = ok ? (int)v[H * WORDS] : c;
+                const bool swap = v[H * WORDS + 1] != 0 && piv != c;
+#pragma unroll
+                for (int h = 0; h < H; ++h) {
+                    const int k = k0 + 64 * h;
+                    MPF<L> e;
+#pragma unroll
+                    for (int i = 0; i < L; ++i) e.m[i] = v[h * WORDS + i];
+                    e.e = (int)v[h * WORDS + L];
+                    e.neg = (int)v[h * WORDS + L + 1];
+                    if (k < b) {
+                        pr[k] = e;
+                        if (swap && owns(c)) a[(c - r0) * bs + k] = e;
+                    }
+                }
+                if (swap && owns(piv)) {
+#pragma unroll
+                    for (int h = 0; h < H; ++h)
+#pragma unroll
+                        for (int i = 0; i < WORDS; ++i)
+                            p[h * WORDS + i] = k0 + 64 * h < b ? orow + i * PBASE + ((k0 + 64 * h) & (PBASE - 1)) : nullptr;
+                    p[H * WORDS] = nullptr;
+                    p[H * WORDS + 1] = nullptr;
+                    ok &= wait_words<H * WORDS + 2>(p, tag, v, err);
+#pragma unroll
+                    for (int h = 0; h < H; ++h) {
+                        const int k = k0 + 64 * h;
+                        MPF<L> e;
+#pragma unroll
+                        for (int i = 0; i < L; ++i) e.m[i] = v[h * WORDS + i];
+                        e.e = (int)v[h * WORDS + L];
+                        e.neg = (int)v[h * WORDS + L + 1];
+                        if (k < b && k != kc && k != kc + 1) a[(piv - r0) * bs + k] = e;
+                    }
+                }
+                if (!ok && lane == 0) s_fail[kc & 1] = 1;
+            }
         } else if (bulk_kc >= 0) {
-            // warps 1 ..: the deferred update of the other rows by column bulk_kc
-            const int kb = bulk_kc, rest = b - kb - 2;
+            // warps 4 ..: the deferred update of the other rows by column bulk_kc
+            // (from bulk_kc + 3 on: warp 1 took column bulk_kc + 2)
+            const int kb = bulk_kc, rest = b - kb - 3;
             const MPF<L>* pk = prow[kb & 1];
-            const int total = (nr - bulk_lo) * rest;
-            for (int p = tid - 32; p < total; p += T - 32) {
-                const int r = bulk_lo + p / rest, k = kb + 2 + (p - (p / rest) * rest);
+            const int total = rest > 0 ? (nr - bulk_lo) * rest : 0;
+            for (int p = tid - 128; p < total; p += T - 128) {
+                const int r = bulk_lo + p / rest, k = kb + 3 + (p - (p / rest) * rest);
                 if (r == bulk_pa || r == bulk_pb) continue;
                 a[r * bs + k] = mpf_fms_oolv<L>(a[r * bs + k], a[r * bs + kb], pk[k]);
             }
         }
         __syncthreads();
-        if (s_fail) return;
-        const int piv = s_piv;
-        if (tid == 0) s_pivs[kc] = piv;
-        const bool zero = mpf_zero<L>(pr[kc]);
-        if (g == 0 && tid == 0) {
-            ipiv[c] = piv + 1;
-            if (zero && *info == 0) *info = c + 1;
-        }
-        if (!zero && piv != c) {
-            if (owner(c) == g)
-                for (int k = tid; k < b; k += T) a[(c - r0) * bs + k] = pr[k];
-            if (owner(piv) == g)
-                for (int k = tid; k < b; k += T) a[(piv - r0) * bs + k] = otmp[k];
-        }
-        __syncthreads();
-        const int lo = max(r0, c + 1) - r0;
-        const int cols = b - kc - 1;
-        if (!zero) {
-            // multipliers, then the next column first (its candidate is needed next)
-            for (int r = lo + tid; r < nr; r += T) {
-                mpf_mul_ool<L>(&a[r * bs + kc], &a[r * bs + kc], &rec);
-                if (cols > 0) a[r * bs + kc + 1] = mpf_fms_oolv<L>(a[r * bs + kc + 1], a[r * bs + kc], pr[kc + 1]);
+        if (s_fail[kc & 1]) return;
+        if (last) break;
+        const bool zero = s_zero != 0;
+        const int pa = s_cand >= 0 ? s_cand - r0 : -1;
+        const int pb = owns(c + 1) ? c + 1 - r0 : -1;
+        if (warp == 0) {
+            publish_rec(cand, kc + 1);
+        } else {
+            if (pub >= 0) {
+                publish_rows(kc, zero, pa, pb);
+            } else if (warp == 1 && !zero && kc + 2 < b) {
+                for (int r = lo + lane; r < nr; r += 32)
+                    if (r != pa && r != pb)
+                        a[r * bs + kc + 2] = mpf_fms_oolv<L>(a[r * bs + kc + 2], a[r * bs + kc], pr[kc + 2]);
             }
+            bar_arrive(BAR_COL, T);
         }
-        __syncthreads();
-        if (cols == 0) break;
-        // warp 0: the next candidate
-        if (tid < 32) candidate(kc + 1, c + 1);
-        __syncthreads();
-        // the rows the next step reads from this block: the candidate and (from
-        // its owner) row c + 1, which the pivot will replace
-        const int pa = ci >= 0 ? ci - r0 : -1;
-        const int pb = owner(c + 1) == g ? c + 1 - r0 : -1;
-        const int rest = cols - 1;
-        if (tid == 0) {
-            // the candidate's reciprocal and stamp B, beside the priority rows
-            publish_rec(kc + 1);
-        } else if (tid >= 32) {
-            if (!zero && rest > 0 && (warp & 3) != 0) {
-                const int nprio = (pa >= 0 ? 1 : 0) + (pb >= 0 && pb != pa ? 1 : 0);
-                const int pt = (warp - 1 - (warp >> 2)) * 32 + (tid & 31);
-                for (int p = pt; p < nprio * rest; p += NPRIO_T) {
-                    const int which = p / rest, k = kc + 2 + (p - which * rest);
-                    const int r = (which == 0 && pa >= 0) ? pa : pb;
-                    a[r * bs + k] = mpf_fms_oolv<L>(a[r * bs + k], a[r * bs + kc], pr[k]);
-                }
-            }
-            bar_rest();
-            // publish the candidate row of column kc + 1 and, from its owner,
-            // row c + 1; then stamp A with the key
-            CoopSlot<L>& slot = sc->part[(kc + 1) & 1][g];
-            const int wi = ci;
-            if (wi >= 0)
-                for (int k = tid - 32; k < b; k += T - 32) slot.row[k] = a[(wi - r0) * bs + k];
-            if (pb >= 0)
-                for (int k = tid - 32; k < b; k += T - 32) sc->orow[(kc + 1) & 1][k] = a[pb * bs + k];
-            if (tid == 32) slot.idx = wi;
-            bar_rest();
-            if (tid == 32) {
-                __threadfence();
-                const unsigned long long key = wi >= 0 ? mpf_key<L>(cv) : 0ull;
-                *reinterpret_cast<volatile unsigned long long*>(&slot.stamp) =
-                    ((unsigned long long)((c + 2) & 0xfffff) << STAMP_SHIFT) | key;
-            }
-        }
-        bulk_kc = (!zero && rest > 0) ? kc : -1;
+        bulk_kc = zero ? -1 : kc;
         bulk_lo = lo;
         bulk_pa = pa;
         bulk_pb = pb;
@@ -769,20 +952,6 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) base_block_coop_kernel(
     for (int p = tid; p < nr * b; p += T) {
         const int r = p / b, k = p - r * b;
         mpf_to_exp<L, N>(a[r * bs + k], elem(A, lda, N, r0 + r, c0 + k));
-    }
-    // the interchanges of this base block on the rest of the outer panel
-    // (columns [p0, c0) and [c0 + b, p1)), one column per thread
-    const int left = c0 - p0, span = left + (p1 - c0 - b);
-    for (int t = g * T + tid; t < span; t += G * T) {
-        const int j = t < left ? p0 + t : c0 + b + (t - left);
-        for (int kc = 0; kc < b; ++kc) {
-            const int pv = s_pivs[kc], c = c0 + kc;
-            if (pv == c) continue;
-            double* x = elem(A, lda, N, c, j);
-            double* y = elem(A, lda, N, pv, j);
-#pragma unroll
-            for (int q = 0; q < N; ++q) { const double tt = x[q]; x[q] = y[q]; y[q] = tt; }
-        }
     }
 }
 
@@ -804,45 +973,52 @@ __global__ void laswp_kernel(double* A, long long lda, int j0, int j1, int k0, i
 }
 
 // Interchanges k in [k0, k1) (ipiv 1-based) applied to columns [j0, j1) as one
-// permutation: every block replays the swaps on the few affected rows (a
-// shared-memory hash map: position -> row whose contents end up there), then
-// gathers those rows of its LCT columns into shared memory and writes them
-// back permuted.  Replaces the column-serial swap chain.
+// permutation: one block lists the (destination, source) row pairs, then every
+// block of laswp_apply_kernel gathers those rows of its LCT columns into shared
+// memory and writes them back permuted.  Replaces the column-serial swap chain.
 
-// one block: the (destination, source) row pairs of the interchanges
-__global__ void __launch_bounds__(256) laswp_list_kernel(int k0, int k1, const int* ipiv, int* list) {
-    __shared__ int hkey[LHASH], hval[LHASH];
+// Position k < b stands for row k0 + k, position b + j for a row p >= k1 first
+// named by interchange j.  The threads find each interchange's positions; one
+// thread then replays the swaps on the contents (two shared-memory loads and
+// stores a swap, the next positions loaded ahead).  With a hash map filled by that
+// thread the list took 50 us for 256 interchanges.
+__global__ void __launch_bounds__(LMAXB) laswp_list_kernel(int k0, int k1, const int* ipiv, int* list) {
+    __shared__ int piv[LMAXB], slot[LMAXB + 1], val[2 * LMAXB], row[2 * LMAXB];
     __shared__ int cnt;
-    for (int i = threadIdx.x; i < LHASH; i += blockDim.x) hkey[i] = -1;
-    if (threadIdx.x == 0) cnt = 0;
+    const int b = k1 - k0, t = threadIdx.x;
+    if (t < b) piv[t] = ipiv[k0 + t] - 1;
+    if (t == 0) cnt = 0;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        auto slot = [&](int row) {
-            int h = (int)(((unsigned)row * 2654435761u) & (LHASH - 1));
-            while (hkey[h] != -1 && hkey[h] != row) h = (h + 1) & (LHASH - 1);
-            return h;
-        };
-        for (int k = k0; k < k1; ++k) {
-            const int p = ipiv[k] - 1;
-            if (p == k) continue;
-            const int sk = slot(k);
-            if (hkey[sk] == -1) { hkey[sk] = k; hval[sk] = k; }
-            const int sp = slot(p);
-            if (hkey[sp] == -1) { hkey[sp] = p; hval[sp] = p; }
-            const int t = hval[sk];
-            hval[sk] = hval[sp];
-            hval[sp] = t;
+    if (t < b) {
+        const int p = piv[t];
+        int j = t;
+        if (p >= k1)
+            for (j = 0; piv[j] != p; ++j) {}
+        slot[t] = p < k1 ? p - k0 : b + j;
+        row[t] = val[t] = k0 + t;
+        row[b + t] = p >= k1 && j == t ? p : -1;
+        val[b + t] = p;
+    }
+    __syncthreads();
+    if (t == 0) {
+        int nxt = slot[0];
+        for (int k = 0; k < b; ++k) {
+            const int sl = nxt;
+            nxt = slot[k + 1];  // (one past the end is in bounds)
+            const int x = val[k], y = val[sl];
+            val[k] = y;
+            val[sl] = x;
         }
     }
     __syncthreads();
-    for (int h = threadIdx.x; h < LHASH; h += blockDim.x)
-        if (hkey[h] != -1 && hval[h] != hkey[h]) {
+    for (int q = t; q < 2 * b; q += blockDim.x)
+        if (row[q] >= 0 && val[q] != row[q]) {
             const int c = atomicAdd(&cnt, 1);
-            list[1 + 2 * c] = hkey[h];
-            list[2 + 2 * c] = hval[h];
+            list[1 + 2 * c] = row[q];
+            list[2 + 2 * c] = val[q];
         }
     __syncthreads();
-    if (threadIdx.x == 0) list[0] = cnt;
+    if (t == 0) list[0] = cnt;
 }
 
 template <int N>
@@ -880,7 +1056,7 @@ void laswp2(double* A, long long lda, int ja0, int ja1, int jb0, int jb1, int k0
         if (jb1 > jb0) laswp_kernel<N><<<(jb1 - jb0 + 127) / 128, 128, 0, s>>>(A, lda, jb0, jb1, k0, k1, ipiv);
         return;
     }
-    laswp_list_kernel<<<1, 256, 0, s>>>(k0, k1, ipiv, list);
+    laswp_list_kernel<<<1, (k1 - k0 + 31) / 32 * 32, 0, s>>>(k0, k1, ipiv, list);
     const size_t smem = sizeof(double) * 2 * (k1 - k0) * LCT * N;
     raise_smem_limit((const void*)laswp_apply_kernel<N>, (int)(sizeof(double) * 2 * LMAXB * LCT * N));
     if (ja1 > ja0) laswp_apply_kernel<N><<<(ja1 - ja0 + LCT - 1) / LCT, 256, smem, s>>>(A, lda, ja0, ja1, list);
@@ -1003,8 +1179,8 @@ void trsm_base(const double* T, long long ldt, double* X, long long ldx, int b, 
 // Launch the cooperative base-block kernel; returns false when the slice of
 // rows does not fit in shared memory (the caller then uses column kernels).
 template <int N>
-bool base_block_coop(double* A, long long lda, int n, int c0, int b, int p0, int p1, int* ipiv,
-                     int* info, void* scratch, int min_rows, cudaStream_t s) {
+bool base_block_coop(double* A, long long lda, int n, int c0, int b, int* ipiv, int* info, void* scratch,
+                     int min_rows, cudaStream_t s) {
     constexpr int L = Limbs<N>::L;
     const int sms = device_sms();
     // at least min_rows rows per block: a small panel takes a few SMs and
@@ -1017,11 +1193,13 @@ bool base_block_coop(double* A, long long lda, int n, int c0, int b, int p0, int
         if (G > g_rows) G = g_rows < 1 ? 1 : g_rows;
         const int rows = (n - c0 + G - 1) / G;
         const size_t smem = sizeof(MPF<L>) * (size_t)rows * (b + 1);
-        if (smem > 200 * 1024 / per_sm) continue;
-        raise_smem_limit((const void*)base_block_coop_kernel<N>, (int)(smem < 1024 ? 1024 : smem));
+        if (rows > 256 || smem > 200 * 1024 / per_sm) continue;
+        // rows per lane of warp 0: two keep its values in registers (n to 9728 at
+        // one block per SM); more rows only meet narrow blocks
+        const auto kernel = rows <= 64 ? base_block_coop_kernel<N, 2> : base_block_coop_kernel<N, 8>;
+        raise_smem_limit((const void*)kernel, (int)(smem < 1024 ? 1024 : smem));
         int active = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&active, base_block_coop_kernel<N>, COOP_THREADS,
-                                                      smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&active, kernel, COOP_THREADS, smem);
         if (active * sms < G) continue;
         auto* sc = reinterpret_cast<CoopScratch<L>*>(scratch);
         // cooperative launch (all blocks co-resident), also valid under stream capture
@@ -1035,7 +1213,7 @@ bool base_block_coop(double* A, long long lda, int n, int c0, int b, int p0, int
         attr[0].val.cooperative = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        if (cudaLaunchKernelEx(&cfg, base_block_coop_kernel<N>, A, lda, n, c0, b, p0, p1, rows, ipiv, info, sc) !=
+        if (cudaLaunchKernelEx(&cfg, kernel, A, lda, n, c0, b, rows, ipiv, info, sc) !=
             cudaSuccess) {
             cudaGetLastError();
             return false;
@@ -1112,9 +1290,14 @@ void panel_rec(Ctx& c, int r, int b, int p0, int p1) {
     // in shared memory (else the block is split further)
     if (b <= coop_width(c, r)) {
         c.h->phase(PH_PANEL);
-        if (base_block_coop<N>(c.A, c.lda, c.n, r, b, p0, p1, c.ipiv, &c.sc->info, c.h->coop_scratch,
+        if (base_block_coop<N>(c.A, c.lda, c.n, r, b, c.ipiv, &c.sc->info, c.h->coop_scratch,
                                c.h->coop_min_rows, s)) {
             c.h->count(1);
+            if (p0 < r || r + b < p1) {
+                c.h->phase(PH_OTHER);
+                laswp2<N>(c.A, c.lda, p0, r, r + b, p1, r, r + b, c.ipiv, c.sc->plist, s);
+                c.h->count(1 + (p0 < r) + (r + b < p1));
+            }
             c.h->stats.panel_launches += 1;
             return;
         }
@@ -1217,7 +1400,7 @@ size_t align256(size_t v) { return (v + 255) / 256 * 256; }
 }  // namespace
 
 int lu_scratch(ozlu_handle* h, LuScratch** out);
-int coop_reset(ozlu_handle* h, int nc, cudaStream_t s);
+int coop_reset(ozlu_handle* h, int nc, int n, cudaStream_t s);
 
 namespace {
 // info of one factorisation: the first zero pivot (1-based), or
@@ -1253,7 +1436,7 @@ int wait_expiry_selftest(ozlu_handle* h, int which, long long limit, int* out) {
     int* gerr = err_word(h);
     if (!gerr) return OZLU_ERR_NOMEM;
     if (cudaMemsetAsync(sc, 0, sizeof(LuScratch), s)) return OZLU_ERR_CUDA;
-    if ((rc = coop_reset(h, 4, s))) return rc;
+    if ((rc = coop_reset(h, 4, 1, s))) return rc;
     if ((rc = clear_err_word(h))) return rc;
     // the candidate area of the scratch (zeroed above) holds a stamp word that
     // nothing writes and the kernel's flag
@@ -1293,7 +1476,7 @@ int getrf_one(ozlu_handle* h, int nc, int p, int n, double* A, long long lda, in
     // rank-1 update of the whole trailing matrix in expansion arithmetic
     if (opts && opts->native == 2) nb = 1;
     if (cudaMemsetAsync(sc, 0, sizeof(LuScratch), s)) return OZLU_ERR_CUDA;
-    if ((rc = coop_reset(h, nc, s))) return rc;
+    if ((rc = coop_reset(h, nc, n, s))) return rc;
     if ((rc = clear_err_word(h))) return rc;
     if (n > 0) {
         switch (nc) {
@@ -1337,14 +1520,19 @@ int lu_scratch(ozlu_handle* h, LuScratch** out) {
     return OZLU_OK;
 }
 
-// the error word and the slot stamps start at zero for every factorisation
-int coop_reset(ozlu_handle* h, int nc, cudaStream_t s) {
+// the error word and the tagged words of the blocks a panel of n rows can have
+// start at zero for every factorisation
+int coop_reset(ozlu_handle* h, int nc, int n, cudaStream_t s) {
+    int G = (n + h->coop_min_rows - 1) / h->coop_min_rows;
+    if (G > 2 * device_sms()) G = 2 * device_sms();
+    if (G > COOP_MAXG) G = COOP_MAXG;
+    const dim3 grid(G < 1 ? 1 : G, COOP_DEPTH);
     // the slot layout is that of the panel kernel's limb count for nc
     constexpr int L2 = Limbs<2>::L, L3 = Limbs<3>::L, L4 = Limbs<4>::L;
     switch (nc) {
-        case 2: coop_reset_kernel<L2><<<1, 2 * COOP_MAXG, 0, s>>>((CoopScratch<L2>*)h->coop_scratch); break;
-        case 3: coop_reset_kernel<L3><<<1, 2 * COOP_MAXG, 0, s>>>((CoopScratch<L3>*)h->coop_scratch); break;
-        default: coop_reset_kernel<L4><<<1, 2 * COOP_MAXG, 0, s>>>((CoopScratch<L4>*)h->coop_scratch); break;
+        case 2: coop_reset_kernel<L2><<<grid, 256, 0, s>>>((CoopScratch<L2>*)h->coop_scratch); break;
+        case 3: coop_reset_kernel<L3><<<grid, 256, 0, s>>>((CoopScratch<L3>*)h->coop_scratch); break;
+        default: coop_reset_kernel<L4><<<grid, 256, 0, s>>>((CoopScratch<L4>*)h->coop_scratch); break;
     }
     h->count(1);
     return cudaGetLastError() == cudaSuccess ? OZLU_OK : OZLU_ERR_CUDA;

@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(1024) mp_shift_kernel(MPView A, int m, MPView 
 // complement with a constant per modulus (ConvMod::k4, picked by a one-hot
 // dot product).  Bound by integer issue.  A block covers eight consecutive rows,
 // so that the limb sectors of A's columns are shared in L1.
-// 512 x 512 each, p = 1024, FP8 digits: @@@ us with the exponents; the former
+// 512 x 512 each, p = 1024, FP8 digits: 273 us with the exponents; the former
 // kernel (a warp per element, a lane per residue, the table in constant memory
 // read at 32 addresses at once) 3836 us.
 // E = 4 where that leaves two blocks of 256 threads per SM, else E = 1 and the

@@ -11,6 +11,7 @@
 
 #include <stdint.h>
 
+#include "carry.cuh"
 #include "mp_device.cuh"
 
 namespace ozlu {
@@ -37,67 +38,54 @@ __device__ __forceinline__ MPF<L> mpf_make_zero() {
     return r;
 }
 
-// Round the W-word magnitude X (top word nonzero or all zero) to L words:
-// normalise, keep the top 32 L bits, round to nearest even with a sticky.
-// `ex` is the exponent such that value = X * 2^(ex - 32 W).
+// The rounding of a normalised W-word magnitude X 2^(ex - 32 W) to its top L
+// words, to nearest even with a sticky for what lies below X: one carry chain
 template <int L, int W>
-__device__ __forceinline__ MPF<L> mpf_round(uint32_t (&X)[W], int ex, int neg, bool sticky_in) {
+__device__ __forceinline__ MPF<L> mpf_round_top(const uint32_t (&X)[W], int ex, int neg, bool sticky) {
     MPF<L> r;
-    r.neg = neg;
-    const int bl = bit_length<W>(X);
-    if (bl == 0) {
-        r = mpf_make_zero<L>();
-        return r;
-    }
-    // shift left so that the top bit is bit 32W-1
-    const int sh = 32 * W - bl;
-    if (sh > 0 && sh < 32) {
-        // common case: the top word is nonzero, a funnel shift of every word
-#pragma unroll
-        for (int i = W - 1; i > 0; --i) X[i] = __funnelshift_l(X[i - 1], X[i], sh);
-        X[0] <<= sh;
-    } else if (sh >= 32) {
-        // whole words by a logarithmic shifter (selects, no dynamic indexing), then bits
-        const int q = sh >> 5, rr = sh & 31;
-#pragma unroll
-        for (int s = 8; s >= 1; s >>= 1) {
-            if (s < W) {
-                const bool on = (q & s) != 0;
-#pragma unroll
-                for (int i = W - 1; i >= 0; --i) X[i] = on ? (i >= s ? X[i - s] : 0u) : X[i];
-            }
-        }
-#pragma unroll
-        for (int i = W - 1; i > 0; --i) X[i] = __funnelshift_l(X[i - 1], X[i], rr);
-        X[0] <<= rr;
-    }
-    ex -= sh;
-    // top L words; round bit = top bit of word W-L-1; sticky = the rest
-    bool rbit = false, sticky = sticky_in;
+    uint32_t up = 0;
     if (W > L) {
-        rbit = (X[W - L - 1] >> 31) != 0;
-        sticky |= (X[W - L - 1] & 0x7fffffffu) != 0;
+        uint32_t low = X[W - L - 1] & 0x7fffffffu;
 #pragma unroll
-        for (int i = 0; i < W - L - 1; ++i) sticky |= X[i] != 0;
+        for (int i = 0; i < W - L - 1; ++i) low |= X[i];
+        up = (X[W - L - 1] >> 31) & ((low != 0 || sticky) ? 1u : X[W - L] & 1u);
     }
+    r.m[0] = add_first(X[W - L], up);
 #pragma unroll
-    for (int i = 0; i < L; ++i) r.m[i] = X[W - L + i];
+    for (int i = 1; i < L; ++i) r.m[i] = add_next(X[W - L + i], 0u);
     // X * 2^(ex - 32 W) with the top L words kept: m * 2^(ex - 32 L)
     r.e = ex;
-    if (rbit && (sticky || (r.m[0] & 1u))) {
-        uint64_t c = 1;
-#pragma unroll
-        for (int i = 0; i < L; ++i) {
-            const uint64_t s = (uint64_t)r.m[i] + c;
-            r.m[i] = (uint32_t)s;
-            c = s >> 32;
-        }
-        if (c) {  // carried out: 1000...0
-            r.m[L - 1] = 0x80000000u;
-            r.e += 1;
-        }
+    r.neg = neg;
+    if (r.m[L - 1] == 0) {  // carried out: 1000...0
+        r.m[L - 1] = 0x80000000u;
+        r.e += 1;
     }
     return r;
+}
+
+// Round the W-word magnitude X (any leading zeros) to L words: normalise, keep
+// the top 32 L bits, round to nearest even with a sticky.  `ex` is the exponent
+// such that value = X * 2^(ex - 32 W).  Whole zero words at the top come only
+// from a cancellation of 32 bits or more: they are shifted out one at a time.
+template <int L, int W>
+__device__ __forceinline__ MPF<L> mpf_round(uint32_t (&X)[W], int ex, int neg, bool sticky_in) {
+    if (X[W - 1] == 0) {
+        uint32_t any = 0;
+#pragma unroll
+        for (int i = 0; i < W - 1; ++i) any |= X[i];
+        if (any == 0) return mpf_make_zero<L>();
+        do {
+#pragma unroll
+            for (int i = W - 1; i > 0; --i) X[i] = X[i - 1];
+            X[0] = 0;
+            ex -= 32;
+        } while (X[W - 1] == 0);
+    }
+    const int sh = __clz(X[W - 1]);
+#pragma unroll
+    for (int i = W - 1; i > 0; --i) X[i] = __funnelshift_l(X[i - 1], X[i], sh);
+    X[0] <<= sh;
+    return mpf_round_top<L, W>(X, ex - sh, neg, sticky_in);
 }
 
 // from an expansion of N binary64 components (sticky-truncated to 32(L+2) bits,
@@ -196,30 +184,52 @@ __device__ __forceinline__ int mpf_abs_cmp(const MPF<L>& a, const MPF<L>& b) {
     return 0;
 }
 
-// Exact product of two L-word magnitudes (2 L words): column sums of the
-// 32-bit halves of the limb products (independent, each below
-// 2^(33 + log2 L)), then one carry pass.  (Carry-flag chains of 32-bit
-// multiply-adds measured slower on GB300: they serialise on the flag.)
-template <int L>
-__device__ __forceinline__ void mul_words(const uint32_t (&a)[L], const uint32_t (&b)[L], uint32_t (&P)[2 * L]) {
-    uint64_t S[2 * L];
+// Words K0 .. NA + NB - 1 of the product of an NA-word and an NB-word magnitude
+// (exact for K0 = 0; else without the products below column K0, whose carry is
+// under min(NA, NB) units of word K0).  Every 64-bit product a_i b_j is added at
+// word i + j; those at even and at odd distance from K0 have an accumulator of
+// their own, so that a row of each is one chain of wide multiply-adds on
+// aligned word pairs (one instruction a product), and the two are added at the
+// end.  7 x 7 words: 91 instructions and 315 cycles on one warp; the column sums
+// of 32-bit halves that stood here before, 181 and 410.
+template <int NA, int NB, int K0>
+__device__ __forceinline__ void mul_words(const uint32_t (&a)[NA], const uint32_t (&b)[NB],
+                                          uint32_t (&P)[NA + NB - K0]) {
+    constexpr int W = NA + NB - K0;
+    uint32_t E[W + 1], O[W + 1];  // O: word k + 1 at O[k]
 #pragma unroll
-    for (int k = 0; k < 2 * L; ++k) S[k] = 0;
-#pragma unroll
-    for (int i = 0; i < L; ++i)
-#pragma unroll
-        for (int j = 0; j < L; ++j) {
-            const uint64_t t = (uint64_t)a[i] * b[j];
-            S[i + j] += (uint32_t)t;
-            S[i + j + 1] += t >> 32;
-        }
-    uint64_t c = 0;
-#pragma unroll
-    for (int k = 0; k < 2 * L; ++k) {
-        const uint64_t v = S[k] + c;
-        P[k] = (uint32_t)v;
-        c = v >> 32;
+    for (int k = 0; k <= W; ++k) {
+        E[k] = 0;
+        O[k] = 0;
     }
+#pragma unroll
+    for (int i = 0; i < NA; ++i) {
+        int last = -1;
+#pragma unroll
+        for (int j = 0; j < NB; ++j) {
+            const int k = i + j - K0;
+            if (k < 0 || (k & 1)) continue;
+            E[k] = last < 0 ? mad_lo_first(a[i], b[j], E[k]) : mad_lo_next(a[i], b[j], E[k]);
+            E[k + 1] = mad_hi_next(a[i], b[j], E[k + 1]);
+            last = k;
+        }
+        // the word above a row's chain has only taken such carries so far
+        if (last >= 0 && last + 2 < W) E[last + 2] = add_last(E[last + 2], 0u);
+        last = -1;
+#pragma unroll
+        for (int j = 0; j < NB; ++j) {
+            const int k = i + j - K0;
+            if (k < 0 || !(k & 1)) continue;
+            O[k - 1] = last < 0 ? mad_lo_first(a[i], b[j], O[k - 1]) : mad_lo_next(a[i], b[j], O[k - 1]);
+            O[k] = mad_hi_next(a[i], b[j], O[k]);
+            last = k;
+        }
+        if (last >= 0 && last + 2 < W) O[last + 1] = add_last(O[last + 1], 0u);
+    }
+    P[0] = E[0];
+    P[1] = add_first(E[1], O[0]);
+#pragma unroll
+    for (int k = 2; k < W; ++k) P[k] = add_next(E[k], O[k - 1]);
 }
 
 // a * b, rounded to L words
@@ -227,9 +237,13 @@ template <int L>
 __device__ __forceinline__ MPF<L> mpf_mul(const MPF<L>& a, const MPF<L>& b) {
     if (mpf_zero<L>(a) || mpf_zero<L>(b)) return mpf_make_zero<L>();
     uint32_t P[2 * L];
-    mul_words<L>(a.m, b.m, P);
-    // value = P * 2^(a.e + b.e - 64 L) = P * 2^((a.e + b.e) - 32 * 2L)
-    return mpf_round<L, 2 * L>(P, a.e + b.e, a.neg ^ b.neg, false);
+    mul_words<L, L, 0>(a.m, b.m, P);
+    // value = P * 2^((a.e + b.e) - 32 * 2L), P in [2^(64 L - 2), 2^(64 L)): one bit at most
+    const int sh = P[2 * L - 1] >> 31 ? 0 : 1;
+#pragma unroll
+    for (int i = 2 * L - 1; i > 0; --i) P[i] = __funnelshift_l(P[i - 1], P[i], sh);
+    P[0] <<= sh;
+    return mpf_round_top<L, 2 * L>(P, a.e + b.e - sh, a.neg ^ b.neg, false);
 }
 
 // a + b, rounded to L words (guard words and a sticky keep it correctly rounded)
@@ -314,151 +328,90 @@ __device__ __forceinline__ MPF<L> mpf_sub(const MPF<L>& a, const MPF<L>& b) {
     return mpf_add<L>(a, mpf_neg<L>(b));
 }
 
-// Y >>= d bits (d >= 0) by a logarithmic word shifter and a funnel shift;
-// sticky collects the bits shifted out
-template <int W>
-__device__ __forceinline__ void shr_sticky(uint32_t (&Y)[W], int d, bool& sticky) {
-    if (d >= 32 * W) {
-        bool any = false;
-#pragma unroll
-        for (int i = 0; i < W; ++i) {
-            any |= Y[i] != 0;
-            Y[i] = 0;
-        }
-        sticky |= any;
-        return;
-    }
-    const int q = d >> 5, r = d & 31;
-#pragma unroll
-    for (int s = 16; s >= 1; s >>= 1) {
-        if (s < W) {
-            const bool on = (q & s) != 0;
-            uint32_t lost = 0;
-#pragma unroll
-            for (int i = 0; i < s; ++i) lost |= Y[i];
-            sticky |= on && lost != 0;
-#pragma unroll
-            for (int i = 0; i < W; ++i) Y[i] = on ? (i + s < W ? Y[i + s] : 0u) : Y[i];
-        }
-    }
-    sticky |= r != 0 && (Y[0] & ((1u << r) - 1u)) != 0;
-#pragma unroll
-    for (int i = 0; i < W - 1; ++i) Y[i] = __funnelshift_r(Y[i], Y[i + 1], r);
-    Y[W - 1] >>= r;
-}
-
-// (-1)^xn X 2^(ex - 32 W) + (-1)^yn Y 2^(ey - 32 W), both W-word magnitudes
-// normalised (top bit set) or zero (xz, yz), rounded to L words; ysticky:
-// Y stands for a value with more nonzero bits below its last word
-template <int L, int W>
-__device__ __forceinline__ MPF<L> add_windows(uint32_t (&X)[W], int ex, int xn, bool xz, uint32_t (&Y)[W], int ey,
-                                              int yn, bool yz, bool ysticky) {
-    if (yz) return mpf_round<L, W>(X, ex, xn, false);
-    if (xz) return mpf_round<L, W>(Y, ey, yn, ysticky);
-    bool swap = ey > ex;  // |Y| > |X|
-    if (ey == ex) {
-        int cmp = 0;
-#pragma unroll
-        for (int i = W - 1; i >= 0; --i)
-            if (cmp == 0 && X[i] != Y[i]) cmp = X[i] > Y[i] ? 1 : -1;
-        swap = cmp < 0;
-    }
-    uint32_t A[W], B[W];
-#pragma unroll
-    for (int i = 0; i < W; ++i) {
-        A[i] = swap ? Y[i] : X[i];
-        B[i] = swap ? X[i] : Y[i];
-    }
-    const int ea = swap ? ey : ex, eb = swap ? ex : ey;
-    const int an = swap ? yn : xn, bn = swap ? xn : yn;
-    bool sticky = swap ? false : ysticky;
-    shr_sticky<W>(B, ea - eb, sticky);
-    if (an == bn) {
-        uint64_t c = 0;
-#pragma unroll
-        for (int i = 0; i < W; ++i) {
-            const uint64_t s = (uint64_t)A[i] + B[i] + c;
-            A[i] = (uint32_t)s;
-            c = s >> 32;
-        }
-        if (c) {
-            sticky |= (A[0] & 1u) != 0;
-#pragma unroll
-            for (int i = 0; i < W - 1; ++i) A[i] = (A[i] >> 1) | (A[i + 1] << 31);
-            A[W - 1] = (A[W - 1] >> 1) | 0x80000000u;
-            return mpf_round<L, W>(A, ea + 1, an, sticky);
-        }
-        return mpf_round<L, W>(A, ea, an, sticky);
-    }
-    // the exact difference is A - B - delta with 0 <= delta < 1 unit of the
-    // window: A - B - 1 plus a set sticky stands for it whenever delta > 0
-    uint64_t brw = sticky ? 1u : 0u;
-#pragma unroll
-    for (int i = 0; i < W; ++i) {
-        const uint64_t s = (uint64_t)A[i] - B[i] - brw;
-        A[i] = (uint32_t)s;
-        brw = (s >> 63) & 1u;
-    }
-    // a borrow out means A == B with the sticky set: the exact difference is
-    // below one unit of the window's last word (zero for an exact
-    // cancellation such as c = a b) and is returned as zero
-    if (brw) return mpf_make_zero<L>();
-    return mpf_round<L, W>(A, ea, an, sticky);
-}
-
-// c - a b with one rounding: the product's top L + 2 words (words L - 2 ..
-// 2L - 1 of the 2L-word product, from the limb products that reach them; the
-// carry lost from the words below is under 2^5 units of the lowest window
-// word) are added to c in an (L + 2)-word window, the lower words counting as
-// a set sticky.  The result is the correctly rounded c - a b unless the exact
-// value lies within about 2^-58 of a unit of its last word from a rounding
-// boundary.
+// c - a b with one rounding: the product's top L + 2 words (from the columns
+// that reach them and one guard column; what is left out is under 2^-28 of
+// the lowest window word) meet c in an (L + 2)-word window, the lower words
+// counting as a set sticky.  The result is the correctly rounded c - a b unless
+// the exact value lies within about 2^-58 of a unit of its last word from a
+// rounding boundary.  Written for a short dependent chain and few
+// instructions, since the LU's panels and triangular solves run it on one warp
+// or two per scheduler: chains on the carry flag throughout, the alignment by
+// a loop over whole words (the exponents mostly lie within a word or two) and one
+// funnel shift, addition and subtraction as one chain on B or its complement.
+// L = 7: 724 cycles on one warp, 96 SM cycles a warp with 16 of them; the QD
+// triangular solves of the n = 4096 LU went from 14.3 to 10.3 ms with it.
 template <int L>
 __device__ __forceinline__ MPF<L> mpf_fms(const MPF<L>& c, const MPF<L>& a, const MPF<L>& b) {
     static_assert(L >= 4, "two guard words below the product window");
     constexpr int W = L + 2;
     if (mpf_zero<L>(a) || mpf_zero<L>(b)) return c;
-    // window word k = product word k + L - 2: lo(a_i b_j) for i + j >= L - 2,
-    // hi(a_i b_j) for i + j >= L - 3
-    uint64_t S[W + 1];
-#pragma unroll
-    for (int k = 0; k <= W; ++k) S[k] = 0;
-#pragma unroll
-    for (int i = 0; i < L; ++i)
-#pragma unroll
-        for (int j = 0; j < L; ++j) {
-            const int k = i + j - (L - 2);
-            if (k >= 0) {
-                const uint64_t t = (uint64_t)a.m[i] * b.m[j];
-                S[k] += (uint32_t)t;
-                S[k + 1] += t >> 32;
-            } else if (k == -1) {
-                S[0] += __umulhi(a.m[i], b.m[j]);
-            }
-        }
+    uint32_t G[W + 1];
+    mul_words<L, L, L - 3>(a.m, b.m, G);
+    // a b ~ P 2^(ep - 32 W), P the top W words of G, normalised (the top bit may be clear)
+    const int up1 = G[W] >> 31 ? 0 : 1;
     uint32_t P[W];
-    uint64_t cy = 0;
 #pragma unroll
-    for (int k = 0; k < W; ++k) {
-        const uint64_t v = S[k] + cy;
-        P[k] = (uint32_t)v;
-        cy = v >> 32;
+    for (int i = 0; i < W; ++i) P[i] = __funnelshift_l(G[i], G[i + 1], up1);
+    const int ep = a.e + b.e - up1;
+    const int pn = a.neg ^ b.neg ^ 1;
+    if (mpf_zero<L>(c)) return mpf_round_top<L, W>(P, ep, pn, true);
+    // A: the operand of the larger exponent (c on a tie), B the other
+    const bool swap = ep > c.e;
+    uint32_t A[W], B[W];
+#pragma unroll
+    for (int i = 0; i < W; ++i) {
+        const uint32_t cw = i < 2 ? 0u : c.m[i < 2 ? 0 : i - 2];
+        A[i] = swap ? P[i] : cw;
+        B[i] = swap ? cw : P[i];
     }
-    // a b ~ P 2^(ep - 32 W); normalise (the top bit may be clear)
-    int ep = a.e + b.e;
-    if (!(P[W - 1] >> 31)) {
+    const int ea = swap ? ep : c.e;
+    int an = swap ? pn : c.neg;
+    int d = swap ? ep - c.e : c.e - ep;
+    // B >>= d; the bits shifted out and, where B is the product, its words left
+    // out make the sticky
+    bool sticky = !swap;
+    if (d >= 32 * W) {
+        sticky = true;
 #pragma unroll
-        for (int i = W - 1; i > 0; --i) P[i] = __funnelshift_l(P[i - 1], P[i], 1);
-        P[0] <<= 1;
-        ep -= 1;
+        for (int i = 0; i < W; ++i) B[i] = 0;
+    } else {
+        uint32_t lost = 0;
+        for (; d >= 32; d -= 32) {
+            lost |= B[0];
+#pragma unroll
+            for (int i = 0; i < W - 1; ++i) B[i] = B[i + 1];
+            B[W - 1] = 0;
+        }
+        lost |= __funnelshift_r(0u, B[0], d);
+        sticky |= lost != 0;
+#pragma unroll
+        for (int i = 0; i < W - 1; ++i) B[i] = __funnelshift_r(B[i], B[i + 1], d);
+        B[W - 1] >>= d;
     }
-    const bool sticky = true;
-    uint32_t C[W];
-    C[0] = 0;
-    C[1] = 0;
+    // A + B, or A - B - delta with 0 < delta < 1 unit of the window where the
+    // sticky is set: A - B - 1 plus a set sticky stands for it
+    const uint32_t f = c.neg != pn ? 0xffffffffu : 0u;
+    add_first(f, f & (sticky ? 0u : 1u));  // the flag: set for an exact difference
 #pragma unroll
-    for (int i = 0; i < L; ++i) C[i + 2] = c.m[i];
-    return add_windows<L, W>(C, c.e, c.neg, mpf_zero<L>(c), P, ep, a.neg ^ b.neg ^ 1, false, sticky);
+    for (int i = 0; i < W; ++i) A[i] = add_next(A[i], B[i] ^ f);
+    const uint32_t cy = add_last(0u, 0u);
+    if (f == 0) {
+        if (cy) {
+            sticky |= (A[0] & 1u) != 0;
+#pragma unroll
+            for (int i = 0; i < W - 1; ++i) A[i] = __funnelshift_r(A[i], A[i + 1], 1);
+            A[W - 1] = (A[W - 1] >> 1) | 0x80000000u;
+            return mpf_round_top<L, W>(A, ea + 1, an, sticky);
+        }
+    } else if (!cy) {
+        // A < B + delta (equal exponents): B - A of the other sign; zero for an
+        // exact cancellation such as c = a b
+#pragma unroll
+        for (int i = 0; i < W; ++i) A[i] = ~A[i];
+        an ^= 1;
+        sticky = false;
+    }
+    return mpf_round<L, W>(A, ea, an, sticky);
 }
 
 // Out-of-line copies of the fused multiply-subtract and the product.  A kernel
@@ -475,16 +428,6 @@ __device__ __noinline__ MPF<L> mpf_fms_oolv(MPF<L> c, MPF<L> a, MPF<L> b) {
 template <int L>
 __device__ __noinline__ void mpf_mul_ool(MPF<L>* out, const MPF<L>* a, const MPF<L>* b) {
     *out = mpf_mul<L>(*a, *b);
-}
-
-// c - a b by the inline (OOL = false) or the out-of-line copy
-template <int L, bool OOL>
-__device__ __forceinline__ MPF<L> mpf_fms_sel(const MPF<L>& c, const MPF<L>& a, const MPF<L>& b) {
-    if constexpr (OOL) {
-        return mpf_fms_oolv<L>(c, a, b);
-    } else {
-        return mpf_fms<L>(c, a, b);
-    }
 }
 
 template <int L>
@@ -567,21 +510,89 @@ __device__ __forceinline__ MPF<4> mpf_recip_seed(uint64_t T) {
     return r;
 }
 
-// 1 / b on the mantissa f = |b| 2^-e in [1/2, 1), the exponent applied last.
-// From the seed r (above), the residual e = 1 - f r of one fused multiply-
-// subtract (a single rounding) gives r = (1 - e) / f exactly, so
-//   r (1 + e)       = (1 - e^2) / f   (second order),
-//   r (1 + e + e^2) = (1 - e^3) / f   (third order, e^2 from the top word of e),
-// each formed as r + r t by one more fused multiply-subtract.  A 4-word step
-// on the top 128 bits of f goes first (third order, about 180 bits, for
-// L = 4; second order, about 120 bits, otherwise), then one L-word step:
-// second order (about 240 bits) for L <= 7, third order (about 360 bits) for
-// L <= 11; longer formats continue with second-order steps.  Everything runs
-// on the integer pipes apart from one binary32 reciprocal.  OOL: the fused
-// multiply-subtracts through their out-of-line copies.
-template <int L, bool OOL = false>
-__device__ __forceinline__ MPF<L> mpf_recip(const MPF<L>& b) {
-    static_assert(L >= 4, "a 4-word first step");
+// 1 / f for f = F 2^(-32 L) in (1/2, 1), L <= 7, in fixed point: R words with
+// r = R 2^(1 - 32 (L + 1)) in (1, 2), r <= 1 / f, 1 - f r < 2^-(32 L + 4) or
+// 2^-238, whichever is larger.  Newton steps r <- r + r e, e = 1 - f r, whose
+// result (1 - e^2) / f stays below 1 / f; each uses only the words of f and of e
+// that its precision needs, so that the alignments are fixed and nothing is
+// normalised.  On values:
+//   r0  binary32 reciprocal of the top 24 bits plus one       e < 2^-21
+//   r1  32-bit f (plus one unit), one step in 64 bits          e < 2^-30
+//   r2  64-bit f (plus one unit), one step                     e < 2^-59
+//   r3  four words of f (plus one unit), two of r              e < 2^-117
+//   r4  all of f, four words of r
+// 62 wide multiply-adds for L = 7, against four fused multiply-subtracts of
+// general floats before (3413 cycles on one thread with the present ones; 783 now).
+template <int L>
+__device__ __forceinline__ void recip_words(const uint32_t (&F)[L], uint32_t (&R)[L + 1]) {
+    const uint32_t t32 = F[L - 1];
+    const uint64_t T = ((uint64_t)t32 << 32) | F[L - 2];
+    // r0 2^30, a binary32 unit below
+    const uint32_t fb = __float_as_uint(__frcp_rn((float)((t32 >> 8) + 1)));
+    // (1 / (t + 1) in [2^-24, 2^-23): exponent field 103; 2^-24 itself only for t + 1 = 2^24)
+    const uint32_t R0 = (((fb & 0x7fffffu) | 0x800000u) << 7) - 128u;
+    // r1 2^62
+    const uint64_t E1 = (1ull << 62) - ((uint64_t)R0 * t32 + R0);
+    const uint64_t R1 = ((uint64_t)R0 << 32) + (((uint64_t)R0 * (uint32_t)(E1 >> 10)) >> 20);
+    // r2 2^62: E2 = 2^126 - (T + 1) R1
+    const uint64_t plo = T * R1, lo2 = plo + R1;
+    const uint64_t hi2 = __umul64hi(T, R1) + (lo2 < plo ? 1ull : 0ull);
+    const uint64_t elo = 0ull - lo2, ehi = (1ull << 62) - hi2 - (lo2 != 0ull ? 1ull : 0ull);
+    const uint64_t R2 = R1 + (__umul64hi(R1, (ehi << 31) | (elo >> 33)) >> 29);
+    // r3 2^127 in four words: E3 = 2^191 - (F4 + 1) G, G = r2 2^63
+    const uint32_t G[2] = {(uint32_t)(R2 << 1), (uint32_t)(R2 >> 31)};
+    uint32_t F4[4], P3[6], R3[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) F4[i] = F[L - 4 + i];
+    mul_words<4, 2, 0>(F4, G, P3);
+    P3[0] = add_first(P3[0], G[0]);
+    P3[1] = add_next(P3[1], G[1]);
+#pragma unroll
+    for (int i = 2; i < 6; ++i) P3[i] = add_next(P3[i], 0u);
+    {
+        // -P3 = ~P3 + 1; E3 < 2^132: words 2 .. 4
+        add_first(~P3[0], 1u);
+        add_next(~P3[1], 0u);
+        uint32_t E3[3], Q[5];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) E3[i] = add_next(~P3[i + 2], 0u);
+        mul_words<3, 2, 0>(E3, G, Q);
+        // r3 2^127 = G 2^64 + (G E3) 2^-63
+        R3[0] = __funnelshift_r(Q[1], Q[2], 31);
+        R3[1] = __funnelshift_r(Q[2], Q[3], 31);
+        const uint32_t q2 = __funnelshift_r(Q[3], Q[4], 31);
+        R3[2] = add_first(G[0], q2);
+        R3[3] = add_last(G[1], Q[4] >> 31);
+    }
+    // r4: E4 = 2^(32 L + 127) - F R3 < 2^(32 L + 12): words 0 .. L; its top NE
+    // words times R3
+    constexpr int NE = L - 2, WP = L + 4;
+    uint32_t P4[WP], E4[NE], Q[NE + 4];
+    mul_words<L, 4, 0>(F, R3, P4);
+    add_first(~P4[0], 1u);
+#pragma unroll
+    for (int i = 1; i < L + 1 - NE; ++i) add_next(~P4[i], 0u);
+#pragma unroll
+    for (int i = 0; i < NE; ++i) E4[i] = add_next(~P4[L + 1 - NE + i], 0u);
+    mul_words<NE, 4, 0>(E4, R3, Q);
+    // r 2^(32 L + 31) = R3 2^(32 L - 96) + R3 E4 2^-223, E4 here without its low
+    // L + 1 - NE = 3 words: (R3 E4) 2^-127, words from bit 127 on
+    uint32_t q[L + 1];
+#pragma unroll
+    for (int i = 0; i < L + 1; ++i)
+        q[i] = i + 3 < NE + 4 ? __funnelshift_r(Q[i + 3 < NE + 4 ? i + 3 : 0], i + 4 < NE + 4 ? Q[i + 4 < NE + 4 ? i + 4 : 0] : 0u, 31) : 0u;
+    R[0] = L - 3 <= 0 ? add_first(q[0], R3[0]) : q[0];
+#pragma unroll
+    for (int i = 1; i < L + 1; ++i) {
+        if (i < L - 3) R[i] = q[i];
+        else if (i == L - 3) R[i] = add_first(q[i], R3[0]);
+        else R[i] = add_next(q[i], R3[i - (L - 3) < 4 ? i - (L - 3) : 0]);
+    }
+}
+
+// the general-float steps of mpf_recip for L >= 8
+template <int L>
+__device__ __forceinline__ MPF<L> mpf_recip_long(const MPF<L>& b) {
     MPF<4> r4 = mpf_recip_seed(((uint64_t)b.m[L - 1] << 32) | b.m[L - 2]);
     MPF<4> f4;
 #pragma unroll
@@ -589,26 +600,57 @@ __device__ __forceinline__ MPF<L> mpf_recip(const MPF<L>& b) {
     f4.e = 0;
     f4.neg = 0;
     {
-        MPF<4> t4 = mpf_fms_sel<4, OOL>(mpf_one<4>(), f4, r4);
-        if (L == 4) t4 = mpf_add<4>(t4, mpf_top_square<4>(t4));
-        r4 = mpf_fms_sel<4, OOL>(r4, r4, mpf_neg<4>(t4));
+        MPF<4> t4 = mpf_fms<4>(mpf_one<4>(), f4, r4);
+        r4 = mpf_fms<4>(r4, r4, mpf_neg<4>(t4));
     }
     MPF<L> r = mpf_widen<L, 4>(r4);
-    if (L > 4) {
+    {
         MPF<L> f = b;
         f.neg = 0;
         f.e = 0;
-        MPF<L> t = mpf_fms_sel<L, OOL>(mpf_one<L>(), f, r);
-        if (L > 7) t = mpf_add<L>(t, mpf_top_square<L>(t));
-        r = mpf_fms_sel<L, OOL>(r, r, mpf_neg<L>(t));
-        for (int prec = L > 7 ? 360 : 240; prec < 32 * L + 8; prec *= 2) {
-            t = mpf_fms_sel<L, OOL>(mpf_one<L>(), f, r);
-            r = mpf_fms_sel<L, OOL>(r, r, mpf_neg<L>(t));
+        MPF<L> t = mpf_fms<L>(mpf_one<L>(), f, r);
+        t = mpf_add<L>(t, mpf_top_square<L>(t));
+        r = mpf_fms<L>(r, r, mpf_neg<L>(t));
+        for (int prec = 360; prec < 32 * L + 8; prec *= 2) {
+            t = mpf_fms<L>(mpf_one<L>(), f, r);
+            r = mpf_fms<L>(r, r, mpf_neg<L>(t));
         }
     }
     r.e -= b.e;
     r.neg = b.neg;
     return r;
+}
+
+// 1 / b on the mantissa f = |b| 2^-e in [1/2, 1), the exponent applied last.
+// L <= 7 takes the fixed-point steps above; a power of two is exact.  Longer
+// formats work on general floats: from the seed r (above), the residual
+// e = 1 - f r of one fused multiply-subtract (a single rounding) gives
+// r = (1 - e) / f exactly, so
+//   r (1 + e)       = (1 - e^2) / f   (second order),
+//   r (1 + e + e^2) = (1 - e^3) / f   (third order, e^2 from the top word of e),
+// each formed as r + r t by one more fused multiply-subtract: a 4-word step of
+// second order (about 120 bits) on the top 128 bits of f, then one L-word step of
+// third order (about 360 bits) and second-order steps beyond.  Everything runs
+// on the integer pipes apart from one binary32 reciprocal.
+template <int L>
+__device__ __forceinline__ MPF<L> mpf_recip(const MPF<L>& b) {
+    static_assert(L >= 4, "a 4-word first step");
+    if constexpr (L <= 7) {
+        uint32_t low = b.m[L - 1] ^ 0x80000000u;
+#pragma unroll
+        for (int i = 0; i < L - 1; ++i) low |= b.m[i];
+        if (low == 0) {  // 1 / 2^(e - 1) = 2^(1 - e)
+            MPF<L> r = mpf_one<L>();
+            r.e = 2 - b.e;
+            r.neg = b.neg;
+            return r;
+        }
+        uint32_t R[L + 1];
+        recip_words<L>(b.m, R);
+        return mpf_round_top<L, L + 1>(R, 1 - b.e, b.neg, true);
+    } else {
+        return mpf_recip_long<L>(b);
+    }
 }
 
 }  // namespace ozlu
