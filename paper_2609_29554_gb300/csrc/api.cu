@@ -240,6 +240,23 @@ int autotune(ozlu_handle* h, int nc, int p, int m, int n, int k, const double* A
     return OZLU_OK;
 }
 
+// What gemm_device answers for these options at this K without running it: a
+// plan exists (for the autotuner, on any back-end), or why not
+int check_plan(ozlu_handle* h, int p, int K, const ozlu_opts* opts) {
+    const PlanEntry* pe;
+    if (opts && opts->backend != OZLU_BE_AUTO) return plan_for(h, p, K, opts, &pe);
+    const int cand[4] = {OZLU_BE_FP16, OZLU_BE_FP8, OZLU_BE_FP64, OZLU_BE_INT8};
+    int rc = OZLU_OK;
+    for (int be : cand) {
+        ozlu_opts o;
+        memset(&o, 0, sizeof o);
+        if (opts) o = *opts;
+        o.backend = be;
+        if (!(rc = plan_for(h, p, K, &o, &pe))) break;
+    }
+    return rc;
+}
+
 // The device part of one GEMM, all pointers on the device.
 
 int gemm_device(ozlu_handle* h, int nc, int p, int m, int n, int k, int alpha, const double* A,
@@ -425,6 +442,7 @@ int ozlu_destroy(ozlu_handle* h) {
     h->ws.release();
     h->stage.release();
     h->tune_ws.release();
+    h->solve_ws.release();
     h->nb_ws.release();
     if (h->lu_scratch) cudaFree(h->lu_scratch);
     if (h->coop_scratch) cudaFree(h->coop_scratch);

@@ -13,9 +13,10 @@
 // Only (P4) is the update the paper moves to Ozaki scheme II; the recursion
 // puts the larger part of (P1) and (P3) on the same GEMM as well, leaving
 // O(n^2 BASE) operations in FP64 expansion arithmetic (the GB300 FP64 rate is
-// about 1 TFLOP/s).  getrs: interchanges, then blocked forward (unit L) and
-// backward (U) substitution with base triangles in expansion arithmetic and
-// the off-diagonal updates by the Ozaki-II GEMM.
+// about 1 TFLOP/s).  getrs: interchanges, then forward (unit L)
+// and backward (U) substitution: for a few right-hand sides each as one
+// cooperative kernel in multi-limb floats, else blocked, with base triangles in
+// them and the off-diagonal updates by the Ozaki-II GEMM.
 #include <string.h>
 
 #include <tuple>
@@ -991,12 +992,13 @@ __global__ void __launch_bounds__(LMAXB) laswp_list_kernel(int k0, int k1, const
     __syncthreads();
     if (t < b) {
         const int p = piv[t];
+        const bool out = p < k0 || p >= k1;
         int j = t;
-        if (p >= k1)
+        if (out)
             for (j = 0; piv[j] != p; ++j) {}
-        slot[t] = p < k1 ? p - k0 : b + j;
+        slot[t] = out ? b + j : p - k0;
         row[t] = val[t] = k0 + t;
-        row[b + t] = p >= k1 && j == t ? p : -1;
+        row[b + t] = out && j == t ? p : -1;
         val[b + t] = p;
     }
     __syncthreads();
@@ -1174,6 +1176,188 @@ void trsm_base(const double* T, long long ldt, double* X, long long ldx, int b, 
     const size_t smem = sizeof(MPF<L>) * (BASE * BASE + BASE);
     raise_smem_limit((const void*)trsm_base_kernel<N>, (int)smem);
     trsm_base_kernel<N><<<(ncols + wpb - 1) / wpb, 32 * wpb, smem, s>>>(sc, X, ldx, b, ncols, lower, slot);
+}
+
+// ---------------------------------------------------------------------------
+// X <- L^-1 X (unit lower) or U^-1 X for a few right-hand sides as one
+// cooperative kernel per direction.  A block owns 32 rows (block-rows t = g,
+// g + G, ... in the order of the substitution): it subtracts the products with
+// every earlier x as it is announced, then solves its triangle and announces its
+// own rows, SOLVE_PART at a time, as tagged words (as the panel kernel does).
+// Everything is in L-limb floats, X rounded to expansions once per direction.
+//   lane = row; the 16 warps are KW parts of k times the right-hand sides
+//   (KW = 16 / the power of two >= nrhs), each with a partial sum of its own
+//   over all blocks, added once at the end in a fixed order.
+// Bound by latency: of the 24 us (QD) a block-row takes, 19 are its 32 dependent
+// multiply-subtracts (about 1170 cycles each with the broadcast), 3 the last
+// part of x_{t-1} on all warps and 2 the sum of the parts.  The products with
+// all other x and the conversion of the next 32 x 32 factors (SOLVE_BUF buffers)
+// run ahead of the chain.  The warps that solve the triangle, one a right-hand
+// side, issue from different schedulers: on one, three took 1940 cycles a step.
+// The upper triangle is scaled by the reciprocals of its diagonal beforehand (a
+// zero pivot gives 0), so that both directions have unit steps.
+// n = 1500, 3 right-hand sides: QD 2.05 ms, DD 1.43.  By base triangles of 32
+// rows and an Ozaki-II GEMM after each, the form kept above SOLVE_RHS: 7.2 and
+// 5.1, hardly depending on nrhs; here 16 take 5.3 and 3.3, and two rounds of 16
+// would be slower than that form.
+constexpr int SOLVE_RHS = 16;
+constexpr int SOLVE_BUF = 3;
+constexpr int SOLVE_PART = 8;  // rows announced together
+
+template <int L>
+size_t solve_smem(int nrhs) {
+    return sizeof(MPF<L>) * (SOLVE_BUF * BASE * BASE + BASE * BASE + BASE + 16 * 32 + (size_t)SOLVE_BUF * nrhs * BASE);
+}
+
+template <int N, bool LOWER>
+__global__ void __launch_bounds__(512, 1) solve_kernel(const double* T, long long ldt, int n, double* X, long long ldx,
+                                                       int nrhs, int kw, unsigned long long* words, int* err) {
+    constexpr int L = Limbs<N>::L, WORDS = L + 2;
+    extern __shared__ __align__(16) unsigned char smraw[];
+    MPF<L>* lb = reinterpret_cast<MPF<L>*>(smraw);    // [SOLVE_BUF][k][i]
+    MPF<L>* tri = lb + SOLVE_BUF * BASE * BASE;       // [k][i]
+    MPF<L>* rd = tri + BASE * BASE;                   // reciprocal diagonal (upper)
+    MPF<L>* part = rd + BASE;                         // [warp][row]
+    MPF<L>* xs = part + 16 * 32;                      // [SOLVE_BUF][j][k]
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    const int nb = (n + BASE - 1) / BASE, G = gridDim.x;
+    // right-hand side, part of k: the warps of one part issue from different schedulers
+    const int nj = 16 / kw, kp = warp / nj, j = warp - kp * nj;
+    auto row0 = [&](int t) { return (LOWER ? t : nb - 1 - t) * BASE; };
+    // factors of block-row t against block-column s (both in solve order) into a buffer
+    auto convert = [&](int t, int s, int buf) {
+        const int i = row0(t) + lane, c0 = row0(s);
+#pragma unroll 1
+        for (int k = warp; k < BASE; k += 16) {
+            MPF<L> v = mpf_make_zero<L>();
+            if (i < n && c0 + k < n) v = mpf_from_exp<L, N>(T + ((long long)i + (long long)(c0 + k) * ldt) * N);
+            lb[(buf * BASE + k) * BASE + lane] = v;
+        }
+    };
+    for (int t = blockIdx.x; t < nb; t += G) {
+        const int i0 = row0(t), bi = min(BASE, n - i0);
+        __syncthreads();
+        if (!LOWER) {
+            if (tid < BASE) {
+                MPF<L> d = mpf_make_zero<L>();
+                if (tid < bi) d = mpf_from_exp<L, N>(T + ((long long)(i0 + tid) + (long long)(i0 + tid) * ldt) * N);
+                rd[tid] = mpf_zero<L>(d) ? mpf_make_zero<L>() : mpf_recip<L>(d);
+            }
+            __syncthreads();
+        }
+        for (int k = warp; k < BASE; k += 16) {
+            MPF<L> v = mpf_make_zero<L>();
+            if (lane < bi && k < bi && (LOWER ? k < lane : k > lane)) {
+                v = mpf_from_exp<L, N>(T + ((long long)(i0 + lane) + (long long)(i0 + k) * ldt) * N);
+                if (!LOWER) v = mpf_mul<L>(v, rd[lane]);
+            }
+            tri[k * BASE + lane] = v;
+        }
+        MPF<L> acc = mpf_make_zero<L>();
+        if (kp == 0 && j < nrhs && lane < bi)
+            acc = mpf_from_exp<L, N>(X + ((long long)(i0 + lane) + (long long)j * ldx) * N);
+        if (t > 0) convert(t, 0, 0);
+        for (int s = 0; s < t; ++s) {
+            const int buf = s % SOLVE_BUF;
+            if (s + 1 < t) convert(t, s + 1, (s + 1) % SOLVE_BUF);
+            const unsigned long long* w = words + (size_t)s * nrhs * WORDS * BASE;
+            // the newest x in the parts in which it is announced, older ones whole
+            const int parts = s == t - 1 ? BASE / SOLVE_PART : 1, len = BASE / parts;
+            for (int g = 0; g < parts; ++g) {
+                const int k0 = LOWER ? g * len : BASE - (g + 1) * len;
+                WaitBound wb;
+                for (int q = tid; q < nrhs * WORDS * len; q += 512) {
+                    const int k = k0 + q % len, r = q / len;  // r = right-hand side x word
+                    unsigned long long v = ld_relaxed(w + r * BASE + k);
+                    while ((unsigned)(v >> 32) != 1u) {
+                        if (wb.expired(err)) break;  // then the rest is soon done, with wrong numbers
+                        if (s + 2 < t) __nanosleep(500);  // not next in the chain: keep off the L2 lines
+                        v = ld_relaxed(w + r * BASE + k);
+                    }
+                    reinterpret_cast<uint32_t*>(&xs[(buf * nrhs + r / WORDS) * BASE + k])[r % WORDS] = (uint32_t)v;
+                }
+                __syncthreads();
+                if (j < nrhs)
+                    for (int k = k0 + kp; k < k0 + len; k += kw)
+                        acc = mpf_fms<L>(acc, lb[(buf * BASE + k) * BASE + lane], xs[(buf * nrhs + j) * BASE + k]);
+            }
+        }
+        // the partial sums of a right-hand side, pairwise
+        part[warp * 32 + lane] = acc;
+        for (int o = 1; o < kw; o *= 2) {
+            __syncthreads();
+            if ((kp & (2 * o - 1)) == 0) {
+                acc = mpf_add<L>(acc, part[(warp + o * nj) * 32 + lane]);
+                part[warp * 32 + lane] = acc;
+            }
+        }
+        __syncthreads();
+        if (kp == 0 && j < nrhs) {
+            MPF<L> x = acc;
+            if (!LOWER) x = mpf_mul<L>(x, rd[lane]);
+            unsigned long long* w = words + ((size_t)t * nrhs + j) * WORDS * BASE;
+            // (every lane multiplies and selects: a branch would cost more than it saves)
+            for (int g = 0; g < BASE / SOLVE_PART; ++g) {
+                const int first = LOWER ? g * SOLVE_PART : BASE - 1 - g * SOLVE_PART;
+#pragma unroll 1
+                for (int q = 0; q < SOLVE_PART; ++q) {
+                    const int k = LOWER ? first + q : first - q;
+                    const MPF<L> v = mpf_fms<L>(x, tri[k * BASE + lane], mpf_bcast<L>(x, k));
+                    const bool mine = LOWER ? lane > k : lane < k;
+#pragma unroll
+                    for (int i = 0; i < L; ++i) x.m[i] = mine ? v.m[i] : x.m[i];
+                    x.e = mine ? v.e : x.e;
+                    x.neg = mine ? v.neg : x.neg;
+                }
+                if ((LOWER ? lane - first : first - lane) >= 0 && (LOWER ? lane - first : first - lane) < SOLVE_PART)
+#pragma unroll
+                    for (int i = 0; i < WORDS; ++i) st_relaxed(w + i * BASE + lane, (1ull << 32) | mpf_word<L>(x, i));
+            }
+            if (lane < bi) mpf_to_exp<L, N>(x, X + ((long long)(i0 + lane) + (long long)j * ldx) * N);
+        }
+    }
+}
+
+// interchanges k in [0, n) on the right-hand sides, LMAXB at a time
+template <int N>
+void laswp_all(double* B, long long ldb, int nrhs, int n, const int* ipiv, int* list, cudaStream_t s) {
+    for (int k0 = 0; k0 < n; k0 += LMAXB) laswp2<N>(B, ldb, 0, nrhs, 0, 0, k0, k0 + LMAXB < n ? k0 + LMAXB : n, ipiv, list, s);
+}
+
+// both substitutions for nrhs <= SOLVE_RHS.  *launched stays false when the
+// kernel cannot be launched here (the caller then takes the blocked form)
+template <int N>
+int solve_few(const double* LU, long long lda, int n, double* B, long long ldb, int nrhs, void* words, int* err,
+              cudaStream_t s, bool* launched) {
+    constexpr int L = Limbs<N>::L;
+    const int nb = (n + BASE - 1) / BASE, sms = device_sms();
+    int kw = 16;
+    while (16 / kw < nrhs) kw /= 2;
+    const size_t smem = solve_smem<L>(nrhs), half = (size_t)nb * BASE * nrhs * (L + 2);
+    unsigned long long* w = (unsigned long long*)words;
+    if (cudaMemsetAsync(w, 0, 2 * half * sizeof *w, s) != cudaSuccess) return OZLU_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nb < sms ? nb : sms);
+    cfg.blockDim = dim3(512);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const size_t most = solve_smem<L>(SOLVE_RHS);
+    raise_smem_limit((const void*)solve_kernel<N, true>, (int)most);
+    raise_smem_limit((const void*)solve_kernel<N, false>, (int)most);
+    if (cudaLaunchKernelEx(&cfg, solve_kernel<N, true>, LU, lda, n, B, ldb, nrhs, kw, w, err) != cudaSuccess) {
+        cudaGetLastError();
+        return OZLU_OK;
+    }
+    *launched = true;
+    return cudaLaunchKernelEx(&cfg, solve_kernel<N, false>, LU, lda, n, B, ldb, nrhs, kw, w + half, err) == cudaSuccess
+               ? OZLU_OK
+               : OZLU_ERR_CUDA;
 }
 
 // Launch the cooperative base-block kernel; returns false when the slice of
@@ -1370,12 +1554,30 @@ template <int N>
 int getrs_device(ozlu_handle* h, int p, int n, int nrhs, double* LU, long long lda, const int* ipiv,
                  double* B, long long ldb, const ozlu_opts* opts, LuScratch* sc) {
     cudaStream_t s = h->stream;
-    laswp_kernel<N><<<(nrhs + 127) / 128, 128, 0, s>>>(B, ldb, 0, nrhs, 0, n, ipiv);
+    // options that no plan of the updates meets are refused whichever form runs
+    const int refused = n > BASE ? check_plan(h, p, BASE, opts) : OZLU_OK;
+    if (refused) return refused;
+    h->phase(PH_OTHER);
+    laswp_all<N>(B, ldb, nrhs, n, ipiv, sc->plist, s);
+    h->count(2 * ((n + LMAXB - 1) / LMAXB));
     int rc = 0;
+    if (nrhs <= SOLVE_RHS) {
+        constexpr int W = Limbs<N>::L + 2;
+        const size_t rows = (size_t)(n + BASE - 1) / BASE * BASE;
+        bool launched = false;
+        rc = h->solve_ws.ensure(2 * sizeof(unsigned long long) * rows * nrhs * W);
+        h->phase(PH_TRSM);
+        if (!rc) rc = solve_few<N>(LU, lda, n, B, ldb, nrhs, h->solve_ws.base, h->dev_err, s, &launched);
+        if (rc || launched) {
+            h->count(2);
+            h->phase(-1);
+            return !rc && cudaGetLastError() != cudaSuccess ? OZLU_ERR_CUDA : rc;
+        }
+    }
     auto L = [&](long long i, long long j) { return LU + (i + j * lda) * N; };
     auto X = [&](long long i) { return B + i * N; };
     h->phase(PH_TRSM);
-    h->count(1 + 3 * ((n + BASE - 1) / BASE));
+    h->count(4 * ((n + BASE - 1) / BASE));
     for (int r = 0; r < n && !rc; r += BASE) {
         const int b = BASE < n - r ? BASE : n - r;
         trsm_base<N>(L(r, r), lda, X(r), ldb, b, nrhs, 1, sc, s);

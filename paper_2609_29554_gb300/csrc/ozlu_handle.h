@@ -47,6 +47,7 @@ struct ozlu_handle {
     // shape key -> (back-end, slice count) chosen by the autotuner
     std::map<std::tuple<int, int, int, int, int, int>, std::pair<int, int>> tuned;
     std::map<std::tuple<int, int, int, int>, int> tuned_nb;  // (nc, p, log2 n, backend) -> nb
+    ozlu::Workspace solve_ws;  // tagged words of the few-right-hand-side solve
     ozlu::Workspace nb_ws;  // scratch copy of A for the panel-width autotuner
     std::map<std::tuple<int, int, int, int, int, int>, ozlu::PlanEntry> plans;
     ozlu::GemmLayout last;
@@ -99,6 +100,7 @@ int tune_nb(ozlu_handle* h, int nc, int p, int n, const double* A, long long lda
             int* nb_out);
 int getrs_one(ozlu_handle* h, int nc, int p, int n, int nrhs, const double* LU, long long lda, const int* ipiv,
               double* B, long long ldb, const ozlu_opts* opts);
+int check_plan(ozlu_handle* h, int p, int K, const ozlu_opts* opts);
 int gemm_device(ozlu_handle* h, int nc, int p, int m, int n, int k, int alpha, const double* A,
                 long long lda, const double* B, long long ldb, int beta, double* C,
                 long long ldc, const ozlu_opts* opts);
