@@ -34,6 +34,7 @@ constexpr int PIV_THREADS = 256;
 constexpr int PIV_BLOCKS = 152;
 constexpr int MAXPART = 1024;   // block partials of a column step
 constexpr int STEP_ROWS = 16;   // rows per block of a column step
+constexpr int TRSM_WARPS = 16;  // columns per block of a base triangular solve, at most
 constexpr int LCT = 4;          // laswp: columns per block
 constexpr int LMAXB = 512;      // laswp: interchanges per call
 constexpr int TRI_SLOTS = 8;    // triangles of base solves converted ahead (256 / BASE)
@@ -56,7 +57,7 @@ struct LuScratch {
     // triangles of base triangular solves as L-limb floats: [k][i], then the
     // reciprocal diagonal (upper case); slot q holds the q-th diagonal block of
     // a unit lower triangle converted ahead of its recursion
-    unsigned char tri[TRI_SLOTS][(BASE * BASE + BASE) * sizeof(MPF<8>)];
+    alignas(16) unsigned char tri[TRI_SLOTS][(BASE * BASE + BASE) * sizeof(MPF<8>)];
 };
 
 template <int L>
@@ -488,6 +489,15 @@ __device__ __forceinline__ MPF<L> mpf_gather(uint32_t w) {
     v.e = (int)__shfl_sync(0xffffffffu, w, L);
     v.neg = (int)__shfl_sync(0xffffffffu, w, L + 1);
     return v;
+}
+
+// x = v where `on`, by selects
+template <int L>
+__device__ __forceinline__ void mpf_take(MPF<L>& x, const MPF<L>& v, bool on) {
+#pragma unroll
+    for (int i = 0; i < L; ++i) x.m[i] = on ? v.m[i] : x.m[i];
+    x.e = on ? v.e : x.e;
+    x.neg = on ? v.neg : x.neg;
 }
 
 // lane src's float on every lane
@@ -1129,36 +1139,41 @@ __global__ void __launch_bounds__(256) tri_convert_kernel(const double* T, long 
 // floating point.  One warp per column, lane i holding x_i in registers: step
 // k broadcasts the final x_k by warp shuffles and every lane below (lower) or
 // above (upper) row k subtracts l_ik x_k, so the b steps need no block-wide
-// barrier and the warps of a block progress independently.  The triangle is
-// read from shared memory column by column ([k][i], conflict-free).
+// barrier and the warps of a block progress independently.  The triangle comes
+// to shared memory by asynchronous copies while X is converted, and is read
+// column by column ([k][i], conflict-free).  The warps stay converged (every
+// lane multiplies and selects).
 template <int N>
-__global__ void __launch_bounds__(256) trsm_base_kernel(const LuScratch* sc, double* X, long long ldx, int b,
-                                                        int ncols, int lower, int slot) {
+__global__ void __launch_bounds__(TRSM_WARPS * 32) trsm_base_kernel(const LuScratch* sc, double* X, long long ldx,
+                                                                    int b, int ncols, int lower, int slot) {
     constexpr int L = Limbs<N>::L;
     extern __shared__ __align__(16) unsigned char smraw[];
     MPF<L>* sl = reinterpret_cast<MPF<L>*>(smraw);   // [k][i]
     MPF<L>* rd = sl + BASE * BASE;                   // reciprocal diagonal (upper)
-    const int row = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int row = threadIdx.x & 31, w = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
     const int col = blockIdx.x * (blockDim.x >> 5) + w;
-    const MPF<L>* tl = reinterpret_cast<const MPF<L>*>(sc->tri[slot]);
-    for (int idx = threadIdx.x; idx < BASE * BASE; idx += blockDim.x) sl[idx] = tl[idx];
-    if (!lower)
-        for (int k = threadIdx.x; k < b; k += blockDim.x) rd[k] = tl[BASE * BASE + k];
-    __syncthreads();
-    if (col >= ncols) return;  // whole warps: col is uniform in a warp
+    constexpr int CHUNKS = (BASE * BASE + BASE) * (int)sizeof(MPF<L>) / 16;
+    static_assert((BASE * BASE + BASE) * sizeof(MPF<L>) % 16 == 0, "whole 16-byte pieces");
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(smraw);
+    for (int i = threadIdx.x; i < CHUNKS; i += blockDim.x)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16 * i), "l"(sc->tri[slot] + 16 * i)
+                     : "memory");
+    const bool mine = row < b && col < ncols;
     double* xp = X + ((long long)row + (long long)col * ldx) * N;
-    MPF<L> x = row < b ? mpf_from_exp<L, N>(xp) : mpf_make_zero<L>();
+    MPF<L> x = mine ? mpf_from_exp<L, N>(xp) : mpf_make_zero<L>();
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+#pragma unroll 1
     for (int s = 0; s < b; ++s) {
         const int k = lower ? s : b - 1 - s;
-        if (!lower && row == k) x = mpf_mul<L>(x, rd[k]);
-        MPF<L> xk;
-#pragma unroll
-        for (int q = 0; q < L; ++q) xk.m[q] = __shfl_sync(0xffffffffu, x.m[q], k);
-        xk.e = __shfl_sync(0xffffffffu, x.e, k);
-        xk.neg = __shfl_sync(0xffffffffu, x.neg, k);
-        if (row < b && (lower ? row > k : row < k)) x = mpf_fms<L>(x, sl[k * BASE + row], xk);
+        if (!lower) {
+            const MPF<L> v = mpf_mul<L>(x, rd[k]);
+            mpf_take<L>(x, v, row == k);
+        }
+        const MPF<L> v = mpf_fms<L>(x, sl[k * BASE + row], mpf_bcast<L>(x, k));
+        mpf_take<L>(x, v, lower ? row > k : row < k);
     }
-    if (row < b) mpf_to_exp<L, N>(x, xp);
+    if (mine) mpf_to_exp<L, N>(x, xp);
 }
 
 // slot < 0: convert the triangle into slot 0 first; else it is in `slot`
@@ -1171,8 +1186,9 @@ void trsm_base(const double* T, long long ldt, double* X, long long ldx, int b, 
         tri_convert_kernel<N><<<(b * b + 255) / 256, 256, 0, s>>>(T, ldt, b, lower, sc);
         slot = 0;
     }
-    // 8 columns (warps) per block, fewer when that leaves SMs idle
-    const int wpb = ncols >= 8 * 152 ? 8 : (ncols >= 4 * 152 ? 4 : 2);
+    // every SM the same number of columns: blocks of equal size, one or two an SM
+    const int sms = device_sms(), per = (ncols + TRSM_WARPS * sms - 1) / (TRSM_WARPS * sms) * sms;
+    const int wpb = (ncols + per - 1) / per;
     const size_t smem = sizeof(MPF<L>) * (BASE * BASE + BASE);
     raise_smem_limit((const void*)trsm_base_kernel<N>, (int)smem);
     trsm_base_kernel<N><<<(ncols + wpb - 1) / wpb, 32 * wpb, smem, s>>>(sc, X, ldx, b, ncols, lower, slot);
@@ -1304,11 +1320,7 @@ __global__ void __launch_bounds__(512, 1) solve_kernel(const double* T, long lon
                 for (int q = 0; q < SOLVE_PART; ++q) {
                     const int k = LOWER ? first + q : first - q;
                     const MPF<L> v = mpf_fms<L>(x, tri[k * BASE + lane], mpf_bcast<L>(x, k));
-                    const bool mine = LOWER ? lane > k : lane < k;
-#pragma unroll
-                    for (int i = 0; i < L; ++i) x.m[i] = mine ? v.m[i] : x.m[i];
-                    x.e = mine ? v.e : x.e;
-                    x.neg = mine ? v.neg : x.neg;
+                    mpf_take<L>(x, v, LOWER ? lane > k : lane < k);
                 }
                 if ((LOWER ? lane - first : first - lane) >= 0 && (LOWER ? lane - first : first - lane) < SOLVE_PART)
 #pragma unroll

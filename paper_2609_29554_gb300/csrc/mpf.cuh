@@ -88,14 +88,31 @@ __device__ __forceinline__ MPF<L> mpf_round(uint32_t (&X)[W], int ex, int neg, b
     return mpf_round_top<L, W>(X, ex - sh, neg, sticky_in);
 }
 
+// X += (neg ? -1 : 1) * mag * 2^pos (mod 2^(32 W)), pos >= 0, as one carry chain
+template <int W>
+__device__ __forceinline__ void mpf_acc(uint32_t (&X)[W], uint64_t mag, int pos, bool neg) {
+    const int q = pos >> 5;
+    const uint32_t m0 = (uint32_t)mag, m1 = (uint32_t)(mag >> 32), nm = neg ? 0xffffffffu : 0u;
+    const uint32_t lo = __funnelshift_l(0u, m0, pos & 31), mid = __funnelshift_l(m0, m1, pos & 31),
+                   hi = __funnelshift_l(m1, 0u, pos & 31);
+    add_first(nm, nm & 1u);  // the flag: 1 for the complement
+#pragma unroll
+    for (int i = 0; i < W; ++i)
+        X[i] = add_next(X[i], (i == q ? lo : i == q + 1 ? mid : i == q + 2 ? hi : 0u) ^ nm);
+}
+
 // from an expansion of N binary64 components (sticky-truncated to 32(L+2) bits,
-// then rounded to L words)
+// then rounded to L words).  The components are added with their sign relative
+// to the first one's, so that the sum of a normalised expansion is positive.
 template <int L, int N>
 __device__ __forceinline__ MPF<L> mpf_from_exp(const double* x) {
     constexpr int W = L + 2;
     if (x[0] == 0.0) return mpf_make_zero<L>();
-    const int top = frexp_exp(x[0]) + 1;  // |value| < 2^top
-    const int base = top - 32 * W;        // bit 0 of the window
+    const uint64_t b0 = (uint64_t)__double_as_longlong(x[0]);
+    const int be = (int)((b0 >> 52) & 0x7ff);
+    const int top = (be >= 1 && be <= 2046 ? be - 1022 : frexp_exp(x[0])) + 1;  // |value| < 2^top
+    const int base = top - 32 * W;  // bit 0 of the window
+    int neg = (int)(b0 >> 63);
     uint32_t X[W];
 #pragma unroll
     for (int i = 0; i < W; ++i) X[i] = 0;
@@ -113,56 +130,81 @@ __device__ __forceinline__ MPF<L> mpf_from_exp(const double* x) {
             mant >>= -s;
             s = 0;
         }
-        add_shifted<W>(X, mant, s, ng);
+        mpf_acc<W>(X, mant, s, ng != (neg != 0));
     }
-    int neg = 0;
-    if (is_negative<W>(X)) {
+    if (is_negative<W>(X)) {  // not normalised: the rest outweighs the first component
         negate<W>(X);
-        neg = 1;
-        // a dropped positive remainder of a negative sum rounds the magnitude up
+        neg ^= 1;
     }
     return mpf_round<L, W>(X, top, neg, sticky);
 }
 
-// successive round-to-nearest-even into N binary64 components
+// q 2^e for q <= 2^53 (one rounding, for a subnormal result)
+__device__ __forceinline__ double mpf_make_double(uint64_t q, int e, bool neg) {
+    // 2^52 <= q <= 2^53 and a normal result: the biased exponent less one, plus
+    // q with its top bit as it is
+    if (q >> 52 && e >= -1073 && e <= 969)
+        return __longlong_as_double((long long)((((uint64_t)(e + 1074) << 52) + q) | ((uint64_t)neg << 63)));
+    const double x = scalbn((double)q, e);
+    return neg ? -x : x;
+}
+
+// successive round-to-nearest-even into N binary64 components.  The magnitude
+// is kept normalised: a component takes its top 53 bits, what is left of it (or
+// what is missing, after a rounding up) moves to the top by 53 bits and its
+// leading zeros.  Integer pipes only.
 template <int L, int N>
 __device__ __forceinline__ void mpf_to_exp(const MPF<L>& a, double* out) {
-    uint32_t mag[L];
+    uint32_t m[L];
 #pragma unroll
-    for (int i = 0; i < L; ++i) mag[i] = a.m[i];
+    for (int i = 0; i < L; ++i) m[i] = a.m[i];
     bool neg = a.neg != 0;
-    const int E = a.e - 32 * L;
+    int e = a.e;  // |value| = m 2^(e - 32 L)
 #pragma unroll
     for (int c = 0; c < N; ++c) {
-        const int Lb = bit_length<L>(mag);
-        double x = 0.0;
-        if (Lb > 0) {
-            if (Lb <= 53) {
-                const uint64_t q = (uint64_t)field32<L>(mag, 0) | ((uint64_t)field32<L>(mag, 32) << 32);
-                x = scalbn((double)(q & ((1ull << 53) - 1)), E);
-#pragma unroll
-                for (int i = 0; i < L; ++i) mag[i] = 0;
-                if (neg) x = -x;
-            } else {
-                const int sh = Lb - 53;
-                uint64_t q = ((uint64_t)field32<L>(mag, sh) | ((uint64_t)field32<L>(mag, sh + 32) << 32)) &
-                             ((1ull << 53) - 1);
-                const bool rb = bit_at<L>(mag, sh - 1) != 0;
-                const bool st = any_below<L>(mag, sh - 1);
-                mask_below<L>(mag, sh);
-                if (rb && (st || (q & 1))) {
-                    q += 1;
-                    complement_below<L>(mag, sh);
-                    x = scalbn((double)q, E + sh);
-                    if (neg) x = -x;
-                    neg = !neg;
-                } else {
-                    x = scalbn((double)q, E + sh);
-                    if (neg) x = -x;
-                }
-            }
+        if (m[L - 1] == 0) {  // exhausted (or zero)
+            out[c] = 0.0;
+            continue;
         }
-        out[c] = x;
+        const uint64_t hi = ((uint64_t)m[L - 1] << 32) | m[L - 2];
+        uint64_t q = hi >> 11;
+        const uint32_t low = m[L - 2] & 0x7ffu;
+        uint32_t any = low & 0x3ffu;
+#pragma unroll
+        for (int i = 0; i < L - 2; ++i) any |= m[i];
+        const bool up = (low & 0x400u) && (any || (q & 1));
+        q += up;
+        out[c] = mpf_make_double(q, e - 53, neg);
+        if (c + 1 == N) break;
+        // the rest r 2^-53, or 2^-53 - r after a rounding up: complemented
+        // words below the 53 bits, moved up by 53 bits
+        const uint32_t nm = up ? 0xffffffffu : 0u;
+        uint32_t t[L];
+        m[L - 1] = 0;
+        m[L - 2] &= 0x7ffu;
+        add_first(nm, nm & 1u);
+#pragma unroll
+        for (int i = 0; i < L - 1; ++i) t[i] = add_next(m[i] ^ nm, 0u);
+        t[L - 2] &= 0x7ffu;
+#pragma unroll
+        for (int i = L - 1; i > 1; --i) m[i] = __funnelshift_l(t[i - 2], t[i - 1], 21);
+        m[1] = t[0] << 21;
+        m[0] = 0;
+        e -= 53;
+        neg ^= up;
+        // leading zeros: whole words, then bits
+#pragma unroll 1
+        for (int w = 0; w < L - 1 && m[L - 1] == 0; ++w) {
+#pragma unroll
+            for (int i = L - 1; i > 0; --i) m[i] = m[i - 1];
+            m[0] = 0;
+            e -= 32;
+        }
+        const int sh = __clz(m[L - 1]) & 31;
+#pragma unroll
+        for (int i = L - 1; i > 0; --i) m[i] = __funnelshift_l(m[i - 1], m[i], sh);
+        m[0] <<= sh;
+        e -= sh;
     }
 }
 
