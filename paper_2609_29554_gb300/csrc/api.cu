@@ -319,7 +319,8 @@ int gemm_device(ozlu_handle* h, int nc, int p, int m, int n, int k, int alpha, c
     uint8_t* T = (uint8_t*)(base + L.t);
     const int prev = h->open_phase;
     h->phase(PH_CONVERT);
-    launch_shifts(A, lda, m, B, ldb, n, nc, k, pl->Q, mu, nu, nullptr, s);
+    launch_shifts(A, lda, m, B, ldb, n, nc, k, pl->Q, mu, nu, h->clear_err ? derr : nullptr, s);
+    h->clear_err = false;
     if (mode == 3) {
         launch_convert64(A, lda, nc, m, k, false, mu, *tab, Kpad, Mpad, (double*)RA, s);
         launch_convert64(B, ldb, nc, k, n, true, nu, *tab, Kpad, Npad, (double*)RB, s);
@@ -519,10 +520,17 @@ int ozlu_gemm(ozlu_handle* h, int nc, int p, int m, int n, int k, int alpha, con
     if (!C && m && n) return -13;
     if (ldc < (m > 1 ? m : 1)) return -14;
     if (cudaSetDevice(h->device) != cudaSuccess) return OZLU_ERR_CUDA;
-    int rc0 = clear_err_word(h);
-    if (rc0) return rc0;
+    // the product's first kernel clears the error word, or this where none runs
+    if (!err_word(h)) return OZLU_ERR_NOMEM;
+    auto product = [&](const double* a, const double* b, double* c) -> int {
+        h->clear_err = true;
+        const int rc = gemm_device(h, nc, p, m, n, k, alpha, a, lda, b, ldb, beta, c, ldc, opts);
+        const int rc1 = h->clear_err ? clear_err_word(h) : OZLU_OK;
+        h->clear_err = false;
+        return rc ? rc : rc1;
+    };
     const bool dA = !A || is_device_ptr(A), dB = !B || is_device_ptr(B), dC = !C || is_device_ptr(C);
-    if (dA && dB && dC) return gemm_device(h, nc, p, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, opts);
+    if (dA && dB && dC) return product(A, B, C);
     // stage host operands through a second device buffer
     const size_t ea = (size_t)lda * (k ? k : 1) * nc, eb = (size_t)ldb * (n ? n : 1) * nc,
                  ec = (size_t)ldc * (n ? n : 1) * nc;
@@ -542,7 +550,7 @@ int ozlu_gemm(ozlu_handle* h, int nc, int p, int m, int n, int k, int alpha, con
         if (beta && cudaMemcpyAsync(sC, C, sizeof(double) * ec, cudaMemcpyHostToDevice, s)) return OZLU_ERR_CUDA;
         gC = sC;
     }
-    rc = gemm_device(h, nc, p, m, n, k, alpha, gA, lda, gB, ldb, beta, gC, ldc, opts);
+    rc = product(gA, gB, gC);
     if (rc) return rc;
     if (!dC && cudaMemcpyAsync(C, sC, sizeof(double) * ec, cudaMemcpyDeviceToHost, s)) return OZLU_ERR_CUDA;
     return cuda_rc(cudaStreamSynchronize(s));

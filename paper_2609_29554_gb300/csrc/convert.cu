@@ -2,6 +2,7 @@
 // centered residue planes (Sec. 3.1, Sec. 3.2 Eq. (2), Sec. 3.3 Eq. (12)).
 #include <limits.h>
 
+#include "launch.cuh"
 #include "conv_device.cuh"
 #include "mp_device.cuh"
 #include "ozlu_internal.h"
@@ -21,10 +22,11 @@ constexpr int NO_EXP = INT_MIN;
 // `clear` (may be null): the device error word, zeroed for a new call.
 constexpr int SHIFT_THREADS = 1024;
 
-__global__ void __launch_bounds__(SHIFT_THREADS) shift_kernel(const double* __restrict__ A, long long lda, int m,
-                                                              const double* __restrict__ B, long long ldb, int n,
-                                                              int nc, int k, int Q, int* __restrict__ mu,
-                                                              int* __restrict__ nu, int blocks_a, int* clear) {
+__global__ void __launch_bounds__(SHIFT_THREADS) shift_kernel(const double* A, long long lda, int m,
+                                                              const double* B, long long ldb, int n,
+                                                              int nc, int k, int Q, int* mu,
+                                                              int* nu, int blocks_a, int* clear) {
+    chain_enter();
     __shared__ int red[32][33];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (clear && blockIdx.x == 0 && threadIdx.x == 0) *clear = 0;
@@ -36,7 +38,7 @@ __global__ void __launch_bounds__(SHIFT_THREADS) shift_kernel(const double* __re
             const long long step = lda * nc;
 #pragma unroll 4
             for (int h = warp; h < k; h += 32) {
-                const double v = __ldg(x + h * step);
+                const double v = *(x + h * step);
                 if (v != 0.0) E = max(E, frexp_exp(v));
             }
         }
@@ -53,7 +55,7 @@ __global__ void __launch_bounds__(SHIFT_THREADS) shift_kernel(const double* __re
         const double* x = B + (long long)j * ldb * nc;
 #pragma unroll 4
         for (int h = lane; h < k; h += 32) {
-            const double v = __ldg(x + (long long)h * nc);
+            const double v = *(x + (long long)h * nc);
             if (v != 0.0) E = max(E, frexp_exp(v));
         }
         E = __reduce_max_sync(0xffffffffu, E);
@@ -90,9 +92,10 @@ __device__ __forceinline__ int centered_residue64(const uint32_t (&mag)[MAXD], b
 // padded rows are left as they are (they only reach discarded outputs).
 template <int H>
 __global__ void __launch_bounds__(256) convert64_kernel(
-    const double* __restrict__ X, long long ld, int nc, int R, int K, int is_b,
-    const int* __restrict__ shifts, const __grid_constant__ DevTable tab, int Kpad, int Rpad,
-    double* __restrict__ planes) {
+    const double* X, long long ld, int nc, int R, int K, int is_b,
+    const int* shifts, const __grid_constant__ DevTable tab, int Kpad, int Rpad,
+    double* planes) {
+    chain_enter();
     const int h = blockIdx.x * 32 + (threadIdx.x & 31);
     const int r = blockIdx.y * 8 + (threadIdx.x >> 5);
     if (h >= Kpad || r >= R) return;
@@ -210,6 +213,7 @@ struct ConvArgs {
 template <int MODE, int NWX, int NW, int E>
 __global__ void __launch_bounds__(256) convert_kernel(const __grid_constant__ ConvArgs a,
                                                       const __grid_constant__ ConvTab tab) {
+    chain_enter();
     const bool is_b = (int)blockIdx.x >= a.blocks_a;
     const int HG = a.Kpad / E;
     const long long idx = (long long)((int)blockIdx.x - (is_b ? a.blocks_a : 0)) * 256 + threadIdx.x;
@@ -227,7 +231,7 @@ __global__ void __launch_bounds__(256) convert_kernel(const __grid_constant__ Co
 #pragma unroll
             for (int i = 0; i < NWX; ++i) V[e][i] = 0;
             if (h0 + e < a.K)
-                for (int c = 0; c < a.nc; ++c) add_component<NWX>(V[e], __ldg(x + e * step + c), shift);
+                for (int c = 0; c < a.nc; ++c) add_component<NWX>(V[e], *(x + e * step + c), shift);
         }
     }
     const int S = tab.S, w = tab.w;
@@ -287,7 +291,7 @@ void launch_conv(ConvArgs a, const ConvTab& t, cudaStream_t s) {
         const long long ta = (long long)a.m * (a.Kpad / E), tb = (long long)a.n * (a.Kpad / E);
         a.blocks_a = (int)((ta + 255) / 256);
         a.lper = t.N;
-        convert_kernel<MODE, NWX, NW, E><<<a.blocks_a + (unsigned)((tb + 255) / 256), 256, 0, s>>>(a, t);
+        launch(convert_kernel<MODE, NWX, NW, E>, a.blocks_a + (unsigned)((tb + 255) / 256), 256, 0, s, a, t);
         return;
     }
     const long long ta = (long long)a.m * a.Kpad, tb = (long long)a.n * a.Kpad;
@@ -298,7 +302,7 @@ void launch_conv(ConvArgs a, const ConvTab& t, cudaStream_t s) {
     if (split > 8) split = 8;
     if (split > t.N) split = t.N;
     a.lper = (t.N + split - 1) / split;
-    convert_kernel<MODE, NWX, NW, 1><<<dim3(blocks, (t.N + a.lper - 1) / a.lper), 256, 0, s>>>(a, t);
+    launch(convert_kernel<MODE, NWX, NW, 1>, dim3(blocks, (t.N + a.lper - 1) / a.lper), 256, 0, s, a, t);
 }
 
 template <int MODE>
@@ -319,7 +323,7 @@ void launch_conv_mode(const ConvArgs& a, const ConvTab& t, cudaStream_t s) {
 void launch_shifts(const double* A, long long lda, int m, const double* B, long long ldb, int n, int nc, int k, int Q,
                    int* mu, int* nu, int* clear, cudaStream_t s) {
     const int ba = (m + 31) / 32, bb = (n + 31) / 32;
-    shift_kernel<<<ba + bb, SHIFT_THREADS, 0, s>>>(A, lda, m, B, ldb, n, nc, k, Q, mu, nu, ba, clear);
+    launch(shift_kernel, ba + bb, SHIFT_THREADS, 0, s, A, lda, m, B, ldb, n, nc, k, Q, mu, nu, ba, clear);
 }
 
 void launch_convert(const double* A, long long lda, int m, const double* B, long long ldb, int n, int nc, int k,
@@ -343,14 +347,14 @@ void launch_convert64(const double* X, long long ld, int nc, int rows, int cols,
     switch (tab.H) {
 #define OZLU_CONV(HH) \
     case HH: \
-        convert64_kernel<HH><<<grid, 256, 0, s>>>(X, ld, nc, R, K, is_b ? 1 : 0, shifts, tab, Kpad, Rpad, planes); \
+        launch(convert64_kernel<HH>, grid, 256, 0, s, X, ld, nc, R, K, is_b ? 1 : 0, shifts, tab, Kpad, Rpad, planes); \
         break;
         OZLU_CONV(2) OZLU_CONV(3) OZLU_CONV(4) OZLU_CONV(5) OZLU_CONV(6)
         OZLU_CONV(7) OZLU_CONV(8) OZLU_CONV(9) OZLU_CONV(10) OZLU_CONV(11) OZLU_CONV(12)
         OZLU_CONV(13) OZLU_CONV(14) OZLU_CONV(15)
 #undef OZLU_CONV
         default:
-            convert64_kernel<16><<<grid, 256, 0, s>>>(X, ld, nc, R, K, is_b ? 1 : 0, shifts, tab, Kpad, Rpad, planes);
+            launch(convert64_kernel<16>, grid, 256, 0, s, X, ld, nc, R, K, is_b ? 1 : 0, shifts, tab, Kpad, Rpad, planes);
     }
 }
 

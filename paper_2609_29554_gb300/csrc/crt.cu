@@ -16,6 +16,7 @@
 //
 // The group accumulators live in registers (WG is a template parameter, so
 // the word loops unroll).
+#include "launch.cuh"
 #include "crt_kernel.cuh"
 
 namespace ozlu {
@@ -189,10 +190,11 @@ __device__ __forceinline__ void wide_round_out(const Wide& X, bool neg, int E, i
 // need shifts by run-time amounts, live in shared memory, one column per
 // thread ([word][thread]).
 template <int WG>
-__global__ void __launch_bounds__(CT) crt64_kernel(const uint32_t* __restrict__ T, int m, int n,
-                                                   const int* __restrict__ mu, const int* __restrict__ nu,
+__global__ void __launch_bounds__(CT) crt64_kernel(const uint32_t* T, int m, int n,
+                                                   const int* mu, const int* nu,
                                                    const __grid_constant__ DevTable tab, int nc, int alpha,
-                                                   int beta, double* __restrict__ C, long long ldc) {
+                                                   int beta, double* C, long long ldc) {
+    chain_enter();
     __shared__ uint32_t sx[WACC * CT];
     __shared__ uint32_t ss[MAXWG * CT];
     const long long e = (long long)blockIdx.x * CT + threadIdx.x;
@@ -278,11 +280,11 @@ void launch_crt64(const uint32_t* T, int m, int n, const int* mu, const int* nu,
     const unsigned grid = (unsigned)((mn + CT - 1) / CT);
     switch (tab.WG) {
 #define OZLU_WG(W) \
-    case W: crt64_kernel<W><<<grid, CT, 0, s>>>(T, m, n, mu, nu, tab, nc, alpha, beta, C, ldc); break;
+    case W: launch(crt64_kernel<W>, grid, CT, 0, s, T, m, n, mu, nu, tab, nc, alpha, beta, C, ldc); break;
         OZLU_WG(5) OZLU_WG(6) OZLU_WG(7) OZLU_WG(8) OZLU_WG(9) OZLU_WG(10) OZLU_WG(11) OZLU_WG(12) OZLU_WG(13)
         OZLU_WG(14) OZLU_WG(15) OZLU_WG(16)
 #undef OZLU_WG
-        default: crt64_kernel<4><<<grid, CT, 0, s>>>(T, m, n, mu, nu, tab, nc, alpha, beta, C, ldc); break;
+        default: launch(crt64_kernel<4>, grid, CT, 0, s, T, m, n, mu, nu, tab, nc, alpha, beta, C, ldc); break;
     }
 }
 

@@ -3,6 +3,7 @@
 // (two translation units compile side by side).
 #pragma once
 
+#include "launch.cuh"
 #include "carry.cuh"
 #include "mp_device.cuh"
 #include "ozlu_internal.h"
@@ -92,14 +93,14 @@ struct Fetch {
             const uint32_t* tp = (const uint32_t*)a.T + ((long long)gi * tab.NT + 4 * b) * a.mn + e;
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                t[i] = 4 * b + i < tab.NT ? __ldg(tp) : 0u;
+                t[i] = 4 * b + i < tab.NT ? *tp : 0u;
                 tp += a.mn;
             }
         } else {
             const uint8_t* tp = (const uint8_t*)a.T + ((long long)gi * tab.N + 12 * b) * a.mn + e;
 #pragma unroll
             for (int i = 0; i < (PACK ? 4 : 12); ++i) {
-                t[i] = 12 * b + i < tab.N ? (uint32_t)__ldg(tp) : 0u;
+                t[i] = 12 * b + i < tab.N ? (uint32_t)*tp : 0u;
                 tp += a.mn;
             }
         }
@@ -324,6 +325,7 @@ __device__ __noinline__ void crt_one_wide(const CrtArgs& a, const CrtTab& tab, l
 template <int WG, int NW, bool PACK>
 __global__ void __launch_bounds__(CT, min_blocks<NW, PACK>()) crt_kernel(const __grid_constant__ CrtArgs a,
                                                  const __grid_constant__ CrtTab tab) {
+    chain_enter();
     const long long e = (long long)blockIdx.x * CT + threadIdx.x;
     if (e >= a.mn) return;
     if (!crt_one<WG, NW, PACK>(a, tab, e)) crt_one_wide<WG, PACK>(a, tab, e);
@@ -335,10 +337,10 @@ void launch_crt_wg(const CrtArgs& a, const CrtTab& tab, cudaStream_t s) {
     // words for P_int with its sign and 30 bits or more above it for the old C
     const int need = (tab.pint_bits + 1 + 30 + 31) / 32;
 #define OZLU_NW(W) \
-    if (WG < W && need <= W) return crt_kernel<WG, WG < W ? W : WACC, PACK><<<grid, CT, 0, s>>>(a, tab), void();
+    if (WG < W && need <= W) return launch(crt_kernel<WG, WG < W ? W : WACC, PACK>, grid, CT, 0, s, a, tab), void();
     OZLU_NW(10) OZLU_NW(11) OZLU_NW(12) OZLU_NW(13) OZLU_NW(14)
 #undef OZLU_NW
-    crt_kernel<WG, WACC, PACK><<<grid, CT, 0, s>>>(a, tab);
+    launch(crt_kernel<WG, WACC, PACK>, grid, CT, 0, s, a, tab);
 }
 
 template <bool PACK>

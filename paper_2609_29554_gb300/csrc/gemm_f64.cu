@@ -8,6 +8,7 @@
 // 32-bit word.  The tile loop is a plain shared-memory DFMA GEMM: on GB300
 // the binary64 rate (about 1 TFLOP/s) makes this back-end a reference point
 // for the autotuner rather than a contender.
+#include "launch.cuh"
 #include "mp_device.cuh"
 #include "ozlu_internal.h"
 
@@ -21,11 +22,12 @@ __device__ __forceinline__ long long mod_signed(long long v, long long m) {
     return r < 0 ? r + m : r;
 }
 
-__global__ void __launch_bounds__(THREADS) gemm_f64_kernel(const double* __restrict__ RA,
-                                                           const double* __restrict__ RB, int m, int n,
+__global__ void __launch_bounds__(THREADS) gemm_f64_kernel(const double* RA,
+                                                           const double* RB, int m, int n,
                                                            int Mpad, int Npad, int Kpad,
                                                            const __grid_constant__ DevTable tab,
-                                                           uint32_t* __restrict__ T) {
+                                                           uint32_t* T) {
+    chain_enter();
     __shared__ double sa[BK][BM + 1];
     __shared__ double sb[BK][BN + 1];
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
@@ -91,7 +93,7 @@ __global__ void __launch_bounds__(THREADS) gemm_f64_kernel(const double* __restr
 void launch_gemm_f64(const double* RA, const double* RB, int m, int n, int Mpad, int Npad, int Kpad,
                      const DevTable& tab, uint32_t* T, cudaStream_t s) {
     dim3 grid(Mpad / BM, Npad / BN, tab.N * tab.G);
-    gemm_f64_kernel<<<grid, THREADS, 0, s>>>(RA, RB, m, n, Mpad, Npad, Kpad, tab, T);
+    launch(gemm_f64_kernel, grid, THREADS, 0, s, RA, RB, m, n, Mpad, Npad, Kpad, tab, T);
 }
 
 }  // namespace ozlu

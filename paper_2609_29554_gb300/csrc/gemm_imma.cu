@@ -25,6 +25,7 @@
 // residues are combined.  t_l (< 2^14) is stored as 16 bits.
 #include <string.h>
 
+#include "launch.cuh"
 #include "mp_device.cuh"
 #include "ozlu_internal.h"
 
@@ -84,8 +85,9 @@ __device__ __forceinline__ uint32_t smod(int c, uint32_t m, uint32_t magic) {
 
 template <bool EXT>
 __global__ void __launch_bounds__(THREADS) gemm_imma_kernel(
-    const int8_t* __restrict__ RA, const int8_t* __restrict__ RB, int m, int n, int Mpad,
-    int Npad, int Kpad, const __grid_constant__ DevTable tab, const ExtDev ext, void* __restrict__ Tout) {
+    const int8_t* RA, const int8_t* RB, int m, int n, int Mpad,
+    int Npad, int Kpad, const __grid_constant__ DevTable tab, const ExtDev ext, void* Tout) {
+    chain_enter();
     extern __shared__ __align__(128) uint8_t smem[];
     constexpr int P = EXT ? 3 : 1;  // residue planes per modulus
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -269,8 +271,9 @@ constexpr int NBN = 16, NTHREADS = 128;
 constexpr int NTILE_B = NBN * BK;  // 1 KiB
 
 __global__ void __launch_bounds__(NTHREADS) gemm_imma_narrow_kernel(
-    const int8_t* __restrict__ RA, const int8_t* __restrict__ RB, int m, int n, int Mpad, int Npad, int Kpad,
-    const __grid_constant__ DevTable tab, uint8_t* __restrict__ T) {
+    const int8_t* RA, const int8_t* RB, int m, int n, int Mpad, int Npad, int Kpad,
+    const __grid_constant__ DevTable tab, uint8_t* T) {
+    chain_enter();
     extern __shared__ __align__(128) uint8_t smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int tm = blockIdx.x, tn = blockIdx.y;
@@ -387,7 +390,7 @@ void launch_gemm_imma(const int8_t* RA, const int8_t* RB, int m, int n, int Mpad
     dim3 grid(Mpad / BM, Npad / BN, tab.N * tab.G);
     ExtDev none;
     memset(&none, 0, sizeof none);
-    gemm_imma_kernel<false><<<grid, THREADS, smem, s>>>(RA, RB, m, n, Mpad, Npad, Kpad, tab, none, T);
+    launch(gemm_imma_kernel<false>, grid, THREADS, smem, s, RA, RB, m, n, Mpad, Npad, Kpad, tab, none, T);
 }
 
 // n <= 16: the B planes hold Npad = n rounded up to 16 rows
@@ -395,7 +398,7 @@ void launch_gemm_imma_narrow(const int8_t* RA, const int8_t* RB, int m, int n, i
                              const DevTable& tab, uint8_t* T, cudaStream_t s) {
     const int smem = STAGES * (TILE_BYTES + NTILE_B);  // 36 KB
     dim3 grid(Mpad / BM, Npad / NBN, tab.N * tab.G);
-    gemm_imma_narrow_kernel<<<grid, NTHREADS, smem, s>>>(RA, RB, m, n, Mpad, Npad, Kpad, tab, T);
+    launch(gemm_imma_narrow_kernel, grid, NTHREADS, smem, s, RA, RB, m, n, Mpad, Npad, Kpad, tab, T);
 }
 
 void launch_gemm_imma_ext(const int8_t* RA, const int8_t* RB, int m, int n, int Mpad, int Npad, int Kpad,
@@ -403,7 +406,7 @@ void launch_gemm_imma_ext(const int8_t* RA, const int8_t* RB, int m, int n, int 
     const int smem = STAGES * 2 * TILE_BYTES;  // 64 KB (the 32 KB t tile reuses it)
     raise_smem_limit((const void*)gemm_imma_kernel<true>, smem);
     dim3 grid(Mpad / BM, Npad / BN, ext.N * ext.G);
-    gemm_imma_kernel<true><<<grid, THREADS, smem, s>>>(RA, RB, m, n, Mpad, Npad, Kpad, tab, ext, T);
+    launch(gemm_imma_kernel<true>, grid, THREADS, smem, s, RA, RB, m, n, Mpad, Npad, Kpad, tab, ext, T);
 }
 
 }  // namespace ozlu

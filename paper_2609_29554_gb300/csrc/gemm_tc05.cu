@@ -42,6 +42,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include "launch.cuh"
 #include "ozlu_internal.h"
 #include "tables.h"
 
@@ -172,8 +173,8 @@ __device__ __forceinline__ uint32_t floor_mod_bits(float v, float m, float invu)
 template <bool FP8, bool PACK>
 __global__ void __launch_bounds__(THREADS, 1) gemm_tc05_kernel(
     const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int m, int n,
-    int Mpad, int Npad, int KB, const __grid_constant__ GemmTab tab, void* __restrict__ T,
-    int* __restrict__ err) {
+    int Mpad, int Npad, int KB, const __grid_constant__ GemmTab tab, void* T,
+    int* err) {
     constexpr int P = FP8 ? 3 : 1;                // planes (products per modulus)
     constexpr int LG = PACK ? 3 : 1;              // moduli per unit
     constexpr uint32_t TMEM_COLS = NBUF * BN;
@@ -231,6 +232,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc05_kernel(
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n");
     const uint32_t tmem = *tmem_slot;
+    chain_enter();  // (the set-up above runs beside the conversion)
 
     if (warp == 0) {
         // position in the smem ring: stage s, parity of its pass; `issued`
@@ -446,7 +448,7 @@ int launch_gemm_tc05(bool fp8, bool pack, const void* RA, const void* RB, int m,
     dim3 grid((unsigned)(units < sms ? units : sms));
     auto go = [&](auto kernel) {
         raise_smem_limit((const void*)kernel, (int)smem);
-        kernel<<<grid, THREADS, smem, s>>>(ta, tb, m, n, Mpad, Npad, KB, tab, T, err);
+        launch(kernel, grid, THREADS, smem, s, ta, tb, m, n, Mpad, Npad, KB, tab, T, err);
     };
     if (fp8) pack ? go(gemm_tc05_kernel<true, true>) : go(gemm_tc05_kernel<true, false>);
     else pack ? go(gemm_tc05_kernel<false, true>) : go(gemm_tc05_kernel<false, false>);

@@ -21,6 +21,7 @@
 
 #include <tuple>
 
+#include "launch.cuh"
 #include "expansion.cuh"
 #include "mpf.cuh"
 #include "ozlu_handle.h"
@@ -139,6 +140,7 @@ template <int N>
 __global__ void __launch_bounds__(PIV_THREADS) pivot_kernel(double* A, long long lda, int n, int c,
                                                             int p0, int p1, int* ipiv,
                                                             LuScratch* sc) {
+    chain_enter();
     __shared__ double sv[PIV_THREADS][N];
     __shared__ int si[PIV_THREADS];
     __shared__ bool last;
@@ -218,6 +220,7 @@ template <int N>
 __global__ void __launch_bounds__(128) column_step_kernel(double* A, long long lda, int n, int c,
                                                           int c1, int p0, int p1, int* ipiv,
                                                           LuScratch* sc) {
+    chain_enter();
     constexpr int L = Limbs<N>::L;
     __shared__ MPF<L> urow[BASE];
     __shared__ MPF<L> lrow[STEP_ROWS];
@@ -970,6 +973,7 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) base_block_coop_kernel(
 template <int N>
 __global__ void laswp_kernel(double* A, long long lda, int j0, int j1, int k0, int k1,
                              const int* ipiv) {
+    chain_enter();
     const int j = j0 + blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= j1) return;
     for (int k = k0; k < k1; ++k) {
@@ -994,6 +998,7 @@ __global__ void laswp_kernel(double* A, long long lda, int j0, int j1, int k0, i
 // stores a swap, the next positions loaded ahead).  With a hash map filled by that
 // thread the list took 50 us for 256 interchanges.
 __global__ void __launch_bounds__(LMAXB) laswp_list_kernel(int k0, int k1, const int* ipiv, int* list) {
+    chain_enter();
     __shared__ int piv[LMAXB], slot[LMAXB + 1], val[2 * LMAXB], row[2 * LMAXB];
     __shared__ int cnt;
     const int b = k1 - k0, t = threadIdx.x;
@@ -1036,6 +1041,7 @@ __global__ void __launch_bounds__(LMAXB) laswp_list_kernel(int k0, int k1, const
 template <int N>
 __global__ void __launch_bounds__(256) laswp_apply_kernel(double* A, long long lda, int j0, int j1,
                                                           const int* list) {
+    chain_enter();
     extern __shared__ __align__(16) double buf[];  // [entry][col][N]
     const int ne = list[0];
     const int jb = j0 + blockIdx.x * LCT;
@@ -1064,15 +1070,15 @@ void laswp2(double* A, long long lda, int ja0, int ja1, int jb0, int jb1, int k0
             int* list, cudaStream_t s) {
     if (k1 <= k0 || (ja1 <= ja0 && jb1 <= jb0)) return;
     if (k1 - k0 > LMAXB) {
-        if (ja1 > ja0) laswp_kernel<N><<<(ja1 - ja0 + 127) / 128, 128, 0, s>>>(A, lda, ja0, ja1, k0, k1, ipiv);
-        if (jb1 > jb0) laswp_kernel<N><<<(jb1 - jb0 + 127) / 128, 128, 0, s>>>(A, lda, jb0, jb1, k0, k1, ipiv);
+        if (ja1 > ja0) launch(laswp_kernel<N>, (ja1 - ja0 + 127) / 128, 128, 0, s, A, lda, ja0, ja1, k0, k1, ipiv);
+        if (jb1 > jb0) launch(laswp_kernel<N>, (jb1 - jb0 + 127) / 128, 128, 0, s, A, lda, jb0, jb1, k0, k1, ipiv);
         return;
     }
-    laswp_list_kernel<<<1, (k1 - k0 + 31) / 32 * 32, 0, s>>>(k0, k1, ipiv, list);
+    launch(laswp_list_kernel, 1, (k1 - k0 + 31) / 32 * 32, 0, s, k0, k1, ipiv, list);
     const size_t smem = sizeof(double) * 2 * (k1 - k0) * LCT * N;
     raise_smem_limit((const void*)laswp_apply_kernel<N>, (int)(sizeof(double) * 2 * LMAXB * LCT * N));
-    if (ja1 > ja0) laswp_apply_kernel<N><<<(ja1 - ja0 + LCT - 1) / LCT, 256, smem, s>>>(A, lda, ja0, ja1, list);
-    if (jb1 > jb0) laswp_apply_kernel<N><<<(jb1 - jb0 + LCT - 1) / LCT, 256, smem, s>>>(A, lda, jb0, jb1, list);
+    if (ja1 > ja0) launch(laswp_apply_kernel<N>, (ja1 - ja0 + LCT - 1) / LCT, 256, smem, s, A, lda, ja0, ja1, list);
+    if (jb1 > jb0) launch(laswp_apply_kernel<N>, (jb1 - jb0 + LCT - 1) / LCT, 256, smem, s, A, lda, jb0, jb1, list);
 }
 
 // Native trailing update for the blocked-naive comparison (Sec. 3.4):
@@ -1082,6 +1088,7 @@ template <int N>
 __global__ void __launch_bounds__(256) naive_update_kernel(const double* A, long long lda, const double* B,
                                                            long long ldb, double* C, long long ldc, int m,
                                                            int n, int k) {
+    chain_enter();
     __shared__ double sa[16][16][N];
     __shared__ double sb[16][16][N];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -1120,6 +1127,7 @@ __global__ void __launch_bounds__(256) naive_update_kernel(const double* A, long
 template <int N>
 __global__ void __launch_bounds__(256) tri_convert_kernel(const double* T, long long ldt, int b, int lower,
                                                           LuScratch* sc) {
+    chain_enter();
     constexpr int L = Limbs<N>::L;
     const int q = blockIdx.y;
     T += ((long long)q * b + (long long)q * b * ldt) * N;
@@ -1146,6 +1154,7 @@ __global__ void __launch_bounds__(256) tri_convert_kernel(const double* T, long 
 template <int N>
 __global__ void __launch_bounds__(TRSM_WARPS * 32) trsm_base_kernel(const LuScratch* sc, double* X, long long ldx,
                                                                     int b, int ncols, int lower, int slot) {
+    chain_enter();
     constexpr int L = Limbs<N>::L;
     extern __shared__ __align__(16) unsigned char smraw[];
     MPF<L>* sl = reinterpret_cast<MPF<L>*>(smraw);   // [k][i]
@@ -1183,7 +1192,7 @@ void trsm_base(const double* T, long long ldt, double* X, long long ldx, int b, 
     if (ncols <= 0 || b <= 0) return;
     constexpr int L = Limbs<N>::L;
     if (slot < 0) {
-        tri_convert_kernel<N><<<(b * b + 255) / 256, 256, 0, s>>>(T, ldt, b, lower, sc);
+        launch(tri_convert_kernel<N>, (b * b + 255) / 256, 256, 0, s, T, ldt, b, lower, sc);
         slot = 0;
     }
     // every SM the same number of columns: blocks of equal size, one or two an SM
@@ -1191,7 +1200,7 @@ void trsm_base(const double* T, long long ldt, double* X, long long ldx, int b, 
     const int wpb = (ncols + per - 1) / per;
     const size_t smem = sizeof(MPF<L>) * (BASE * BASE + BASE);
     raise_smem_limit((const void*)trsm_base_kernel<N>, (int)smem);
-    trsm_base_kernel<N><<<(ncols + wpb - 1) / wpb, 32 * wpb, smem, s>>>(sc, X, ldx, b, ncols, lower, slot);
+    launch(trsm_base_kernel<N>, (ncols + wpb - 1) / wpb, 32 * wpb, smem, s, sc, X, ldx, b, ncols, lower, slot);
 }
 
 // ---------------------------------------------------------------------------
@@ -1450,7 +1459,7 @@ void trsm_rec(Ctx& c, long long r, int b, long long j0, int ncols, bool lower, l
     if (lower && r_top < 0 && b > BASE && (b & (b - 1)) == 0 && b / BASE <= TRI_SLOTS) {
         // every leaf's triangle in one launch, ahead of the recursion
         c.h->phase(PH_TRSM);
-        tri_convert_kernel<N><<<dim3((BASE * BASE + 255) / 256, b / BASE), 256, 0, c.h->stream>>>(
+        launch(tri_convert_kernel<N>, dim3((BASE * BASE + 255) / 256, b / BASE), 256, 0, c.h->stream, 
             at(c, r, r), c.lda, BASE, 1, c.sc);
         c.h->count(1);
         r_top = r;
@@ -1505,14 +1514,14 @@ void panel_rec(Ctx& c, int r, int b, int p0, int p1) {
             const int rows = c.n - r;
             const int blocks = rows > PIV_THREADS * PIV_BLOCKS ? PIV_BLOCKS
                                                                : (rows + PIV_THREADS - 1) / PIV_THREADS;
-            pivot_kernel<N><<<blocks, PIV_THREADS, 0, s>>>(c.A, c.lda, c.n, r, p0, p1, c.ipiv, c.sc);
+            launch(pivot_kernel<N>, blocks, PIV_THREADS, 0, s, c.A, c.lda, c.n, r, p0, p1, c.ipiv, c.sc);
         }
         for (int col = r; col < r + b; ++col) {
             const int rows = c.n - col - 1;
             if (rows <= 0) break;
             int blocks = (rows + STEP_ROWS - 1) / STEP_ROWS;
             if (blocks > MAXPART) blocks = MAXPART;
-            column_step_kernel<N><<<blocks, 128, 0, s>>>(c.A, c.lda, c.n, col, r + b, p0, p1, c.ipiv,
+            launch(column_step_kernel<N>, blocks, 128, 0, s, c.A, c.lda, c.n, col, r + b, p0, p1, c.ipiv,
                                                           c.sc);
         }
         return;
@@ -1548,7 +1557,7 @@ int getrf_device(ozlu_handle* h, int p, int n, double* A, long long lda, int* ip
                 h->phase(PH_GEMM);
                 const int mm = n - r0 - b;
                 dim3 grid((mm + 15) / 16, (mm + 15) / 16);
-                naive_update_kernel<N><<<grid, 256, 0, s>>>(at(c, r0 + b, r0), lda, at(c, r0, r0 + b), lda,
+                launch(naive_update_kernel<N>, grid, 256, 0, s, at(c, r0 + b, r0), lda, at(c, r0, r0 + b), lda,
                                                             at(c, r0 + b, r0 + b), lda, mm, mm, b);
                 h->count(1);
             } else if (!c.rc) {

@@ -25,6 +25,7 @@
 
 #include <math.h>
 
+#include "launch.cuh"
 #include "conv_device.cuh"
 #include "mp_device.cuh"
 #include "ozlu_handle.h"
@@ -66,6 +67,7 @@ __device__ __forceinline__ uint32_t mant32(const MPView& X, long long x, long lo
 // about a load latency per element.
 __global__ void __launch_bounds__(1024) mp_shift_kernel(MPView A, int m, MPView B, int n, int k, int Q, int* mu,
                                                          int* nu, int blocks_a) {
+    chain_enter();
     __shared__ int red[32][33];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int E = INT_MIN;
@@ -130,6 +132,7 @@ struct MpConvArgs {
 template <int NW, bool FP8, int E>
 __global__ void __launch_bounds__(256) mp_convert_kernel(const __grid_constant__ MpConvArgs a,
                                                          const __grid_constant__ ConvTab tab) {
+    chain_enter();
     const bool is_b = (int)blockIdx.x >= a.blocks_a;
     const int bid = (int)blockIdx.x - (is_b ? a.blocks_a : 0);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -166,13 +169,13 @@ __global__ void __launch_bounds__(256) mp_convert_kernel(const __grid_constant__
         for (int e = 0; e < E; ++e) {
             const int pos = t * w + sh[e];
             const int q = pos >> 5, rr = pos & 31;
-            uint32_t v = live[e] && q >= 0 && q < L ? __ldg(lp[e] + (long long)q * X.plane) : 0u;
+            uint32_t v = live[e] && q >= 0 && q < L ? *(lp[e] + (long long)q * X.plane) : 0u;
             uint64_t c = carry[e];
             bool lowzero = true;
 #pragma unroll
             for (int i = 0; i < NW; ++i) {
                 const int qn = q + i + 1;
-                const uint32_t nx = live[e] && qn >= 0 && qn < L ? __ldg(lp[e] + (long long)qn * X.plane) : 0u;
+                const uint32_t nx = live[e] && qn >= 0 && qn < L ? *(lp[e] + (long long)qn * X.plane) : 0u;
                 uint32_t d = __funnelshift_r(v, nx, rr);
                 v = nx;
                 if (i == NW - 1) d &= mk;
@@ -214,10 +217,11 @@ __global__ void __launch_bounds__(256) mp_convert_kernel(const __grid_constant__
 // (i, j, l, g), the pair terms and K summed in int32 on the integer pipe.
 constexpr int KSMALL = 8;
 
-__global__ void __launch_bounds__(256) small_k_gemm_kernel(const int8_t* __restrict__ RA,
-                                                           const int8_t* __restrict__ RB, int m, int n, int K,
+__global__ void __launch_bounds__(256) small_k_gemm_kernel(const int8_t* RA,
+                                                           const int8_t* RB, int m, int n, int K,
                                                            const __grid_constant__ DevTable tab,
-                                                           uint8_t* __restrict__ T) {
+                                                           uint8_t* T) {
+    chain_enter();
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long mn = (long long)m * n;
     if (idx >= mn * tab.N * tab.G) return;
@@ -260,8 +264,9 @@ __device__ __forceinline__ uint32_t reduce64(unsigned long long a, uint32_t m, u
     return mod_small(hi * two32 + lo, m, magic);
 }
 
-__global__ void mp_convert_ext_kernel(MPView X, int R, int Kc, int is_b, const int* __restrict__ shifts,
-                                      const ExtDev E, int Kpad, int Rpad, int8_t* __restrict__ planes) {
+__global__ void mp_convert_ext_kernel(MPView X, int R, int Kc, int is_b, const int* shifts,
+                                      const ExtDev E, int Kpad, int Rpad, int8_t* planes) {
+    chain_enter();
     extern __shared__ uint32_t dsm[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
     const int groups = (Kc + 31) / 32;  // 32-position groups per row (the K padding is zeroed by the host)
@@ -465,10 +470,11 @@ __device__ void mp_finish(const Acc& A, int NW, long long E, int alpha, int beta
 
 
 template <int WG>
-__global__ void __launch_bounds__(MPCT) mp_crt_kernel(const uint8_t* __restrict__ T, int m, int nchunk, int j0,
-                                                      const int* __restrict__ mu, const int* __restrict__ nu,
+__global__ void __launch_bounds__(MPCT) mp_crt_kernel(const uint8_t* T, int m, int nchunk, int j0,
+                                                      const int* mu, const int* nu,
                                                       const __grid_constant__ DevTable tab, int NW, int alpha,
                                                       int beta, MPView C, int p) {
+    chain_enter();
     extern __shared__ uint32_t accsm[];
     const long long e = (long long)blockIdx.x * MPCT + threadIdx.x;
     const long long mn = (long long)m * nchunk;
@@ -535,10 +541,11 @@ __global__ void __launch_bounds__(MPCT) mp_crt_kernel(const uint8_t* __restrict_
 // rounding of mp_finish.
 constexpr int XCH = 8;
 
-__global__ void __launch_bounds__(MPCT) mp_crt_ext_kernel(const uint16_t* __restrict__ T, int m, int nchunk, int j0,
-                                                          const int* __restrict__ mu, const int* __restrict__ nu,
+__global__ void __launch_bounds__(MPCT) mp_crt_ext_kernel(const uint16_t* T, int m, int nchunk, int j0,
+                                                          const int* mu, const int* nu,
                                                           const ExtDev E, int NW, int alpha, int beta, MPView C,
                                                           int p) {
+    chain_enter();
     extern __shared__ uint32_t accsm[];
     const long long e = (long long)blockIdx.x * MPCT + threadIdx.x;
     const long long mn = (long long)m * nchunk;
@@ -674,6 +681,7 @@ __device__ __forceinline__ uint32_t win_bits(const uint32_t* A, int NW, long lon
 template <int WG>
 __global__ void __launch_bounds__(32 * CWC) mp_crt_warp_kernel(const __grid_constant__ MpCrtArgs a,
                                                                const __grid_constant__ CrtTab tab) {
+    chain_enter();
     extern __shared__ uint32_t cwsm[];
     __shared__ uint32_t sM[MAXTRI][WG];  // P / m_q (lanes read different triples)
     __shared__ uint32_t sc[3 * MAXTRI];
@@ -702,9 +710,9 @@ __global__ void __launch_bounds__(32 * CWC) mp_crt_warp_kernel(const __grid_cons
         if (gi < G) {
             const uint8_t* tp = a.T + (size_t)gi * tab.N * a.mn + e;
             for (int q = part; q < tab.NT; q += parts) {
-                uint32_t u = (uint32_t)__ldg(tp + (size_t)(3 * q) * a.mn) * sc[3 * q];
-                if (3 * q + 1 < tab.N) u += (uint32_t)__ldg(tp + (size_t)(3 * q + 1) * a.mn) * sc[3 * q + 1];
-                if (3 * q + 2 < tab.N) u += (uint32_t)__ldg(tp + (size_t)(3 * q + 2) * a.mn) * sc[3 * q + 2];
+                uint32_t u = (uint32_t)*(tp + (size_t)(3 * q) * a.mn) * sc[3 * q];
+                if (3 * q + 1 < tab.N) u += (uint32_t)*(tp + (size_t)(3 * q + 1) * a.mn) * sc[3 * q + 1];
+                if (3 * q + 2 < tab.N) u += (uint32_t)*(tp + (size_t)(3 * q + 2) * a.mn) * sc[3 * q + 2];
 #pragma unroll
                 for (int k = 0; k < WG; ++k) acc[k] += (uint64_t)u * sM[q][k];
                 F = fmaf((float)u, si[q], F);
@@ -845,7 +853,7 @@ void convert_nw(MpConvArgs a, const ConvTab& t, cudaStream_t s) {
     if (a.Kp % 4 == 0 && ((long long)a.m + a.n) * a.Kp >= 4ll * 512 * sms) {
         a.blocks_a = blocks(a.m, 4);
         a.lper = t.N;
-        mp_convert_kernel<NW, FP8, 4><<<a.blocks_a + blocks(a.n, 4), 256, 0, s>>>(a, t);
+        launch(mp_convert_kernel<NW, FP8, 4>, a.blocks_a + blocks(a.n, 4), 256, 0, s, a, t);
         return;
     }
     a.blocks_a = blocks(a.m, 1);
@@ -855,7 +863,7 @@ void convert_nw(MpConvArgs a, const ConvTab& t, cudaStream_t s) {
     if (split > 16) split = 16;
     if (split > t.N) split = t.N;
     a.lper = (t.N + split - 1) / split;
-    mp_convert_kernel<NW, FP8, 1><<<dim3(nb, (t.N + a.lper - 1) / a.lper), 256, 0, s>>>(a, t);
+    launch(mp_convert_kernel<NW, FP8, 1>, dim3(nb, (t.N + a.lper - 1) / a.lper), 256, 0, s, a, t);
 }
 
 // rows [0, m) of A's planes and [0, n) of B's (padded rows reach discarded
@@ -882,12 +890,12 @@ void crt_wg(const uint8_t* T, int m, int nchunk, int j0, const int* mu, const in
     if (mn < MP_WARP_CRT && wsm <= 200 * 1024) {
         const MpCrtArgs a{T, mu, nu, mn, m, j0, NW, alpha, beta, p, C};
         raise_smem_limit((const void*)mp_crt_warp_kernel<WG>, (int)wsm);
-        mp_crt_warp_kernel<WG><<<(unsigned)((mn + CWC - 1) / CWC), 32 * CWC, wsm, s>>>(a, ct);
+        launch(mp_crt_warp_kernel<WG>, (unsigned)((mn + CWC - 1) / CWC), 32 * CWC, wsm, s, a, ct);
         return;
     }
     const size_t smem = sizeof(uint32_t) * (size_t)NW * MPCT;
     raise_smem_limit((const void*)mp_crt_kernel<WG>, (int)smem);
-    mp_crt_kernel<WG><<<(unsigned)((mn + MPCT - 1) / MPCT), MPCT, smem, s>>>(T, m, nchunk, j0, mu, nu, tab, NW,
+    launch(mp_crt_kernel<WG>, (unsigned)((mn + MPCT - 1) / MPCT), MPCT, smem, s, T, m, nchunk, j0, mu, nu, tab, NW,
                                                                             alpha, beta, C, p);
 }
 
@@ -971,7 +979,7 @@ void mp_convert_ext(const MPView& X, int R, int Kc, int is_b, const int* shifts,
     while (warps > 1 && (size_t)warps * E.WD * 32 * 4 > 200 * 1024) warps /= 2;
     const size_t smem = (size_t)warps * E.WD * 32 * 4;
     raise_smem_limit((const void*)mp_convert_ext_kernel, (int)smem);
-    mp_convert_ext_kernel<<<(unsigned)((tasks + warps - 1) / warps), 32 * warps, smem, s>>>(X, R, Kc, is_b, shifts, E,
+    launch(mp_convert_ext_kernel, (unsigned)((tasks + warps - 1) / warps), 32 * warps, smem, s, X, R, Kc, is_b, shifts, E,
                                                                                            Kpad, Rpad, planes);
 }
 
@@ -1017,7 +1025,7 @@ int mp_gemm_ext(ozlu_handle* h, int p, int S, int m, int n, int k, int alpha, co
     const int prev = h->open_phase;
     h->phase(PH_CONVERT);
     const int ba = (m + 31) / 32, bb = (n + 31) / 32;
-    mp_shift_kernel<<<ba + bb, 1024, 0, s>>>(vA, m, vB, n, k, pl->Q, mu, nu, ba);
+    launch(mp_shift_kernel, ba + bb, 1024, 0, s, vA, m, vB, n, k, pl->Q, mu, nu, ba);
     mp_convert_ext(vA, m, k, 0, mu, E, Kpad, Mpad, RA, s);
     h->count(2);
     for (long long j0 = 0; j0 < n; j0 += nch) {
@@ -1029,7 +1037,7 @@ int mp_gemm_ext(ozlu_handle* h, int p, int S, int m, int n, int k, int alpha, co
         launch_gemm_imma_ext(RA, RB, m, nc, Mpad, ncp, Kpad, tab, E, T, s);
         h->phase(PH_CRT);
         const long long mn = (long long)m * nc;
-        mp_crt_ext_kernel<<<(unsigned)((mn + MPCT - 1) / MPCT), MPCT, crt_smem, s>>>(T, m, nc, (int)j0, mu, nu, E,
+        launch(mp_crt_ext_kernel, (unsigned)((mn + MPCT - 1) / MPCT), MPCT, crt_smem, s, T, m, nc, (int)j0, mu, nu, E,
                                                                                      NW, alpha, beta, vC, p);
         h->count(3);
         h->stats.gemm_launches += 1;
@@ -1167,7 +1175,7 @@ int mp_gemm_device(ozlu_handle* h, int p, int m, int n, int k, int alpha, const 
     h->phase(PH_CONVERT);
     {
         const int nc0 = (int)(n < nch ? n : nch), ba = (m + 31) / 32, bb = (n + 31) / 32;
-        mp_shift_kernel<<<ba + bb, 1024, 0, s>>>(vA, m, vB, n, k, pl->Q, mu, nu, ba);
+        launch(mp_shift_kernel, ba + bb, 1024, 0, s, vA, m, vB, n, k, pl->Q, mu, nu, ba);
         mp_convert(vA, m, vB, nc0, k, mu, nu, pe->conv, Kpad, Mpad, (nc0 + rowq - 1) / rowq * rowq, RA, RB, fp8, s);
     }
     h->count(2);
@@ -1184,7 +1192,7 @@ int mp_gemm_device(ozlu_handle* h, int p, int m, int n, int k, int alpha, const 
             if ((rc = launch_gemm_tc05(true, false, RA, RB, m, nc, Mpad, ncp, Kpad, pe->gemm, T, derr, s))) return rc;
         } else if (smallk) {
             const long long work = (long long)m * nc * pl->N * pl->G;
-            small_k_gemm_kernel<<<(unsigned)((work + 255) / 256), 256, 0, s>>>(RA, RB, m, nc, k, *tab, T);
+            launch(small_k_gemm_kernel, (unsigned)((work + 255) / 256), 256, 0, s, RA, RB, m, nc, k, *tab, T);
         } else if (narrow) {
             launch_gemm_imma_narrow(RA, RB, m, nc, Mpad, ncp, Kpad, *tab, T, s);
         } else {

@@ -20,6 +20,7 @@
 
 #include <utility>
 
+#include "launch.cuh"
 #include "mp_device.cuh"
 #include "ozlu_handle.h"
 
@@ -61,6 +62,7 @@ __device__ int mp_abs_cmp(const MPV& A, long long x, const MPV& B, long long y) 
 // pivot of column c over rows [c, n): one block; ipiv[c] = piv + 1, info
 constexpr int PT = 512;
 __global__ void __launch_bounds__(PT) mp_pivot_kernel(MPV A, int n, int c, int* piv_out, int* ipiv, int* info) {
+    chain_enter();
     __shared__ int best[PT];
     int bi = -1;
     for (int i = c + threadIdx.x; i < n; i += PT) {
@@ -106,6 +108,7 @@ __device__ void swap_elem(const MPV& A, long long x, long long y) {
 
 // rows r and *piv exchanged over columns [j0, j1)
 __global__ void mp_swap_kernel(MPV A, int r, const int* piv, int j0, int j1) {
+    chain_enter();
     const int j = j0 + blockIdx.x * blockDim.x + threadIdx.x;
     const int p = *piv;
     if (j >= j1 || p == r) return;
@@ -114,6 +117,7 @@ __global__ void mp_swap_kernel(MPV A, int r, const int* piv, int j0, int j1) {
 
 // interchanges k in [k0, k1) (ipiv 1-based) on columns [j0, j1), one column per thread
 __global__ void mp_laswp_kernel(MPV A, int k0, int k1, const int* ipiv, int j0, int j1) {
+    chain_enter();
     const int j = j0 + blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= j1) return;
     for (int k = k0; k < k1; ++k) {
@@ -162,6 +166,7 @@ __device__ void blk_mul(const uint32_t* X, int nx, const uint32_t* Y, int ny, ui
 //   T = F Y 2^-(32 L) ~ f y 2^(32 W),  E = 2^(32 W) - T,  Y += Y E 2^-(32 W)
 // from a binary64 start; `iters` steps double the 53 correct bits each.
 __global__ void __launch_bounds__(RT) mp_recip_kernel(MPV A, long long x, MPV R, int iters) {
+    chain_enter();
     extern __shared__ unsigned long long rsm[];
     const int La = A.L, W = R.L;
     unsigned long long* S = rsm;                          // La + 2 W + 4 column sums
@@ -244,6 +249,7 @@ __global__ void __launch_bounds__(RT) mp_recip_kernel(MPV A, long long x, MPV R,
 
 // copy an m x n block (D, S with the same L)
 __global__ void mp_copy_kernel(MPV S, MPV D, int m, int n) {
+    chain_enter();
     const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (long long)m * n) return;
     const long long i = e % m, j = e / m;
@@ -310,7 +316,7 @@ int mp_reciprocal(Ctx& c, const ozlu_mp_matrix& M, long long i, long long j) {
     for (int prec = 53; prec < c.p + 40; prec *= 2) ++iters;
     const size_t smem = sizeof(unsigned long long) * (La + 2 * W + 4) + sizeof(uint32_t) * (La + 3 * (W + 1));
     cudaFuncSetAttribute(mp_recip_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    mp_recip_kernel<<<1, RT, smem, c.h->stream>>>(dv(M), i + j * M.ld, dv(c.sc->x), iters);
+    launch(mp_recip_kernel, 1, RT, smem, c.h->stream, dv(M), i + j * M.ld, dv(c.sc->x), iters);
     c.h->count(1);
     return cudaGetLastError() == cudaSuccess ? OZLU_OK : OZLU_ERR_CUDA;
 }
@@ -334,7 +340,7 @@ int mp_scale(Ctx& c, const ozlu_mp_matrix& M, long long r0, long long j0, int m,
     }
     if (rc) return rc;
     const long long cnt = (long long)m * nc;
-    mp_copy_kernel<<<(unsigned)((cnt + 127) / 128), 128, 0, s>>>(dv(blk), dv(sub(M, r0, j0)), m, nc);
+    launch(mp_copy_kernel, (unsigned)((cnt + 127) / 128), 128, 0, s, dv(blk), dv(sub(M, r0, j0)), m, nc);
     c.h->count(1);
     return cudaGetLastError() == cudaSuccess ? OZLU_OK : OZLU_ERR_CUDA;
 }
@@ -374,8 +380,8 @@ void mp_panel(Ctx& c, int r, int b, int p0, int p1) {
     if (c.rc) return;
     cudaStream_t s = c.h->stream;
     if (b == 1) {
-        mp_pivot_kernel<<<1, PT, 0, s>>>(dv(c.A), c.n, r, c.sc->piv, c.ipiv, c.info);
-        mp_swap_kernel<<<(p1 - p0 + 127) / 128, 128, 0, s>>>(dv(c.A), r, c.sc->piv, p0, p1);
+        launch(mp_pivot_kernel, 1, PT, 0, s, dv(c.A), c.n, r, c.sc->piv, c.ipiv, c.info);
+        launch(mp_swap_kernel, (p1 - p0 + 127) / 128, 128, 0, s, dv(c.A), r, c.sc->piv, p0, p1);
         c.h->count(2);
         // the zero-pivot flag is on the device: skip the scaling only when the
         // pivot is exactly zero (the host cannot see it without a sync), so
@@ -438,9 +444,9 @@ extern "C" int ozlu_mp_getrf(ozlu_handle* h, int p, int n, const ozlu_mp_matrix*
         mp_panel(c, r0, b, r0, r0 + b);
         if (c.rc) break;
         // interchanges of this panel on the columns left and right of it
-        if (r0 > 0) mp_laswp_kernel<<<(r0 + 127) / 128, 128, 0, s>>>(dv(c.A), r0, r0 + b, ipiv, 0, r0);
+        if (r0 > 0) launch(mp_laswp_kernel, (r0 + 127) / 128, 128, 0, s, dv(c.A), r0, r0 + b, ipiv, 0, r0);
         if (r0 + b < n)
-            mp_laswp_kernel<<<(n - r0 - b + 127) / 128, 128, 0, s>>>(dv(c.A), r0, r0 + b, ipiv, r0 + b, n);
+            launch(mp_laswp_kernel, (n - r0 - b + 127) / 128, 128, 0, s, dv(c.A), r0, r0 + b, ipiv, r0 + b, n);
         h->count(2);
         if (r0 + b < n) {
             mp_trsm_lower(c, c.A, r0, b, c.A, r0, r0 + b, n - r0 - b);
@@ -469,7 +475,7 @@ extern "C" int ozlu_mp_getrs(ozlu_handle* h, int p, int n, int nrhs, const ozlu_
     int rc = sc.alloc(B->L, nrhs > n ? nrhs : n);
     if (rc) return rc;
     Ctx c{h, p, *LU, n, const_cast<int*>(ipiv), nullptr, &sc};
-    mp_laswp_kernel<<<(nrhs + 127) / 128, 128, 0, s>>>(dv(*B), 0, n, ipiv, 0, nrhs);
+    launch(mp_laswp_kernel, (nrhs + 127) / 128, 128, 0, s, dv(*B), 0, n, ipiv, 0, nrhs);
     h->count(1);
     mp_trsm_lower(c, *LU, 0, n, *B, 0, 0, nrhs);
     mp_trsm_upper(c, *LU, 0, n, *B, 0, 0, nrhs);

@@ -52,6 +52,7 @@ struct ozlu_handle {
     std::map<std::tuple<int, int, int, int, int, int>, ozlu::PlanEntry> plans;
     ozlu::GemmLayout last;
     int* dev_err = nullptr;  // device error word of the tensor-core GEMMs
+    bool clear_err = false;  // the next product starts by zeroing it
     bool timing = false;
     ozlu_stats stats = {};
     void* lu_scratch = nullptr;  // pivot-search scratch of ozlu_getrf
