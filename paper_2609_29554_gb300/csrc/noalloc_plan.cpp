@@ -15,27 +15,29 @@ namespace {
 
 constexpr int PW = 16;  // words of P (54 moduli of <= 8 bits: <= 432 bits)
 
-bool is_prime_na(int v) {
-    if (v < 2) return false;
-    for (int d = 2; d * d <= v; ++d)
-        if (v % d == 0) return false;
-    return true;
-}
-
 // the 54 maximal prime powers <= 255, descending (Sec. 3.2)
-int int8_moduli_na(int* out) {
+struct Moduli {
+    int v[64] = {};
     int cnt = 0;
-    for (int q = 2; q <= 255; ++q) {
-        if (!is_prime_na(q)) continue;
-        int v = q;
-        while (v * q <= 255) v *= q;
-        out[cnt++] = v;
+    constexpr Moduli() {
+        for (int q = 2; q <= 255; ++q) {
+            bool prime = true;
+            for (int d = 2; d * d <= q; ++d) prime = prime && q % d != 0;
+            if (!prime) continue;
+            int w = q;
+            while (w * q <= 255) w *= q;
+            v[cnt++] = w;
+        }
+        for (int i = 0; i < cnt; ++i)
+            for (int j = i + 1; j < cnt; ++j)
+                if (v[j] > v[i]) {
+                    const int t = v[i];
+                    v[i] = v[j];
+                    v[j] = t;
+                }
     }
-    for (int i = 0; i < cnt; ++i)
-        for (int j = i + 1; j < cnt; ++j)
-            if (out[j] > out[i]) { const int t = out[i]; out[i] = out[j]; out[j] = t; }
-    return cnt;
-}
+};
+constexpr Moduli MODS;
 
 int inv_mod_na(int a, int m) {
     long long t = 0, nt = 1, r = m, nr = a % m;
@@ -53,8 +55,8 @@ int inv_mod_na(int a, int m) {
 int plan_noalloc(int p, int K, DevTable& t, int& Kpad_out, int* pint_out) {
     memset(&t, 0, sizeof t);
     if (p < 1 || K < 1) return OZLU_ERR_CAPACITY;
-    int mods[64];
-    const int nm = int8_moduli_na(mods);
+    const int* mods = MODS.v;
+    const int nm = MODS.cnt;
     const int slack = (int)ceil(log2(2.0 * K) - 1e-12) + 16;
     const int Kpad = (K + 127) / 128 * 128;
     for (int S = 1; S <= 64; ++S) {
@@ -86,26 +88,34 @@ int plan_noalloc(int p, int K, DevTable& t, int& Kpad_out, int* pint_out) {
                 c = v >> 32;
             }
         }
+        int np = PW;
+        while (P[np - 1] == 0) --np;
         t.N = N; t.WG = WG; t.H = H; t.S = S; t.w = w; t.g0 = g0; t.G = G; t.Q = w * S; t.WX = WX;
         for (int l = 0; l < N; ++l) {
             const uint32_t m = (uint32_t)mods[l];
-            uint32_t M[PW];
-            uint64_t rem = 0;
-            for (int wd = PW - 1; wd >= 0; --wd) {
-                const uint64_t cur = (rem << 32) | P[wd];
-                M[wd] = (uint32_t)(cur / m);
-                rem = cur % m;
-            }
-            uint64_t mm = 0;
-            for (int wd = PW - 1; wd >= 0; --wd) mm = ((mm << 32) | M[wd]) % m;
+            const uint32_t magic = (uint32_t)(((1ull << 32) + m - 1) / m);
+            // floor(x / m) for x < 2^24
+            auto quot = [&](uint32_t x) { return (uint32_t)(((uint64_t)x * magic) >> 32); };
+            // M = P / m by halves from the top, and M mod m beside it
+            uint32_t M[PW] = {0};
+            uint32_t rem = 0, mm = 0;
+            for (int wd = np - 1; wd >= 0; --wd)
+                for (int h = 16; h >= 0; h -= 16) {
+                    const uint32_t cur = (rem << 16) | ((P[wd] >> h) & 0xffffu), q = quot(cur);
+                    rem = cur - q * m;
+                    M[wd] |= q << h;
+                    const uint32_t x = (mm << 16) | q;
+                    mm = x - quot(x) * m;
+                }
             t.mod[l] = (int)m;
             t.y[l] = inv_mod_na((int)mm, (int)m);
-            t.magic[l] = (uint32_t)(((1ull << 32) + m - 1) / m);
+            t.magic[l] = magic;
             t.invm[l] = 1.0f / (float)m;
-            uint64_t r = 1 % m;
+            uint32_t r = 1 % m;
             for (int j = 0; j < MAXH; ++j) {
-                t.pow16[l][j] = (uint32_t)r;
-                r = (r << 16) % m;
+                t.pow16[l][j] = r;
+                r <<= 16;
+                r -= quot(r) * m;
             }
             for (int wd = 0; wd < MAXWG; ++wd) t.Mlow[l][wd] = wd < PW ? M[wd] : 0u;
         }

@@ -13,13 +13,15 @@ void fill_conv(const DevTable& t, ConvTab& c) {
     for (int l = 0; l < t.N; ++l) {
         ConvMod& k = c.mod[l];
         const uint32_t m = (uint32_t)t.mod[l];
-        uint32_t pw = 1 % m;  // 2^b mod m
-        for (int b = 0; b <= 32 * CONV_WORDS; ++b) {
-            if ((b & 7) == 0 && b < 32 * CONV_WORDS) k.p8[b >> 5] |= pw << (b & 31);
-            if (b == t.w) k.wrapc = (m - pw) % m;
-            if (b == 32 * c.NW) k.topc = (m - pw) % m;
-            pw += pw;
-            if (pw >= m) pw -= m;
+        // x mod m for x < 2^24
+        auto red = [&](uint32_t x) { return x - (uint32_t)(((uint64_t)x * t.magic[l]) >> 32) * m; };
+        auto neg = [&](uint32_t x) { return x ? m - x : 0u; };
+        uint32_t pw = 1 % m;  // 2^(8 b) mod m
+        for (int b = 0; b <= 4 * CONV_WORDS; ++b) {
+            if (b < 4 * CONV_WORDS) k.p8[b >> 2] |= pw << (8 * (b & 3));
+            if (b == t.w >> 3) k.wrapc = neg(red(pw << (t.w & 7)));
+            if (b == 4 * c.NW) k.topc = neg(pw);
+            pw = red(pw << 8);
         }
         const uint32_t kneg = (1 + k.topc) % m;
         k.k4 = (k.wrapc << 8) | (kneg << 16) | ((kneg + m - k.wrapc) % m << 24);
@@ -36,19 +38,22 @@ void fill_crt(const DevTable& t, int pint_bits, CrtTab& c) {
     memset(&c, 0, sizeof c);
     c.N = t.N; c.NT = (t.N + 2) / 3; c.WG = t.WG; c.G = t.G; c.w = t.w; c.g0 = t.g0;
     c.pint_bits = pint_bits;
+    uint32_t mq[MAXTRI];  // products of triples, below 2^24
     for (int q = 0; q < c.NT; ++q) {
-        uint32_t mq = 1;
-        for (int l = 3 * q; l < 3 * q + 3 && l < t.N; ++l) mq *= (uint32_t)t.mod[l];
-        for (int l = 3 * q; l < 3 * q + 3 && l < t.N; ++l) c.coef[l] = mq / (uint32_t)t.mod[l];
-        c.inv[q] = 1.0f / (float)mq;
-        // P / m_q as the product of the other moduli, modulo 2^(32 MAXWG)
+        mq[q] = 1;
+        for (int l = 3 * q; l < 3 * q + 3 && l < t.N; ++l) mq[q] *= (uint32_t)t.mod[l];
+        for (int l = 3 * q; l < 3 * q + 3 && l < t.N; ++l) c.coef[l] = mq[q] / (uint32_t)t.mod[l];
+        c.inv[q] = 1.0f / (float)mq[q];
+    }
+    for (int q = 0; q < c.NT; ++q) {
+        // P / m_q as the product of the other triples, modulo 2^(32 MAXWG)
         uint32_t* M = c.Mt[q];
         M[0] = 1;
-        for (int l = 0; l < t.N; ++l) {
-            if (l / 3 == q) continue;
+        for (int j = 0; j < c.NT; ++j) {
+            if (j == q) continue;
             uint64_t cy = 0;
             for (int k = 0; k < MAXWG; ++k) {
-                cy += (uint64_t)M[k] * (uint32_t)t.mod[l];
+                cy += (uint64_t)M[k] * mq[j];
                 M[k] = (uint32_t)cy;
                 cy >>= 32;
             }
