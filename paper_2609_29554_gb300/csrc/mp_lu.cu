@@ -91,38 +91,39 @@ __global__ void __launch_bounds__(PT) mp_pivot_kernel(MPV A, int n, int c, int* 
     }
 }
 
-__device__ void swap_elem(const MPV& A, long long x, long long y) {
-    for (int k = 0; k < A.L; ++k) {
-        uint32_t* a = A.limbs + (long long)k * A.plane;
-        const uint32_t t = a[x];
-        a[x] = a[y];
-        a[y] = t;
-    }
-    int t = A.exps[x];
-    A.exps[x] = A.exps[y];
-    A.exps[y] = t;
-    t = A.signs[x];
-    A.signs[x] = A.signs[y];
-    A.signs[y] = t;
+// word w of element x: its limbs, then exponent and sign (L + 2 words)
+__device__ __forceinline__ uint32_t* elem_word(const MPV& A, long long x, int w) {
+    if (w < A.L) return A.limbs + (long long)w * A.plane + x;
+    return (uint32_t*)(w == A.L ? A.exps : A.signs) + x;
 }
 
-// rows r and *piv exchanged over columns [j0, j1)
+// rows r and *piv exchanged over columns [j0, j1): a thread a word of a column
 __global__ void mp_swap_kernel(MPV A, int r, const int* piv, int j0, int j1) {
     chain_enter();
-    const int j = j0 + blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = j0 + blockIdx.x * blockDim.x + threadIdx.x, w = blockIdx.y;
     const int p = *piv;
     if (j >= j1 || p == r) return;
-    swap_elem(A, (long long)r + (long long)j * A.ld, (long long)p + (long long)j * A.ld);
+    uint32_t* x = elem_word(A, (long long)r + (long long)j * A.ld, w);
+    uint32_t* y = elem_word(A, (long long)p + (long long)j * A.ld, w);
+    const uint32_t t = *x;
+    *x = *y;
+    *y = t;
 }
 
-// interchanges k in [k0, k1) (ipiv 1-based) on columns [j0, j1), one column per thread
+// interchanges k in [k0, k1) (ipiv 1-based) on columns [j0, j1): a thread a
+// word of a column
 __global__ void mp_laswp_kernel(MPV A, int k0, int k1, const int* ipiv, int j0, int j1) {
     chain_enter();
-    const int j = j0 + blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = j0 + blockIdx.x * blockDim.x + threadIdx.x, w = blockIdx.y;
     if (j >= j1) return;
+    uint32_t* col = elem_word(A, (long long)j * A.ld, w);
     for (int k = k0; k < k1; ++k) {
         const int p = ipiv[k] - 1;
-        if (p != k) swap_elem(A, (long long)k + (long long)j * A.ld, (long long)p + (long long)j * A.ld);
+        if (p != k) {
+            const uint32_t t = col[k];
+            col[k] = col[p];
+            col[p] = t;
+        }
     }
 }
 
@@ -130,32 +131,58 @@ __global__ void mp_laswp_kernel(MPV A, int k0, int k1, const int* ipiv, int j0, 
 // number (one block of RT threads, words in shared memory).
 constexpr int RT = 256;
 
+// warp 0: words w_0, w_1, ... (value(k) below 2^32 + 2^31, k < n) with their
+// carries resolved, 32 at a time: a word generates a carry from 2^32 on and
+// passes one on at 2^32 - 1, so that all carries of a round are one addition of
+// the two ballots; put(k, word)
+template <typename V, typename P>
+__device__ __forceinline__ void warp_carries(int n, uint32_t cin, V value, P put) {
+    const int lane = threadIdx.x & 31;
+    for (int k0 = 0; k0 < n; k0 += 32) {
+        const int k = k0 + lane;
+        const uint64_t v = k < n ? value(k) : 0;
+        const uint32_t gen = __ballot_sync(0xffffffffu, (v >> 32) != 0);
+        const uint32_t pass = __ballot_sync(0xffffffffu, (uint32_t)v == 0xffffffffu && (v >> 32) == 0);
+        const uint64_t c = ((((uint64_t)gen << 1) | cin) + pass) ^ pass;  // carries into the lanes
+        if (k < n) put(k, (uint32_t)v + (uint32_t)(c >> lane & 1));
+        cin = (uint32_t)(c >> 32) & 1u;
+    }
+}
+
 // out[0, olen) = (X[0, nx) * Y[0, ny)) >> (32 shift), truncated: column sums
-// of the 32-bit halves of the limb products by all threads (64-bit, below
-// 2^(33 + log2 n)), then one thread propagates the carries
+// of the 32-bit halves of the limb products (64-bit, below 2^(32 + log2 n) a
+// part), `parts` = 4: low and high halves, even and odd terms, by different
+// threads (1: where the sums would not fit in shared memory); then one warp
+// adds the parts and resolves the carries
 __device__ void blk_mul(const uint32_t* X, int nx, const uint32_t* Y, int ny, uint32_t* out, int shift, int olen,
-                        unsigned long long* S) {
-    const int ncol = nx + ny;
-    for (int k = threadIdx.x; k < ncol; k += RT) {
+                        unsigned long long* S, int parts) {
+    const int ncol = nx + ny, step = parts > 1 ? 2 : 1;
+    for (int q = threadIdx.x; q < ncol * parts; q += RT) {
+        const int k = q % ncol, part = q / ncol;
         unsigned long long acc = 0;
-        const int i0 = max(0, k - ny + 1), i1 = min(nx - 1, k);
-        for (int i = i0; i <= i1; ++i) acc += (uint32_t)((uint64_t)X[i] * Y[k - i]);
-        const int j0 = max(0, k - 1 - ny + 1), j1 = min(nx - 1, k - 1);
-        for (int i = j0; i <= j1; ++i) acc += (uint64_t)X[i] * Y[k - 1 - i] >> 32;
-        S[k] = acc;
+        if (parts == 1 || part < 2) {
+            const int i0 = max(0, k - ny + 1), i1 = min(nx - 1, k);
+            for (int i = i0 + (part & 1); i <= i1; i += step) acc += (uint32_t)((uint64_t)X[i] * Y[k - i]);
+        }
+        if (parts == 1 || part >= 2) {
+            const int j0 = max(0, k - 1 - ny + 1), j1 = min(nx - 1, k - 1);
+            for (int i = j0 + (part & 1); i <= j1; i += step) acc += (uint64_t)X[i] * Y[k - 1 - i] >> 32;
+        }
+        S[q] = acc;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long c = 0;
-        for (int k = 0; k < ncol; ++k) {
-            const unsigned long long v = S[k] + c;
-            if (k >= shift && k - shift < olen) out[k - shift] = (uint32_t)v;
-            c = v >> 32;
-        }
-        for (int k = ncol; k - shift < olen; ++k) {
-            if (k >= shift) out[k - shift] = (uint32_t)c;
-            c = 0;
-        }
+    if (threadIdx.x < 32) {
+        auto col = [&](int k) -> uint64_t {
+            uint64_t v = 0;
+            if (k >= 0 && k < ncol)
+                for (int q = 0; q < parts; ++q) v += S[q * ncol + k];
+            return v;
+        };
+        const int n = max(ncol, shift + olen);
+        warp_carries(n, 0u, [&](int k) { return (uint64_t)(uint32_t)col(k) + (col(k - 1) >> 32); },
+                     [&](int k, uint32_t v) {
+                         if (k >= shift && k - shift < olen) out[k - shift] = v;
+                     });
     }
     __syncthreads();
 }
@@ -164,25 +191,37 @@ __device__ void blk_mul(const uint32_t* X, int nx, const uint32_t* Y, int ny, ui
 // Newton's iteration on the mantissa in fixed point: with f = |a| 2^-e in
 // [1/2, 1) (F = its L limbs) and y ~ 1/f (Y = y 2^(32 W), W = R.L):
 //   T = F Y 2^-(32 L) ~ f y 2^(32 W),  E = 2^(32 W) - T,  Y += Y E 2^-(32 W)
-// from a binary64 start; `iters` steps double the 53 correct bits each.
-__global__ void __launch_bounds__(RT) mp_recip_kernel(MPV A, long long x, MPV R, int iters) {
+// from a binary64 start; `iters` steps double the 53 correct bits each.  1 / 0
+// is set to 0 (its pivot's column is not scaled, a solve's unknown becomes 0).
+// Latency of one block: with the carries of every product, negation and sum
+// resolved by one warp at a time the 1216-bit reciprocal takes 32 us; by one
+// thread, word after word, it took 48.
+__global__ void __launch_bounds__(RT) mp_recip_kernel(MPV A, long long x, MPV R, int iters, int parts) {
     chain_enter();
     extern __shared__ unsigned long long rsm[];
     const int La = A.L, W = R.L;
-    unsigned long long* S = rsm;                          // La + 2 W + 4 column sums
-    uint32_t* F = (uint32_t*)(S + La + 2 * W + 4);        // La
+    unsigned long long* S = rsm;                             // parts x (La + 2 W + 4) column sums
+    uint32_t* F = (uint32_t*)(S + parts * (La + 2 * W + 4)); // La
     uint32_t* Y = F + La;                                 // W + 1
     uint32_t* T = Y + W + 1;                              // W + 1
     uint32_t* U = T + W + 1;                              // W + 1
     for (int k = threadIdx.x; k < La; k += RT) F[k] = A.limbs[(long long)k * A.plane + x];
+    for (int k = threadIdx.x; k <= W; k += RT) Y[k] = 0;
     __syncthreads();
+    if (F[La - 1] == 0) {
+        for (int k = threadIdx.x; k < W; k += RT) R.limbs[(long long)k * R.plane] = 0;
+        if (threadIdx.x == 0) {
+            R.exps[0] = 0;
+            R.signs[0] = 0;
+        }
+        return;
+    }
     if (threadIdx.x == 0) {
         const uint64_t top = ((uint64_t)F[La - 1] << 32) | (La > 1 ? F[La - 2] : 0u);
         const double f = (double)(top >> 11) * 0x1p-53;
         int ey;
         const double fr = frexp(1.0 / f, &ey);         // 1/f = fr 2^ey, ey in {1, 2}
         const uint64_t m53 = (uint64_t)ldexp(fr, 53);  // 1/f = m53 2^(ey - 53)
-        for (int k = 0; k <= W; ++k) Y[k] = 0;
         const int pos = 32 * W + ey - 53;             // bit of Y holding m53's bit 0
         const int q = pos >> 5, r = pos & 31;
         Y[q] = (uint32_t)(m53 << r);
@@ -191,72 +230,51 @@ __global__ void __launch_bounds__(RT) mp_recip_kernel(MPV A, long long x, MPV R,
     }
     __syncthreads();
     for (int it = 0; it < iters; ++it) {
-        blk_mul(F, La, Y, W + 1, T, La, W + 1, S);      // T = F Y >> 32 La
-        if (threadIdx.x == 0) {
+        blk_mul(F, La, Y, W + 1, T, La, W + 1, S, parts);  // T = F Y >> 32 La
+        if (threadIdx.x < 32) {
             // E = 2^(32 W) - T (two's complement in W + 1 words), sign, |E| into T
-            uint64_t c = 1;
-            for (int k = 0; k <= W; ++k) {
-                const uint32_t o = k == W ? 1u : 0u;
-                const uint64_t v = (uint64_t)o + (uint32_t)~T[k] + c;
-                T[k] = (uint32_t)v;
-                c = v >> 32;
-            }
+            auto wk = [&](int k) { return (uint64_t)(uint32_t)~T[k] + (k == W ? 1u : 0u); };
+            auto to_t = [&](int k, uint32_t v) { T[k] = v; };
+            warp_carries(W + 1, 1u, wk, to_t);
+            __syncwarp();
             const bool eneg = (T[W] >> 31) != 0;
-            if (eneg) {
-                uint64_t c2 = 1;
-                for (int k = 0; k <= W; ++k) {
-                    const uint64_t v = (uint64_t)(uint32_t)~T[k] + c2;
-                    T[k] = (uint32_t)v;
-                    c2 = v >> 32;
-                }
-            }
-            U[0] = eneg ? 1u : 0u;  // sign, read below
+            __syncwarp();
+            if (eneg) warp_carries(W + 1, 1u, [&](int k) { return (uint64_t)(uint32_t)~T[k]; }, to_t);
+            if (threadIdx.x == 0) U[0] = eneg ? 1u : 0u;  // sign, read below
         }
         __syncthreads();
         const bool eneg = U[0] != 0;
         __syncthreads();
-        blk_mul(Y, W + 1, T, W + 1, U, W, W + 1, S);     // U = Y |E| >> 32 W
-        if (threadIdx.x == 0) {
-            uint64_t c = eneg ? 1u : 0u;
-            for (int k = 0; k <= W; ++k) {
-                const uint32_t u = eneg ? ~U[k] : U[k];
-                const uint64_t v = (uint64_t)Y[k] + u + c;
-                Y[k] = (uint32_t)v;
-                c = v >> 32;
-            }
-        }
+        blk_mul(Y, W + 1, T, W + 1, U, W, W + 1, S, parts);  // U = Y |E| >> 32 W
+        if (threadIdx.x < 32)
+            warp_carries(W + 1, eneg ? 1u : 0u, [&](int k) { return (uint64_t)Y[k] + (eneg ? ~U[k] : U[k]); },
+                         [&](int k, uint32_t v) { Y[k] = v; });
         __syncthreads();
     }
-    // normalise Y (value y 2^(32 W), y in (1, 2]) into R's W limbs, truncating
+    // normalise Y (value y 2^(32 W), y in (1, 2]) into R's W limbs, truncating:
+    // Y's top bit is in its word W or W - 1
+    const int b = Y[W] ? 32 * W + 32 - __clz(Y[W]) : 32 * W - __clz(Y[W - 1]);
+    const int first = b - 32 * W;  // Y bit at R's limb 0, bit 0
+    for (int k = threadIdx.x; k < W; k += RT) {
+        const int pos = first + 32 * k;
+        const int q = pos >> 5, r = pos & 31;
+        const uint32_t lo = (q >= 0 && q <= W) ? Y[q] : 0u, hi = (q + 1 >= 0 && q + 1 <= W) ? Y[q + 1] : 0u;
+        R.limbs[(long long)k * R.plane] = r ? (lo >> r) | (hi << (32 - r)) : lo;
+    }
     if (threadIdx.x == 0) {
-        int b = 0;
-        for (int k = W; k >= 0; --k)
-            if (Y[k]) {
-                b = 32 * k + 32 - __clz(Y[k]);
-                break;
-            }
-        const int first = b - 32 * W;  // Y bit at R's limb 0, bit 0
-        for (int k = 0; k < W; ++k) {
-            const int pos = first + 32 * k;
-            const int q = pos >> 5, r = pos & 31;
-            const uint32_t lo = (q >= 0 && q <= W) ? Y[q] : 0u, hi = (q + 1 >= 0 && q + 1 <= W) ? Y[q + 1] : 0u;
-            R.limbs[(long long)k * R.plane] = r ? (lo >> r) | (hi << (32 - r)) : lo;
-        }
         R.exps[0] = b - 32 * W - A.exps[x];
         R.signs[0] = A.signs[x];
     }
 }
 
-// copy an m x n block (D, S with the same L)
-__global__ void mp_copy_kernel(MPV S, MPV D, int m, int n) {
+// copy an m x n block (D, S with the same L), a thread a word of an element;
+// not where *skip is set (the zero-pivot flag; null: always)
+__global__ void mp_copy_kernel(MPV S, MPV D, int m, int n, const int* skip) {
     chain_enter();
     const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (long long)m * n) return;
+    if (e >= (long long)m * n || (skip && *skip)) return;
     const long long i = e % m, j = e / m;
-    const long long xs = i + j * S.ld, xd = i + j * D.ld;
-    for (int k = 0; k < D.L; ++k) D.limbs[(long long)k * D.plane + xd] = S.limbs[(long long)k * S.plane + xs];
-    D.exps[xd] = S.exps[xs];
-    D.signs[xd] = S.signs[xs];
+    *elem_word(D, i + j * D.ld, blockIdx.y) = *elem_word(S, i + j * S.ld, blockIdx.y);
 }
 
 // scratch p-bit elements of one factorisation or solve: x, y, z, two (one
@@ -314,16 +332,22 @@ int mp_reciprocal(Ctx& c, const ozlu_mp_matrix& M, long long i, long long j) {
     const int W = c.sc->x.L, La = M.L;
     int iters = 0;
     for (int prec = 53; prec < c.p + 40; prec *= 2) ++iters;
-    const size_t smem = sizeof(unsigned long long) * (La + 2 * W + 4) + sizeof(uint32_t) * (La + 3 * (W + 1));
-    cudaFuncSetAttribute(mp_recip_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch(mp_recip_kernel, 1, RT, smem, c.h->stream, dv(M), i + j * M.ld, dv(c.sc->x), iters);
+    auto bytes = [&](int parts) {
+        return sizeof(unsigned long long) * parts * (La + 2 * W + 4) + sizeof(uint32_t) * (La + 3 * (W + 1));
+    };
+    const int parts = bytes(4) <= 200 * 1024 ? 4 : 1;
+    const size_t smem = bytes(parts);
+    if (smem > 48 * 1024)
+        cudaFuncSetAttribute(mp_recip_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    launch(mp_recip_kernel, 1, RT, smem, c.h->stream, dv(M), i + j * M.ld, dv(c.sc->x), iters, parts);
     c.h->count(1);
     return cudaGetLastError() == cudaSuccess ? OZLU_OK : OZLU_ERR_CUDA;
 }
 
 // rows [r0, r0 + m) x columns [j0, j0 + nc) of A scaled by sc->x (through
-// the scratch block): A <- A * x
-int mp_scale(Ctx& c, const ozlu_mp_matrix& M, long long r0, long long j0, int m, int nc, bool row_vector) {
+// the scratch block): A <- A * x, unless *skip (may be null) is set on the device
+int mp_scale(Ctx& c, const ozlu_mp_matrix& M, long long r0, long long j0, int m, int nc, bool row_vector,
+             const int* skip) {
     if (m <= 0 || nc <= 0) return OZLU_OK;
     cudaStream_t s = c.h->stream;
     Scratch& sc = *c.sc;
@@ -340,7 +364,7 @@ int mp_scale(Ctx& c, const ozlu_mp_matrix& M, long long r0, long long j0, int m,
     }
     if (rc) return rc;
     const long long cnt = (long long)m * nc;
-    launch(mp_copy_kernel, (unsigned)((cnt + 127) / 128), 128, 0, s, dv(blk), dv(sub(M, r0, j0)), m, nc);
+    launch(mp_copy_kernel, dim3((unsigned)((cnt + 127) / 128), M.L + 2), 128, 0, s, dv(blk), dv(sub(M, r0, j0)), m, nc, skip);
     c.h->count(1);
     return cudaGetLastError() == cudaSuccess ? OZLU_OK : OZLU_ERR_CUDA;
 }
@@ -364,7 +388,7 @@ void mp_trsm_upper(Ctx& c, const ozlu_mp_matrix& M, long long r, int b, const oz
     if (c.rc || b <= 0 || ncols <= 0) return;
     if (b == 1) {
         c.rc = mp_reciprocal(c, M, r, r);
-        if (!c.rc) c.rc = mp_scale(c, X, xr, j0, 1, ncols, true);
+        if (!c.rc) c.rc = mp_scale(c, X, xr, j0, 1, ncols, true, nullptr);
         return;
     }
     const int b1 = b / 2;
@@ -381,22 +405,13 @@ void mp_panel(Ctx& c, int r, int b, int p0, int p1) {
     cudaStream_t s = c.h->stream;
     if (b == 1) {
         launch(mp_pivot_kernel, 1, PT, 0, s, dv(c.A), c.n, r, c.sc->piv, c.ipiv, c.info);
-        launch(mp_swap_kernel, (p1 - p0 + 127) / 128, 128, 0, s, dv(c.A), r, c.sc->piv, p0, p1);
+        launch(mp_swap_kernel, dim3((p1 - p0 + 127) / 128, c.A.L + 2), 128, 0, s, dv(c.A), r, c.sc->piv, p0, p1);
         c.h->count(2);
-        // the zero-pivot flag is on the device: skip the scaling only when the
-        // pivot is exactly zero (the host cannot see it without a sync), so
-        // the reciprocal of a zero pivot is avoided by checking on the host
-        // once per column (a short copy; factorisations of singular matrices
-        // keep going as in LAPACK)
-        int flag = 0;
-        if (cudaMemcpyAsync(&flag, c.sc->piv + 1, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaStreamSynchronize(s) != cudaSuccess) {
-            c.rc = OZLU_ERR_CUDA;
-            return;
-        }
-        if (flag) return;
+        // the zero-pivot flag stays on the device: the scaled column is only
+        // copied back where the pivot is not exactly zero (factorisations of
+        // singular matrices keep going as in LAPACK)
         c.rc = mp_reciprocal(c, c.A, r, r);
-        if (!c.rc) c.rc = mp_scale(c, c.A, r + 1, r, c.n - r - 1, 1, false);
+        if (!c.rc) c.rc = mp_scale(c, c.A, r + 1, r, c.n - r - 1, 1, false, c.sc->piv + 1);
         return;
     }
     const int b1 = b / 2;
@@ -444,9 +459,9 @@ extern "C" int ozlu_mp_getrf(ozlu_handle* h, int p, int n, const ozlu_mp_matrix*
         mp_panel(c, r0, b, r0, r0 + b);
         if (c.rc) break;
         // interchanges of this panel on the columns left and right of it
-        if (r0 > 0) launch(mp_laswp_kernel, (r0 + 127) / 128, 128, 0, s, dv(c.A), r0, r0 + b, ipiv, 0, r0);
+        if (r0 > 0) launch(mp_laswp_kernel, dim3((r0 + 127) / 128, c.A.L + 2), 128, 0, s, dv(c.A), r0, r0 + b, ipiv, 0, r0);
         if (r0 + b < n)
-            launch(mp_laswp_kernel, (n - r0 - b + 127) / 128, 128, 0, s, dv(c.A), r0, r0 + b, ipiv, r0 + b, n);
+            launch(mp_laswp_kernel, dim3((n - r0 - b + 127) / 128, c.A.L + 2), 128, 0, s, dv(c.A), r0, r0 + b, ipiv, r0 + b, n);
         h->count(2);
         if (r0 + b < n) {
             mp_trsm_lower(c, c.A, r0, b, c.A, r0, r0 + b, n - r0 - b);
@@ -475,7 +490,7 @@ extern "C" int ozlu_mp_getrs(ozlu_handle* h, int p, int n, int nrhs, const ozlu_
     int rc = sc.alloc(B->L, nrhs > n ? nrhs : n);
     if (rc) return rc;
     Ctx c{h, p, *LU, n, const_cast<int*>(ipiv), nullptr, &sc};
-    launch(mp_laswp_kernel, (nrhs + 127) / 128, 128, 0, s, dv(*B), 0, n, ipiv, 0, nrhs);
+    launch(mp_laswp_kernel, dim3((nrhs + 127) / 128, B->L + 2), 128, 0, s, dv(*B), 0, n, ipiv, 0, nrhs);
     h->count(1);
     mp_trsm_lower(c, *LU, 0, n, *B, 0, 0, nrhs);
     mp_trsm_upper(c, *LU, 0, n, *B, 0, 0, nrhs);
