@@ -56,7 +56,8 @@ enum {
     OZLU_BE_AUTO = 0, /* measured choice per shape: each feasible back-end is timed on
                          the first call of a shape (the call then waits for the
                          stream) and the fastest is cached in the handle          */
-    OZLU_BE_INT8 = 1, /* centered residues in int8, exact int32 accumulation          */
+    OZLU_BE_INT8 = 1, /* centered residues within int8, sums below 2^31 (computed
+                         exactly by binary16 tensor products, folded in parts)    */
     OZLU_BE_FP8 = 2,  /* balanced base-17 digits in E4M3, Eq. (15), fp32 accumulation */
     OZLU_BE_FP64 = 3, /* residues of ~23-bit primes in binary64, Eq. (17)             */
     OZLU_BE_FP16 = 4  /* centered residues in binary16, fp32 accumulation, Eq. (14)   */

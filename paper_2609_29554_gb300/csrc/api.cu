@@ -166,7 +166,7 @@ int autotune(ozlu_handle* h, int nc, int p, int m, int n, int k, const double* A
     // and the Eq. (Lhint) cost ratios r (the paper's 30 for INT8-class
     // engines, 17.9 for binary64)
     const int cand_be[4] = {OZLU_BE_FP16, OZLU_BE_FP8, OZLU_BE_INT8, OZLU_BE_FP64};
-    const double rate[4] = {600.0, 1700.0 / 3.0, 150.0, 1.0};
+    const double rate[4] = {600.0, 1700.0 / 3.0, 600.0, 1.0};
     const double rcost[4] = {30.0, 30.0, 30.0, 17.9};
     struct Cand { int be, S; double model; };
     std::vector<Cand> cands;
@@ -188,6 +188,12 @@ int autotune(ozlu_handle* h, int nc, int p, int m, int n, int k, const double* A
             ts.nslice = S;
             Plan ps;
             if (make_plan(p, k, &ts, ps) != OZLU_OK) continue;
+            if (t.backend == OZLU_BE_INT8) {  // the FP16 candidate of this S, if any, runs the same kernels
+                ozlu_opts tf = ts;
+                tf.backend = OZLU_BE_FP16;
+                Plan pf;
+                if (make_plan(p, k, &tf, pf) == OZLU_OK) continue;
+            }
             const double model = 2.0 * m * n * (double)k * ps.N * ps.pair_terms / (rate[c] * 1e12);
             cands.push_back({cand_be[c], S, model});
             best_model = std::min(best_model, model);
@@ -287,30 +293,52 @@ int gemm_device(ozlu_handle* h, int nc, int p, int m, int n, int k, int alpha, c
     const Plan* pl = &pe->plan;
     const DevTable* tab = &pe->table;
     const int be = pl->backend;
-    const int mode = be == OZLU_BE_INT8 ? 0 : be == OZLU_BE_FP8 ? 1 : be == OZLU_BE_FP16 ? 2 : 3;
-    const int P = mode == 1 ? 3 : 1, esz = mode == 2 ? 2 : (mode == 3 ? 8 : 1);
     const int Mpad = (m + 127) / 128 * 128, Npad = (n + 127) / 128 * 128;
-    // K padded to the GEMM's step: 64 elements (INT8, FP16; the binary64 kernel
-    // takes any), 128 for FP8 (the accumulator conditions hold for the plan's 128)
-    const int Kpad = mode == 1 ? pl->Kpad : (k + 63) / 64 * 64;
     GemmLayout& L = h->last;
-    L.m = m; L.n = n; L.k = k; L.Mpad = Mpad; L.Npad = Npad; L.Kpad = Kpad;
+    L.m = m; L.n = n; L.k = k; L.Mpad = Mpad; L.Npad = Npad;
     L.N = pl->N; L.S = pl->S; L.G = pl->G; L.backend = be;
-    size_t off = 0;
-    L.mu = off; off = align_up(off + sizeof(int) * m);
-    L.nu = off; off = align_up(off + sizeof(int) * n);
-    L.ra = off; off = align_up(off + (size_t)pl->N * pl->S * P * Mpad * Kpad * esz);
-    L.rb = off; off = align_up(off + (size_t)pl->N * pl->S * P * Npad * Kpad * esz);
-    // t values: bytes, 32-bit words (binary64), or a word per triple of moduli
-    const bool pack = (mode == 1 || mode == 2) && tc05_packs(pe->gemm, Mpad, Npad);
-    const size_t tval = pack ? 4 * (size_t)pe->gemm.NT : (size_t)pl->N * (mode == 3 ? 4 : 1);
-    L.t = off;  off = align_up(off + (size_t)pl->G * tval * m * n);
-    L.pack = pack;
+    // An INT8 plan's residue products run as binary16 ones on tcgen05 (mode 2),
+    // exactly and to the same t values: residues up to 127 are binary16 numbers,
+    // and sums longer than binary32 holds exactly are folded in parts.  The int8
+    // tensor rate of this GPU is far below the binary16 one: TD, 1777 x 611 x
+    // 389, 672 us for the products by mma.sync on int8 and 100 by this, 809 and
+    // 225 in all; QD, 1024^3, 620 us in all by the FP8 plan, 480 by this.
+    // mma.sync (mode 0) is left for where the larger residues do not fit in
+    // memory, and for the allocation-free product's fixed scratch.
+    int mode = be == OZLU_BE_FP8 ? 1 : be == OZLU_BE_FP64 ? 3 : 2;
+    int Kpad = 0;
+    bool pack = false;
+    auto layout = [&]() -> size_t {
+        const int P = mode == 1 ? 3 : 1, esz = mode == 2 ? 2 : (mode == 3 ? 8 : 1);
+        // K padded to the GEMM's step: 64 elements (INT8, FP16; the binary64 kernel
+        // takes any), 128 for FP8 (the accumulator conditions hold for the plan's 128)
+        Kpad = mode == 1 ? pl->Kpad : (k + 63) / 64 * 64;
+        L.Kpad = Kpad;
+        L.mode = mode;
+        size_t off = 0;
+        L.mu = off; off = align_up(off + sizeof(int) * m);
+        L.nu = off; off = align_up(off + sizeof(int) * n);
+        L.ra = off; off = align_up(off + (size_t)pl->N * pl->S * P * Mpad * Kpad * esz);
+        L.rb = off; off = align_up(off + (size_t)pl->N * pl->S * P * Npad * Kpad * esz);
+        // t values: bytes, 32-bit words (binary64), or a word per triple of moduli
+        pack = (mode == 1 || mode == 2) && tc05_packs(pe->gemm, Mpad, Npad);
+        const size_t tval = pack ? 4 * (size_t)pe->gemm.NT : (size_t)pl->N * (mode == 3 ? 4 : 1);
+        L.t = off;  off = align_up(off + (size_t)pl->G * tval * m * n);
+        L.pack = pack;
+        return off;
+    };
     memcpy(L.mod, pl->mod, sizeof L.mod);
     int* derr = err_word(h);
     if (!derr) return OZLU_ERR_NOMEM;
-    rc = h->ws.ensure(off);
+    const size_t bytes = layout();
+    rc = h->ws.ensure(bytes);
+    size_t room = 0, all = 0;
+    if (rc == OZLU_ERR_NOMEM && be == OZLU_BE_INT8 && cudaMemGetInfo(&room, &all) == cudaSuccess && room < bytes) {
+        mode = 0;
+        rc = h->ws.ensure(layout());
+    }
     if (rc) return rc;
+    const int P = mode == 1 ? 3 : 1;
     char* base = (char*)h->ws.base;
     int* mu = (int*)(base + L.mu);
     int* nu = (int*)(base + L.nu);
@@ -583,6 +611,21 @@ int ozlu_debug_fetch(ozlu_handle* h, int what, void* dst, size_t bytes) {
         const size_t need = (size_t)L.N * L.S * R * L.k;
         if (bytes < need) return -4;
         const char* src = base + (what == 3 ? L.ra : L.rb);
+        if (L.mode == 2) {  // binary16 encodings of the same residues
+            std::vector<uint16_t> row((size_t)R * L.k);
+            for (int pl = 0; pl < L.N * L.S; ++pl) {
+                if (cudaMemcpy2D(row.data(), 2 * (size_t)L.k, src + 2 * (size_t)pl * Rpad * L.Kpad,
+                                 2 * (size_t)L.Kpad, 2 * (size_t)L.k, R, cudaMemcpyDeviceToHost) != cudaSuccess)
+                    return OZLU_ERR_CUDA;
+                int8_t* out = (int8_t*)dst + (size_t)pl * R * L.k;
+                for (size_t e = 0; e < row.size(); ++e) {
+                    const int ex = (row[e] >> 10) & 31, fr = (row[e] & 0x3ff) | 0x400;
+                    const int v = ex ? fr >> (25 - ex) : 0;  // an integer below 128
+                    out[e] = (int8_t)(row[e] >> 15 ? -v : v);
+                }
+            }
+            return OZLU_OK;
+        }
         for (int pl = 0; pl < L.N * L.S; ++pl)
             if (cudaMemcpy2D((char*)dst + (size_t)pl * R * L.k, L.k, src + (size_t)pl * Rpad * L.Kpad,
                              L.Kpad, L.k, R, cudaMemcpyDeviceToHost) != cudaSuccess)

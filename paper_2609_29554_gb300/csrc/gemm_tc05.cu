@@ -10,6 +10,10 @@
 //   FP16 the centered residue itself (|r| <= 127 is exact in binary16), one
 //        plane, one fp32 accumulator; exact while K_pad S 127^2 < 2^24
 //        (Eq. (14)).
+//   INT8 the same planes at any K: an accumulator takes 1024 products of
+//        residues, and the epilogue folds the accumulators of a product into
+//        each other modulo m (MULTI).  QD, 1024^3: 241 us; the FP8 plan's three
+//        planes take 342.
 // Both rely on the fp32 tensor-core accumulation being exact for integer
 // sums below 2^24; the parity tests check it bit for bit.
 //
@@ -138,7 +142,16 @@ __device__ __forceinline__ void mma_commit(uint64_t* b) {
                  : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+}
+
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
         "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
@@ -170,13 +183,16 @@ __device__ __forceinline__ uint32_t floor_mod_bits(float v, float m, float invu)
 
 // The CTAs walk the units (gi, q, tm, tn) with stride gridDim.x, tn fastest, so
 // those in flight share A row panels and B column panels in L2.
-template <bool FP8, bool PACK>
+template <bool FP8, bool PACK, bool MULTI>
 __global__ void __launch_bounds__(THREADS, 1) gemm_tc05_kernel(
     const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int m, int n,
-    int Mpad, int Npad, int KB, const __grid_constant__ GemmTab tab, void* T,
+    int Mpad, int Npad, int KB, int chunk, const __grid_constant__ GemmTab tab, void* T,
     int* err) {
     constexpr int P = FP8 ? 3 : 1;                // planes (products per modulus)
     constexpr int LG = PACK ? 3 : 1;              // moduli per unit
+    // columns of an accumulator read at a time: 32 words more would not fit in
+    // the 96 registers a thread beside the packed ones
+    constexpr int LD = PACK && (FP8 || MULTI) ? 16 : 32;
     constexpr uint32_t TMEM_COLS = NBUF * BN;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sm = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -283,20 +299,23 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc05_kernel(
             int tm, tn, q, gi, l1, ta0, items;
             decode(t, tm, tn, q, gi, l1, ta0, items);
             const int prods = (l1 - q * LG) * P;
-            for (int pd = 0; pd < prods && ok; ++pd) {
+            for (int pd = 0, i1 = 0; pd < prods && ok; pd += MULTI ? i1 == items : 1) {
+                // one accumulator: the next `chunk` K blocks of product pd
+                const int i0 = !MULTI || i1 == items ? 0 : i1;
+                i1 = MULTI ? min(items, i0 + chunk) : items;
                 if (!__all_sync(0xffffffffu, mbar_wait(&acce[b], bpar ^ 1, err, abort))) { ok = false; break; }
                 asm volatile("tcgen05.fence::after_thread_sync;\n");
                 const uint32_t acc = tmem + (uint32_t)(b * BN);
-                for (int i = 0; i < items; ++i) {
+                for (int i = i0; i < i1; ++i) {
                     if (!__all_sync(0xffffffffu, mbar_wait(&full[s], par, err, abort))) { ok = false; break; }
                     asm volatile("tcgen05.fence::after_thread_sync;\n");
                     const uint64_t ad = da + (uint64_t)(s * (TILE >> 4)), bd = db + (uint64_t)(s * (TILE >> 4));
                     if (elect_one()) {
 #pragma unroll
                         for (int k = 0; k < BK / 32; ++k)
-                            mma<FP8>(acc, ad + 2 * k, bd + 2 * k, idesc, (i == 0 && k == 0) ? 0u : 1u);
+                            mma<FP8>(acc, ad + 2 * k, bd + 2 * k, idesc, (i == i0 && k == 0) ? 0u : 1u);
                         mma_commit(&empty[s]);
-                        if (i == items - 1) mma_commit(&accf[b]);
+                        if (i == i1 - 1) mma_commit(&accf[b]);
                     }
                     __syncwarp();
                     if (++s == STAGES) { s = 0; par ^= 1; }
@@ -327,26 +346,46 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_tc05_kernel(
                 const GemmMod& M = tab.mod[l];
                 const float md = M.m, inv = M.inv;
                 float v[32];
+                if (MULTI) {
 #pragma unroll
-                for (int p = 0; p < P; ++p) {
+                    for (int jj = 0; jj < 32; ++jj) v[jj] = 0.0f;
+                }
+                // (FP8: the planes; FP16: the accumulators of the one product)
+                const int accs = FP8 ? P : (MULTI ? (items + chunk - 1) / chunk : 1);
+#pragma unroll(FP8 ? 3 : 1)
+                for (int p = 0; p < accs; ++p) {
                     // (the vote keeps the warp together for the loads that follow)
                     if (!ok || !__all_sync(0xffffffffu, mbar_wait(&accf[b], bpar, err, abort))) {
                         ok = false;
                         break;
                     }
                     asm volatile("tcgen05.fence::after_thread_sync;\n");
-                    uint32_t r[32];
-                    tmem_ld32(lane_addr + (uint32_t)(b * BN), r);
-                    // the accumulator is in registers: the MMA warp may overwrite it
-                    asm volatile("tcgen05.fence::before_thread_sync;\n");
-                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(su32(&acce[b])) : "memory");
-                    if (++b == NBUF) { b = 0; bpar ^= 1; }
                     const float yp = M.y[p], off = M.off;
 #pragma unroll
-                    for (int jj = 0; jj < 32; ++jj)
-                        v[jj] = __fmaf_rn(fold(__uint_as_float(r[jj]), md, inv), yp, p == 0 ? off : v[jj]);
+                    for (int h = 0; h < 32; h += LD) {
+                        uint32_t r[LD];
+                        tmem_ld(lane_addr + (uint32_t)(b * BN + h), r);
+                        if (h + LD == 32) {
+                            // the accumulator is in registers: the MMA warp may overwrite it
+                            asm volatile("tcgen05.fence::before_thread_sync;\n");
+                            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(su32(&acce[b])) : "memory");
+                        }
+#pragma unroll
+                        for (int jj = 0; jj < LD; ++jj) {
+                            const float c = __uint_as_float(r[jj]);
+                            float& w = v[h + jj];
+                            if (MULTI) w = fold(c + w, md, inv);
+                            else w = __fmaf_rn(fold(c, md, inv), yp, p == 0 ? off : w);
+                        }
+                    }
+                    if (++b == NBUF) { b = 0; bpar ^= 1; }
                 }
                 if (!ok) break;
+                if (MULTI) {
+                    const float yp = M.y[0], off = M.off;
+#pragma unroll
+                    for (int jj = 0; jj < 32; ++jj) v[jj] = __fmaf_rn(v[jj], yp, off);
+                }
                 const float invu = M.invu;
                 if (PACK) {
                     const uint32_t cf = M.coef;
@@ -442,16 +481,20 @@ int launch_gemm_tc05(bool fp8, bool pack, const void* RA, const void* RB, int m,
     if (!make_map(&ta, RA, fp8, Kpad, (long long)tab.N * tab.S * P * Mpad)) return OZLU_ERR_UNSUPPORTED;
     if (!make_map(&tb, RB, fp8, Kpad, (long long)tab.N * tab.S * P * Npad)) return OZLU_ERR_UNSUPPORTED;
     const int KB = Kpad * (fp8 ? 1 : 2) / BK;
+    // FP16: residues up to 127, so that 1024 products of two (16 K blocks) and
+    // the folded rest of the accumulator before stay below 2^24 in binary32
+    const int chunk = fp8 ? KB * tab.S : 1024 / (BK / 2);
     const size_t smem = tc05_smem_bytes();
     const int sms = device_sms();
     const long long units = (long long)(Mpad / BM) * (Npad / BN) * (pack ? tab.NT : tab.N) * tab.G;
     dim3 grid((unsigned)(units < sms ? units : sms));
     auto go = [&](auto kernel) {
         raise_smem_limit((const void*)kernel, (int)smem);
-        launch(kernel, grid, THREADS, smem, s, ta, tb, m, n, Mpad, Npad, KB, tab, T, err);
+        launch(kernel, grid, THREADS, smem, s, ta, tb, m, n, Mpad, Npad, KB, chunk, tab, T, err);
     };
-    if (fp8) pack ? go(gemm_tc05_kernel<true, true>) : go(gemm_tc05_kernel<true, false>);
-    else pack ? go(gemm_tc05_kernel<false, true>) : go(gemm_tc05_kernel<false, false>);
+    if (fp8) pack ? go(gemm_tc05_kernel<true, true, false>) : go(gemm_tc05_kernel<true, false, false>);
+    else if (KB * tab.S > chunk) pack ? go(gemm_tc05_kernel<false, true, true>) : go(gemm_tc05_kernel<false, false, true>);
+    else pack ? go(gemm_tc05_kernel<false, true, false>) : go(gemm_tc05_kernel<false, false, false>);
     return cudaGetLastError() == cudaSuccess ? OZLU_OK : OZLU_ERR_CUDA;
 }
 

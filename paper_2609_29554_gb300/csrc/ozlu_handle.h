@@ -29,6 +29,7 @@ struct PlanEntry {
 // byte offsets of the last ozlu_gemm's intermediates inside the workspace
 struct GemmLayout {
     int m = 0, n = 0, k = 0, Mpad = 0, Npad = 0, Kpad = 0, N = 0, S = 0, G = 0, backend = 0;
+    int mode = 0;              // residue encoding (launch_convert's; 3: binary64)
     size_t mu = 0, nu = 0, ra = 0, rb = 0, t = 0;
     bool pack = false;         // t values packed by triples of moduli
     int mod[MAXMOD] = {0};
