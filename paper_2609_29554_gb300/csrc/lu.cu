@@ -1389,8 +1389,11 @@ bool base_block_coop(double* A, long long lda, int n, int c0, int b, int* ipiv, 
     constexpr int L = Limbs<N>::L;
     const int sms = device_sms();
     // at least min_rows rows per block: a small panel takes a few SMs and
-    // leaves the rest to concurrent work (the batched driver runs instances
-    // side by side and asks for 32, single factorisations for 16)
+    // leaves the rest to concurrent work.  Fewer rows a block shorten the trailing
+    // updates beside the chain, more leave fewer keys to read: QD n = 1000, 6.59 ms
+    // with 6 rows, 6.61 with 8, 6.91 with 12, 7.40 with 16, 9.7 with 32.  The batched
+    // driver runs instances side by side and asks for 32 (48 uneven TD systems from
+    // CUDA graphs 21.3 ms, with 24 rows 22.2), single factorisations for 8.
     const int g_rows = (n - c0 + min_rows - 1) / min_rows;
     for (int per_sm = 1; per_sm <= 2; ++per_sm) {
         int G = sms * per_sm;
