@@ -115,7 +115,9 @@ __global__ void __launch_bounds__(1024) mp_shift_kernel(MPView A, int m, MPView 
 // kernel (a warp per element, a lane per residue, the table in constant memory
 // read at 32 addresses at once) 3836 us.
 // E = 4 where that leaves two blocks of 256 threads per SM, else E = 1 and the
-// moduli split over gridDim.y (digits formed again in each slice).
+// moduli split over gridDim.y (digits formed again in each slice); that form is
+// bound by the latency of its digits: a column of a 1216-bit LU, 8.4 us with the
+// next digit's words in flight, 10.0 without.
 struct MpConvArgs {
     MPView A, B;
     const int* mu;
@@ -163,19 +165,39 @@ __global__ void __launch_bounds__(256) mp_convert_kernel(const __grid_constant__
     }
     const int l0 = blockIdx.y * a.lper, l1 = min(tab.N, l0 + a.lper);
     const uint32_t mk = (1u << (w - 32 * (NW - 1))) - 1u;  // bits of the digit's last word below w
+    // one element a thread (few elements: bound by latency): the next digit's
+    // words are in flight while this one's residues are formed
+    constexpr bool AHEAD = E == 1;
+    uint32_t nxt[AHEAD ? NW + 1 : 1];
+    auto fetch = [&](int t) {
+        const int q = (t * w + sh[0]) >> 5;
+#pragma unroll
+        for (int i = 0; i < (AHEAD ? NW + 1 : 1); ++i)
+            nxt[i] = live[0] && q + i >= 0 && q + i < L ? *(lp[0] + (long long)(q + i) * X.plane) : 0u;
+    };
+    if (AHEAD) fetch(0);
     for (int t = 0; t < S; ++t) {
-        uint32_t D[E][NW], f[E];
+        uint32_t D[E][NW], f[E], cur[AHEAD ? NW + 1 : 1];
+        if (AHEAD) {
+#pragma unroll
+            for (int i = 0; i < (AHEAD ? NW + 1 : 1); ++i) cur[i] = nxt[i];
+            if (t + 1 < S) fetch(t + 1);
+        }
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             const int pos = t * w + sh[e];
             const int q = pos >> 5, rr = pos & 31;
-            uint32_t v = live[e] && q >= 0 && q < L ? *(lp[e] + (long long)q * X.plane) : 0u;
+            uint32_t v;
+            if (AHEAD) v = cur[0];
+            else v = live[e] && q >= 0 && q < L ? *(lp[e] + (long long)q * X.plane) : 0u;
             uint64_t c = carry[e];
             bool lowzero = true;
 #pragma unroll
             for (int i = 0; i < NW; ++i) {
                 const int qn = q + i + 1;
-                const uint32_t nx = live[e] && qn >= 0 && qn < L ? *(lp[e] + (long long)qn * X.plane) : 0u;
+                uint32_t nx;
+                if (AHEAD) nx = cur[AHEAD ? i + 1 : 0];
+                else nx = live[e] && qn >= 0 && qn < L ? *(lp[e] + (long long)qn * X.plane) : 0u;
                 uint32_t d = __funnelshift_r(v, nx, rr);
                 v = nx;
                 if (i == NW - 1) d &= mk;

@@ -129,7 +129,7 @@ __global__ void mp_laswp_kernel(MPV A, int k0, int k1, const int* ipiv, int j0, 
 
 // Block-cooperative fixed-point arithmetic for the reciprocal of one p-bit
 // number (one block of RT threads, words in shared memory).
-constexpr int RT = 256;
+constexpr int RT = 384;
 
 // warp 0: words w_0, w_1, ... (value(k) below 2^32 + 2^31, k < n) with their
 // carries resolved, 32 at a time: a word generates a carry from 2^32 on and
@@ -162,10 +162,12 @@ __device__ void blk_mul(const uint32_t* X, int nx, const uint32_t* Y, int ny, ui
         unsigned long long acc = 0;
         if (parts == 1 || part < 2) {
             const int i0 = max(0, k - ny + 1), i1 = min(nx - 1, k);
+#pragma unroll 4
             for (int i = i0 + (part & 1); i <= i1; i += step) acc += (uint32_t)((uint64_t)X[i] * Y[k - i]);
         }
         if (parts == 1 || part >= 2) {
             const int j0 = max(0, k - 1 - ny + 1), j1 = min(nx - 1, k - 1);
+#pragma unroll 4
             for (int i = j0 + (part & 1); i <= j1; i += step) acc += (uint64_t)X[i] * Y[k - 1 - i] >> 32;
         }
         S[q] = acc;
@@ -194,7 +196,7 @@ __device__ void blk_mul(const uint32_t* X, int nx, const uint32_t* Y, int ny, ui
 // from a binary64 start; `iters` steps double the 53 correct bits each.  1 / 0
 // is set to 0 (its pivot's column is not scaled, a solve's unknown becomes 0).
 // Latency of one block: with the carries of every product, negation and sum
-// resolved by one warp at a time the 1216-bit reciprocal takes 32 us; by one
+// resolved by one warp at a time the 1216-bit reciprocal takes 25 us; by one
 // thread, word after word, it took 48.
 __global__ void __launch_bounds__(RT) mp_recip_kernel(MPV A, long long x, MPV R, int iters, int parts) {
     chain_enter();
