@@ -97,6 +97,7 @@ int Workspace::ensure(size_t bytes) {
     if (base) cudaFree(base);
     base = nullptr;
     cap = 0;
+    ++moves;
     size_t want = bytes + bytes / 8;
     if (!dev_alloc(&base, want)) {
         if (!dev_alloc(&base, bytes)) {

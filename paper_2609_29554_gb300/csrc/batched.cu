@@ -109,6 +109,14 @@ ozlu_stats sub_counters(ozlu_handle* h) {
     return c;
 }
 
+// how often the workspaces that a captured call uses have moved
+unsigned long long sub_moves(ozlu_handle* h) {
+    unsigned long long m = 0;
+    for (int k = 0; k < NSUB; ++k)
+        if (h->sub[k]) m += h->sub[k]->ws.moves + h->sub[k]->solve_ws.moves;
+    return m;
+}
+
 // eager, capture or replay, keyed by the batch description; a replay adds
 // the counters the captured call recorded, so the statistics count the
 // kernels a replay runs.  The capture runs on a library-owned stream (the
@@ -119,6 +127,12 @@ int run_batched(ozlu_handle* h, const std::vector<long long>& key, bool graph,
     auto issue = [&]() { return issue_on(h->stream); };
     if (!graph) return issue();
     auto g = h->graphs.find(key);
+    if (g != h->graphs.end() && g->second.exec && g->second.moves != sub_moves(h)) {
+        // a larger call has replaced a workspace since: capture again
+        cudaGraphExecDestroy(g->second.exec);
+        h->graphs.erase(g);
+        g = h->graphs.end();
+    }
     if (g != h->graphs.end()) {
         if (!g->second.exec) {  // capture failed before: stay eager
             h->stats.graph_status = g->second.status;
@@ -145,7 +159,7 @@ int run_batched(ozlu_handle* h, const std::vector<long long>& key, bool graph,
     }
     auto fail = [&](cudaError_t e) -> int {
         cudaGetLastError();
-        h->graphs[key] = {nullptr, {}, -(int)e};
+        h->graphs[key] = {nullptr, {}, -(int)e, 0};
         h->stats.graph_status = -(int)e;
         return issue();
     };
@@ -179,7 +193,7 @@ int run_batched(ozlu_handle* h, const std::vector<long long>& key, bool graph,
     const cudaError_t ie = cudaGraphInstantiate(&ex, gr, 0);
     cudaGraphDestroy(gr);
     if (ie != cudaSuccess) return fail(ie);
-    h->graphs[key] = {ex, work, 1};
+    h->graphs[key] = {ex, work, 1, sub_moves(h)};
     h->stats.graph_status = 1;
     return cudaGraphLaunch(ex, h->stream) == cudaSuccess ? OZLU_OK : OZLU_ERR_CUDA;
 }

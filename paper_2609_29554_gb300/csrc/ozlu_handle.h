@@ -14,6 +14,7 @@ namespace ozlu {
 struct Workspace {
     void* base = nullptr;
     size_t cap = 0;
+    unsigned long long moves = 0;  // times the buffer has been replaced
     int ensure(size_t bytes);
     void release();
 };
@@ -79,6 +80,7 @@ struct ozlu_handle {
         cudaGraphExec_t exec;  // null: capture failed, the batch runs eagerly
         ozlu_stats work;       // counters of the captured call, added on each replay
         int status;            // graph_status of ozlu_stats
+        unsigned long long moves = 0;  // of the sub-handles' workspaces, whose addresses it holds
     };
     std::map<std::vector<long long>, Graph> graphs;
     std::map<std::vector<long long>, int> warm;
