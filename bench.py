@@ -496,11 +496,11 @@ def roofline(st, a, peaks, src, fms=None, steps=None):
     L = {2: 4, 3: 6, 4: 7}[nc]
     if dom == "gemm":
         achieved = st.gemm_ops / (st.gemm_ms * 1e-3) / 1e12
-        peak = {"int8": IMMA_PEAK, "fp8": 2 * peaks["bf16_tflops"], "fp16": peaks["bf16_tflops"],
-                "fp64": 1.0}[be]
-        r = {"kernel": {"int8": "gemm_imma_kernel", "fp64": "gemm_f64_kernel"}.get(be, "gemm_tc05_kernel"),
+        # (INT8 plans run as binary16 products)
+        peak = {"fp8": 2 * peaks["bf16_tflops"], "fp64": 1.0}.get(be, peaks["bf16_tflops"])
+        r = {"kernel": "gemm_f64_kernel" if be == "fp64" else "gemm_tc05_kernel",
              "bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-             "peak_source": src if be in ("fp8", "fp16") else "own probe"}
+             "peak_source": src if be != "fp64" else "own probe"}
     elif dom == "convert":
         achieved = st.convert_bytes / (st.convert_ms * 1e-3) / 1e9
         r = {"kernel": "convert_kernel", "bound": "hbm", "achieved": achieved,
