@@ -131,7 +131,7 @@ struct MpConvArgs {
     int lper;      // moduli per gridDim.y slice
 };
 
-template <int NW, bool FP8, int E>
+template <int NW, int MODE, int E>
 __global__ void __launch_bounds__(256) mp_convert_kernel(const __grid_constant__ MpConvArgs a,
                                                          const __grid_constant__ ConvTab tab) {
     chain_enter();
@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(256) mp_convert_kernel(const __grid_constant__
             uint32_t res[E];
 #pragma unroll
             for (int e = 0; e < E; ++e) res[e] = conv_residue<NW>(D[e], M, __dp4a(f[e], M.k4, M.half));
-            store_residues<FP8 ? 1 : 0, E>(is_b ? a.RB : a.RA, (size_t)(l * S + t), plane, off, M, res);
+            store_residues<MODE, E>(is_b ? a.RB : a.RA, (size_t)(l * S + t), plane, off, M, res);
         }
     }
 }
@@ -861,7 +861,7 @@ __global__ void __launch_bounds__(32 * CWC) mp_crt_warp_kernel(const __grid_cons
     }
 }
 
-template <int NW, bool FP8>
+template <int NW, int MODE>
 void convert_nw(MpConvArgs a, const ConvTab& t, cudaStream_t s) {
     const int sms = device_sms();
     auto blocks = [&](int R, int E) {
@@ -875,7 +875,7 @@ void convert_nw(MpConvArgs a, const ConvTab& t, cudaStream_t s) {
     if (a.Kp % 4 == 0 && ((long long)a.m + a.n) * a.Kp >= 4ll * 512 * sms) {
         a.blocks_a = blocks(a.m, 4);
         a.lper = t.N;
-        launch(mp_convert_kernel<NW, FP8, 4>, a.blocks_a + blocks(a.n, 4), 256, 0, s, a, t);
+        launch(mp_convert_kernel<NW, MODE, 4>, a.blocks_a + blocks(a.n, 4), 256, 0, s, a, t);
         return;
     }
     a.blocks_a = blocks(a.m, 1);
@@ -885,19 +885,20 @@ void convert_nw(MpConvArgs a, const ConvTab& t, cudaStream_t s) {
     if (split > 16) split = 16;
     if (split > t.N) split = t.N;
     a.lper = (t.N + split - 1) / split;
-    launch(mp_convert_kernel<NW, FP8, 1>, dim3(nb, (t.N + a.lper - 1) / a.lper), 256, 0, s, a, t);
+    launch(mp_convert_kernel<NW, MODE, 1>, dim3(nb, (t.N + a.lper - 1) / a.lper), 256, 0, s, a, t);
 }
 
 // rows [0, m) of A's planes and [0, n) of B's (padded rows reach discarded
 // outputs), zeros in the K padding; m = 0: B alone
 void mp_convert(const MPView& A, int m, const MPView& B, int n, int K, const int* mu, const int* nu, const ConvTab& t,
-                int Kp, int Mpad, int Npad, int8_t* RA, int8_t* RB, bool fp8, cudaStream_t s) {
+                int Kp, int Mpad, int Npad, int8_t* RA, int8_t* RB, int mode, cudaStream_t s) {
     const MpConvArgs a{A, B, mu, nu, RA, RB, m, n, K, Kp, Mpad, Npad, 0, 0, 0, 0};
     switch (t.NW) {
 #define OZ_N(NN)                                                                       \
     case NN:                                                                           \
-        if (fp8) convert_nw<NN, true>(a, t, s);                                        \
-        else convert_nw<NN, false>(a, t, s);                                           \
+        if (mode == 0) convert_nw<NN, 0>(a, t, s);                                     \
+        else if (mode == 1) convert_nw<NN, 1>(a, t, s);                                \
+        else convert_nw<NN, 2>(a, t, s);                                               \
         break;
         OZ_N(1) OZ_N(2) OZ_N(3) OZ_N(4) OZ_N(5) OZ_N(6) OZ_N(7) OZ_N(8)
 #undef OZ_N
@@ -950,6 +951,7 @@ int mp_plan_for(ozlu_handle* h, int p, int K, const PlanEntry** out) {
         fill_conv(e.table, e.conv);
         fill_crt(e.table, e.plan.pint_bits, e.crt);
         fill_gemm(e.table, true, e.gemm);
+        fill_gemm(e.table, false, e.gemm16);
         it = h->plans.emplace(key, e).first;
     }
     *out = &it->second;
@@ -1073,7 +1075,7 @@ int mp_gemm_ext(ozlu_handle* h, int p, int S, int m, int n, int k, int alpha, co
 int mp_gemm_device(ozlu_handle* h, int p, int m, int n, int k, int alpha, const ozlu_mp_matrix& A,
                    const ozlu_mp_matrix& B, int beta, const ozlu_mp_matrix& C);
 
-// INT8 (mma.sync) or FP8 (tcgen05) residues for a wide p-bit product, by
+// INT8 (as binary16 products) or FP8 residues for a wide p-bit product, by
 // measurement: both run the same plan (identical results) into a scratch C,
 // once untimed and once timed; the faster is cached per (p, k, log2 m, log2 n)
 int mp_tune_backend(ozlu_handle* h, int p, int m, int n, int k, const ozlu_mp_matrix& A, const ozlu_mp_matrix& B,
@@ -1154,36 +1156,52 @@ int mp_gemm_device(ozlu_handle* h, int p, int m, int n, int k, int alpha, const 
     // n <= 16: 128 x 16 tiles and B planes of 16 rows
     const bool narrow = n <= 16;
     const MPView vA = view_of(A, 0), vB = view_of(B, 0), vC = view_of(C, 0);
-    // FP8 (balanced base-17 digits on tcgen05, three planes per residue, the
-    // same plan and so the same results) for wide products when chosen and
-    // admissible: fp32 accumulations below 2^24
+    // FP8 (balanced base-17 digits, three planes per residue, the same plan and so
+    // the same results) for wide products when chosen and admissible: fp32
+    // accumulations below 2^24
     int be = h->mp_opts.backend;
     const int kp128 = (k + 127) / 128 * 128;
     const bool fp8_ok = !smallk && !narrow && (double)kp128 * pl->S * 225.0 < ldexp(1.0, 24);
     if (be == OZLU_BE_AUTO && fp8_ok) {
         if ((rc = mp_tune_backend(h, p, m, n, k, A, B, &be))) return rc;
     }
-    const bool fp8 = be == OZLU_BE_FP8 && fp8_ok;
-    const int P = fp8 ? 3 : 1;
-    const int Kpad = smallk ? k : (fp8 ? kp128 : (k + 63) / 64 * 64), Mpad = smallk ? m : (m + 127) / 128 * 128;
-    const size_t planesN = (size_t)pl->N * pl->S * P;
+    // residue encoding (store_residues): FP8 digits; INT8 as binary16 for wide
+    // products, as ozlu_gemm does (512 x 512 x 512 at 1024 bits: 752 us, by the FP8
+    // plan's three planes 940), int8 for the others and where the larger planes do
+    // not fit
+    int mode = be == OZLU_BE_FP8 && fp8_ok ? 1 : (smallk || narrow ? 0 : 2);
+    const int P = mode == 1 ? 3 : 1;
+    const int Kpad = smallk ? k : (mode == 1 ? kp128 : (k + 63) / 64 * 64), Mpad = smallk ? m : (m + 127) / 128 * 128;
     const int rowq = smallk ? 1 : (narrow ? 16 : 128);
-    // column chunk: t values of one chunk below 4 GiB and B planes below 2 GiB
     const size_t tcol = (size_t)pl->G * pl->N * m;
-    long long nch = (long long)(((size_t)4 << 30) / (tcol ? tcol : 1));
-    const long long bcap = (long long)(((size_t)2 << 30) / (planesN * Kpad)) / 128 * 128;
-    if (nch > bcap) nch = bcap;
-    nch = nch / 128 * 128;
-    if (nch < 128) nch = 128;
-    if (nch > n) nch = n;
-    const int Ncpad = (int)((nch + rowq - 1) / rowq * rowq);
-    size_t off = 0;
-    const size_t o_mu = off; off = up256(off + sizeof(int) * (size_t)m);
-    const size_t o_nu = off; off = up256(off + sizeof(int) * (size_t)n);
-    const size_t o_ra = off; off = up256(off + planesN * Mpad * Kpad);
-    const size_t o_rb = off; off = up256(off + planesN * (size_t)Ncpad * Kpad);
-    const size_t o_t = off;  off = up256(off + tcol * (size_t)nch);
-    if ((rc = h->ws.ensure(off))) return rc;
+    long long nch = 0;
+    size_t o_mu = 0, o_nu = 0, o_ra = 0, o_rb = 0, o_t = 0;
+    auto layout = [&]() -> size_t {
+        const size_t planesN = (size_t)pl->N * pl->S * P * (mode == 2 ? 2 : 1);  // in bytes an element
+        // column chunk: t values of one chunk below 4 GiB and B planes below 2 GiB
+        nch = (long long)(((size_t)4 << 30) / (tcol ? tcol : 1));
+        const long long bcap = (long long)(((size_t)2 << 30) / (planesN * Kpad)) / 128 * 128;
+        if (nch > bcap) nch = bcap;
+        nch = nch / 128 * 128;
+        if (nch < 128) nch = 128;
+        if (nch > n) nch = n;
+        const int Ncpad = (int)((nch + rowq - 1) / rowq * rowq);
+        size_t off = 0;
+        o_mu = off; off = up256(off + sizeof(int) * (size_t)m);
+        o_nu = off; off = up256(off + sizeof(int) * (size_t)n);
+        o_ra = off; off = up256(off + planesN * Mpad * Kpad);
+        o_rb = off; off = up256(off + planesN * (size_t)Ncpad * Kpad);
+        o_t = off;  off = up256(off + tcol * (size_t)nch);
+        return off;
+    };
+    const size_t bytes = layout();
+    rc = h->ws.ensure(bytes);
+    size_t room = 0, all = 0;
+    if (rc == OZLU_ERR_NOMEM && mode == 2 && cudaMemGetInfo(&room, &all) == cudaSuccess && room < bytes) {
+        mode = 0;
+        rc = h->ws.ensure(layout());
+    }
+    if (rc) return rc;
     char* base = (char*)h->ws.base;
     int* mu = (int*)(base + o_mu);
     int* nu = (int*)(base + o_nu);
@@ -1192,13 +1210,13 @@ int mp_gemm_device(ozlu_handle* h, int p, int m, int n, int k, int alpha, const 
     uint8_t* T = (uint8_t*)(base + o_t);
     const int NW = mp_window_words(*pl);
     int* derr = nullptr;
-    if (fp8 && !(derr = err_word(h))) return OZLU_ERR_NOMEM;
+    if (mode && !(derr = err_word(h))) return OZLU_ERR_NOMEM;
     const int prev = h->open_phase;
     h->phase(PH_CONVERT);
     {
         const int nc0 = (int)(n < nch ? n : nch), ba = (m + 31) / 32, bb = (n + 31) / 32;
         launch(mp_shift_kernel, ba + bb, 1024, 0, s, vA, m, vB, n, k, pl->Q, mu, nu, ba);
-        mp_convert(vA, m, vB, nc0, k, mu, nu, pe->conv, Kpad, Mpad, (nc0 + rowq - 1) / rowq * rowq, RA, RB, fp8, s);
+        mp_convert(vA, m, vB, nc0, k, mu, nu, pe->conv, Kpad, Mpad, (nc0 + rowq - 1) / rowq * rowq, RA, RB, mode, s);
     }
     h->count(2);
     for (long long j0 = 0; j0 < n; j0 += nch) {
@@ -1206,12 +1224,14 @@ int mp_gemm_device(ozlu_handle* h, int p, int m, int n, int k, int alpha, const 
         const int ncp = (nc + rowq - 1) / rowq * rowq;
         h->phase(PH_CONVERT);
         if (j0 > 0) {
-            mp_convert(vA, 0, view_of(B, j0 * B.ld), nc, k, mu, nu + j0, pe->conv, Kpad, Mpad, ncp, RA, RB, fp8, s);
+            mp_convert(vA, 0, view_of(B, j0 * B.ld), nc, k, mu, nu + j0, pe->conv, Kpad, Mpad, ncp, RA, RB, mode, s);
             h->count(1);
         }
         h->phase(PH_GEMM);
-        if (fp8) {
-            if ((rc = launch_gemm_tc05(true, false, RA, RB, m, nc, Mpad, ncp, Kpad, pe->gemm, T, derr, s))) return rc;
+        if (mode) {
+            if ((rc = launch_gemm_tc05(mode == 1, false, RA, RB, m, nc, Mpad, ncp, Kpad,
+                                       mode == 1 ? pe->gemm : pe->gemm16, T, derr, s)))
+                return rc;
         } else if (smallk) {
             const long long work = (long long)m * nc * pl->N * pl->G;
             launch(small_k_gemm_kernel, (unsigned)((work + 255) / 256), 256, 0, s, RA, RB, m, nc, k, *tab, T);
@@ -1226,7 +1246,7 @@ int mp_gemm_device(ozlu_handle* h, int p, int m, int n, int k, int alpha, const 
         h->stats.gemm_launches += 1;
         h->stats.crt_launches += 1;
         h->stats.gemm_ops += 2.0 * m * nc * (double)k * pl->N * pl->pair_terms * P;
-        h->stats.last_backend = fp8 ? OZLU_BE_FP8 : OZLU_BE_INT8;
+        h->stats.last_backend = mode == 1 ? OZLU_BE_FP8 : OZLU_BE_INT8;
     }
     h->phase(prev);
     return cudaGetLastError() == cudaSuccess ? OZLU_OK : OZLU_ERR_CUDA;

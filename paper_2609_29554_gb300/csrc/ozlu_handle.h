@@ -25,6 +25,7 @@ struct PlanEntry {
     ConvTab conv;
     CrtTab crt;
     GemmTab gemm;  // tensor-core epilogue
+    GemmTab gemm16;  // p-bit plans: of binary16 products (gemm: of FP8 ones)
 };
 
 // byte offsets of the last ozlu_gemm's intermediates inside the workspace

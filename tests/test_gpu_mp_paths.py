@@ -43,6 +43,7 @@ def _norm(pair, L):
 @pytest.mark.parametrize("m,n,k,p,beta", [
     (160, 161, 1000, 100, 0), (161, 160, 1021, 200, 1),     # four elements a thread
     (5, 6, 33, 31, 1), (4, 3, 9, 320, 1), (3, 4, 8, 700, 1), (2, 3, 7, 1216, 1), (1, 2, 1, 2000, 0),
+    (20, 17, 300, 700, 1), (3, 18, 65, 1216, 0),            # wide: accumulators folded
     (128, 128, 4, 150, 1), (127, 129, 4, 150, 1)])          # a thread and a warp per output
 def test_conversion_and_crt_forms(m, n, k, p, beta):
     rng = random.Random(m * 1000 + p)
