@@ -249,7 +249,7 @@ extern "C" int ozlu_getrf_batched(ozlu_handle* h, int nc, int p, int count, cons
     }
     const auto lists = assign(count, n);
     // concurrent instances take fewer SMs per panel (32 rows per block at least;
-    // 256 TD instances: 576 ms against 643 ms with 16); a single instance keeps 16
+    // 256 TD instances: 576 ms against 643 ms with 16); a single instance keeps 8
     for (int k = 0; k < NSUB; ++k) h->sub[k]->coop_min_rows = count > 1 ? 32 : 8;
     auto issue = [&](cudaStream_t root) -> int {
         return fork_join(h, root, lists, [&](ozlu_handle* s, int i) -> int {

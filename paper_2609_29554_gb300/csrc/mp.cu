@@ -643,10 +643,7 @@ void zero_k_padding(int8_t* planes, long long count, int R, int Rpad, int Kc, in
 // one thread (about 20 us for 80 words).
 constexpr int CWC = 4;  // warps per block
 // outputs below which a warp takes each (above, a thread each: mp_crt_kernel)
-#ifndef MP_WARP_CRT_N
-#define MP_WARP_CRT_N 16384
-#endif
-constexpr long long MP_WARP_CRT = MP_WARP_CRT_N;
+constexpr long long MP_WARP_CRT = 16384;
 
 struct MpCrtArgs {
     const uint8_t* T;

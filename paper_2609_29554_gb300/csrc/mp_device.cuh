@@ -114,19 +114,6 @@ __device__ __forceinline__ uint32_t bit_at(const uint32_t (&X)[W], int pos) {
     return v;
 }
 
-// any bit set below position pos
-template <int W>
-__device__ __forceinline__ bool any_below(const uint32_t (&X)[W], int pos) {
-    bool any = false;
-#pragma unroll
-    for (int wd = 0; wd < W; ++wd) {
-        const int lo = 32 * wd;
-        if (pos >= lo + 32) any |= X[wd] != 0;
-        else if (pos > lo) any |= (X[wd] & ((1u << (pos - lo)) - 1u)) != 0;
-    }
-    return any;
-}
-
 // keep only the bits below position pos
 template <int W>
 __device__ __forceinline__ void mask_below(uint32_t (&X)[W], int pos) {

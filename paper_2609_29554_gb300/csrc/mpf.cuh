@@ -365,11 +365,6 @@ __device__ __forceinline__ MPF<L> mpf_add(const MPF<L>& a, const MPF<L>& b) {
     return mpf_round<L, W>(X, x.e, x.neg, sticky);
 }
 
-template <int L>
-__device__ __forceinline__ MPF<L> mpf_sub(const MPF<L>& a, const MPF<L>& b) {
-    return mpf_add<L>(a, mpf_neg<L>(b));
-}
-
 // c - a b with one rounding: the product's top L + 2 words (from the columns
 // that reach them and one guard column; what is left out is under 2^-28 of
 // the lowest window word) meet c in an (L + 2)-word window, the lower words
@@ -465,11 +460,6 @@ __device__ __forceinline__ MPF<L> mpf_fms(const MPF<L>& c, const MPF<L>& a, cons
 template <int L>
 __device__ __noinline__ MPF<L> mpf_fms_oolv(MPF<L> c, MPF<L> a, MPF<L> b) {
     return mpf_fms<L>(c, a, b);
-}
-
-template <int L>
-__device__ __noinline__ void mpf_mul_ool(MPF<L>* out, const MPF<L>* a, const MPF<L>* b) {
-    *out = mpf_mul<L>(*a, *b);
 }
 
 template <int L>
