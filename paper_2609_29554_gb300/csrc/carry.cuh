@@ -32,7 +32,7 @@ OZ_CHAIN3(mad_hi_next, "madc.hi.cc.u32")   // high word of a b, plus c and the f
 #undef OZ_CHAIN
 #undef OZ_CHAIN3
 #else
-static uint32_t oz_carry_flag;
+static thread_local uint32_t oz_carry_flag;
 __device__ __forceinline__ uint32_t oz_chain(uint64_t s) {
     oz_carry_flag = (uint32_t)(s >> 32);
     return (uint32_t)s;

@@ -267,6 +267,8 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) base_block_coop_kernel(
     constexpr int T = COOP_THREADS;
     constexpr int BAR_PIVOT = 1;  // warps 0 .. 3: the pivot's slot is known
     constexpr int BAR_COL = 2;    // column kc + 2 is updated (warp 0 waits, the others arrive)
+    constexpr int BAR_ROWS = 3;   // the pair of rows is published (warps 1 .. 3 wait, its publishers arrive)
+    constexpr int ROWS_T = (3 + 8) * 32;
     extern __shared__ __align__(16) unsigned char smraw[];
     MPF<L>* a = reinterpret_cast<MPF<L>*>(smraw);  // [r][k], r < rows_per_block, k < b
     // rows padded to b + 1 entries: threads on consecutive rows of one column
@@ -350,7 +352,10 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) base_block_coop_kernel(
     // four warps each for the candidate row (pub 0 .. 3) and, in its owner, row
     // c0 + kc + 1 (pub 4 .. 7): update it by column kc (kc < 0 or zero: no update)
     // and publish it for column kc + 1.  None of them shares warp 0's scheduler,
-    // where the reciprocal runs at the same time.
+    // where the reciprocal runs at the same time.  They read and write the two rows
+    // in shared memory, which the next column's multipliers and interchange write
+    // too: those wait for them at BAR_ROWS (a word in the exchange says that its own
+    // element is done, not that the row's multiplier has been read by all).
     const int pub = (warp & 3) == 0 || warp < 5 || warp > 14 ? -1 : (warp - 5) - ((warp - 5) >> 2);
     auto publish_rows = [&](int kc, bool zero, int pa, int pb) {
         const unsigned long long tag = (unsigned long long)(unsigned)(c0 + kc + 2) << 32;
@@ -384,7 +389,10 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) base_block_coop_kernel(
     if (warp == 0) {
         publish_rec(cand, 0);
     } else {
-        if (pub >= 0) publish_rows(-1, true, s_cand >= 0 ? s_cand - r0 : -1, owns(c0) ? c0 - r0 : -1);
+        if (pub >= 0) {
+            publish_rows(-1, true, s_cand >= 0 ? s_cand - r0 : -1, owns(c0) ? c0 - r0 : -1);
+            bar_arrive(BAR_ROWS, ROWS_T);
+        }
         bar_arrive(BAR_COL, T);
     }
 
@@ -556,6 +564,7 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) base_block_coop_kernel(
                         if (zero && *info == 0) *info = c + 1;
                     }
                 }
+                bar_sync(BAR_ROWS, ROWS_T);
                 if (!zero)
                     for (int r = lane; r < nr; r += 32)
                         if (r >= lo) a[r * bs + kc] = mpf_mul<L>(piv != c && r0 + r == piv ? ox : a[r * bs + kc], rec);
@@ -575,6 +584,7 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) base_block_coop_kernel(
                 bool ok = wait_words<H * WORDS + 2>(p, tag, v, err);
                 const int piv = ok ? (int)v[H * WORDS] : c;
                 const bool swap = v[H * WORDS + 1] != 0 && piv != c;
+                bar_sync(BAR_ROWS, ROWS_T);
 #pragma unroll
                 for (int h = 0; h < H; ++h) {
                     const int k = k0 + 64 * h;
@@ -633,6 +643,7 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) base_block_coop_kernel(
         } else {
             if (pub >= 0) {
                 publish_rows(kc, zero, pa, pb);
+                bar_arrive(BAR_ROWS, ROWS_T);
             } else if (warp == 1 && !zero && kc + 2 < b) {
                 for (int r = lo + lane; r < nr; r += 32)
                     if (r != pa && r != pb)
