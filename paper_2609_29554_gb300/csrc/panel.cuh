@@ -34,9 +34,12 @@ __device__ __forceinline__ double* elem(double* A, long long lda, int nc, long l
 //   warps 4 ..  the trailing update of the last column, then the two rows other
 //               blocks may need from this one (its candidate and the row the
 //               pivot will replace), published as they are formed.
-// The next column is updated as y - (x u) / p with x u formed while the
-// reciprocal is on its way (one rounding more of 2^-(32 L), 32 L >= 53 nc + 12);
-// the multipliers x / p are off the chain.
+// The next column is updated as y - l u with the multiplier l = x (1 / p) that is
+// stored, one rounding like every other element; l is formed again on warp 0 when
+// the reciprocal arrives.  (y - (x u) (1 / p), with x u ready by then, is a product
+// shorter on the chain, QD n = 1000 / 4096 6.63 / 50.7 ms against 6.68 / 50.9, but
+// rounds both factors: backward error of the n = 4096 LU at cond 1e40, sampled,
+// 1.74e-66 against 1.39e-66.)
 //
 // Blocks exchange 64-bit words whose upper half is a tag (the column) and whose
 // lower half is data, so that a word announces itself: readers poll the words
@@ -503,13 +506,9 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) base_block_coop_kernel(
             const int piv = ok ? (int)w[0] : c;
             const MPF<L> u = mpf_gather<L>(w[1]), ox = mpf_gather<L>(w[2]), oy = mpf_gather<L>(w[3]);
             const bool swapped = piv != c && owns(piv);
-            MPF<L> s[Q];
 #pragma unroll
-            for (int q = 0; q < Q; ++q) {
+            for (int q = 0; q < Q; ++q)
                 if (swapped && lane + 32 * q == piv - r0) x[q] = ox;
-                s[q] = mpf_make_zero<L>();
-                if (32 * q < nr) s[q] = mpf_mul<L>(x[q], u);
-            }
             __syncwarp();
             {
                 const unsigned long long* p[1] = {word ? &ws.rec[word ? lane : 0] : nullptr};
@@ -517,6 +516,11 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) base_block_coop_kernel(
             }
             const MPF<L> rec = mpf_gather<L>(wr[0]);
             const bool zero = mpf_zero<L>(rec);
+            if (!last) {  // the multipliers
+#pragma unroll
+                for (int q = 0; q < Q; ++q)
+                    if (32 * q < nr) x[q] = mpf_mul<L>(x[q], rec);
+            }
             bar_sync(BAR_COL, T);  // column kc + 1 carries the updates up to kc - 1
             if (lane == 0) {
                 s_zero = zero ? 1 : 0;
@@ -537,7 +541,7 @@ __global__ void __launch_bounds__(COOP_THREADS, 1) base_block_coop_kernel(
                     y[q].e = from ? oy.e : old.e;
                     y[q].neg = from ? oy.neg : old.neg;
                     if (!zero) {
-                        y[q] = mpf_fms<L>(y[q], s[q], rec);
+                        y[q] = mpf_fms<L>(y[q], x[q], u);
                         if (r >= lo && r < nr) a[r * bs + kc + 1] = y[q];
                     }
                 }

@@ -6,7 +6,8 @@
 // N components, n rows, b columns, `rows` rows a block; order "even" lets the warps
 // go on in turn, "late" holds one warp after another back as long as possible
 // (the seed says which order of preference), "mixed" draws a new preference every
-// few steps.  Prints the interchanges, info and the factored panel's words.
+// few steps; "plain" is no run of the kernel but the same factorisation as a plain
+// loop, one element after another.  Prints the interchanges, info and the factored panel's words.
 #include "cuda_host.h"
 
 #include <algorithm>
@@ -42,6 +43,33 @@ static host::Order make_order(const std::string& kind, uint64_t seed, int warps)
     };
 }
 
+// columns in turn: the pivot (lowest row on ties), the multipliers x (1 / p), every
+// other element y - l u; each operation rounded to L words
+template <int N>
+static void plain(double* A, int n, int b, int* ipiv, int* info) {
+    constexpr int L = Limbs<N>::L;
+    std::vector<MPF<L>> a((size_t)n * b);
+    for (size_t e = 0; e < a.size(); ++e) a[e] = mpf_from_exp<L, N>(A + e * N);
+    auto at = [&](int i, int j) -> MPF<L>& { return a[(size_t)j * n + i]; };
+    for (int c = 0; c < b; ++c) {
+        int p = c;
+        for (int i = c + 1; i < n; ++i)
+            if (mpf_abs_cmp<L>(at(i, c), at(p, c)) > 0) p = i;
+        ipiv[c] = p + 1;
+        if (mpf_zero<L>(at(p, c))) {
+            if (*info == 0) *info = c + 1;
+            continue;
+        }
+        for (int k = 0; k < b; ++k) std::swap(at(c, k), at(p, k));
+        const MPF<L> r = mpf_recip<L>(at(c, c));
+        for (int i = c + 1; i < n; ++i) {
+            at(i, c) = mpf_mul<L>(at(i, c), r);
+            for (int k = c + 1; k < b; ++k) at(i, k) = mpf_fms<L>(at(i, k), at(i, c), at(c, k));
+        }
+    }
+    for (size_t e = 0; e < a.size(); ++e) mpf_to_exp<L, N>(a[e], A + e * N);
+}
+
 template <int N>
 static void go(int n, int b, int rows, const std::string& order, uint64_t seed) {
     constexpr int L = Limbs<N>::L;
@@ -65,7 +93,8 @@ static void go(int n, int b, int rows, const std::string& order, uint64_t seed) 
     auto* sc = new CoopScratch<L>();
     memset((void*)sc, 0, sizeof *sc);
     std::vector<std::thread> blocks;
-    for (int k = 0; k < G; ++k)
+    if (order == "plain") plain<N>(A.data(), n, b, ipiv.data(), &info);
+    for (int k = 0; k < G && order != "plain"; ++k)
         blocks.emplace_back([&, k] {
             blockIdx.x = (unsigned)k;
             gridDim.x = (unsigned)G;

@@ -7,6 +7,7 @@ barriers and exchanged words leave open is thereby taken to its extremes; the
 interchanges and every word of the factored panel must not depend on it, nor on how
 the rows are spread over blocks.
 """
+import hashlib
 import os
 import shutil
 import subprocess
@@ -30,7 +31,8 @@ def panel(tmp_path_factory):
     def run(nc, n, b, rows, order, seed):
         r = subprocess.run([exe, str(nc), str(n), str(b), str(rows), order, str(seed)], check=True,
                            capture_output=True, text=True, timeout=120)
-        return r.stdout
+        head, pivots, words = r.stdout.splitlines()
+        return head, pivots, hashlib.sha256(words.encode()).hexdigest()
     return run
 
 
@@ -42,7 +44,7 @@ def panel(tmp_path_factory):
 ])
 def test_result_does_not_depend_on_the_order_of_the_warps(panel, nc, n, b, rows):
     want = panel(nc, n, b, rows, "even", 0)
-    assert want.startswith("error 0 info 0\n")
+    assert want[0] == "error 0 info 0"
     for seed in range(1, 9):
         for order in ("late", "mixed"):
             assert panel(nc, n, b, rows, order, seed) == want, (order, seed)
@@ -52,3 +54,9 @@ def test_result_does_not_depend_on_the_rows_a_block(panel):
     want = panel(2, 128, 128, 128, "even", 0)
     for rows in (8, 24, 64):
         assert panel(2, 128, 128, rows, "late", rows) == want, rows
+
+
+@pytest.mark.parametrize("nc,n,b,rows", [(2, 100, 100, 50), (3, 65, 65, 33), (4, 90, 77, 30), (4, 64, 64, 64)])
+def test_the_panel_is_the_plain_factorisation(panel, nc, n, b, rows):
+    # every element one rounding of y - l u with the multiplier that is stored
+    assert panel(nc, n, b, rows, "mixed", 3) == panel(nc, n, b, rows, "plain", 0)
