@@ -543,11 +543,11 @@ __device__ __forceinline__ MPF<4> mpf_recip_seed(uint64_t T) {
 }
 
 // 1 / f for f = F 2^(-32 L) in (1/2, 1), L <= 7, in fixed point: R words with
-// r = R 2^(1 - 32 (L + 1)) in (1, 2), r <= 1 / f, 1 - f r < 2^-(32 L + 4) or
-// 2^-238, whichever is larger.  Newton steps r <- r + r e, e = 1 - f r, whose
-// result (1 - e^2) / f stays below 1 / f; each uses only the words of f and of e
-// that its precision needs, so that the alignments are fixed and nothing is
-// normalised.  On values:
+// r = R 2^(1 - 32 (L + 1)) in (1, 2), r < 1 / f, 1 - f r < 2^-(32 L + 28).
+// Newton steps r <- r + r e, e = 1 - f r, whose result (1 - e^2) / f stays below
+// 1 / f (with the e^2 of the last one added, L = 7, (1 - e^3) / f); each uses only
+// the words of f and of e that its precision needs, so that the alignments are
+// fixed and nothing is normalised.  On values:
 //   r0  binary32 reciprocal of the top 24 bits plus one       e < 2^-21
 //   r1  32-bit f (plus one unit), one step in 64 bits          e < 2^-30
 //   r2  64-bit f (plus one unit), one step                     e < 2^-59
@@ -606,6 +606,14 @@ __device__ __forceinline__ void recip_words(const uint32_t (&F)[L], uint32_t (&R
     for (int i = 1; i < L + 1 - NE; ++i) add_next(~P4[i], 0u);
 #pragma unroll
     for (int i = 0; i < NE; ++i) E4[i] = add_next(~P4[L + 1 - NE + i], 0u);
+    if (L >= 7) {
+        // the step's third-order term e^2 (2^-234 at most, below the words kept for
+        // L <= 6): e = t 2^-147 from the top 32 bits, e^2 in units of E4's word 0
+        const uint32_t t = __funnelshift_r(E4[NE - 2], E4[NE - 1], 12);
+        E4[0] = add_first(E4[0], __umulhi(t, t) >> (L >= 7 ? 231 - 32 * L : 0));
+#pragma unroll
+        for (int i = 1; i < NE; ++i) E4[i] = add_next(E4[i], 0u);
+    }
     mul_words<NE, 4, 0>(E4, R3, Q);
     // r 2^(32 L + 31) = R3 2^(32 L - 96) + R3 E4 2^-223, E4 here without its low
     // L + 1 - NE = 3 words: (R3 E4) 2^-127, words from bit 127 on
