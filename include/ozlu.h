@@ -357,6 +357,10 @@ int ozlu_mp_getrs(ozlu_handle* handle, int p, int n, int nrhs, const ozlu_mp_mat
  * the calls that needed them return OZLU_ERR_NOMEM; 0 turns it off.  The
  * counter is process-wide.  Returns 0, or -1 for count < 0.
  *
+ * ozlu_debug_limit_alloc: the library's device allocations of `bytes` or more
+ * fail, as on a device with little free memory; 0 turns it off.  Process-wide.
+ * Returns 0, or -1 for bytes < 0.
+ *
  * ozlu_debug_wait_expiry: runs one of the library's bounded device waits on
  * the handle's stream with a short limit, on a flag or barrier that nothing
  * sets, and then the LU's finish step that turns the error word into info:
@@ -372,6 +376,7 @@ int ozlu_mp_getrs(ozlu_handle* handle, int p, int n, int nrhs, const ozlu_mp_mat
  * ozlu_getrf or ozlu_getrs call clears both error words.
  */
 int ozlu_debug_fail_alloc(int count);
+int ozlu_debug_limit_alloc(long long bytes);
 int ozlu_debug_wait_expiry(ozlu_handle* handle, int which, long long limit, int* out);
 
 /* Version string of the library. */

@@ -18,6 +18,7 @@ int cuda_rc(cudaError_t e) { return e == cudaSuccess ? OZLU_OK : OZLU_ERR_CUDA; 
 
 namespace {
 std::atomic<int> g_fail_allocs{0};  // allocations still to fail (test injection)
+std::atomic<long long> g_alloc_limit{0};  // size from which allocations fail; 0: none (test injection)
 std::mutex g_attr_mutex;
 std::map<std::pair<const void*, int>, int> g_smem_set;  // (kernel, device) -> bytes set
 constexpr int MAX_DEVICES = 64;
@@ -28,6 +29,8 @@ bool dev_alloc(void** p, size_t bytes) {
     *p = nullptr;
     for (int v = g_fail_allocs.load(); v > 0; v = g_fail_allocs.load())
         if (g_fail_allocs.compare_exchange_weak(v, v - 1)) return false;
+    const long long limit = g_alloc_limit.load();
+    if (limit > 0 && bytes >= (size_t)limit) return false;
     if (cudaMalloc(p, bytes) != cudaSuccess) {
         cudaGetLastError();
         *p = nullptr;
@@ -108,6 +111,10 @@ int Workspace::ensure(size_t bytes) {
     }
     cap = want;
     return OZLU_OK;
+}
+
+int ensure_unmoved(const ozlu_handle* h, Workspace& ws, size_t bytes) {
+    return h->capturing && bytes > ws.cap ? RC_WOULD_MOVE : ws.ensure(bytes);
 }
 
 void Workspace::release() {
@@ -309,7 +316,8 @@ int gemm_device(ozlu_handle* h, int nc, int p, int m, int n, int k, int alpha, c
     int mode = be == OZLU_BE_FP8 ? 1 : be == OZLU_BE_FP64 ? 3 : 2;
     int Kpad = 0;
     bool pack = false;
-    auto layout = [&]() -> size_t {
+    auto layout = [&](bool narrow) -> size_t {
+        if (narrow) mode = 0;
         const int P = mode == 1 ? 3 : 1, esz = mode == 2 ? 2 : (mode == 3 ? 8 : 1);
         // K padded to the GEMM's step: 64 elements (INT8, FP16; the binary64 kernel
         // takes any), 128 for FP8 (the accumulator conditions hold for the plan's 128)
@@ -331,14 +339,7 @@ int gemm_device(ozlu_handle* h, int nc, int p, int m, int n, int k, int alpha, c
     memcpy(L.mod, pl->mod, sizeof L.mod);
     int* derr = err_word(h);
     if (!derr) return OZLU_ERR_NOMEM;
-    const size_t bytes = layout();
-    rc = h->ws.ensure(bytes);
-    size_t room = 0, all = 0;
-    if (rc == OZLU_ERR_NOMEM && be == OZLU_BE_INT8 && cudaMemGetInfo(&room, &all) == cudaSuccess && room < bytes) {
-        mode = 0;
-        rc = h->ws.ensure(layout());
-    }
-    if (rc) return rc;
+    if ((rc = fit_workspace(h, be == OZLU_BE_INT8, layout))) return rc;
     const int P = mode == 1 ? 3 : 1;
     char* base = (char*)h->ws.base;
     int* mu = (int*)(base + L.mu);
@@ -431,6 +432,12 @@ const char* ozlu_version(void) { return "ozlu 0.2 (sm_103a)"; }
 int ozlu_debug_fail_alloc(int count) {
     if (count < 0) return -1;
     g_fail_allocs.store(count);
+    return OZLU_OK;
+}
+
+int ozlu_debug_limit_alloc(long long bytes) {
+    if (bytes < 0) return -1;
+    g_alloc_limit.store(bytes);
     return OZLU_OK;
 }
 

@@ -169,6 +169,7 @@ int run_batched(ozlu_handle* h, const std::vector<long long>& key, bool graph,
     const cudaError_t be = cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeRelaxed);
     if (be != cudaSuccess) return fail(be);
     const ozlu_stats before = sub_counters(h);
+    const unsigned long long moves = sub_moves(h);
     h->capturing = true;
     const int rc = issue_on(h->cap_stream);
     h->capturing = false;
@@ -183,6 +184,11 @@ int run_batched(ozlu_handle* h, const std::vector<long long>& key, bool graph,
     const cudaError_t ce = cudaStreamEndCapture(h->cap_stream, &gr);
     if (rc || ce != cudaSuccess || !gr) {
         if (gr) cudaGraphDestroy(gr);
+        if (rc == RC_WOULD_MOVE) {  // a workspace has to grow first: run eagerly, capture the next call
+            cudaGetLastError();
+            h->stats.graph_status = 0;
+            return issue();
+        }
         if (rc) {
             cudaGetLastError();
             return rc;
@@ -193,7 +199,7 @@ int run_batched(ozlu_handle* h, const std::vector<long long>& key, bool graph,
     const cudaError_t ie = cudaGraphInstantiate(&ex, gr, 0);
     cudaGraphDestroy(gr);
     if (ie != cudaSuccess) return fail(ie);
-    h->graphs[key] = {ex, work, 1, sub_moves(h)};
+    h->graphs[key] = {ex, work, 1, moves};
     h->stats.graph_status = 1;
     return cudaGraphLaunch(ex, h->stream) == cudaSuccess ? OZLU_OK : OZLU_ERR_CUDA;
 }

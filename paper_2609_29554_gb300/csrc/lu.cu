@@ -950,7 +950,7 @@ int getrs_device(ozlu_handle* h, int p, int n, int nrhs, double* LU, long long l
         constexpr int W = Limbs<N>::L + 2;
         const size_t rows = (size_t)(n + BASE - 1) / BASE * BASE;
         bool launched = false;
-        rc = h->solve_ws.ensure(2 * sizeof(unsigned long long) * rows * nrhs * W);
+        rc = ensure_unmoved(h, h->solve_ws, 2 * sizeof(unsigned long long) * rows * nrhs * W);
         h->phase(PH_TRSM);
         if (!rc) rc = solve_few<N>(LU, lda, n, B, ldb, nrhs, h->solve_ws.base, h->dev_err, s, &launched);
         if (rc || launched) {

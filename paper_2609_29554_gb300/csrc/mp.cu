@@ -1173,7 +1173,8 @@ int mp_gemm_device(ozlu_handle* h, int p, int m, int n, int k, int alpha, const 
     const size_t tcol = (size_t)pl->G * pl->N * m;
     long long nch = 0;
     size_t o_mu = 0, o_nu = 0, o_ra = 0, o_rb = 0, o_t = 0;
-    auto layout = [&]() -> size_t {
+    auto layout = [&](bool narrower) -> size_t {
+        if (narrower) mode = 0;
         const size_t planesN = (size_t)pl->N * pl->S * P * (mode == 2 ? 2 : 1);  // in bytes an element
         // column chunk: t values of one chunk below 4 GiB and B planes below 2 GiB
         nch = (long long)(((size_t)4 << 30) / (tcol ? tcol : 1));
@@ -1191,14 +1192,7 @@ int mp_gemm_device(ozlu_handle* h, int p, int m, int n, int k, int alpha, const 
         o_t = off;  off = up256(off + tcol * (size_t)nch);
         return off;
     };
-    const size_t bytes = layout();
-    rc = h->ws.ensure(bytes);
-    size_t room = 0, all = 0;
-    if (rc == OZLU_ERR_NOMEM && mode == 2 && cudaMemGetInfo(&room, &all) == cudaSuccess && room < bytes) {
-        mode = 0;
-        rc = h->ws.ensure(layout());
-    }
-    if (rc) return rc;
+    if ((rc = fit_workspace(h, mode == 2, layout))) return rc;
     char* base = (char*)h->ws.base;
     int* mu = (int*)(base + o_mu);
     int* nu = (int*)(base + o_nu);

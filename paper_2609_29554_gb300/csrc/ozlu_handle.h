@@ -54,6 +54,7 @@ struct ozlu_handle {
     ozlu::Workspace nb_ws;  // scratch copy of A for the panel-width autotuner
     std::map<std::tuple<int, int, int, int, int, int>, ozlu::PlanEntry> plans;
     ozlu::GemmLayout last;
+    size_t wide_refused = (size_t)-1;  // smallest workspace with binary16 residues that was not to be had
     int* dev_err = nullptr;  // device error word of the tensor-core GEMMs
     bool clear_err = false;  // the next product starts by zeroing it
     bool timing = false;
@@ -114,5 +115,33 @@ int* err_word(ozlu_handle* h);
 int mp_gemm_device(ozlu_handle* h, int p, int m, int n, int k, int alpha, const ozlu_mp_matrix& A,
                    const ozlu_mp_matrix& B, int beta, const ozlu_mp_matrix& C);
 int clear_err_word(ozlu_handle* h);
+// A capture holds the addresses of its workspaces, so none moves meanwhile: a call
+// that would have to grow one returns this, and the captured call runs eagerly
+constexpr int RC_WOULD_MOVE = -1000;
+int ensure_unmoved(const ozlu_handle* h, Workspace& ws, size_t bytes);
+// The workspace of one product.  layout(narrow) sets the product's offsets and
+// returns the bytes; `either`: its residues can be int8 (narrow) instead of
+// binary16, half the bytes, where those do not fit.  What has been refused once
+// is not asked for again, so that a repeated call neither moves the workspace nor
+// pays for allocations; a workspace never ends smaller than it was.
+template <typename F>
+int fit_workspace(ozlu_handle* h, bool either, F layout) {
+    Workspace& ws = h->ws;
+    size_t bytes = layout(false);
+    if (bytes <= ws.cap) return OZLU_OK;
+    if (either && (h->capturing || bytes >= h->wide_refused)) {
+        bytes = layout(true);
+        either = false;
+    }
+    const size_t had = ws.cap;
+    int rc = ensure_unmoved(h, ws, bytes);
+    if (rc == OZLU_ERR_NOMEM && either) {
+        h->wide_refused = bytes;
+        bytes = layout(true);
+        rc = had > bytes ? ws.ensure(had) : rc;
+        if (rc) rc = ws.ensure(bytes);
+    }
+    return rc;
+}
 int cuda_rc(cudaError_t e);
 }  // namespace ozlu

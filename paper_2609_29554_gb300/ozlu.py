@@ -92,6 +92,7 @@ SIGNATURES = {
     "ozlu_mp_set_opts": (_I, [_P, ctypes.POINTER(ozlu_opts)]),
     "ozlu_mp_plan_opts": (_I, [_I, _I, ctypes.POINTER(ozlu_opts), ctypes.POINTER(ozlu_plan_info)]),
     "ozlu_debug_fail_alloc": (_I, [_I]),
+    "ozlu_debug_limit_alloc": (_I, [_L]),
     "ozlu_debug_wait_expiry": (_I, [_P, _I, _L, _P]),
 }
 
@@ -247,6 +248,10 @@ def ozlu_debug_fetch(h, what, out: np.ndarray):
 
 def ozlu_debug_fail_alloc(count):
     _check("ozlu_debug_fail_alloc", lib().ozlu_debug_fail_alloc(int(count)))
+
+
+def ozlu_debug_limit_alloc(bytes):
+    _check("ozlu_debug_limit_alloc", lib().ozlu_debug_limit_alloc(int(bytes)))
 
 
 def ozlu_debug_wait_expiry(h, which, limit):
