@@ -293,7 +293,9 @@ extern "C" int ozlu_getrs_batched(ozlu_handle* h, int nc, int p, int count, cons
     for (int i = 0; i < count; ++i) {
         key.push_back(n[i]);
         key.push_back((long long)LU[i]);
+        key.push_back(lda[i]);
         key.push_back((long long)B[i]);
+        key.push_back(ldb[i]);
         key.push_back((long long)ipiv[i]);
     }
     const auto lists = assign(count, n);
