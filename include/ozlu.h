@@ -144,6 +144,9 @@ int ozlu_getrf(ozlu_handle* handle, int nc, int p, int n, double* A, long long l
 /*
  * Solve A X = B from ozlu_getrf's factors (P b, forward L, backward U).
  *   LU, ipiv  as returned by ozlu_getrf;  B n x nrhs, overwritten by X.
+ * A bounded device wait that gave up leaves X wrong: with host arguments the call
+ * returns OZLU_ERR_TIMEOUT, otherwise (batched and captured calls too) the error
+ * word has it, ozlu_debug_fetch what = 6.
  */
 int ozlu_getrs(ozlu_handle* handle, int nc, int p, int n, int nrhs,
                const double* LU, long long lda, const int* ipiv,
@@ -189,8 +192,9 @@ int ozlu_getrs_batched(ozlu_handle* handle, int nc, int p, int count, const int*
  *   5 t values      uint8 [gi][l][j][i] (column-major m x n per plane);
  *                   uint32 for the binary64 back-end
  *   6 device error word (int32): 0, or OZLU_ERR_TIMEOUT when a bounded
- *     wait inside a tensor-core GEMM gave up since the start of the last
- *     ozlu_gemm, ozlu_getrf or ozlu_getrs call on this handle
+ *     wait inside a tensor-core GEMM or a solve gave up since the start of the
+ *     last ozlu_gemm, ozlu_getrf, ozlu_getrs (also batched or captured) or p-bit
+ *     call on this handle
  * Residues (3, 4) are available for the INT8 back-end only.
  * bytes must be at least the size of the requested array.
  */
@@ -300,7 +304,8 @@ int ozlu_mp_gemm(ozlu_handle* handle, int p, int m, int n, int k, int alpha, con
  * row interchange, and its scaling by the reciprocal of the pivot (Newton's
  * iteration in fixed point by one thread block).  ipiv (device, n ints,
  * 1-based) and info (device int: 0, or the first exactly zero pivot) as in
- * ozlu_getrf; nb = 0 picks 128.
+ * ozlu_getrf; nb = 0 picks 128.  Waits for the stream, as ozlu_mp_getrs does;
+ * both return OZLU_ERR_TIMEOUT when a bounded device wait gave up.
  */
 int ozlu_mp_getrf(ozlu_handle* handle, int p, int n, const ozlu_mp_matrix* A, int* ipiv, int nb,
                   int* info);
@@ -374,10 +379,16 @@ int ozlu_mp_getrs(ozlu_handle* handle, int p, int n, int nrhs, const ozlu_mp_mat
  * ozlu_getrf does with host arguments), 0 if it did not, -i for an invalid
  * argument i, or OZLU_ERR_CUDA / OZLU_ERR_NOMEM.  The next ozlu_gemm,
  * ozlu_getrf or ozlu_getrs call clears both error words.
+ *
+ * ozlu_debug_wait_limit: from now on a device wait that runs out goes before every
+ * solve (after `limit` ns) and before every wide p-bit product (after `limit`
+ * polls) of the handle, so that the call reports it; 0 turns it off.  Returns 0,
+ * -1 or -2.
  */
 int ozlu_debug_fail_alloc(int count);
 int ozlu_debug_limit_alloc(long long bytes);
 int ozlu_debug_wait_expiry(ozlu_handle* handle, int which, long long limit, int* out);
+int ozlu_debug_wait_limit(ozlu_handle* handle, long long limit);
 
 /* Version string of the library. */
 const char* ozlu_version(void);

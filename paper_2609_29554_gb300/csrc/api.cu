@@ -92,7 +92,15 @@ int* err_word(ozlu_handle* h) {
 int clear_err_word(ozlu_handle* h) {
     int* e = err_word(h);
     if (!e) return OZLU_ERR_NOMEM;
+    h->err_subs = 0;
     return cudaMemsetAsync(e, 0, sizeof(int), h->stream) == cudaSuccess ? OZLU_OK : OZLU_ERR_CUDA;
+}
+
+int finish_call(ozlu_handle* h) {
+    int err = 0;
+    if (h->dev_err && cudaMemcpyAsync(&err, h->dev_err, sizeof err, cudaMemcpyDeviceToHost, h->stream) != cudaSuccess)
+        return OZLU_ERR_CUDA;
+    return cudaStreamSynchronize(h->stream) == cudaSuccess ? err : OZLU_ERR_CUDA;
 }
 
 int Workspace::ensure(size_t bytes) {
@@ -488,6 +496,13 @@ int ozlu_destroy(ozlu_handle* h) {
     return OZLU_OK;
 }
 
+int ozlu_debug_wait_limit(ozlu_handle* h, long long limit) {
+    if (!h) return -1;
+    if (limit < 0) return -2;
+    h->wait_limit = limit;
+    return OZLU_OK;
+}
+
 int ozlu_set_stream(ozlu_handle* h, void* stream) {
     if (!h) return -1;
     h->stream = (cudaStream_t)stream;
@@ -560,6 +575,7 @@ int ozlu_gemm(ozlu_handle* h, int nc, int p, int m, int n, int k, int alpha, con
     if (!err_word(h)) return OZLU_ERR_NOMEM;
     auto product = [&](const double* a, const double* b, double* c) -> int {
         h->clear_err = true;
+        h->err_subs = 0;
         const int rc = gemm_device(h, nc, p, m, n, k, alpha, a, lda, b, ldb, beta, c, ldc, opts);
         const int rc1 = h->clear_err ? clear_err_word(h) : OZLU_OK;
         h->clear_err = false;
@@ -589,7 +605,7 @@ int ozlu_gemm(ozlu_handle* h, int nc, int p, int m, int n, int k, int alpha, con
     rc = product(gA, gB, gC);
     if (rc) return rc;
     if (!dC && cudaMemcpyAsync(C, sC, sizeof(double) * ec, cudaMemcpyDeviceToHost, s)) return OZLU_ERR_CUDA;
-    return cuda_rc(cudaStreamSynchronize(s));
+    return finish_call(h);
 }
 
 int ozlu_debug_fetch(ozlu_handle* h, int what, void* dst, size_t bytes) {
@@ -600,11 +616,15 @@ int ozlu_debug_fetch(ozlu_handle* h, int what, void* dst, size_t bytes) {
     if (what == 6) {
         if (bytes < sizeof(int)) return -4;
         if (cudaStreamSynchronize(h->stream)) return OZLU_ERR_CUDA;
-        if (!h->dev_err) {
-            *(int*)dst = 0;
-            return OZLU_OK;
+        // the handle's own word, or those of the sub-handles that ran its last call
+        int err = 0;
+        for (int k = -1; k < MAX_SUB && !err; ++k) {
+            ozlu_handle* s = k < 0 ? (h->err_subs ? nullptr : h) : (h->err_subs >> k & 1 ? h->sub[k] : nullptr);
+            if (s && s->dev_err && cudaMemcpy(&err, s->dev_err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
+                return OZLU_ERR_CUDA;
         }
-        return cuda_rc(cudaMemcpy(dst, h->dev_err, sizeof(int), cudaMemcpyDeviceToHost));
+        *(int*)dst = err;
+        return OZLU_OK;
     }
     if (!base) return OZLU_ERR_CAPACITY;
     if (cudaStreamSynchronize(h->stream)) return OZLU_ERR_CUDA;

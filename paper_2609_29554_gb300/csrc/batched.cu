@@ -61,6 +61,15 @@ std::vector<std::vector<int>> assign(int count, const int* n) {
     return lists;
 }
 
+// the sub-handles (bits) on which instances run
+uint32_t used_subs(const std::vector<std::vector<int>>& lists, const int* n) {
+    static_assert(NSUB <= 32, "a bit each");
+    uint32_t m = 0;
+    for (int k = 0; k < NSUB; ++k)
+        if (!lists[k].empty() && n[lists[k][0]] > 0) m |= 1u << k;  // (largest first)
+    return m;
+}
+
 // fork from `root` onto the sub-streams, issue the instances round-robin
 // (one instance per stream in turn, so that a full launch queue never holds
 // one stream's work alone), then join every forked stream back into `root`
@@ -74,6 +83,7 @@ int fork_join(ozlu_handle* h, cudaStream_t root, const std::vector<std::vector<i
         if (cudaStreamWaitEvent(s->stream, h->fork, 0) != cudaSuccess) return OZLU_ERR_CUDA;
         s->capturing = h->capturing;
         s->timing = h->timing && !h->capturing;
+        s->wait_limit = h->wait_limit;
         rounds = std::max(rounds, lists[k].size());
     }
     int rc = OZLU_OK;
@@ -254,6 +264,7 @@ extern "C" int ozlu_getrf_batched(ozlu_handle* h, int nc, int p, int count, cons
         }
     }
     const auto lists = assign(count, n);
+    h->err_subs = used_subs(lists, n);
     // concurrent instances take fewer SMs per panel (32 rows per block at least;
     // 256 TD instances: 576 ms against 643 ms with 16); a single instance keeps 8
     for (int k = 0; k < NSUB; ++k) h->sub[k]->coop_min_rows = count > 1 ? 32 : 8;
@@ -299,10 +310,15 @@ extern "C" int ozlu_getrs_batched(ozlu_handle* h, int nc, int p, int count, cons
         key.push_back((long long)ipiv[i]);
     }
     const auto lists = assign(count, n);
+    // a stream's error word is cleared by its first instance and then kept
+    std::vector<char> first(count, 0);
+    for (const auto& l : lists)
+        if (!l.empty()) first[l[0]] = 1;
+    h->err_subs = used_subs(lists, n);
     auto issue = [&](cudaStream_t root) -> int {
         return fork_join(h, root, lists, [&](ozlu_handle* s, int i) -> int {
             if (n[i] == 0) return (int)OZLU_OK;
-            return getrs_one(s, nc, p, n[i], nrhs, LU[i], lda[i], ipiv[i], B[i], ldb[i], &o);
+            return getrs_one(s, nc, p, n[i], nrhs, LU[i], lda[i], ipiv[i], B[i], ldb[i], &o, first[i]);
         });
     };
     return run_batched(h, key, o.graph != 0, issue);

@@ -707,6 +707,15 @@ void laswp_all(double* B, long long ldb, int nrhs, int n, const int* ipiv, int* 
     for (int k0 = 0; k0 < n; k0 += LMAXB) laswp2<N>(B, ldb, 0, nrhs, 0, 0, k0, k0 + LMAXB < n ? k0 + LMAXB : n, ipiv, list, s);
 }
 
+// Self-test of the panel kernel's bounded wait: one thread waits with
+// wait_stamp for a stamp that nothing writes (a zeroed word, column 1), with a
+// short limit, into the panel's own error word; out[0] = 1 if it gave up.
+__global__ void stamp_expiry_selftest_kernel(const unsigned long long* word, unsigned long long limit_ns,
+                                             int* err, int* out) {
+    if (threadIdx.x != 0) return;
+    out[0] = wait_stamp(word, 1u, err, limit_ns) == 0 ? 1 : 0;
+}
+
 // both substitutions for nrhs <= SOLVE_RHS.  *launched stays false when the
 // kernel cannot be launched here (the caller then takes the blocked form)
 template <int N>
@@ -942,6 +951,9 @@ int getrs_device(ozlu_handle* h, int p, int n, int nrhs, double* LU, long long l
     // options that no plan of the updates meets are refused whichever form runs
     const int refused = n > BASE ? check_plan(h, p, BASE, opts) : OZLU_OK;
     if (refused) return refused;
+    if (h->wait_limit)  // test hook: a wait that runs out, on a word that nothing writes
+        stamp_expiry_selftest_kernel<<<1, 32, 0, s>>>((const unsigned long long*)(h->dev_err + 8), (unsigned long long)h->wait_limit,
+                                                       h->dev_err, h->dev_err + 1);
     h->phase(PH_OTHER);
     laswp_all<N>(B, ldb, nrhs, n, ipiv, sc->plist, s);
     h->count(2 * ((n + LMAXB - 1) / LMAXB));
@@ -1000,14 +1012,6 @@ __global__ void finish_kernel(int* info_out, const LuScratch* sc, const int* coo
     *info_out = v;
 }
 
-// Self-test of the panel kernel's bounded wait: one thread waits with
-// wait_stamp for a stamp that nothing writes (a zeroed word, column 1), with a
-// short limit, into the panel's own error word; out[0] = 1 if it gave up.
-__global__ void stamp_expiry_selftest_kernel(const unsigned long long* word, unsigned long long limit_ns,
-                                             int* err, int* out) {
-    if (threadIdx.x != 0) return;
-    out[0] = wait_stamp(word, 1u, err, limit_ns) == 0 ? 1 : 0;
-}
 }  // namespace
 
 int launch_mbar_expiry_selftest(long long limit, int* err, int* out, cudaStream_t s);
@@ -1079,11 +1083,11 @@ int getrf_one(ozlu_handle* h, int nc, int p, int n, double* A, long long lda, in
 }
 
 int getrs_one(ozlu_handle* h, int nc, int p, int n, int nrhs, const double* LU, long long lda, const int* ipiv,
-              double* B, long long ldb, const ozlu_opts* opts) {
+              double* B, long long ldb, const ozlu_opts* opts, bool clear) {
     LuScratch* sc;
     int rc = lu_scratch(h, &sc);
     if (rc) return rc;
-    if ((rc = clear_err_word(h))) return rc;
+    if (clear && (rc = clear_err_word(h))) return rc;
     switch (nc) {
         case 2: return getrs_device<2>(h, p, n, nrhs, (double*)LU, lda, ipiv, B, ldb, opts, sc);
         case 3: return getrs_device<3>(h, p, n, nrhs, (double*)LU, lda, ipiv, B, ldb, opts, sc);
@@ -1314,6 +1318,6 @@ extern "C" int ozlu_getrs(ozlu_handle* h, int nc, int p, int n, int nrhs, const 
     }
     if (rc) return rc;
     if (!dB && cudaMemcpyAsync(B, gB, bbytes, cudaMemcpyDeviceToHost, s)) return OZLU_ERR_CUDA;
-    if (!dL || !dP || !dB) return cuda_rc(cudaStreamSynchronize(s));
+    if (!dL || !dP || !dB) return finish_call(h);
     return OZLU_OK;
 }

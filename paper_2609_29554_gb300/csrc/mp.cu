@@ -64,11 +64,13 @@ __device__ __forceinline__ uint32_t mant32(const MPView& X, long long x, long lo
 // (S1) of both operands in one launch: blocks [0, blocks_a) take 32 rows of A
 // each (32 warps share the columns), the others 32 columns of B, one a warp.
 // Four elements in flight per thread; one thread walking a whole row took
-// about a load latency per element.
+// about a load latency per element.  `clear` (may be null): the device error word,
+// zeroed for a new call.
 __global__ void __launch_bounds__(1024) mp_shift_kernel(MPView A, int m, MPView B, int n, int k, int Q, int* mu,
-                                                         int* nu, int blocks_a) {
+                                                         int* nu, int blocks_a, int* clear) {
     chain_enter();
     __shared__ int red[32][33];
+    if (clear && blockIdx.x == 0 && threadIdx.x == 0) *clear = 0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int E = INT_MIN;
     if ((int)blockIdx.x < blocks_a) {
@@ -1046,7 +1048,7 @@ int mp_gemm_ext(ozlu_handle* h, int p, int S, int m, int n, int k, int alpha, co
     const int prev = h->open_phase;
     h->phase(PH_CONVERT);
     const int ba = (m + 31) / 32, bb = (n + 31) / 32;
-    launch(mp_shift_kernel, ba + bb, 1024, 0, s, vA, m, vB, n, k, pl->Q, mu, nu, ba);
+    launch(mp_shift_kernel, ba + bb, 1024, 0, s, vA, m, vB, n, k, pl->Q, mu, nu, ba, nullptr);
     mp_convert_ext(vA, m, k, 0, mu, E, Kpad, Mpad, RA, s);
     h->count(2);
     for (long long j0 = 0; j0 < n; j0 += nch) {
@@ -1071,6 +1073,7 @@ int mp_gemm_ext(ozlu_handle* h, int p, int S, int m, int n, int k, int alpha, co
 
 int mp_gemm_device(ozlu_handle* h, int p, int m, int n, int k, int alpha, const ozlu_mp_matrix& A,
                    const ozlu_mp_matrix& B, int beta, const ozlu_mp_matrix& C);
+int launch_mbar_expiry_selftest(long long limit, int* err, int* out, cudaStream_t s);
 
 // INT8 (as binary16 products) or FP8 residues for a wide p-bit product, by
 // measurement: both run the same plan (identical results) into a scratch C,
@@ -1206,7 +1209,9 @@ int mp_gemm_device(ozlu_handle* h, int p, int m, int n, int k, int alpha, const 
     h->phase(PH_CONVERT);
     {
         const int nc0 = (int)(n < nch ? n : nch), ba = (m + 31) / 32, bb = (n + 31) / 32;
-        launch(mp_shift_kernel, ba + bb, 1024, 0, s, vA, m, vB, n, k, pl->Q, mu, nu, ba);
+        launch(mp_shift_kernel, ba + bb, 1024, 0, s, vA, m, vB, n, k, pl->Q, mu, nu, ba, h->clear_err ? h->dev_err : nullptr);
+        h->clear_err = false;
+        if (mode && h->wait_limit && (rc = launch_mbar_expiry_selftest(h->wait_limit, derr, derr + 1, s))) return rc;
         mp_convert(vA, m, vB, nc0, k, mu, nu, pe->conv, Kpad, Mpad, (nc0 + rowq - 1) / rowq * rowq, RA, RB, mode, s);
     }
     h->count(2);
@@ -1282,5 +1287,12 @@ extern "C" int ozlu_mp_gemm(ozlu_handle* h, int p, int m, int n, int k, int alph
     if (beta != 0 && beta != 1) return -9;
     if (!mp_valid(C, p, m, n)) return -10;
     if (cudaSetDevice(h->device) != cudaSuccess) return OZLU_ERR_CUDA;
-    return mp_gemm_device(h, p, m, n, k, alpha, *A, *B, beta, *C);
+    // the product's first kernel clears the error word, or this where none runs
+    if (!err_word(h)) return OZLU_ERR_NOMEM;
+    h->clear_err = true;
+    h->err_subs = 0;
+    const int rc = mp_gemm_device(h, p, m, n, k, alpha, *A, *B, beta, *C);
+    const int rc1 = h->clear_err ? clear_err_word(h) : OZLU_OK;
+    h->clear_err = false;
+    return rc ? rc : rc1;
 }

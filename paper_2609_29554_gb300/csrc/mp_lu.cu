@@ -454,6 +454,7 @@ extern "C" int ozlu_mp_getrf(ozlu_handle* h, int p, int n, const ozlu_mp_matrix*
     if (n == 0) return OZLU_OK;
     Scratch sc;
     int rc = sc.alloc(A->L, n);
+    if (!rc) rc = clear_err_word(h);
     if (rc) return rc;
     Ctx c{h, p, *A, n, ipiv, info, &sc};
     for (int r0 = 0; r0 < n && !c.rc; r0 += nb) {
@@ -472,7 +473,7 @@ extern "C" int ozlu_mp_getrf(ozlu_handle* h, int p, int n, const ozlu_mp_matrix*
                                       1, sub(c.A, r0 + b, r0 + b));
         }
     }
-    if (!c.rc && cudaStreamSynchronize(s) != cudaSuccess) c.rc = OZLU_ERR_CUDA;
+    if (!c.rc) c.rc = finish_call(h);
     return c.rc;
 }
 
@@ -490,12 +491,13 @@ extern "C" int ozlu_mp_getrs(ozlu_handle* h, int p, int n, int nrhs, const ozlu_
     cudaStream_t s = h->stream;
     Scratch sc;
     int rc = sc.alloc(B->L, nrhs > n ? nrhs : n);
+    if (!rc) rc = clear_err_word(h);
     if (rc) return rc;
     Ctx c{h, p, *LU, n, const_cast<int*>(ipiv), nullptr, &sc};
     launch(mp_laswp_kernel, dim3((nrhs + 127) / 128, B->L + 2), 128, 0, s, dv(*B), 0, n, ipiv, 0, nrhs);
     h->count(1);
     mp_trsm_lower(c, *LU, 0, n, *B, 0, 0, nrhs);
     mp_trsm_upper(c, *LU, 0, n, *B, 0, 0, nrhs);
-    if (!c.rc && cudaStreamSynchronize(s) != cudaSuccess) c.rc = OZLU_ERR_CUDA;
+    if (!c.rc) c.rc = finish_call(h);
     return c.rc;
 }

@@ -57,6 +57,8 @@ struct ozlu_handle {
     size_t wide_refused = (size_t)-1;  // smallest workspace with binary16 residues that was not to be had
     int* dev_err = nullptr;  // device error word of the tensor-core GEMMs
     bool clear_err = false;  // the next product starts by zeroing it
+    uint32_t err_subs = 0;   // sub-handles whose error words stand for it (a batched or captured call)
+    long long wait_limit = 0;  // test hook: ozlu_debug_wait_limit
     bool timing = false;
     ozlu_stats stats = {};
     void* lu_scratch = nullptr;  // pivot-search scratch of ozlu_getrf
@@ -105,7 +107,7 @@ int getrf_one(ozlu_handle* h, int nc, int p, int n, double* A, long long lda, in
 int tune_nb(ozlu_handle* h, int nc, int p, int n, const double* A, long long lda, const ozlu_opts* opts,
             int* nb_out);
 int getrs_one(ozlu_handle* h, int nc, int p, int n, int nrhs, const double* LU, long long lda, const int* ipiv,
-              double* B, long long ldb, const ozlu_opts* opts);
+              double* B, long long ldb, const ozlu_opts* opts, bool clear);
 int check_plan(ozlu_handle* h, int p, int K, const ozlu_opts* opts);
 int gemm_device(ozlu_handle* h, int nc, int p, int m, int n, int k, int alpha, const double* A,
                 long long lda, const double* B, long long ldb, int beta, double* C,
@@ -115,6 +117,9 @@ int* err_word(ozlu_handle* h);
 int mp_gemm_device(ozlu_handle* h, int p, int m, int n, int k, int alpha, const ozlu_mp_matrix& A,
                    const ozlu_mp_matrix& B, int beta, const ozlu_mp_matrix& C);
 int clear_err_word(ozlu_handle* h);
+// waits for the handle's stream; OZLU_ERR_TIMEOUT if a bounded device wait of the
+// call gave up
+int finish_call(ozlu_handle* h);
 // A capture holds the addresses of its workspaces, so none moves meanwhile: a call
 // that would have to grow one returns this, and the captured call runs eagerly
 constexpr int RC_WOULD_MOVE = -1000;

@@ -94,6 +94,7 @@ SIGNATURES = {
     "ozlu_debug_fail_alloc": (_I, [_I]),
     "ozlu_debug_limit_alloc": (_I, [_L]),
     "ozlu_debug_wait_expiry": (_I, [_P, _I, _L, _P]),
+    "ozlu_debug_wait_limit": (_I, [_P, _L]),
 }
 
 
@@ -259,6 +260,10 @@ def ozlu_debug_wait_expiry(h, which, limit):
     out = np.zeros(3, dtype=np.int32)
     rc = lib().ozlu_debug_wait_expiry(h, which, int(limit), out.ctypes.data)
     return rc, tuple(int(v) for v in out)
+
+
+def ozlu_debug_wait_limit(h, limit):
+    _check("ozlu_debug_wait_limit", lib().ozlu_debug_wait_limit(h, int(limit)))
 
 
 def ozlu_set_timing(h, enable):
