@@ -324,6 +324,7 @@ int gemm_device(ozlu_handle* h, int nc, int p, int m, int n, int k, int alpha, c
     int mode = be == OZLU_BE_FP8 ? 1 : be == OZLU_BE_FP64 ? 3 : 2;
     int Kpad = 0;
     bool pack = false;
+    double residue_bytes = 0.0, t_bytes = 0.0;  // of the layout, for the counters
     auto layout = [&](bool narrow) -> size_t {
         if (narrow) mode = 0;
         const int P = mode == 1 ? 3 : 1, esz = mode == 2 ? 2 : (mode == 3 ? 8 : 1);
@@ -342,6 +343,8 @@ int gemm_device(ozlu_handle* h, int nc, int p, int m, int n, int k, int alpha, c
         const size_t tval = pack ? 4 * (size_t)pe->gemm.NT : (size_t)pl->N * (mode == 3 ? 4 : 1);
         L.t = off;  off = align_up(off + (size_t)pl->G * tval * m * n);
         L.pack = pack;
+        residue_bytes = (double)pl->N * pl->S * P * ((double)Mpad + Npad) * Kpad * esz;
+        t_bytes = (double)pl->G * tval * m * n;
         return off;
     };
     memcpy(L.mod, pl->mod, sizeof L.mod);
@@ -383,9 +386,8 @@ int gemm_device(ozlu_handle* h, int nc, int p, int m, int n, int k, int alpha, c
     h->stats.last_backend = be;
     h->stats.last_nslice = pl->S;
     h->stats.gemm_ops += 2.0 * m * n * (double)k * pl->N * pl->pair_terms * P;
-    h->stats.crt_bytes += (double)pl->G * pl->N * m * n + 8.0 * nc * m * n * (beta ? 2 : 1);
-    h->stats.convert_bytes += 8.0 * nc * ((double)m * k + (double)k * n) +
-                              (double)pl->N * pl->S * ((double)Mpad + Npad) * Kpad;
+    h->stats.crt_bytes += t_bytes + 8.0 * nc * m * n * (beta ? 2 : 1);
+    h->stats.convert_bytes += 8.0 * nc * ((double)m * k + (double)k * n) + residue_bytes;
     h->count(mode == 3 ? 5 : 4);
     if (cudaGetLastError() != cudaSuccess) return OZLU_ERR_CUDA;
     return OZLU_OK;
