@@ -231,8 +231,10 @@ def main_pbit(a, rank, world, local, ozlu, torch):
     flops = 2.0 * n ** 3 / 3.0
     value = job_value(flops, world, ms_max)
     achieved = st.gemm_ops / (st.gemm_ms * 1e-3) / 1e12 if st.gemm_ms else 0.0
-    rf = {"kernel": "gemm_imma_kernel", "bound": "tensor", "achieved": achieved, "peak": IMMA_PEAK,
-          "unit": "TOPS", "peak_source": "own mma.sync s8 probe", "frac": achieved / IMMA_PEAK,
+    # (nearly all operations are in the wide products, on the tensor-core kernel)
+    peaks, src = measured_peaks()
+    rf = {"kernel": "gemm_tc05_kernel", "bound": "tensor", "achieved": achieved, "peak": peaks["bf16_tflops"],
+          "unit": "TFLOP/s", "peak_source": src, "frac": achieved / peaks["bf16_tflops"],
           "traffic": None, "phase_ms_per_step": {k: v / a.steps for k, v in r["phases"].items()},
           "note": "phase events over the timed steps (eager calls)"}
     line = {"metric": METRIC, "value": value, "unit": "Gflop/s", "n_gpus": world, "steps": a.steps,
@@ -432,31 +434,27 @@ def run_reference(a):
 
 # ------------------------------------------------------------------ roofline --
 # Peaks for the integer and binary64 pipes come from this repository's own
-# probes on a GB300 (register-only loops): IMAD 18.9 T/s,
-# mma.sync s8 151.6 TOPS.  Tensor-core peaks scale the measured bf16 number
-# by the nominal ratios (fp8 = 2x, fp16 = 1x).
+# probe on a GB300 (register-only loops): IMAD 18.9 T/s.  Tensor-core peaks scale
+# the measured bf16 number by the nominal ratios (fp8 = 2x, fp16 = 1x).
 IMAD_PEAK = 18.9        # T IMAD/s
-IMMA_PEAK = 151.6       # TOPS (mma.sync s8)
 # DRAM bytes (read + write) per launch of the cooperative panel kernel, the
 # mean over the base-block launches of one factorisation (dram__bytes_read.sum
-# + dram__bytes_write.sum from one ncu capture, profiles/; taken at n = 2048,
-# where the traffic is 0.56 MB + 5.12 KB per row of the base block, and scaled
-# to the 2112 rows of an average n = 4096 launch), keyed by (n, nc, nb, panel
-# width), with the digest of the kernel source the counters were taken on: a
-# changed kernel reports null until it is captured again
-PANEL_TRAFFIC = {(4096, 4, 256, 0): (11.36e6, "bbd712b36bcf70cf")}
+# + dram__bytes_write.sum from one ncu capture, profiles/; taken at
+# n = 2048, where the traffic is 0.12 MB + 4.15 KB per row of the base block, and
+# scaled to the 2112 rows of an average n = 4096 launch), keyed by (n, nc, nb,
+# panel width), with the digest of the kernel source the counters were taken on:
+# a changed kernel reports null until it is captured again
+PANEL_TRAFFIC = {(4096, 4, 256, 0): (8.88e6, "32f3b78dad5d7153")}
 PBASE = 128     # widest base block of the cooperative panel kernel
 
 
 def panel_source_digest():
     """sha256 (16 hex digits) of the panel kernel's source: the text of
-    base_block_coop_kernel in lu.cu and the multi-limb arithmetic it uses."""
+    base_block_coop_kernel in panel.cuh and the multi-limb arithmetic it uses."""
     import hashlib
     csrc = os.path.join(ROOT, "paper_2609_29554_gb300", "csrc")
-    lu = open(os.path.join(csrc, "lu.cu")).read()
-    i = lu.find("base_block_coop_kernel(")
-    j = lu.find("// Apply interchanges", i)
-    body = lu[i:j] if i >= 0 and j > i else lu
+    panel = open(os.path.join(csrc, "panel.cuh")).read()
+    body = panel[panel.index("base_block_coop_kernel("):]
     mpf = open(os.path.join(csrc, "mpf.cuh")).read()
     return hashlib.sha256((body + mpf).encode()).hexdigest()[:16]
 

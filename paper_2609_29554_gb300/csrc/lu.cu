@@ -582,10 +582,19 @@ void trsm_base(const double* T, long long ldt, double* X, long long ldx, int b, 
 // side, issue from different schedulers: on one, three took 1940 cycles a step.
 // The upper triangle is scaled by the reciprocals of its diagonal beforehand (a
 // zero pivot gives 0), so that both directions have unit steps.
-// n = 1500, 3 right-hand sides: QD 2.05 ms, DD 1.43.  By base triangles of 32
-// rows and an Ozaki-II GEMM after each, the form kept above SOLVE_RHS: 7.2 and
-// 5.1, hardly depending on nrhs; here 16 take 5.3 and 3.3, and two rounds of 16
-// would be slower than that form.
+// The other form, kept above SOLVE_RHS: base triangles of 32 rows and an Ozaki-II
+// GEMM after each, its time hardly depending on nrhs.  Milliseconds, here / there,
+// for 1, 8, 9 and 16 right-hand sides:
+//   QD n =   256   0.42 / 0.81   0.58 / 0.82   0.78 / 0.83   0.96 / 0.83
+//      n =  1024   1.6 / 3.6     2.2 / 3.6     3.2 / 3.6     3.9 / 3.6
+//      n =  4096   5.7 / 17.9    8.2 / 18.1   11.4 / 18.1   14.3 / 18.5
+//      n = 16384  22.8 / 130    51 / 133      75 / 134      94 / 140
+//   DD n =   256   0.31 / 0.59   0.39 / 0.59   0.52 / 0.59   0.62 / 0.60
+//      n =  4096   4.1 / 12.2    5.3 / 12.3    7.3 / 12.3    8.9 / 12.6
+// so 13 to 16 lose up to a sixth below n = 1500 or so.  They take it all the same:
+// X is rounded to expansions once per direction, not after every 32 rows, and the
+// mean error is 3 to 50 times smaller (n = 60 to 1500), the largest one too.  Two
+// rounds of 16 would be slower than the other form.
 constexpr int SOLVE_RHS = 16;
 constexpr int SOLVE_BUF = 3;
 constexpr int SOLVE_PART = 8;  // rows announced together
@@ -763,7 +772,10 @@ bool base_block_coop(double* A, long long lda, int n, int c0, int b, int* ipiv, 
     // updates beside the chain, more leave fewer keys to read: QD n = 1000, 6.59 ms
     // with 6 rows, 6.61 with 8, 6.91 with 12, 7.40 with 16, 9.7 with 32.  The batched
     // driver runs instances side by side and asks for 32 (48 uneven TD systems from
-    // CUDA graphs 21.3 ms, with 24 rows 22.2), single factorisations for 8.
+    // CUDA graphs 21.3 ms, with 24 rows 22.2), single factorisations for 8.  A program
+    // that factors on several handles at once is served less well by 8: milliseconds
+    // per QD factorisation on 1, 2, 4 and 8 streams, n = 300 1.63, 0.85, 0.48, 0.39 (16
+    // rows: 1.87, 0.96, 0.51, 0.30), n = 1000 6.2, 4.0, 3.9, 3.9 (7.1, 3.9, 2.7, 2.6).
     const int g_rows = (n - c0 + min_rows - 1) / min_rows;
     for (int per_sm = 1; per_sm <= 2; ++per_sm) {
         int G = sms * per_sm;

@@ -5,7 +5,7 @@
 // exact (or sticky-truncated) result to L words, round to nearest even.
 // The arithmetic runs on the integer pipes (IMAD), which on GB300 issue
 // about 40 times the binary64 FMA rate; the LU panel uses it for DD/TD/QD
-// elements at 32 L >= 53 nc + 22 bits and converts to and from the
+// elements at 32 L >= 53 nc + 12 bits and converts to and from the
 // expansion format (successive round-to-nearest on the way out).
 #pragma once
 
@@ -451,12 +451,10 @@ __device__ __forceinline__ MPF<L> mpf_fms(const MPF<L>& c, const MPF<L>& a, cons
     return mpf_round<L, W>(A, ea, an, sticky);
 }
 
-// Out-of-line copies of the fused multiply-subtract and the product.  A kernel
-// whose warps run several of them at once on different code paths (the LU
-// panel) then keeps one copy of each in the instruction cache instead of one
-// per call site.  The fused multiply-subtract takes its operands and returns
-// its result by value (in registers); the product works on operands in
-// memory (shared memory in the panel), by address.
+// An out-of-line copy of the fused multiply-subtract.  A kernel whose warps run
+// several at once on different code paths (the LU panel) then keeps one copy in the
+// instruction cache instead of one per call site.  Operands and result go by
+// value, in registers.
 template <int L>
 __device__ __noinline__ MPF<L> mpf_fms_oolv(MPF<L> c, MPF<L> a, MPF<L> b) {
     return mpf_fms<L>(c, a, b);

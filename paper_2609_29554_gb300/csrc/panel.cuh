@@ -52,9 +52,9 @@ __device__ __forceinline__ double* elem(double* A, long long lda, int nc, long l
 // need of column kc.  The words are zeroed before every factorisation and tags are
 // column numbers, so a stale word never matches.
 //
-// Measured, QD panels of the n = 1000 / 4096 LU (nb = 256): 5.2 / 23.8 ms, from 13.0 /
-// 58.7 ms with a stamp over a fenced row and the exchange, the reciprocal and the
-// multipliers on the same warp in turn (5.0 against 13 us a column at n = 1000).
+// Measured, QD panels of the n = 1000 / 4096 LU (nb = 256): 4.2 / 21.6 ms (4.2 us a
+// column at n = 1000), from 13.0 / 58.7 ms with a stamp over a fenced row and the
+// exchange, the reciprocal and the multipliers on the same warp in turn.
 //
 // The interchanges of the columns outside the base block are applied once,
 // after the last column, as one permutation (laswp2; by one thread per column
